@@ -299,50 +299,136 @@ __device__ __noinline__ int riemann_jac(double g, double rl, double ul, double p
 }
 
 // ------------------------------------------------------------------ face flux adjoints
+// Cotangents (rho, u, p)_L, (rho, u, p)_R of the Riemann solution for the
+// cotangents (rb, ub, pb) of the face state, by the six-tangent Jacobian, and
+// the side; out of line, by value: the faces that near_riemann hands back.
+struct RFaceVjp {
+  double rho, u, p, b[6];
+  int side;
+  unsigned status;
+};
+struct FluxCot {  // cotangent of the flux in face order: mass, normal and transverse momenta, energy
+  double m, n, t1, t2, e;
+};
+// Cotangents of the face state's own values, F = (m, m u + p, m ut1, m ut2,
+// H u) with m = rho u, H = rho K + g / (g - 1) p, K = |v|^2 / 2.
+__device__ __forceinline__ void flux_state_vjp(double g_gm1, double rho, double u, double p, double ut1, double ut2,
+                                               const FluxCot& F, double& rb, double& ub, double& pb, double& ut1b,
+                                               double& ut2b) {
+  const double m = rho * u, K = 0.5 * fma(u, u, fma(ut1, ut1, ut2 * ut2));
+  const double mb = fma(F.e, K, fma(F.n, u, fma(F.t1, ut1, fma(F.t2, ut2, F.m))));  // d/dm, with H u = m K + g/(g-1) p u
+  const double Fm = F.e * m, Fp = F.e * g_gm1;
+  rb = mb * u;
+  ub = fma(F.n, m, fma(Fp, p, fma(Fm, u, mb * rho)));
+  pb = fma(Fp, u, F.n);
+  ut1b = fma(F.t1, m, Fm * ut1);
+  ut2b = fma(F.t2, m, Fm * ut2);
+}
+static __device__ __noinline__ RFaceVjp riemann_vjp_general(double g, double rl, double ul, double pl, double l1,
+                                                            double l2, double rr, double ur, double pr, double r1,
+                                                            double r2, const FluxCot F) {
+  RFaceVjp o;
+  o.status = 0;
+  J6 Rs, Us, Ps;
+  o.side = g == 1.4 ? riemann_jac<true>(g, rl, ul, pl, rr, ur, pr, Rs, Us, Ps, o.status)
+                    : riemann_jac<false>(g, rl, ul, pl, rr, ur, pr, Rs, Us, Ps, o.status);
+  o.rho = Rs.v;
+  o.u = Us.v;
+  o.p = Ps.v;
+  double rb, ub, pb, t1b, t2b;
+  const double ut1 = o.side < 0 ? l1 : (o.side > 0 ? r1 : 0.0), ut2 = o.side < 0 ? l2 : (o.side > 0 ? r2 : 0.0);
+  flux_state_vjp(g / (g - 1.0), o.rho, o.u, o.p, ut1, ut2, F, rb, ub, pb, t1b, t2b);
+#pragma unroll
+  for (int q = 0; q < 6; ++q) o.b[q] = rb * Rs.d[q] + ub * Us.d[q] + pb * Ps.d[q];
+  return o;
+}
+
 // Cotangents of the primitive face states (u, v, w, P, rho in the field
-// slots) for a cotangent Fb on the gas flux gas_face_flux<D>(WL, WR).
+// slots) for a cotangent Fb on the gas flux F(WL, WR) of gas_face_flux.
+//
+// Near p_K the reverse of the star state is closed: with f_K = x p_K irc_K
+// S(x), df_K/drho_K = -f_K / (2 rho_K) at fixed p* and p_K (f ~ rho^-1/2) and
+// p* f_K' + p_K df_K/dp_K = f_K / 2 (f has the dimension of (p/rho)^1/2), and
+// the cotangent of p* passes to the side states through f_L + f_R + u_R - u_L
+// = 0.  About 40 FP64 operations after the forward's 55, where six tangents
+// carried through the solution took over a thousand.
 template <int D>
-__device__ __noinline__ void gas_flux_vjp(double g, const double* WL, const double* WR, const double* Fb, double* WLb,
-                                          double* WRb, unsigned& status) {
+__device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL, const double* WR, const double* Fb,
+                                             double* WLb, double* WRb, unsigned& status) {
   constexpr int n = Axes<D>::n, t1 = Axes<D>::t1, t2 = Axes<D>::t2;
 #pragma unroll
   for (int f = 0; f < 5; ++f) WLb[f] = WRb[f] = 0.0;
   const double rl = WL[RHO], rr = WR[RHO], pl = WL[EN], pr = WR[EN];
-  if (!(rl > 0.0) || !(rr > 0.0) || !(pl > 0.0) || !(pr > 0.0)) return;  // zero flux
-  J6 Rs, Us, Ps;
-  const int side = g == 1.4 ? riemann_jac<true>(g, rl, WL[n], pl, rr, WR[n], pr, Rs, Us, Ps, status)
-                            : riemann_jac<false>(g, rl, WL[n], pl, rr, WR[n], pr, Rs, Us, Ps, status);
-  double ut1 = 0.0, ut2 = 0.0;
-  if (side < 0) { ut1 = WL[t1]; ut2 = WL[t2]; }
-  else if (side > 0) { ut1 = WR[t1]; ut2 = WR[t2]; }
-  const double rho = Rs.v, u = Us.v, p = Ps.v;
-  const double m = rho * u;
-  const double K = 0.5 * (u * u + ut1 * ut1 + ut2 * ut2);
-  const double H = rho * K + p / (g - 1.0) + p;
-  const double FE = Fb[EN];
-  // F = (m, m u + p, m ut1, m ut2, H u) in (RHO, n, t1, t2, EN)
-  const double mb = Fb[RHO] + Fb[n] * u + Fb[t1] * ut1 + Fb[t2] * ut2;
-  const double ub = Fb[n] * m + FE * (H + u * rho * u) + mb * rho;
-  const double rb = FE * u * K + mb * u;
-  const double pb = Fb[n] + FE * u * (1.0 / (g - 1.0) + 1.0);
-  const double ut1b = Fb[t1] * m + FE * u * rho * ut1;
-  const double ut2b = Fb[t2] * m + FE * u * rho * ut2;
-  double w[6];
-#pragma unroll
-  for (int q = 0; q < 6; ++q) w[q] = rb * Rs.d[q] + ub * Us.d[q] + pb * Ps.d[q];
-  WLb[RHO] = w[0];
-  WLb[n] = w[1];
-  WLb[EN] = w[2];
-  WRb[RHO] = w[3];
-  WRb[n] = w[4];
-  WRb[EN] = w[5];
-  if (side < 0) {
-    WLb[t1] = ut1b;
-    WLb[t2] = ut2b;
-  } else if (side > 0) {
-    WRb[t1] = ut1b;
-    WRb[t2] = ut2b;
+  if (!positive(rl) || !positive(rr) || !positive(pl) || !positive(pr)) return;  // zero flux
+  const FluxCot F{Fb[RHO], Fb[n], Fb[t1], Fb[t2], Fb[EN]};
+  const double dP = pr - pl;
+  NearStar<double> s;
+  const int kind = near_riemann<double>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, narrow(WL[n]),
+                                        narrow(WR[n]), s);
+  if (kind == NEAR_GENERAL) {
+    const RFaceVjp o = riemann_vjp_general(C.gamma, rl, WL[n], pl, WL[t1], WL[t2], rr, WR[n], pr, WR[t1], WR[t2], F);
+    status |= o.status;
+    WLb[RHO] = o.b[0];
+    WLb[n] = o.b[1];
+    WLb[EN] = o.b[2];
+    WRb[RHO] = o.b[3];
+    WRb[n] = o.b[4];
+    WRb[EN] = o.b[5];
+    const double m = o.rho * o.u, Fm = F.e * m;
+    if (o.side < 0) {
+      WLb[t1] = F.t1 * m + Fm * WL[t1];
+      WLb[t2] = F.t2 * m + Fm * WL[t2];
+    } else if (o.side > 0) {
+      WRb[t1] = F.t1 * m + Fm * WR[t1];
+      WRb[t2] = F.t2 * m + Fm * WR[t2];
+    }
+    return;
   }
+  const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L, star = kind >= NEAR_STAR_L;
+  const double rk = left ? rl : rr;
+  const double rho = star ? rk + s.drho : rk, u = star ? s.us : (left ? WL[n] : WR[n]);
+  const double p = star ? pl + s.d : (left ? pl : pr);
+  double rb, ub, pb, t1b, t2b;
+  flux_state_vjp(C.g_gm1, rho, u, p, left ? WL[t1] : WR[t1], left ? WL[t2] : WR[t2], F, rb, ub, pb, t1b, t2b);
+  double lr = 0.0, lu = 0.0, lp = 0.0, qr = 0.0, qu = 0.0, qp = 0.0;  // cotangents of (rho, u, p)_L and _R
+  if (star) {
+    const double yl = s.d * s.ipl, yr = (s.d - dP) * s.ipr;
+    const bool sl = !sign_bit(yl), sr = !sign_bit(yr);
+    const double tl = s.ircl * near_sum(C.tf, C.t, C.tt, sl, yl), tr = s.ircr * near_sum(C.tf, C.t, C.tt, sr, yr);
+    // rho* = rho_K (1 + x D(x)), x = p*/p_K - 1
+    const double x = left ? yl : yr, ipk = left ? s.ipl : s.ipr;
+    const double hb = rb * rk * (near_sum(C.df, C.h, C.ht, left ? sl : sr, x) * ipk);
+    const double rkb = rb * (rho * recip(rk)), pkb = -hb * (1.0 + x);
+    const double gu = 0.5 * ub;
+    const double psb = pb + hb + gu * (tr - tl);
+    const double lam = -psb * recip(tl + tr);
+    const double fl = lam - gu, fr = lam + gu;  // cotangents of f_L, f_R
+    lu = gu - lam;
+    qu = gu + lam;
+    // 1 / (2 rho_K) = gamma p_K irc_K^2 / 2
+    const double hg = -0.5 * C.gamma;
+    lr = fl * s.fl * (hg * pl * (s.ircl * s.ircl)) + (left ? rkb : 0.0);
+    qr = fr * s.fr * (hg * pr * (s.ircr * s.ircr)) + (left ? 0.0 : rkb);
+    lp = fl * fma(-p, tl, 0.5 * s.fl) * s.ipl + (left ? pkb : 0.0);
+    qp = fr * fma(-p, tr, 0.5 * s.fr) * s.ipr + (left ? 0.0 : pkb);
+  } else {
+    lr = left ? rb : 0.0;
+    lu = left ? ub : 0.0;
+    lp = left ? pb : 0.0;
+    qr = left ? 0.0 : rb;
+    qu = left ? 0.0 : ub;
+    qp = left ? 0.0 : pb;
+  }
+  WLb[RHO] = lr;
+  WLb[n] = lu;
+  WLb[EN] = lp;
+  WRb[RHO] = qr;
+  WRb[n] = qu;
+  WRb[EN] = qp;
+  WLb[t1] = left ? t1b : 0.0;
+  WLb[t2] = left ? t2b : 0.0;
+  WRb[t1] = left ? 0.0 : t1b;
+  WRb[t2] = left ? 0.0 : t2b;
 }
 
 // Cotangents of the dust face primitives (u, v, w, rho_d) for a cotangent Fb
@@ -351,8 +437,8 @@ template <int D>
 __device__ __forceinline__ void dust_flux_vjp(const double* WL, const double* WR, const double* Fb, double* WLb,
                                               double* WRb) {
   constexpr int n = Axes<D>::n, t1 = Axes<D>::t1, t2 = Axes<D>::t2;
-  const double ml = WL[3] * (WL[n] > 0.0 ? WL[n] : 0.0);
-  const double mr = WR[3] * (WR[n] < 0.0 ? WR[n] : 0.0);
+  const double ml = WL[3] * pos_part(WL[n]);
+  const double mr = WR[3] * neg_part(WR[n]);
   const double mlb = Fb[3] + Fb[n] * WL[n] + Fb[t1] * WL[t1] + Fb[t2] * WL[t2];
   const double mrb = Fb[3] + Fb[n] * WR[n] + Fb[t1] * WR[t1] + Fb[t2] * WR[t2];
   WLb[3] = 0.0;
@@ -363,51 +449,39 @@ __device__ __forceinline__ void dust_flux_vjp(const double* WL, const double* WR
   WRb[n] = Fb[n] * mr;
   WRb[t1] = Fb[t1] * mr;
   WRb[t2] = Fb[t2] * mr;
-  if (WL[n] > 0.0) {
+  if (positive(WL[n])) {
     WLb[3] += mlb * WL[n];
     WLb[n] += mlb * WL[3];
   }
-  if (WR[n] < 0.0) {
+  if (positive(-WR[n])) {
     WRb[3] += mrb * WR[n];
     WRb[n] += mrb * WR[3];
   }
 }
 
 // ------------------------------------------------------------------ reconstruction adjoint
+// Limiter products of the axis-0 weights (w6 w0, w6 w1, w7 w0, w7 w1).
+__device__ __forceinline__ void limiter_weights(const double* w, double* lw) {
+  lw[0] = w[6] * w[0];
+  lw[1] = w[6] * w[1];
+  lw[2] = w[7] * w[0];
+  lw[3] = w[7] * w[1];
+}
 // Cotangents (bm, b0, bp) of the three cell deviations for cotangents gm, gp
-// on the face values qm, qp of parabola(em, e0, ep, w); branches of the
-// forward values.
-__device__ __forceinline__ void parabola_vjp(double em, double e0, double ep, const double* w, double gm, double gp,
+// on the face values, at the branches br that parabola_branches took: each
+// face value is e0 -/+ (alpha dm + beta dp) with the branch's two weights.
+template <bool UNI>
+__device__ __forceinline__ void parabola_vjp(unsigned br, const double* w, const double* lw, double gm, double gp,
                                              double& bm, double& b0, double& bp) {
-  const double sm = (e0 - em) * w[0];
-  const double sp = (ep - e0) * w[1];
-  const double s = minmod(sm, sp);
-  const double a = (sp - sm) * w[2];
-  const double b = (sp * w[3] + sm * w[4]) * w[2];
-  double ab = 0.0, bb = 0.0, sb = 0.0;
-  {
-    const double A = w[5] * (a * w[5] + b), B = s * w[7];
-    if (A * B > 0.0) {
-      if (fabs(A) < fabs(B)) { ab += gm * w[5] * w[5]; bb += gm * w[5]; }
-      else sb += gm * w[7];
-    }
-  }
-  {
-    const double A = w[6] * (a * w[6] + b), B = s * w[8];
-    if (A * B > 0.0) {
-      if (fabs(A) < fabs(B)) { ab += gp * w[6] * w[6]; bb += gp * w[6]; }
-      else sb += gp * w[8];
-    }
-  }
-  double smb = -ab * w[2] + bb * w[4] * w[2];
-  double spb = ab * w[2] + bb * w[3] * w[2];
-  if (sm * sp > 0.0) {
-    if (fabs(sm) < fabs(sp)) smb += sb;
-    else spb += sb;
-  }
-  bm = -smb * w[0];
-  bp = spb * w[1];
-  b0 = gm + gp + smb * w[0] - spb * w[1];
+  const bool live = br & 1, first = br & 2, A = br & 4, B = br & 8;
+  const double am = !live ? 0.0 : (A ? (UNI ? 0.375 : w[2]) : (first ? (UNI ? 1.0 : lw[0]) : 0.0));
+  const double ap = !live ? 0.0 : (A ? (UNI ? 0.125 : w[3]) : (first ? 0.0 : (UNI ? 1.0 : lw[1])));
+  const double cm = !live ? 0.0 : (B ? (UNI ? 0.125 : w[4]) : (first ? (UNI ? 1.0 : lw[2]) : 0.0));
+  const double cp = !live ? 0.0 : (B ? (UNI ? 0.375 : w[5]) : (first ? 0.0 : (UNI ? 1.0 : lw[3])));
+  const double dmb = fma(gp, cm, -(gm * am)), dpb = fma(gp, cp, -(gm * ap));
+  bm = -dmb;
+  bp = dpb;
+  b0 = (gm + gp) + (dmb - dpb);
 }
 
 // ------------------------------------------------------------------ drag and source adjoints
@@ -418,104 +492,81 @@ __device__ __forceinline__ double drag_vjp(const DevGrid& g, int i, const double
 #pragma unroll
   for (int f = 0; f < 9; ++f) li[f] = lo[f];
   const double rg = U[RHO], rd = U[DRHO];
-  if (!(rd > 0.0) || !(rg > 0.0)) return 0.0;
-  double ts, cs = 0.0;
-  bool stokes_regime = false;  // drag law 2 above r_p = 9 lambda / 4 (the forward's branch)
-  if (d.law == 0) {
-    if (g.geom == GEOM_CYL) {
-      const double r = g.rc[i + GH];
-      ts = d.stokes / sqrt(g.gm / (r * r * r));
-    } else {
-      ts = d.stokes;
-    }
-  } else {
-    cs = sqrt(g.gamma * gas_pressure(g.gamma, U[MU], U[MV], U[MW], U[EN], rg) / rg);
-    ts = d.rhos_rp / (rg * cs);
-    stokes_regime = d.law == 2 && d.kappa * rg > 2.25;
-    if (stokes_regime) ts = ts * ((4.0 / 9.0) * (d.kappa * rg));
-  }
-  const double kk = tau * (1.0 + rd / rg) / ts;
-  const double mu = rg * rd / (rg + rd);
-  const double relax = kk / (1.0 + kk);
-  const double K = mu * relax;
+  if (!positive(rd) || !positive(rg)) return 0.0;
+  const double ig = recip(rg), id = recip(rd);
+  double P = 0.0;
+  if (d.law != 0) P = (g.gamma - 1.0) * fma(-0.5 * ig, fma(U[MU], U[MU], fma(U[MV], U[MV], U[MW] * U[MW])), U[EN]);
+  const double a = tau * inv_stopping_time<true>(g, i, rg, P, d, 0);
+  // the momentum that changes hands is K (v_d - v_g), K = rho_d a / (1 + k),
+  // k = a (1 + rho_d / rho_g)
+  const double eps = rd * ig, q = recip(1.0 + fma(a, eps, a)), aq = a * q, K = rd * aq;
   const double e = lo[EN];
   double Kb = 0.0, rgb = 0.0, rdb = 0.0;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const double vg = U[MU + c] / rg;
-    const double vd = U[DMU + c] / rd;
+    const double vg = U[MU + c] * ig;
+    const double vd = U[DMU + c] * id;
     const double dv = vd - vg;
-    const double X = mu * dv * relax;
-    const double ugp = U[MU + c] + X;
-    const double dE = 0.5 * X * (ugp / rg + vg);
-    const double Xb = lo[MU + c] - lo[DMU + c] + e * ugp / rg;
-    li[MU + c] += e * X / rg;
-    rgb -= e * dE / rg;
-    Kb += Xb * dv;
-    const double dvb = Xb * K;
-    li[DMU + c] += dvb / rd;
-    rdb -= dvb * vd / rd;
-    li[MU + c] -= dvb / rg;
-    rgb += dvb * vg / rg;
+    const double X = K * dv;
+    const double vp = fma(X, ig, vg);
+    const double dE = 0.5 * X * (vp + vg);
+    const double Xb = fma(e, vp, lo[MU + c] - lo[DMU + c]);
+    const double dvb = Xb * K, dg = dvb * ig, dd = dvb * id;
+    li[MU + c] += fma(e * X, ig, -dg);
+    li[DMU + c] += dd;
+    rgb += fma(dg, vg, -(e * dE * ig));
+    rdb = fma(-dd, vd, rdb);
+    Kb = fma(Xb, dv, Kb);
   }
-  const double mub = Kb * relax;
-  const double relaxb = Kb * mu;
-  const double kkb = relaxb / ((1.0 + kk) * (1.0 + kk));
-  const double s = rg + rd;
-  rgb += mub * rd * rd / (s * s);
-  rdb += mub * rg * rg / (s * s);
-  rdb += kkb * tau / (rg * ts);
-  rgb -= kkb * tau * rd / (rg * rg * ts);
-  const double tsb = -kkb * kk / ts;
-  if (d.law == 1 || d.law == 2) {
-    // t_s = rhos_rp / (rho_g c_s), c_s = sqrt(gamma P / rho_g); in the Stokes
-    // regime t_s = (4/9) kappa rhos_rp / c_s, with no explicit rho_g
-    if (!stokes_regime) rgb -= tsb * ts / rg;
-    const double csb = -tsb * ts / cs;
-    const double Pb = csb * g.gamma / (2.0 * cs * rg);
-    rgb -= csb * cs / (2.0 * rg);
-    const double gm1 = g.gamma - 1.0;
+  rdb = fma(Kb * aq, fma(-aq, eps, 1.0), rdb);
+  rgb = fma(Kb * (K * aq), eps * ig, rgb);
+  const double ab = Kb * (rd * (q * q)), aab = ab * a;  // cotangent of a, times a
+  if (d.law != 0) {
+    // 1 / t_s = rho_g c_s / rhos_rp with c_s = sqrt(gamma P / rho_g); in the
+    // Stokes regime (drag law 2 above r_p = 9 lambda / 4, the forward's branch)
+    // 1 / t_s = (9/4) c_s / (kappa rhos_rp), with no explicit rho_g
+    const bool stokes_regime = d.law == 2 && positive(d.kappa * rg - 2.25);
+    if (!stokes_regime) rgb = fma(aab, ig, rgb);
+    const double Pb = 0.5 * aab * recip(P), gm1 = g.gamma - 1.0;
+    rgb = fma(-0.5 * aab, ig, rgb);
     li[EN] += Pb * gm1;
     double k2 = 0.0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const double v = U[MU + c] / rg;
+      const double v = U[MU + c] * ig;
       li[MU + c] -= Pb * gm1 * v;
-      k2 += v * v;
+      k2 = fma(v, v, k2);
     }
     rgb += Pb * gm1 * 0.5 * k2;
   }
   li[RHO] += rgb;
   li[DRHO] += rdb;
-  return tsb * ts / d.stokes;  // t_s is proportional to St in every law
+  return -aab * d.ist[0];  // t_s is proportional to St in every law: -a a_b = t_s t_s_b
 }
 
 // out += s S'(U)^T for the App. B sources at a cell (cylindrical only).
 __device__ __forceinline__ void sources_vjp(const DevGrid& g, int i, int k, const double* U, const double* s,
                                             double* out) {
-  const double r = g.rc[i + GH];
-  const double z = g.x0[2] + (k + 0.5) * g.dx[2];
-  const double R2 = r * r + z * z;
-  const double R3 = R2 * sqrt(R2);
-  const double fr = -g.gm * r / R3, fz = -g.gm * z / R3;
-  const double Om = g.omega;
-  const double A1 = fr + Om * Om * r;
+  const double ir = g.ir[i], Om2 = 2.0 * g.omega;
+  const size_t o = (size_t)k * g.nr + i;
+  const double A1 = g.grav[o], fz = g.grav[(size_t)g.nz * g.nr + o];
   const double gm1 = g.gamma - 1.0;
   {
-    const double ir = 1.0 / U[RHO];
-    const double u = U[MU] * ir, v = U[MV] * ir, w = U[MW] * ir;
-    out[MU] += s[MU] * (-gm1 * u / r) + s[MV] * (-v / r - 2.0 * Om) + s[EN] * A1;
-    out[MV] += s[MU] * (2.0 * v / r + 2.0 * Om - gm1 * v / r) + s[MV] * (-u / r);
-    out[MW] += s[MU] * (-gm1 * w / r) + s[EN] * fz;
-    out[EN] += s[MU] * gm1 / r;
-    out[RHO] += s[MU] * (-v * v / r + gm1 * 0.5 * (u * u + v * v + w * w) / r + A1) + s[MV] * (u * v / r) + s[MW] * fz;
+    const double iq = recip(U[RHO]);
+    const double u = U[MU] * iq, v = U[MV] * iq, w = U[MW] * iq;
+    const double sg = s[MU] * (gm1 * ir), vr = v * ir, ur = u * ir;
+    out[MU] += fma(s[EN], A1, -fma(sg, u, s[MV] * (vr + Om2)));
+    out[MV] += fma(s[MU], fma(2.0, vr, Om2), -fma(sg, v, s[MV] * ur));
+    out[MW] += fma(s[EN], fz, -(sg * w));
+    out[EN] += sg;
+    out[RHO] += fma(s[MU], fma(-v, vr, A1), fma(0.5 * sg, fma(u, u, fma(v, v, w * w)), fma(s[MV] * u, vr, s[MW] * fz)));
   }
-  if (g.nf > 5 && U[DRHO] > 0.0) {
-    const double ir = 1.0 / U[DRHO];
-    const double u = U[DMU] * ir, v = U[DMV] * ir;
-    out[DMU] += s[DMV] * (-v / r - 2.0 * Om);
-    out[DMV] += s[DMU] * (2.0 * v / r + 2.0 * Om) + s[DMV] * (-u / r);
-    out[DRHO] += s[DMU] * (-v * v / r + A1) + s[DMV] * (u * v / r) + s[DMW] * fz;
+  if (g.nf > 5 && positive(U[DRHO])) {
+    const double iq = recip(U[DRHO]);
+    const double u = U[DMU] * iq, v = U[DMV] * iq, vr = v * ir;
+    out[DMU] -= s[DMV] * (vr + Om2);
+    out[DMV] += fma(s[DMU], fma(2.0, vr, Om2), -(s[DMV] * (u * ir)));
+    out[DRHO] += fma(s[DMU], fma(-v, vr, A1), fma(s[DMV] * u, vr, s[DMW] * fz));
   }
 }
 
@@ -706,8 +757,12 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
       const double v = RC == RECON_PRIM ? W[f] : U[f];
       dst[(size_t)f * PE * NLP] = g.has_eq ? v - e0[((size_t)f * g.nz + c[2]) * g.nr + c[0]] : v;
     }
+    if (NF == 9) {  // the dust as primitives (u, v, w, rho_d)
+      const double rd = a.E[DRHO][lin], id = positive(rd) ? recip(rd) : 0.0;
 #pragma unroll
-    for (int f = 5; f < NF; ++f) dst[(size_t)f * PE * NLP] = a.E[f][lin];
+      for (int q = 0; q < 3; ++q) dst[(size_t)(DMU + q) * PE * NLP] = a.E[DMU + q][lin] * id;
+      dst[(size_t)DRHO * PE * NLP] = rd;
+    }
   }
   for (int idx = threadIdx.x; idx < PM * NL; idx += NT) {
     const int pos = D == 0 ? idx % PM : idx / NL;
@@ -759,52 +814,53 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
     if (D == 1) return tc[((size_t)f * g.nz + ck) * g.nr + ci];
     return tz[((size_t)f * (g.nz + 1) + clampi(fd, 0, g.nz)) * g.nr + ci];
   };
-  double w[9];
-  parabola_weights<double, D>(g.rcoef, gi, g.nr, g.dx[D], w);
+  constexpr bool UNI = D != 0;
+  double w[RCW], lw[4];
+  parabola_weights<double, D>(g.rcoef, gi, g.nr, w);
+  if (!UNI) limiter_weights(w, lw);
 
-  // ---- forward reconstruction of this lane's cell
-  double qm[5], qp[5];
-  bool shaped = false;
-#pragma unroll
-  for (int f = 0; f < 5; ++f) shaped |= parabola(sv(f, p), sv(f, p + 1), sv(f, p + 2), w, qm[f], qp[f]);
+  // ---- forward reconstruction of this lane's cell: the primitives of the
+  // right state of its lower face (WR, 1 / rho irm) and of the left state of
+  // its upper face (WP, irp), and the branches taken
+  double WR[5], WP[5], irm = 0.0, irp = 0.0;
+  unsigned br[9];
   bool fallback = false;
-  if (shaped && line_ok) {
-    if (RC == RECON_PRIM) {
-      fallback = !(eq_face(RHO, c) + qm[RHO] > 0.0 && eq_face(RHO, c + 1) + qp[RHO] > 0.0 &&
-                   eq_face(EN, c) + qm[EN] > 0.0 && eq_face(EN, c + 1) + qp[EN] > 0.0);
-    } else {
+  {
+    double qm[5], qp[5];
+#pragma unroll
+    for (int f = 0; f < 5; ++f)
+      br[f] = parabola_branches<UNI>(sv(f, p), sv(f, p + 1), sv(f, p + 2), w, qm[f], qp[f]);
+    auto face_states = [&]() {
       double Um[5], Up[5];
 #pragma unroll
       for (int f = 0; f < 5; ++f) {
         Um[f] = eq_face(f, c) + qm[f];
         Up[f] = eq_face(f, c + 1) + qp[f];
       }
-      double Wm[5], Wp[5];  // the forward's test, on the same converted states
-      gas_prim(gam, Um, Wm);
-      gas_prim(gam, Up, Wp);
-      fallback = !(Um[RHO] > 0.0 && Up[RHO] > 0.0 && Wm[EN] > 0.0 && Wp[EN] > 0.0);
-    }
-    if (fallback) {
+      if (RC == RECON_PRIM) {
+#pragma unroll
+        for (int f = 0; f < 5; ++f) {
+          WR[f] = Um[f];
+          WP[f] = Up[f];
+        }
+      } else {
+        irm = gas_prim(gam, Um, WR);
+        irp = gas_prim(gam, Up, WP);
+      }
+      return positive(Um[RHO]) && positive(Up[RHO]) && positive(WR[EN]) && positive(WP[EN]);
+    };
+    if (!face_states() && line_ok) {  // the forward's positivity fallback: flat departures
+      fallback = true;
 #pragma unroll
       for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sv(f, p + 1);
+      face_states();
     }
   }
-  double dm[4], dp[4], pm[4], p0[4], pp[4];
+  double dm[4], dp[4];
   if (NF == 9) {
-    pm[3] = sv(8, p);
-    p0[3] = sv(8, p + 1);
-    pp[3] = sv(8, p + 2);
-    const double im = pm[3] > 0.0 ? 1.0 / pm[3] : 0.0;
-    const double i0 = p0[3] > 0.0 ? 1.0 / p0[3] : 0.0;
-    const double ip = pp[3] > 0.0 ? 1.0 / pp[3] : 0.0;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      pm[q] = sv(5 + q, p) * im;
-      p0[q] = sv(5 + q, p + 1) * i0;
-      pp[q] = sv(5 + q, p + 2) * ip;
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) parabola(pm[q], p0[q], pp[q], w, dm[q], dp[q]);
+    for (int q = 0; q < 4; ++q)
+      br[5 + q] = parabola_branches<UNI>(sv(5 + q, p), sv(5 + q, p + 1), sv(5 + q, p + 2), w, dm[q], dp[q]);
   }
 
   // ---- the face below this cell: cotangents of its two states
@@ -813,25 +869,13 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
   double Fb[9];
 #pragma unroll
   for (int f = 0; f < NF; ++f) Fb[f] = has_face ? area * (sm(f, p) - sm(f, p > 0 ? p - 1 : 0)) : 0.0;
-  double ULb[5], URb[5];
+  double ULb[5], URb[5];  // of the left state (the lane below's WP) and of this lane's WR
   {
-    double UL[5], UR[5];
+    double WL[5];
 #pragma unroll
-    for (int f = 0; f < 5; ++f) {
-      const double ql = __shfl_up_sync(FULL, qp[f], 1, L);
-      const double e0 = eq_face(f, c);
-      UL[f] = e0 + ql;
-      UR[f] = e0 + qm[f];
-    }
-    if (has_face && RC == RECON_PRIM) {
-      gas_flux_vjp<D>(gam, UL, UR, Fb, ULb, URb, status);
-    } else if (has_face) {  // conservative face states: through W = gas_prim(U)
-      double WL[5], WR[5], WLb[5], WRb[5];
-      gas_prim(gam, UL, WL);
-      gas_prim(gam, UR, WR);
-      gas_flux_vjp<D>(gam, WL, WR, Fb, WLb, WRb, status);
-      gas_prim_vjp(gam, UL, WLb, ULb);
-      gas_prim_vjp(gam, UR, WRb, URb);
+    for (int f = 0; f < 5; ++f) WL[f] = __shfl_up_sync(FULL, WP[f], 1, L);
+    if (has_face) {
+      gas_flux_vjp<D>(g.near, WL, WR, Fb, ULb, URb, status);
     } else {
 #pragma unroll
       for (int f = 0; f < 5; ++f) ULb[f] = URb[f] = 0.0;
@@ -851,39 +895,34 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
   }
 
   // ---- cotangents of this cell's face values: lower from its own face, upper from the lane above
-  double tm[9], t0[9], tp[9];  // contributions to cells c - 1, c, c + 1
+  double tm[9], t0[9], tp[9];  // contributions to cells c - 1, c, c + 1 (dust: of the primitives)
+  {
+    double gp[5];
 #pragma unroll
-  for (int f = 0; f < 5; ++f) {
-    const double up = __shfl_down_sync(FULL, ULb[f], 1, L);
-    const double gpf = p < L - 1 ? up : 0.0;
-    if (fallback) {
-      tm[f] = tp[f] = 0.0;
-      t0[f] = URb[f] + gpf;
-    } else {
-      parabola_vjp(sv(f, p), sv(f, p + 1), sv(f, p + 2), w, URb[f], gpf, tm[f], t0[f], tp[f]);
+    for (int f = 0; f < 5; ++f) {
+      const double up = __shfl_down_sync(FULL, ULb[f], 1, L);
+      gp[f] = p < L - 1 ? up : 0.0;
+    }
+    if (RC != RECON_PRIM) {  // through W = gas_prim(U) of the face states
+      prim_vjp(gam, irm, WR, URb);
+      prim_vjp(gam, irp, WP, gp);
+    }
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+      if (fallback) {
+        tm[f] = tp[f] = 0.0;
+        t0[f] = URb[f] + gp[f];
+      } else {
+        parabola_vjp<UNI>(br[f], w, lw, URb[f], gp[f], tm[f], t0[f], tp[f]);
+      }
     }
   }
   if (NF == 9) {
-    double bm[4], b0[4], bp[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const double up = __shfl_down_sync(FULL, WLb[q], 1, L);
-      parabola_vjp(pm[q], p0[q], pp[q], w, WRb[q], p < L - 1 ? up : 0.0, bm[q], b0[q], bp[q]);
+      parabola_vjp<UNI>(br[5 + q], w, lw, WRb[q], p < L - 1 ? up : 0.0, tm[5 + q], t0[5 + q], tp[5 + q]);
     }
-    // primitives (u, v, w, rho_d) back to the conservative dust fields of each cell
-    auto back = [&](const double* b, const double* prim, double* t) {
-      const double inv = prim[3] > 0.0 ? 1.0 / prim[3] : 0.0;  // prim[3] is the density itself
-      double rb = b[3];
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        t[5 + q] = b[q] * inv;
-        rb -= b[q] * prim[q] * inv;
-      }
-      t[8] = rb;
-    };
-    back(bm, pm, tm);
-    back(b0, p0, t0);
-    back(bp, pp, tp);
   }
   double tot[9];
 #pragma unroll
@@ -916,8 +955,17 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
 #pragma unroll
       for (int f = 0; f < 5; ++f) a.lam[f][lin] += tot[f];
     }
+    if (NF == 9) {  // dust: the primitives' cotangents back to (rho_d u, rho_d v, rho_d w, rho_d)
+      const double rd = sv(8, p + 1), id = positive(rd) ? recip(rd) : 0.0;
+      double rb = tot[8];
 #pragma unroll
-    for (int f = 5; f < NF; ++f) a.lam[f][lin] += tot[f];
+      for (int q = 0; q < 3; ++q) {
+        const double m = tot[5 + q] * id;
+        a.lam[5 + q][lin] += m;
+        rb = fma(-m, sv(5 + q, p + 1), rb);
+      }
+      a.lam[DRHO][lin] += rb;
+    }
   }
   if (status) atomicOr(a.status, status);
 }
@@ -934,7 +982,8 @@ static __global__ void __launch_bounds__(ADJ_PT_NT) drag_only_kernel(DevGrid g, 
     double U[9];
 #pragma unroll
     for (int f = 0; f < 9; ++f) U[f] = Y.p[f][lin];
-    apply_drag<true, 1>(g, (int)(lin % g.nr), U, tau, d);
+    const double id = recip(U[DRHO]);
+    apply_drag<true, 1>(g, (int)(lin % g.nr), U, tau, d, recip(U[RHO]), &id);
 #pragma unroll
     for (int f = 0; f < 9; ++f) out.p[f][lin] = U[f];
   }

@@ -4,6 +4,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "riemann_near.cuh"
+
 namespace rossbi {
 
 // Conservative variables in App. B order, then the dust fluid; dust species
@@ -21,7 +23,7 @@ enum { STATUS_NONPHYSICAL = 1u, STATUS_RIEMANN = 2u };
 enum { RECON_CONS = 0, RECON_PRIM = 1 };
 
 constexpr int GH = 2;   // ghost offset of the axis-0 coordinate tables
-constexpr int RCW = 10; // parabola weights per axis-0 cell (9 used)
+constexpr int RCW = 8;  // parabola weights per axis-0 cell
 
 // Grid data the kernels read.  Passed by value as a kernel parameter; the
 // pointers are device tables owned by the host runtime.
@@ -39,7 +41,10 @@ struct DevGrid {
   const double* area_r;  // A of the axis-0 face i - 1/2, i in [0, nr]
   const double* area_t;  // A of an axis-1 face of a cell with radial index i
   const double* area_z;  // A of an axis-2 face of a cell with radial index i
-  const double* maxA;    // largest face area of a cell with radial index i
+  const double* aov;     // largest face area of a cell with radial index i over its volume
+  const double* ir;      // 1 / r of the cell centre (cylindrical)
+  const double* omk;     // Omega_K at the cell centre (cylindrical), 1 in the Box
+  const double* grav;    // [2][nz][nr] cylindrical: f_r + Omega^2 r, f_z at the cell centres
   const double* e0c;     // equilibrium gas state at centres   [5][nz][nr]
   const double* e0r;     // equilibrium gas state at r faces   [5][nz][nr + 1]
   const double* e0z;     // equilibrium gas state at z faces   [5][nz + 1][nr]
@@ -62,6 +67,7 @@ struct DevGrid {
   const float* damp_kf;
   // dust species s has the Stokes number St x st_factor[s] (st_factor[0] = 1)
   double st_factor[ND_MAX];
+  NearCoef near;         // series of the exact Riemann solution near p_K
 };
 
 __host__ __device__ constexpr int pow2ceil(int v) {
@@ -349,26 +355,44 @@ __device__ __forceinline__ int riemann_face_g75(double rl, double ul, double pl,
   return 1;
 }
 
+// The general solver, out of line: faces near a strong wave or in the sonic
+// band.  By value: pointers would keep the callers' face states in memory.
+struct RFace {
+  double rho, u, p;
+  int side;         // -1 left, +1 right, 0 vacuum: whose transverse velocity is carried
+  unsigned status;
+};
+static __device__ __noinline__ RFace riemann_general(double g, double rl, double ul, double pl, double rr, double ur,
+                                                     double pr) {
+  RFace o;
+  o.status = 0;
+  o.side = g == 1.4 ? riemann_face_g75(rl, ul, pl, rr, ur, pr, o.rho, o.u, o.p, o.status)
+                    : riemann_face(g, rl, ul, pl, rr, ur, pr, o.rho, o.u, o.p, o.status);
+  return o;
+}
+
 __device__ __forceinline__ double gas_pressure(double g, double mu, double mv, double mw, double en, double rho) {
   return (g - 1.0) * (en - 0.5 * (mu * mu + mv * mv + mw * mw) / rho);
 }
 
 // Primitive gas state (u, v, w, P, rho), in the field slots MU, MV, MW, EN,
-// RHO, of a conservative gas state.
-__device__ __forceinline__ void gas_prim(double g, const double* U, double* W) {
-  const double ir = 1.0 / U[RHO];  // one division: GB300's FP64 divide is a multi-instruction sequence
+// RHO, of a conservative gas state; returns 1 / rho (NaN for rho = 0, which
+// leaves a P that fails every positivity test).
+__device__ __forceinline__ double gas_prim(double g, const double* U, double* W) {
+  const double ir = recip(U[RHO]);
   W[MU] = U[MU] * ir;
   W[MV] = U[MV] * ir;
   W[MW] = U[MW] * ir;
-  W[EN] = (g - 1.0) * (U[EN] - 0.5 * (U[MU] * U[MU] + U[MV] * U[MV] + U[MW] * U[MW]) * ir);
+  W[EN] = (g - 1.0) * fma(-0.5, fma(U[MU], W[MU], fma(U[MV], W[MV], U[MW] * W[MW])), U[EN]);
   W[RHO] = U[RHO];
+  return ir;
 }
 
 // Cotangent Ub of the conservative gas state U for a cotangent Wb of its
 // primitive state W = gas_prim(U) (the transpose of the conversion's
 // Jacobian at U).
 __device__ __forceinline__ void gas_prim_vjp(double g, const double* U, const double* Wb, double* Ub) {
-  const double ir = 1.0 / U[RHO], gm1 = g - 1.0;
+  const double ir = recip(U[RHO]), gm1 = g - 1.0;
   const double v0 = U[MU] * ir, v1 = U[MV] * ir, v2 = U[MW] * ir;
   const double bP = Wb[EN];
   Ub[MU] = Wb[MU] * ir - gm1 * bP * v0;
@@ -378,43 +402,71 @@ __device__ __forceinline__ void gas_prim_vjp(double g, const double* U, const do
   Ub[RHO] = Wb[RHO] - (Wb[MU] * v0 + Wb[MV] * v1 + Wb[MW] * v2) * ir + gm1 * bP * 0.5 * (v0 * v0 + v1 * v1 + v2 * v2);
 }
 
-// Gas flux F(E*) through a face normal to axis D from the reconstructed left
-// and right primitive states (App. B flux vector; energy flux (E + P) u_n).
+// The same in place, b the cotangent of W on entry and of U on return, from
+// W and ir = 1 / rho.
+__device__ __forceinline__ void prim_vjp(double g, double ir, const double* W, double* b) {
+  const double pb = (g - 1.0) * b[EN];
+  const double k2 = fma(W[MU], W[MU], fma(W[MV], W[MV], W[MW] * W[MW]));
+  const double dot = fma(b[MU], W[MU], fma(b[MV], W[MV], b[MW] * W[MW]));
+  b[RHO] = fma(0.5 * pb, k2, fma(-dot, ir, b[RHO]));
+  b[MU] = fma(b[MU], ir, -(pb * W[MU]));
+  b[MV] = fma(b[MV], ir, -(pb * W[MV]));
+  b[MW] = fma(b[MW], ir, -(pb * W[MW]));
+  b[EN] = pb;
+}
+
+// Gas flux A F(E*) through a face of area A normal to axis D from the
+// reconstructed left and right primitive states (App. B flux vector; energy
+// flux (E + P) u_n).
 template <int D>
-__device__ __forceinline__ void gas_face_flux(double g, const double* WL, const double* WR, double* F,
-                                              unsigned& status) {
+__device__ __forceinline__ void gas_face_flux(const NearCoef& C, double area, const double* WL, const double* WR,
+                                              double* F, unsigned& status) {
   constexpr int n = Axes<D>::n, t1 = Axes<D>::t1, t2 = Axes<D>::t2;
-  const double rl = WL[RHO], rr = WR[RHO], pl = WL[EN], pr = WR[EN];
-  if (!(rl > 0.0) || !(rr > 0.0) || !(pl > 0.0) || !(pr > 0.0)) {
+  if (!positive(WL[RHO]) || !positive(WR[RHO]) || !positive(WL[EN]) || !positive(WR[EN])) {
     status |= STATUS_NONPHYSICAL;
 #pragma unroll
     for (int f = 0; f < 5; ++f) F[f] = 0.0;
     return;
   }
-  double rho, u, p;
-  const int side = g == 1.4 ? riemann_face_g75(rl, WL[n], pl, rr, WR[n], pr, rho, u, p, status)
-                            : riemann_face(g, rl, WL[n], pl, rr, WR[n], pr, rho, u, p, status);
-  double ut1 = 0.0, ut2 = 0.0;
-  if (side < 0) { ut1 = WL[t1]; ut2 = WL[t2]; }
-  else if (side > 0) { ut1 = WR[t1]; ut2 = WR[t2]; }
-  const double m = rho * u;
+  NearStar<double> s;
+  const int kind = near_riemann<double>(C, WL[RHO], WL[n], WL[EN], WR[RHO], WR[n], WR[EN], WR[EN] - WL[EN],
+                                        WR[n] - WL[n], 0.0, false, narrow(WL[n]), narrow(WR[n]), s);
+  const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
+  double rho = left ? WL[RHO] : WR[RHO], u = left ? WL[n] : WR[n], p = left ? WL[EN] : WR[EN];
+  double ut1 = left ? WL[t1] : WR[t1], ut2 = left ? WL[t2] : WR[t2];
+  if (kind >= NEAR_STAR_L) {
+    rho += s.drho;
+    u = s.us;
+    p = WL[EN] + s.d;
+  }
+  if (kind == NEAR_GENERAL) {
+    const RFace o = riemann_general(C.gamma, WL[RHO], WL[n], WL[EN], WR[RHO], WR[n], WR[EN]);
+    status |= o.status;
+    rho = o.rho;
+    u = o.u;
+    p = o.p;
+    ut1 = o.side < 0 ? WL[t1] : (o.side > 0 ? WR[t1] : 0.0);
+    ut2 = o.side < 0 ? WL[t2] : (o.side > 0 ? WR[t2] : 0.0);
+  }
+  const double m = area * (rho * u), pa = area * p;
   F[RHO] = m;
-  F[n] = m * u + p;
+  F[n] = fma(m, u, pa);
   F[t1] = m * ut1;
   F[t2] = m * ut2;
-  F[EN] = (0.5 * rho * (u * u + ut1 * ut1 + ut2 * ut2) + p / (g - 1.0) + p) * u;
+  F[EN] = fma(0.5 * m, fma(u, u, fma(ut1, ut1, ut2 * ut2)), C.g_gm1 * (pa * u));
 }
 
 // Flux of the pressureless dust fluid (Sect. 2.9 "adapted" solver) by kinetic
 // flux-vector splitting (Bouchut, Jin & Li 2003): the matter moving right
 // crosses from the left face state, the matter moving left from the right one.
 // WL, WR hold face primitives (u, v, w, rho_d); F the dust fluxes in the
-// order (rho_d u, rho_d v, rho_d w, rho_d) for a face normal to axis D.
+// order (rho_d u, rho_d v, rho_d w, rho_d), times the face's area, for a face
+// normal to axis D.
 template <int D, class T>
-__device__ __forceinline__ void dust_kinetic_flux(const T* WL, const T* WR, T* F) {
+__device__ __forceinline__ void dust_kinetic_flux(T area, const T* WL, const T* WR, T* F) {
   constexpr int n = Axes<D>::n, t1 = Axes<D>::t1, t2 = Axes<D>::t2;  // 0..2 in the dust block
-  const T ml = WL[3] * (WL[n] > T(0) ? WL[n] : T(0));
-  const T mr = WR[3] * (WR[n] < T(0) ? WR[n] : T(0));
+  const T ml = area * (WL[3] * pos_part(WL[n]));
+  const T mr = area * (WR[3] * neg_part(WR[n]));
   F[3] = ml + mr;
   F[n] = ml * WL[n] + mr * WR[n];
   F[t1] = ml * WL[t1] + mr * WR[t1];
@@ -422,56 +474,44 @@ __device__ __forceinline__ void dust_kinetic_flux(const T* WL, const T* WR, T* F
 }
 
 // ------------------------------------------------------------------ sources
-// App. B sources per unit volume at the cell centre: geometric terms,
-// stellar gravity (Sect. 2.1), the rotating-frame Coriolis / centrifugal
-// terms and, when switched on, the indirect gravity of Sect. 2.10 (force
-// -grad Phi_ind on gas and dust, and its work on the gas); the Box has none.
-// XT = false compiles the optional terms out.
-template <bool XT>
-__device__ __forceinline__ void cell_sources(const DevGrid& g, int i, int j, int k, const double* U, double* S) {
-  const double r = g.rc[i + GH];
-  const double z = g.x0[2] + (k + 0.5) * g.dx[2];
-  const double R2 = r * r + z * z;
-  const double R3 = R2 * sqrt(R2);
-  const double fr = -g.gm * r / R3, fz = -g.gm * z / R3;
-  const double Om = g.omega;
-  {
-    const double rho = U[RHO];
-    const double ir = 1.0 / rho;
-    const double u = U[MU] * ir, v = U[MV] * ir, w = U[MW] * ir;
-    const double P = gas_pressure(g.gamma, U[MU], U[MV], U[MW], U[EN], rho);
-    S[MU] = rho * v * v / r + P / r + rho * fr + 2.0 * Om * rho * v + rho * Om * Om * r;
-    S[MV] = -rho * u * v / r - 2.0 * Om * rho * u;
-    S[MW] = rho * fz;
-    S[EN] = rho * u * (fr + Om * Om * r) + rho * w * fz;
-    S[RHO] = 0.0;
+// G += V S, S the App. B sources per unit volume at the cell centre: geometric
+// terms, stellar gravity (Sect. 2.1), the rotating-frame Coriolis /
+// centrifugal terms and, when switched on, the indirect gravity of Sect. 2.10
+// (force -grad Phi_ind on gas and dust, and its work on the gas); the Box has
+// none.  W: the cell's primitive gas state; Vd: the dust velocities (u, v) of
+// each species, zero where it has no mass.  XT = false compiles the optional
+// terms out.
+template <bool XT, int NF>
+__device__ __forceinline__ void add_sources(const DevGrid& g, int i, int j, int k, const double* U, const double* W,
+                                            const double (*Vd)[2], double* G) {
+  const double V = g.vol[i], ir = g.ir[i], Om2 = 2.0 * g.omega;
+  const size_t o = (size_t)k * g.nr + i;
+  const double a1 = g.grav[o], fz = g.grav[(size_t)g.nz * g.nr + o];
+  double gr = 0.0, gt = 0.0;
+  const bool ind = XT && g.x_ind != 0.0;
+  if (ind) {
+    gr = g.ind_g[j];
+    gt = g.ind_g[g.nth + j];  // grad Phi_ind, (r, theta)
   }
-  for (int b = 5; b < g.nf; b += 4) {  // each dust species
-    const double rho = U[b + 3];
-    if (rho > 0.0) {
-      const double ir = 1.0 / rho;
-      const double u = U[b] * ir, v = U[b + 1] * ir;
-      S[b] = rho * v * v / r + rho * fr + 2.0 * Om * rho * v + rho * Om * Om * r;
-      S[b + 1] = -rho * u * v / r - 2.0 * Om * rho * u;
-      S[b + 2] = rho * fz;
-    } else {
-      S[b] = S[b + 1] = S[b + 2] = 0.0;
-    }
-    S[b + 3] = 0.0;
+  const double ar = XT ? a1 - gr : a1;
+  G[MU] = fma(V, fma(ir, fma(U[MV], W[MV], W[EN]), fma(U[RHO], ar, Om2 * U[MV])), G[MU]);
+  double sv = -U[MU] * fma(W[MV], ir, Om2), se = fma(U[MU], ar, U[MW] * fz);
+  if (ind) {
+    sv -= U[RHO] * gt;
+    se -= U[MV] * gt;
   }
-  if (XT && g.x_ind != 0.0) {
-    const double gr = g.ind_g[j], gt = g.ind_g[g.nth + j];  // grad Phi_ind, (r, theta)
-    const double rho = U[RHO];
-    const double ir = 1.0 / rho;
-    S[MU] -= rho * gr;
-    S[MV] -= rho * gt;
-    S[EN] -= rho * (U[MU] * ir * gr + U[MV] * ir * gt);
-    for (int b = 5; b < g.nf; b += 4) {
-      if (U[b + 3] > 0.0) {
-        S[b] -= U[b + 3] * gr;
-        S[b + 1] -= U[b + 3] * gt;
-      }
-    }
+  G[MV] = fma(V, sv, G[MV]);
+  G[MW] = fma(V, U[RHO] * fz, G[MW]);
+  G[EN] = fma(V, se, G[EN]);
+#pragma unroll
+  for (int b = 5; b < NF; b += 4) {  // each dust species
+    const double v = Vd[(b - 5) / 4][1], rd = U[b + 3];
+    if (!positive(rd)) continue;
+    G[b] = fma(V, fma(U[b + 1], fma(v, ir, Om2), rd * ar), G[b]);
+    double sd = -U[b] * fma(v, ir, Om2);
+    if (ind) sd -= rd * gt;
+    G[b + 1] = fma(V, sd, G[b + 1]);
+    G[b + 2] = fma(V, rd * fz, G[b + 2]);
   }
 }
 
@@ -481,114 +521,121 @@ struct DragArgs {
   double rhos_rp;  // Epstein constant rho_s r_p (drag laws 1 and 2)
   int law;
   double kappa;    // drag law 2: r_p / lambda_0, the mean free path being lambda_0 / rho_g
+  // 1 / (St x factor) and 1 / (rho_s r_p x factor) of each species, formed on
+  // the host: a division per cell and species is eight FP64 operations
+  double ist[ND_MAX], irr[ND_MAX];
 };
 
-// Stopping time of dust species s (Stokes number St x st_factor[s]) in a cell
-// of radial index i with gas state U (Sect. 2.9): drag law 0 t_s = St /
-// Omega_K(r) (the Box: St); laws 1 and 2 Epstein t_s = rho_s r_p /
-// (rho_g c_s), rho_s r_p proportional to St; law 2 (compiled in with XT) adds
-// the Stokes regime of Sect. 2.9: above r_p = 9 lambda / 4 the Epstein time
-// grows by (4/9) r_p / lambda.
+// 1 / t_s of dust species s (Stokes number St x st_factor[s]) in a cell of
+// radial index i with gas density rg and pressure P (Sect. 2.9): drag law 0
+// t_s = St / Omega_K(r) (the Box: St); laws 1 and 2 Epstein t_s = rho_s r_p /
+// (rho_g c_s), rho_s r_p proportional to St, with rho_g c_s = sqrt(gamma P
+// rho_g); law 2 (compiled in with XT) adds the Stokes regime of Sect. 2.9:
+// above r_p = 9 lambda / 4 the Epstein time grows by (4/9) r_p / lambda.
 template <bool XT>
-__device__ __forceinline__ double stopping_time(const DevGrid& g, int i, const double* U, const DragArgs& d, int s) {
-  const double rg = U[RHO];
-  if (d.law == 0) {
-    const double st = d.stokes * g.st_factor[s];
-    if (g.geom == GEOM_CYL) {
-      const double r = g.rc[i + GH];
-      return st / sqrt(g.gm / (r * r * r));
-    }
-    return st;
+__device__ __forceinline__ double inv_stopping_time(const DevGrid& g, int i, double rg, double P, const DragArgs& d,
+                                                    int s) {
+  if (d.law == 0) return g.omk[i] * d.ist[s];
+  double it = root(g.gamma * P * rg) * d.irr[s];
+  if (XT && d.law == 2) {
+    const double x = d.kappa * rg;
+    if (positive(x - 2.25)) it *= 2.25 * recip(x);
   }
-  const double cs = sqrt(g.gamma * gas_pressure(g.gamma, U[MU], U[MV], U[MW], U[EN], rg) / rg);
-  double ts = d.rhos_rp * g.st_factor[s] / (rg * cs);
-  if (XT && d.law == 2 && d.kappa * rg > 2.25) ts = ts * ((4.0 / 9.0) * (d.kappa * rg));
-  return ts;
+  return it;
 }
 
 // Semi-implicit drag over a stage of length tau (Sect. 2.9 drag law).  One
-// dust species: the relative gas-dust velocity relaxes by
-// 1 / (1 + tau (1 + eps) / t_s) at fixed barycentric velocity.  ND > 1
-// species: the backward-Euler system of the gas coupled to each species
-// (no dust-dust exchange) in closed form, v_g' = (rho_g v_g + sum rho_k w_k
-// v_k) / (rho_g + sum rho_k w_k), v_k' = (v_k + a_k v_g') / (1 + a_k), with
-// a_k = tau / t_k and w_k = a_k / (1 + a_k).  The gas energy gains the work
-// done on the gas in both.
+// dust species: the relative gas-dust velocity relaxes by 1 / (1 + k), k =
+// tau (1 + eps) / t_s, at fixed barycentric velocity; with a = tau / t_s the
+// momentum that changes hands is rho_d a / (1 + k) times the velocity
+// difference (no reduced mass to form).  ND > 1 species: the backward-Euler
+// system of the gas coupled to each species (no dust-dust exchange) in closed
+// form, v_g' = (rho_g v_g + sum rho_k w_k v_k) / (rho_g + sum rho_k w_k),
+// v_k' = (v_k + a_k v_g') / (1 + a_k), with a_k = tau / t_k and w_k =
+// a_k / (1 + a_k).  The gas energy gains the work done on the gas in both.
+// ig = 1 / rho_g, id = 1 / rho_d of each species (any value without mass).
 template <bool XT, int ND>
-__device__ __forceinline__ void apply_drag(const DevGrid& g, int i, double* U, double tau, const DragArgs& d) {
+__device__ __forceinline__ void apply_drag(const DevGrid& g, int i, double* U, double tau, const DragArgs& d,
+                                           double ig, const double* id) {
   const double rg = U[RHO];
+  if (!positive(rg)) return;
+  double P = 0.0;
+  if (d.law != 0)
+    P = (g.gamma - 1.0) * fma(-0.5 * ig, fma(U[MU], U[MU], fma(U[MV], U[MV], U[MW] * U[MW])), U[EN]);
   if constexpr (ND == 1) {
     const double rd = U[DRHO];
-    if (!(rd > 0.0) || !(rg > 0.0)) return;
-    const double ts = stopping_time<XT>(g, i, U, d, 0);
-    const double kk = tau * (1.0 + rd / rg) / ts;
-    const double mu = rg * rd / (rg + rd);
-    const double relax = kk / (1.0 + kk);
+    if (!positive(rd)) return;
+    const double a = tau * inv_stopping_time<XT>(g, i, rg, P, d, 0);
+    const double K = rd * a * recip(1.0 + fma(a * rd, ig, a));
     double dE = 0.0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const double vg = U[MU + c] / rg;
-      const double X = mu * (U[DMU + c] / rd - vg) * relax;
+      const double vg = U[MU + c] * ig;
+      const double X = K * fma(U[DMU + c], id[0], -vg);
       U[MU + c] += X;
       U[DMU + c] -= X;
-      dE += 0.5 * X * (U[MU + c] / rg + vg);
+      dE = fma(X, fma(0.5 * ig, X, vg), dE);
     }
     U[EN] += dE;
   } else {
-  if (!(rg > 0.0)) return;
-  double a[ND], num[3], den = rg;
+    double a[ND], h[ND], num[3], den = rg;  // h = 1 / (1 + a), 0 for a species without mass
 #pragma unroll
-  for (int c = 0; c < 3; ++c) num[c] = U[MU + c];
-#pragma unroll
-  for (int s = 0; s < ND; ++s) {
-    const int b = 5 + 4 * s;
-    a[s] = 0.0;
-    if (!(U[b + 3] > 0.0)) continue;
-    a[s] = tau / stopping_time<XT>(g, i, U, d, s);
-    const double w = a[s] / (1.0 + a[s]);
-    den += U[b + 3] * w;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) num[c] += U[b + c] * w;
-  }
-  double dE = 0.0;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const double vg_ex = U[MU + c] / rg;
-    const double vg = num[c] / den;
+    for (int c = 0; c < 3; ++c) num[c] = U[MU + c];
 #pragma unroll
     for (int s = 0; s < ND; ++s) {
       const int b = 5 + 4 * s;
-      if (!(U[b + 3] > 0.0)) continue;
-      U[b + c] = U[b + 3] * ((U[b + c] / U[b + 3] + a[s] * vg) / (1.0 + a[s]));
+      a[s] = h[s] = 0.0;
+      if (!positive(U[b + 3])) continue;
+      a[s] = tau * inv_stopping_time<XT>(g, i, rg, P, d, s);
+      h[s] = recip(1.0 + a[s]);
+      const double w = a[s] * h[s];
+      den = fma(U[b + 3], w, den);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) num[c] = fma(U[b + c], w, num[c]);
     }
-    U[MU + c] = rg * vg;
-    dE += 0.5 * rg * (vg * vg - vg_ex * vg_ex);
-  }
-  U[EN] += dE;
+    const double iden = recip(den);
+    double dE = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double vg = num[c] * iden, m = rg * vg;
+      const double X = m - U[MU + c];  // what the gas gains
+#pragma unroll
+      for (int s = 0; s < ND; ++s) {
+        const int b = 5 + 4 * s;
+        if (!positive(U[b + 3])) continue;
+        U[b + c] = h[s] * fma(U[b + 3] * a[s], vg, U[b + c]);
+      }
+      dE = fma(0.5 * X, fma(U[MU + c], ig, vg), dE);
+      U[MU + c] = m;
+    }
+    U[EN] += dE;
   }
 }
 
 // ------------------------------------------------------------------ CFL
-// Sect. 2.5, Eq. (cfl condition) for one cell of radial index i.
-__device__ __forceinline__ double cell_dt(const DevGrid& g, int i, const double* U) {
-  const double rho = U[RHO];
-  const double vel = sqrt(U[MU] * U[MU] + U[MV] * U[MV] + U[MW] * U[MW]) / rho;
-  const double cs = sqrt(g.gamma * gas_pressure(g.gamma, U[MU], U[MV], U[MW], U[EN], rho) / rho);
-  const double V = g.vol[i], A = g.maxA[i];
-  double dt = g.cfl * V / ((vel + cs) * A);
-  for (int b = 5; b < g.nf; b += 4) {
-    if (!(U[b + 3] > 0.0)) continue;
-    const double vd = sqrt(U[b] * U[b] + U[b + 1] * U[b + 1] + U[b + 2] * U[b + 2]) / U[b + 3];
-    if (vd > 0.0) dt = fmin(dt, g.cfl * V / (vd * A));
+// Sect. 2.5, Eq. (cfl condition): the largest (|v| + c) A / V and |v_d| A / V
+// of one cell of radial index i (the step is N_CFL over their maximum: one
+// division per block instead of one per cell), and whether the cell is not
+// physical.  ig, id: as apply_drag.
+template <int NF>
+__device__ __forceinline__ double cell_rate(const DevGrid& g, int i, const double* U, double ig, const double* id,
+                                            bool& bad) {
+  const double u = U[MU] * ig, v = U[MV] * ig, w = U[MW] * ig;
+  const double q = fma(u, u, fma(v, v, w * w));
+  const double P = (g.gamma - 1.0) * fma(-0.5 * U[RHO], q, U[EN]);
+  bad = !positive(U[RHO]) || !positive(P);
+  double rate = root(g.gamma * P * ig) + (positive(q) ? root(q) : 0.0);
+#pragma unroll
+  for (int b = 5; b < NF; b += 4) {
+    const double j = id[(b - 5) / 4], ud = U[b] * j, vd = U[b + 1] * j, wd = U[b + 2] * j;
+    const double d2 = fma(ud, ud, fma(vd, vd, wd * wd));
+    if (positive(U[b + 3]) && positive(d2)) {
+      const double vel = root(d2);
+      if (mag_less(rate, vel)) rate = vel;
+    }
+    bad |= !non_negative(U[b + 3]);
   }
-  return dt;
-}
-
-__device__ __forceinline__ bool cell_nonphysical(const DevGrid& g, const double* U) {
-  const double P = gas_pressure(g.gamma, U[MU], U[MV], U[MW], U[EN], U[RHO]);
-  bool bad = !(U[RHO] > 0.0) || !(P > 0.0);
-  for (int b = 5; b < g.nf; b += 4) bad |= !(U[b + 3] >= 0.0);
-  return bad;
+  return rate * g.aov[i];
 }
 
 // Positive doubles order like their bit patterns, so a 64-bit integer

@@ -1,0 +1,113 @@
+// Scalar building blocks that keep work off GB300's FP64 pipe.
+//
+// An SM has two FP64 lanes against 128 for FP32 and 64 or more for integers:
+// one FP64 instruction of a warp occupies its pipe for 16 clocks, in which
+// the SM's schedulers could issue 64 others.  What needs no 64-bit rounding
+// (comparisons, selections, conversions between the float types, a Newton
+// correction that is already small) therefore runs on the bits or in float;
+// compares and conversions of doubles would take an FP64 slot each.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace rossbi {
+
+// ---------------------------------------------------------------- doubles by their bits
+__device__ __forceinline__ bool sign_bit(double x) { return __double2hiint(x) < 0; }
+__device__ __forceinline__ bool sign_bit(float x) { return __float_as_int(x) < 0; }
+
+// x > 0, false for NaN (the bits of +inf and below, above +0).
+__device__ __forceinline__ bool positive(double x) {
+  return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+
+// x >= 0, false for NaN.
+__device__ __forceinline__ bool non_negative(double x) {
+  return positive(x) || ((unsigned long long)__double_as_longlong(x) << 1) == 0;
+}
+__device__ __forceinline__ bool non_negative(float x) { return x >= 0.0f; }
+
+// |a| < |b| (magnitudes of non-NaN values order like their bits).
+__device__ __forceinline__ bool mag_less(double a, double b) {
+  return (__double_as_longlong(a) & 0x7fffffffffffffffll) < (__double_as_longlong(b) & 0x7fffffffffffffffll);
+}
+
+// max(x, 0) and min(x, 0)
+__device__ __forceinline__ double pos_part(double x) { return sign_bit(x) ? 0.0 : x; }
+__device__ __forceinline__ double neg_part(double x) { return sign_bit(x) ? x : 0.0; }
+__device__ __forceinline__ float pos_part(float x) { return fmaxf(x, 0.0f); }
+__device__ __forceinline__ float neg_part(float x) { return fminf(x, 0.0f); }
+
+// The smaller of two values of one sign in magnitude.
+__device__ __forceinline__ double min_mag(double a, double b) { return mag_less(a, b) ? a : b; }
+
+// MinMod slope: 0 where the signs differ.
+__device__ __forceinline__ double minmod_bits(double a, double b) {
+  const double m = min_mag(a, b);
+  return (__double2hiint(a) ^ __double2hiint(b)) < 0 ? 0.0 : m;
+}
+
+// min(|a|, |b|) with the sign of a * b (one instruction).
+__device__ __forceinline__ float min_xorsign(float a, float b) {
+  float r;
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+// double -> float by truncation, flushed to 0 below and held at FLT_MAX above
+// float's range; float -> double, exact for normal values, subnormals to 0.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  unsigned b = __funnelshift_l(lo, hi & 0x7fffffffu, 3) - (896u << 23);
+  b = e - 897u < 254u ? b & 0x7fffffffu : (e < 897u ? 0u : 0x7f7fffffu);
+  return __uint_as_float(b | (hi & 0x80000000u));
+}
+__device__ __forceinline__ float narrow(float x) { return x; }
+template <class T> __device__ __forceinline__ T widen(float x);
+template <> __device__ __forceinline__ float widen<float>(float x) { return x; }
+template <> __device__ __forceinline__ double widen<double>(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  const unsigned hi = m < 0x00800000u ? 0u : (m >> 3) + (896u << 20);
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(m < 0x00800000u ? 0u : b << 29));
+}
+
+// ---------------------------------------------------------------- reciprocals
+// One step of the third-order Householder iteration (y (1 + e + e^2) with
+// e = 1 - x y for 1/x; y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 for x^-1/2)
+// from the PTX approximation, whose error of about 2^-20 it takes below
+// 2^-59: three and five FP64 operations, where the correctly rounded division
+// and square root with their scaling take 8 and more.  Zero, infinite and
+// subnormal arguments give NaN: the callers test positivity first.
+__device__ __forceinline__ double recip(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double recip_sqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ float recip(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float recip_sqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// sqrt(x), x > 0
+__device__ __forceinline__ double root(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double t = x * y, e = fma(-t, y, 1.0);
+  return fma(t * e, fma(0.375, e, 0.5), t);
+}
+__device__ __forceinline__ float root(float x) { return x * recip_sqrt(x); }
+
+}  // namespace rossbi

@@ -1,0 +1,222 @@
+// Exact Riemann solution on the face (Sect. 2.6) where the star pressure is
+// close to both side pressures, |x_K| <= 1/32 with x_K = p*/p_K - 1: every
+// face of a smooth flow, and all but a few cells around a strong shock.
+//
+// There the pressure function of a side is f_K = x p_K / (rho_K c_K) S(x),
+// its derivative T(x) / (rho_K c_K) with T = (x S)', and the star density
+// rho_K (1 + x D(x)); S, D are the Taylor series of the rarefaction branch
+// (x <= 0) or of the shock branch, which agree to first order, so that one
+// straight line of code with selected coefficients serves both and the lanes
+// of a warp do not diverge.  With beta = (gamma - 1)/(2 gamma):
+//   rarefaction  S_k = C(beta, k+1)/beta,   D_k = C(1/gamma, k+1),
+//   shock        S_k = C(-1/2, k) ((gamma+1)/(2 gamma))^k,  D_k = (-beta)^k / gamma.
+// The differences that enter (p_R - p_L, u_R - u_L) are the caller's, so the
+// perturbation forms pass theirs exactly.
+//
+// In double the Newton iteration runs in float and its result is corrected by
+// FP64 residuals: step = -F/F' with F in FP64 and the quotient in float.  A
+// step has a relative error of about 2^-21, so the iteration ends once it is
+// below 2^-32 p (one evaluation of F for |x| up to about 2^-11, two up to
+// 1/32) and p* is then exact to the last bits, as the FP64 iteration's is.
+// The series are summed in double to x^5, the rest (below 2^-30 of the sum)
+// in float.
+//
+// What bounds the callers: in FP64 the two-lane FP64 pipe, which sees about
+// 55 operations here against 250 to 300 of the FP64 Newton iteration with its
+// two branches; in float the issue slots.
+#pragma once
+#include "narrow.cuh"
+
+namespace rossbi {
+
+constexpr int NEAR_N = 6;  // FP64 terms of a series
+constexpr int NEAR_T = 5;  // float terms of its tail
+constexpr float NEAR_X = 0.03125f;
+
+// Series coefficients of one gamma, [0] rarefaction, [1] shock (built on the host).
+struct NearCoef {
+  double s[2][NEAR_N], d[2][NEAR_N];
+  float st[2][NEAR_T], dt[2][NEAR_T];  // tails: the terms x^6 ... x^10
+  double t[2][NEAR_N], h[2][NEAR_N];   // (x S)' and (x D)', for the adjoint
+  float tt[2][NEAR_T], ht[2][NEAR_T];
+  float sf[2][5], tf[2][5], df[2][5];  // S, T, D to x^4 in float
+  double gamma, g_gm1;  // gamma, gamma / (gamma - 1)
+  float gammaf;
+};
+
+// Builds the coefficients of gamma (host).
+inline NearCoef near_coef(double gamma) {
+  NearCoef c{};
+  const double beta = (gamma - 1.0) / (2.0 * gamma), alpha = (gamma + 1.0) / (2.0 * gamma), ig = 1.0 / gamma;
+  double bb = beta, bg = ig, bh = 1.0, al = 1.0, be = ig;  // C(beta, k+1), C(1/gamma, k+1), C(-1/2, k), alpha^k, (-beta)^k / gamma
+  for (int k = 0; k < NEAR_N + NEAR_T; ++k) {
+    const double s[2] = {bb / beta, bh * al}, d[2] = {bg, be};
+    for (int q = 0; q < 2; ++q) {
+      if (k < NEAR_N) {
+        c.s[q][k] = s[q];
+        c.d[q][k] = d[q];
+        c.t[q][k] = (k + 1) * s[q];
+        c.h[q][k] = (k + 1) * d[q];
+      } else {
+        c.st[q][k - NEAR_N] = (float)s[q];
+        c.dt[q][k - NEAR_N] = (float)d[q];
+        c.tt[q][k - NEAR_N] = (float)((k + 1) * s[q]);
+        c.ht[q][k - NEAR_N] = (float)((k + 1) * d[q]);
+      }
+      if (k < 5) {
+        c.sf[q][k] = (float)s[q];
+        c.tf[q][k] = (float)((k + 1) * s[q]);
+        c.df[q][k] = (float)d[q];
+      }
+    }
+    bb *= (beta - (k + 1)) / (k + 2);
+    bg *= (ig - (k + 1)) / (k + 2);
+    bh *= (-0.5 - k) / (k + 1);
+    al *= alpha;
+    be *= -beta;
+  }
+  c.gamma = gamma;
+  c.g_gm1 = gamma / (gamma - 1.0);
+  c.gammaf = (float)gamma;
+  return c;
+}
+
+// Float series to x^4; the branches share the first two coefficients.
+__device__ __forceinline__ float near_sum_f(const float (&c)[2][5], bool shock, float x) {
+  float t = shock ? c[1][4] : c[0][4];
+#pragma unroll
+  for (int k = 3; k >= 2; --k) t = fmaf(t, x, shock ? c[1][k] : c[0][k]);
+  return fmaf(fmaf(t, x, c[0][1]), x, c[0][0]);
+}
+__device__ __forceinline__ float near_sum(const float (&c)[2][5], const double (&)[2][NEAR_N],
+                                          const float (&)[2][NEAR_T], bool shock, float x) {
+  return near_sum_f(c, shock, x);
+}
+__device__ __forceinline__ double near_sum(const float (&)[2][5], const double (&c)[2][NEAR_N],
+                                           const float (&ct)[2][NEAR_T], bool shock, double x) {
+  const float xf = narrow(x);
+  float t = shock ? ct[1][NEAR_T - 1] : ct[0][NEAR_T - 1];
+#pragma unroll
+  for (int k = NEAR_T - 2; k >= 0; --k) t = fmaf(t, xf, shock ? ct[1][k] : ct[0][k]);
+  double v = widen<double>(t);
+#pragma unroll
+  for (int k = NEAR_N - 1; k >= 2; --k) v = fma(v, x, shock ? c[1][k] : c[0][k]);
+  return fma(fma(v, x, c[0][1]), x, c[0][0]);
+}
+
+enum { NEAR_GENERAL = 0, NEAR_LEFT = 1, NEAR_RIGHT = 2, NEAR_STAR_L = 3, NEAR_STAR_R = 4 };
+
+// What the solution needs beyond the face state (the adjoint reads it).
+template <class T>
+struct NearStar {
+  T d;          // p* - p_L
+  T us;         // u* about the base velocity of ul, ur
+  T drho;       // rho* - rho_K of the side K that the face lies on
+  T fl, fr;     // pressure functions at p*
+  T ircl, ircr, ipl, ipr;
+};
+
+// Which state is on the face: NEAR_LEFT / NEAR_RIGHT (the side's own, the
+// flow being supersonic), NEAR_STAR_L / NEAR_STAR_R (the star state of that
+// side; s is set), or NEAR_GENERAL: not near, or within the sonic band where
+// a fan or a shock may sit on the face; the caller then takes the general
+// solver.  (rl, pl), (rr, pr): positive densities and pressures; dP = p_R -
+// p_L, ul, ur velocities about u0, dU = u_R - u_L; ulf, urf the full
+// velocities in float.
+template <class T>
+__device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl, T rr, T ur, T pr, T dP, T dU, T u0,
+                                            bool has_u0, float ulf, float urf, NearStar<T>& s) {
+  const float plf = narrow(pl), prf = narrow(pr), rlf = narrow(rl), rrf = narrow(rr);
+  // outside float's comfortable range: the general solver
+  if (!(fmaxf(fmaxf(plf, prf), fmaxf(rlf, rrf)) < 1e30f)) return NEAR_GENERAL;
+  const float gl = C.gammaf * plf, gr = C.gammaf * prf;
+  const float il = recip_sqrt(gl) * recip_sqrt(rlf), ir = recip_sqrt(gr) * recip_sqrt(rrf);  // 1 / (rho c)
+  const float cl = gl * il, cr = gr * ir;
+  const float ipl = recip(plf), ipr = recip(prf);
+  const float dPf = narrow(dP), dUf = narrow(dU);
+  // linear (acoustic) star pressure d = p* - p_L
+  float d = (dPf * ir - dUf) * recip(il + ir);
+  float xl = d * ipl, xr = (d - dPf) * ipr;
+  float X = fabsf(xl) + fabsf(xr);
+  if (!(X <= NEAR_X)) return NEAR_GENERAL;  // NaN too
+  // supersonic by a margin that covers every wave speed at |x| <= 1/32
+  if (ulf >= 1.1f * cl) return NEAR_LEFT;
+  if (-urf >= 1.1f * cr) return NEAR_RIGHT;
+  float fl, fr, tl, tr;
+  if constexpr (sizeof(T) == 4) {
+    // Newton in float: the error after a step is 0.43 step^2 / p at most
+    // ((gamma + 1)/(4 gamma) < 1/2), below the rounding of d once
+    // step^2 < 2^-23 |d| p
+    bool more = true;
+    for (int it = 0; it < 6 && more; ++it) {
+      const bool sl = d > 0.0f, sr = d > dPf;
+      xl = d * ipl;
+      xr = (d - dPf) * ipr;
+      fl = d * il * near_sum_f(C.sf, sl, xl);
+      fr = (d - dPf) * ir * near_sum_f(C.sf, sr, xr);
+      tl = il * near_sum_f(C.tf, sl, xl);
+      tr = ir * near_sum_f(C.tf, sr, xr);
+      const float step = -(fl + fr + dUf) * recip(tl + tr);
+      d += step;
+      fl += tl * step;
+      fr += tr * step;
+      const float scale = fabsf(d) + fabsf(d - dPf);
+      more = !(step * step <= 1.2e-7f * scale * fminf(plf, prf)) && fabsf(step) > 2.4e-7f * scale;
+    }
+    s.d = d;
+    s.fl = fl;
+    s.fr = fr;
+    s.us = 0.5f * ((ul - fl) + (ur + fr));
+    s.ipl = ipl;
+    s.ipr = ipr;
+  } else {
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+      const bool sl = d > 0.0f, sr = d > dPf;
+      xl = d * ipl;
+      xr = (d - dPf) * ipr;
+      tl = il * near_sum_f(C.tf, sl, xl);
+      tr = ir * near_sum_f(C.tf, sr, xr);
+      d -= (d * il * near_sum_f(C.sf, sl, xl) + (d - dPf) * ir * near_sum_f(C.sf, sr, xr) + dUf) * recip(tl + tr);
+    }
+    const float iD = recip(tl + tr), small = 2.3e-10f * fminf(plf, prf);
+    s.ircl = recip_sqrt(C.gamma * (pl * rl));
+    s.ircr = recip_sqrt(C.gamma * (pr * rr));
+    s.ipl = recip(pl);
+    s.ipr = recip(pr);
+    T dd = widen<T>(d), f1 = T(0), f2 = T(0);
+    float step = 0.0f;
+    bool more = true;
+    for (int it = 0; it < 4 && more; ++it) {
+      const T dr = dd - dP;
+      const T yl = dd * s.ipl, yr = dr * s.ipr;
+      const bool sl = !sign_bit(yl), sr = !sign_bit(yr);
+      f1 = dd * s.ircl * near_sum(C.sf, C.s, C.st, sl, yl);
+      f2 = dr * s.ircr * near_sum(C.sf, C.s, C.st, sr, yr);
+      step = -narrow(f1 + f2 + dU) * iD;
+      dd += widen<T>(step);
+      more = !(fabsf(step) <= small);
+    }
+    if (more) return NEAR_GENERAL;
+    s.d = dd;
+    s.fl = f1 + widen<T>(tl * step);
+    s.fr = f2 + widen<T>(tr * step);
+    s.us = T(0.5) * ((ul - s.fl) + (ur + s.fr));
+    d = narrow(dd);
+  }
+  xl = d * ipl;
+  xr = (d - dPf) * ipr;
+  X = fabsf(xl) + fabsf(xr);
+  if (!(X <= 1.25f * NEAR_X)) return NEAR_GENERAL;
+  const bool left = !sign_bit(has_u0 ? u0 + s.us : s.us);
+  // the head of side K is at u_K -/+ c_K, its shock or tail within |x| c_K of
+  // it: the side's own state beyond that band, the star state before it
+  const float v = left ? ulf : -urf, c = left ? cl : cr, band = c * (X + 1e-5f);
+  if (v - c >= band) return left ? NEAR_LEFT : NEAR_RIGHT;
+  if (!(c - v > band)) return NEAR_GENERAL;
+  const T x = left ? s.d * s.ipl : (s.d - dP) * s.ipr;
+  s.drho = (left ? rl : rr) * (x * near_sum(C.df, C.d, C.dt, !sign_bit(x), x));
+  return left ? NEAR_STAR_L : NEAR_STAR_R;
+}
+
+}  // namespace rossbi

@@ -35,7 +35,8 @@ struct rossbi_grid {
   rossbi_disc_params disc{};
   // device tables
   double *d_rc = nullptr, *d_rf = nullptr, *d_rcoef = nullptr, *d_vol = nullptr, *d_ivol = nullptr;
-  double *d_area_r = nullptr, *d_area_t = nullptr, *d_area_z = nullptr, *d_maxA = nullptr;
+  double *d_area_r = nullptr, *d_area_t = nullptr, *d_area_z = nullptr, *d_aov = nullptr;
+  double *d_ir = nullptr, *d_omk = nullptr, *d_grav = nullptr;
   double *d_e0c = nullptr, *d_e0r = nullptr, *d_e0z = nullptr, *d_r0 = nullptr;
   double* d_w0 = nullptr;              // primitive equilibrium tables (centres, r faces, z faces)
   std::vector<double> h_e0c;
@@ -187,19 +188,24 @@ rossbi_status sync_and_status(rossbi_grid* g) {
 }
 
 // ---------------------------------------------------------------- kernels
+template <int NF>
 __global__ void cfl_kernel(DevGrid g, StageArgs a, unsigned long long* slot) {
   __shared__ double red[CFL_NT / 32];
   const size_t ncell = (size_t)g.nr * g.nth * g.nz;
-  double m = INFINITY;
+  double rate = 0.0;
   unsigned status = 0;
   for (size_t lin = blockIdx.x * (size_t)CFL_NT + threadIdx.x; lin < ncell; lin += (size_t)gridDim.x * CFL_NT) {
-    double U[NF_MAX];
-    for (int f = 0; f < g.nf; ++f) U[f] = a.in[f][lin];
-    const int i = (int)(lin % g.nr);
-    if (cell_nonphysical(g, U)) status |= STATUS_NONPHYSICAL;
-    m = fmin(m, cell_dt(g, i, U));
+    double U[NF], id[NF > 5 ? (NF - 5) / 4 : 1];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) U[f] = a.in[f][lin];
+#pragma unroll
+    for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = recip(U[b + 3]);
+    bool bad = false;
+    const double c = cell_rate<NF>(g, (int)(lin % g.nr), U, recip(U[RHO]), id, bad);
+    if (bad) status |= STATUS_NONPHYSICAL;
+    if (positive(c) && mag_less(rate, c)) rate = c;
   }
-  m = block_min<CFL_NT>(m, red);
+  const double m = block_min<CFL_NT>(positive(rate) ? g.cfl / rate : INFINITY, red);
   if (threadIdx.x == 0) atomic_min_pos_double(slot, m);
   if (status) atomicOr(a.status, status);
 }
@@ -525,7 +531,7 @@ rossbi_status build_pert_tables(rossbi_grid* g, PertTables<T>& pt) {
       cudaMemcpy(ar.data(), g->d_area_r, ar.size() * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
       cudaMemcpy(at.data(), g->d_area_t, nr * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
       cudaMemcpy(az.data(), g->d_area_z, nr * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
-      cudaMemcpy(ma.data(), g->d_maxA, nr * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
+      cudaMemcpy(ma.data(), g->d_aov, nr * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
     return ROSSBI_ERR_CUDA;
   for (size_t q = 0; q < rcoef.size(); ++q) h[off_rc + q] = rcoef[q];
   for (int i = 0; i < nr; ++i) {
@@ -597,7 +603,7 @@ rossbi_status build_pert_tables(rossbi_grid* g, PertTables<T>& pt) {
   pt.area_r = b + off_ar;
   pt.area_t = b + off_at;
   pt.area_z = b + off_az;
-  pt.maxA = b + off_ma;
+  pt.aov = b + off_ma;
   pt.omk = b + off_om;
   if (!g->d_fallbacks) {
     CK(cudaMalloc(&g->d_fallbacks, sizeof(unsigned long long)));
@@ -644,7 +650,7 @@ void set_pert_drag(PertArgs<T>& a, const DragArgs& drag) {
 // Drag parameters of a step (Sect. 2.9 drag law; Epstein constant fixed so
 // that the Stokes number holds at r = 1, z = 0).
 rossbi_status drag_args(rossbi_grid* g, const rossbi_dust_params* dust, DragArgs& drag) {
-  drag = DragArgs{0.0, 0.0, 0, 0.0};
+  drag = DragArgs{};
   if (g->nf > 5) {
     drag.stokes = dust->stokes;
     drag.law = dust->drag_law;
@@ -662,6 +668,10 @@ rossbi_status drag_args(rossbi_grid* g, const rossbi_dust_params* dust, DragArgs
       drag.rhos_rp = dust->stokes * rho1 * std::sqrt(g->desc.gamma * p1 / rho1) / std::sqrt(g->desc.gm);
     } else if (dust->drag_law != 0) {
       return ROSSBI_ERR_ARG;
+    }
+    for (int s = 0; s < ND_MAX; ++s) {
+      drag.ist[s] = 1.0 / (drag.stokes * g->dg.st_factor[s]);
+      drag.irr[s] = 1.0 / (drag.rhos_rp * g->dg.st_factor[s]);
     }
   }
   return ROSSBI_OK;
@@ -1017,12 +1027,11 @@ rossbi_status adjoint_step(rossbi_grid* g, void* const* state, double dt, const 
     LamS[f] = g->d_adj + 4 * nfc + f * g->ncell;
   }
   // forward recompute from E^n: the stage kernels with the drag switched off
-  // (t_s = infinity makes apply_drag the identity) give the pre-drag states
+  // (1 / t_s = 0 makes apply_drag the identity) give the pre-drag states
   const int nblocks = n_tiles(g);
   StageArgs a = base_args(g);
   a.drag = drag;
-  a.drag.stokes = INFINITY;
-  a.drag.rhos_rp = INFINITY;
+  for (int sp = 0; sp < ND_MAX; ++sp) a.drag.ist[sp] = a.drag.irr[sp] = 0.0;
   a.dt_host = dt;
   for (int f = 0; f < g->nf; ++f) {
     a.in[f] = (const double*)state[f];
@@ -1154,7 +1163,7 @@ int rossbi_precision(const rossbi_grid* g) { return g ? g->desc.precision : -1; 
 void rossbi_destroy(rossbi_grid* g) {
   if (!g) return;
   double* tabs[] = {g->d_rc, g->d_rf, g->d_rcoef, g->d_vol, g->d_ivol, g->d_area_r, g->d_area_t,
-                    g->d_area_z, g->d_maxA, g->d_e0c, g->d_e0r, g->d_e0z, g->d_r0, g->d_partials, g->d_sums};
+                    g->d_area_z, g->d_aov, g->d_ir, g->d_omk, g->d_grav, g->d_e0c, g->d_e0r, g->d_e0z, g->d_r0, g->d_partials, g->d_sums};
   for (double* p : tabs)
     if (p) cudaFree(p);
   if (g->d_dt) cudaFree(g->d_dt);
@@ -1209,15 +1218,18 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
     const double xm = rc[i - 1 + GH], x0 = rc[i + GH], xp = rc[i + 1 + GH];
     const double fm = rf[i + GH], fp = rf[i + 1 + GH];
     double* w = &rcoef[(size_t)(i + 1) * RCW];
-    w[0] = 1.0 / (x0 - xm);
-    w[1] = 1.0 / (xp - x0);
-    w[2] = 1.0 / (xp - xm);
-    w[3] = x0 - xm;
-    w[4] = xp - x0;
-    w[5] = fm - x0;
-    w[6] = fp - x0;
-    w[7] = -std::min(2.0 * (x0 - fm), x0 - xm);  // limiter reach on the lower side
-    w[8] = std::min(2.0 * (fp - x0), xp - x0);   // and on the upper side
+    // The parabola through the three centres at the face distances hm, hp from
+    // x0, in the differences dm = e0 - em, dp = ep - e0:
+    // q(x0 - hm) = e0 - (w2 dm + w3 dp), q(x0 + hp) = e0 + (w4 dm + w5 dp)
+    const double hm = x0 - fm, hp = fp - x0, dl = x0 - xm, dr = xp - x0, dx = xp - xm;
+    w[0] = 1.0 / dl;
+    w[1] = 1.0 / dr;
+    w[2] = hm * (dr + hm) / (dl * dx);
+    w[3] = hm * (dl - hm) / (dr * dx);
+    w[4] = hp * (dr - hp) / (dl * dx);
+    w[5] = hp * (dl + hp) / (dr * dx);
+    w[6] = std::min(2.0 * hm, dl);  // limiter reach on the lower side
+    w[7] = std::min(2.0 * hp, dr);  // and on the upper side
   }
   std::vector<double> vol(nr), ivol(nr), ar(nr + 1), at(nr), az(nr), maxA(nr);
   if (d.geometry == ROSSBI_GEOM_CYL) {  // Sect. 2.2 finite volumes of the cylindrical mesh
@@ -1239,7 +1251,20 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
       maxA[i] = std::max(ar[i], std::max(at[i], az[i]));
     }
   }
-  for (int i = 0; i < nr; ++i) ivol[i] = 1.0 / vol[i];
+  std::vector<double> ir(nr, 0.0), omk(nr, 1.0), grav((size_t)2 * d.nz * nr, 0.0);
+  for (int i = 0; i < nr; ++i) {
+    ivol[i] = 1.0 / vol[i];
+    maxA[i] /= vol[i];
+    if (d.geometry != ROSSBI_GEOM_CYL) continue;
+    const double r = rc[i + GH];
+    ir[i] = 1.0 / r;
+    omk[i] = std::sqrt(d.gm / (r * r * r));
+    for (int k = 0; k < d.nz; ++k) {  // stellar gravity and the frame's centrifugal term at the cell centres
+      const double z = d.x0[2] + (k + 0.5) * dz, R2 = r * r + z * z, R3 = R2 * std::sqrt(R2);
+      grav[(size_t)k * nr + i] = -d.gm * r / R3 + d.omega_frame * d.omega_frame * r;
+      grav[(size_t)(d.nz + k) * nr + i] = -d.gm * z / R3;
+    }
+  }
   rossbi_status st = ROSSBI_OK;
   do {
     if ((st = upload(&g->d_rc, rc, g->stream)) != ROSSBI_OK) break;
@@ -1250,7 +1275,10 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
     if ((st = upload(&g->d_area_r, ar, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_area_t, at, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_area_z, az, g->stream)) != ROSSBI_OK) break;
-    if ((st = upload(&g->d_maxA, maxA, g->stream)) != ROSSBI_OK) break;
+    if ((st = upload(&g->d_aov, maxA, g->stream)) != ROSSBI_OK) break;
+    if ((st = upload(&g->d_ir, ir, g->stream)) != ROSSBI_OK) break;
+    if ((st = upload(&g->d_omk, omk, g->stream)) != ROSSBI_OK) break;
+    if ((st = upload(&g->d_grav, grav, g->stream)) != ROSSBI_OK) break;
     if (cudaMalloc(&g->d_dt, 3 * sizeof(unsigned long long)) != cudaSuccess) { st = ROSSBI_ERR_OOM; break; }
     if (cudaMalloc(&g->d_sums, NF_MAX * sizeof(double)) != cudaSuccess) { st = ROSSBI_ERR_OOM; break; }
     if (cudaMalloc(&g->d_status, sizeof(unsigned)) != cudaSuccess) { st = ROSSBI_ERR_OOM; break; }
@@ -1289,7 +1317,11 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   dg.area_r = g->d_area_r;
   dg.area_t = g->d_area_t;
   dg.area_z = g->d_area_z;
-  dg.maxA = g->d_maxA;
+  dg.aov = g->d_aov;
+  dg.ir = g->d_ir;
+  dg.omk = g->d_omk;
+  dg.grav = g->d_grav;
+  dg.near = near_coef(d.gamma);
   *out = g;
   return ROSSBI_OK;
 }
@@ -1390,7 +1422,10 @@ rossbi_status rossbi_cfl_dt(rossbi_grid* g, const void* const* state, double* dt
   if (prec == ROSSBI_FP64) {
     StageArgs a = base_args(g);
     for (int f = 0; f < g->nf; ++f) a.in[f] = (const double*)state[f];
-    cfl_kernel<<<blocks, CFL_NT, 0, g->stream>>>(g->dg, a, slot);
+    CK(by_nf(g->nf, [&](auto nf) {
+      cfl_kernel<decltype(nf)::value><<<blocks, CFL_NT, 0, g->stream>>>(g->dg, a, slot);
+      return cudaGetLastError();
+    }));
   } else if (prec == ROSSBI_FP32_PERT) {
     PertArgs<float> a = pert_args<float>(g);
     for (int f = 0; f < g->nf; ++f) a.in[f] = (const float*)state[f];

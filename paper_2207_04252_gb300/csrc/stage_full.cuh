@@ -36,69 +36,92 @@ struct StageArgs {
   int tiles_r, tiles_z;  // tile counts along r and z (block -> tile: r fastest, then z, then theta)
 };
 
-template <class T>
-__device__ __forceinline__ T minmod(T a, T b) {
-  if (a * b <= T(0)) return T(0);
-  return fabs(a) < fabs(b) ? a : b;
-}
-
 // Parabola through three deviations (Sect. 2.7) with the MinMod limiter: each
 // face deviation is limited to minmod(deviation, s h), s the minmod slope and
-// h the signed limiter reach of that side.  w = {1/(x0-xm), 1/(xp-x0),
-// 1/(xp-xm), x0-xm, xp-x0, fm-x0, fp-x0, h-, h+}.  Returns false if flat.
-template <class T>
-__device__ __forceinline__ bool parabola(T em, T e0, T ep, const T* w, T& qm, T& qp) {
-  const T sm = (e0 - em) * w[0];
-  const T sp = (ep - e0) * w[1];
-  const T s = minmod(sm, sp);
-  const T a = (sp - sm) * w[2];
-  const T b = (sp * w[3] + sm * w[4]) * w[2];
-  qm = e0 + minmod(w[5] * (a * w[5] + b), s * w[7]);
-  qp = e0 + minmod(w[6] * (a * w[6] + b), s * w[8]);
-  return s != T(0);
+// h the limiter reach of that side.  With the differences dm = e0 - em and
+// dp = ep - e0 the parabola's face deviations are -(am dm + ap dp) and bm dm +
+// bp dp with positive weights (of the geometry alone, tabulated), so that
+// where dm and dp have one sign they have it too, and the limiter is a
+// minimum of magnitudes: w = {1/(x0-xm), 1/(xp-x0), am, ap, bm, bp, h-, h+}.
+// UNI: a uniform axis, where in units of the spacing am = bp = 3/8, ap = bm =
+// 1/8 and both reaches are 1.  8 (uniform) or 12 FP64 operations; forming the
+// slopes, the curvature and the limiter's products took 17 and four compares.
+template <bool UNI>
+__device__ __forceinline__ void parabola(double em, double e0, double ep, const double* w, double& qm, double& qp) {
+  const double dm = e0 - em, dp = ep - e0;
+  if (UNI) {
+    const double s = minmod_bits(dm, dp), u = 0.125 * (dm + dp);
+    qm = e0 - min_mag(fma(0.25, dm, u), s);
+    qp = e0 + min_mag(fma(0.25, dp, u), s);
+  } else {
+    const double s = minmod_bits(dm * w[0], dp * w[1]);
+    qm = e0 - min_mag(fma(w[2], dm, w[3] * dp), w[6] * s);
+    qp = e0 + min_mag(fma(w[4], dm, w[5] * dp), w[7] * s);
+  }
+}
+template <bool UNI>
+__device__ __forceinline__ void parabola(float em, float e0, float ep, const float* w, float& qm, float& qp) {
+  const float dm = e0 - em, dp = ep - e0;
+  if (UNI) {
+    const float s = fmaxf(min_xorsign(dm, dp), 0.0f), u = 0.125f * (dm + dp);
+    qm = e0 - min_xorsign(fmaf(0.25f, dm, u), s);
+    qp = e0 + min_xorsign(fmaf(0.25f, dp, u), s);
+  } else {
+    const float s = fmaxf(min_xorsign(dm * w[0], dp * w[1]), 0.0f);
+    qm = e0 - min_xorsign(fmaf(w[2], dm, w[3] * dp), w[6] * s);
+    qp = e0 + min_xorsign(fmaf(w[4], dm, w[5] * dp), w[7] * s);
+  }
 }
 
-// Parabola weights of a cell along axis D (axis 0 from the table, uniform axes closed form).
+// The branches of a double-precision parabola, for its adjoint: bit 0 the
+// slopes have one sign (the face values move with the neighbours), bit 1 the
+// lower slope is the smaller, bits 2, 3 the parabola's own lower / upper face
+// value is inside the limiter.
+template <bool UNI>
+__device__ __forceinline__ unsigned parabola_branches(double em, double e0, double ep, const double* w, double& qm,
+                                                      double& qp) {
+  const double dm = e0 - em, dp = ep - e0;
+  double sm = dm, sp = dp, A, B, lo, up;
+  if (UNI) {
+    const double u = 0.125 * (dm + dp);
+    A = fma(0.25, dm, u);
+    B = fma(0.25, dp, u);
+  } else {
+    sm = dm * w[0];
+    sp = dp * w[1];
+    A = fma(w[2], dm, w[3] * dp);
+    B = fma(w[4], dm, w[5] * dp);
+  }
+  const double s = minmod_bits(sm, sp);
+  lo = UNI ? s : w[6] * s;
+  up = UNI ? s : w[7] * s;
+  const bool a = mag_less(A, lo), b = mag_less(B, up);
+  qm = e0 - (a ? A : lo);
+  qp = e0 + (b ? B : up);
+  return (((unsigned long long)__double_as_longlong(s) << 1) != 0 ? 1u : 0u) | (mag_less(sm, sp) ? 2u : 0u) |
+         (a ? 4u : 0u) | (b ? 8u : 0u);
+}
+
+// Parabola weights of a cell of axis 0 (the uniform axes 1, 2 need none).
 template <class T, int D>
-__device__ __forceinline__ void parabola_weights(const T* rcoef, int gi, int nr, T h, T* w) {
+__device__ __forceinline__ void parabola_weights(const T* rcoef, int gi, int nr, T* w) {
   if (D == 0) {
     const int c = gi < -1 ? -1 : (gi > nr ? nr : gi);
     const T* cw = rcoef + (c + 1) * RCW;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) w[q] = cw[q];
-  } else {
-    w[0] = w[1] = T(1) / h;
-    w[2] = T(0.5) / h;
-    w[3] = w[4] = h;
-    w[5] = T(-0.5) * h;
-    w[6] = T(0.5) * h;
-    w[7] = -h;
-    w[8] = h;
+    for (int q = 0; q < RCW; ++q) w[q] = cw[q];
   }
 }
 
-// Primitive dust reconstruction (u, v, w, rho_d) of the cell at s (stride S
-// along the sweep) from the conservative shared-memory fields b .. b + 3 of
-// one dust species (momenta, then density).
-template <class T, int BOX, int S>
+// Dust reconstruction of the cell at s (stride S along the sweep) from the
+// staged primitives (u, v, w, rho_d) in the fields b .. b + 3.
+template <class T, int BOX, int S, bool UNI>
 __device__ __forceinline__ void dust_recon(const T* sE, int sidx, int b, const T* w, T* wm, T* wp) {
-  T pm[4], p0[4], pp[4];
-  const T* r = sE + (b + 3) * BOX + sidx;
-  pm[3] = r[-S];
-  p0[3] = r[0];
-  pp[3] = r[S];
-  const T im = pm[3] > T(0) ? T(1) / pm[3] : T(0);
-  const T i0 = p0[3] > T(0) ? T(1) / p0[3] : T(0);
-  const T ip = pp[3] > T(0) ? T(1) / pp[3] : T(0);
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const T* m = sE + (b + c) * BOX + sidx;
-    pm[c] = m[-S] * im;
-    p0[c] = m[0] * i0;
-    pp[c] = m[S] * ip;
+  for (int q = 0; q < 4; ++q) {
+    const T* r = sE + (b + q) * BOX + sidx;
+    parabola<UNI>(r[-S], r[0], r[S], w, wm[q], wp[q]);
   }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) parabola(pm[q], p0[q], pp[q], w, wm[q], wp[q]);
 }
 
 // Ghost rule of Sect. 2.4 for a cell index possibly outside the domain.
@@ -159,9 +182,9 @@ __device__ __forceinline__ void sweep_full(const StageArgs& a, const double* sE,
     const bool do_acc = line_ok && c >= 0 && c < TD && gd < nd;
     const int sidx = do_recon ? ((z + ZH) * BY + (y + 2)) * BX + (x + 2) : (ZH * BY + 2) * BX + 2;
 
-    // parabola weights of this cell along D
-    double w[9];
-    parabola_weights<double, D>(g.rcoef, gi, g.nr, g.dx[D], w);
+    constexpr bool UNI = D != 0;
+    double w[RCW];
+    parabola_weights<double, D>(g.rcoef, gi, g.nr, w);
     // equilibrium gas state (conservative, or primitive with RC = RECON_PRIM)
     // on the lower face of this cell (index along D = gd) and on its upper
     // face; table indices clamped
@@ -180,74 +203,49 @@ __device__ __forceinline__ void sweep_full(const StageArgs& a, const double* sE,
 
     // ---------------- gas: departures in slots 0..4
     {
-      double qm[5], qp[5];
-      bool shaped = false;
+      double WR[5], WP[5];  // primitives: right state of the lower face, left state of the upper face
+      {
+        double qm[5], qp[5];
 #pragma unroll
-      for (int f = 0; f < 5; ++f) {
-        const double* s = sE + f * BOX + sidx;
-        shaped |= parabola(s[-STRIDE], s[0], s[STRIDE], w, qm[f], qp[f]);
-      }
-      double F[5];
-      if (RC == RECON_PRIM) {
-        if (shaped && do_recon) {  // positivity of both reconstructed face states
-          const bool ok = eq_face(RHO, gd) + qm[RHO] > 0.0 && eq_face(RHO, gd + 1) + qp[RHO] > 0.0 &&
-                          eq_face(EN, gd) + qm[EN] > 0.0 && eq_face(EN, gd + 1) + qp[EN] > 0.0;
-          if (!ok) {
+        for (int f = 0; f < 5; ++f) {
+          const double* s = sE + f * BOX + sidx;
+          parabola<UNI>(s[-STRIDE], s[0], s[STRIDE], w, qm[f], qp[f]);
+        }
+        // face states E0 + q on both faces of this cell (Sect. 2.7); flat
+        // departures if either is not physical
+        auto face_states = [&]() {
+          double Um[5], Up[5];
 #pragma unroll
-            for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + sidx];
+          for (int f = 0; f < 5; ++f) {
+            Um[f] = eq_face(f, gd) + qm[f];
+            Up[f] = eq_face(f, gd + 1) + qp[f];
           }
-        }
-        double UL[5], UR[5];
-#pragma unroll
-        for (int f = 0; f < 5; ++f) {
-          const double ql = __shfl_up_sync(FULL, qp[f], 1, L);
-          const double w0 = do_face ? eq_face(f, gd) : 0.0;
-          UL[f] = w0 + ql;
-          UR[f] = w0 + qm[f];
-        }
-        if (do_face) {
-          gas_face_flux<D>(gam, UL, UR, F, status);
-#pragma unroll
-          for (int f = 0; f < 5; ++f) F[f] *= area;
-        } else {
-#pragma unroll
-          for (int f = 0; f < 5; ++f) F[f] = 0.0;
-        }
-      } else {
-        // face states E0 + q on both faces of this cell (Sect. 2.7 on App. B's
-        // E); flat departures if either is not physical
-        double Um[5], Up[5];
-#pragma unroll
-        for (int f = 0; f < 5; ++f) {
-          Um[f] = eq_face(f, gd) + qm[f];
-          Up[f] = eq_face(f, gd + 1) + qp[f];
-        }
-        double WL[5], WR[5], WP[5];
-        gas_prim(gam, Um, WR);  // right state of the lower face
-        gas_prim(gam, Up, WP);  // left state of the upper face, for the lane above
-        if (shaped && do_recon) {
-          const bool ok = Um[RHO] > 0.0 && Up[RHO] > 0.0 && WR[EN] > 0.0 && WP[EN] > 0.0;
-          if (!ok) {
+          if (RC == RECON_PRIM) {
 #pragma unroll
             for (int f = 0; f < 5; ++f) {
-              const double e = sE[f * BOX + sidx];
-              Um[f] = eq_face(f, gd) + e;
-              Up[f] = eq_face(f, gd + 1) + e;
+              WR[f] = Um[f];
+              WP[f] = Up[f];
             }
+          } else {
             gas_prim(gam, Um, WR);
             gas_prim(gam, Up, WP);
           }
+          return positive(Um[RHO]) && positive(Up[RHO]) && positive(WR[EN]) && positive(WP[EN]);
+        };
+        if (!face_states() && do_recon) {
+#pragma unroll
+          for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + sidx];
+          face_states();
         }
+      }
+      double F[5], WL[5];
 #pragma unroll
-        for (int f = 0; f < 5; ++f) WL[f] = __shfl_up_sync(FULL, WP[f], 1, L);
-        if (do_face) {
-          gas_face_flux<D>(gam, WL, WR, F, status);
+      for (int f = 0; f < 5; ++f) WL[f] = __shfl_up_sync(FULL, WP[f], 1, L);
+      if (do_face) {
+        gas_face_flux<D>(g.near, area, WL, WR, F, status);
+      } else {
 #pragma unroll
-          for (int f = 0; f < 5; ++f) F[f] *= area;
-        } else {
-#pragma unroll
-          for (int f = 0; f < 5; ++f) F[f] = 0.0;
-        }
+        for (int f = 0; f < 5; ++f) F[f] = 0.0;
       }
 #pragma unroll
       for (int f = 0; f < 5; ++f) {
@@ -264,16 +262,14 @@ __device__ __forceinline__ void sweep_full(const StageArgs& a, const double* sE,
 #pragma unroll 1
     for (int b = 5; b < NF; b += 4) {
       double qm[4], qp[4];
-      dust_recon<double, BOX, STRIDE>(sE, sidx, b, w, qm, qp);
+      dust_recon<double, BOX, STRIDE, UNI>(sE, sidx, b, w, qm, qp);
       double F[4];
       {
         double WL[4];
 #pragma unroll
         for (int f = 0; f < 4; ++f) WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
         if (do_face) {
-          dust_kinetic_flux<D>(WL, qm, F);
-#pragma unroll
-          for (int f = 0; f < 4; ++f) F[f] *= area;
+          dust_kinetic_flux<D>(area, WL, qm, F);
         } else {
 #pragma unroll
           for (int f = 0; f < 4; ++f) F[f] = 0.0;
@@ -317,6 +313,45 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   for (int q = 0; q < NT / 32; ++q) s += red[q];
   __syncthreads();
   return s;
+}
+
+// The block's stage-2 results: the sums in FP64 in a fixed order (each thread's
+// partials to shared memory, then NF x 8 threads add NT / 8 of them each and
+// 8-lane shuffles finish; a five-level butterfly in every lane cost the FP64
+// pipe ten times that), and the smallest step length.  smem: NF NT + NT / 32
+// doubles, free once every thread is here.
+template <int NT, int NF>
+__device__ __forceinline__ void block_results(const double* sums, double dtmin, double* red, double* partials) {
+  constexpr int NW = NT / 32, SEG = NT / 8;
+  static_assert(NT % 8 == 0 && NF * 8 <= NT, "reduction layout");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double other = __shfl_xor_sync(0xffffffffu, dtmin, o);
+    if (mag_less(other, dtmin)) dtmin = other;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int f = 0; f < NF; ++f) red[f * NT + threadIdx.x] = sums[f];
+  if (lane == 0) red[NF * NT + warp] = dtmin;
+  __syncthreads();
+  if (threadIdx.x < NF * 8) {
+    const int f = threadIdx.x >> 3, seg = threadIdx.x & 7;
+    const double* src = red + f * NT + seg * SEG;
+    double acc = 0.0;
+#pragma unroll 8
+    for (int u = 0; u < SEG; ++u) acc += src[u];
+    const unsigned grp = 0xffu << (lane & 24);  // this 8-lane group (all of it active)
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) acc += __shfl_down_sync(grp, acc, o, 8);
+    if (seg == 0) partials[(size_t)f * gridDim.x + blockIdx.x] = acc;
+  }
+  if (threadIdx.x == NT - 1) {
+    double m = red[NF * NT];
+    for (int w = 1; w < NW; ++w)
+      if (mag_less(red[NF * NT + w], m)) m = red[NF * NT + w];
+    partials[(size_t)NF * gridDim.x + blockIdx.x] = m;
+  }
 }
 
 // XT: the optional terms (indirect gravity, wave-killing zones) are compiled
@@ -368,8 +403,15 @@ __global__ void __launch_bounds__(NT, 1) stage_full_kernel(const StageArgs a) {
 #pragma unroll
       for (int f = 0; f < 5; ++f) sE[f * BOX + idx] = g.has_eq ? a.in[f][lin] - g.e0c[f * e0s + e0o] : a.in[f][lin];
     }
+    // the dust as primitives (u, v, w, rho_d): converted once per staged cell,
+    // not by every lane that reconstructs from it
 #pragma unroll
-    for (int f = 5; f < NF; ++f) sE[f * BOX + idx] = a.in[f][lin];
+    for (int b = 5; b < NF; b += 4) {
+      const double rd = a.in[b + 3][lin], id = positive(rd) ? recip(rd) : 0.0;
+#pragma unroll
+      for (int c3 = 0; c3 < 3; ++c3) sE[(b + c3) * BOX + idx] = a.in[b + c3][lin] * id;
+      sE[(b + 3) * BOX + idx] = rd;
+    }
   }
   __syncthreads();
   sweep_full<NF, TR, TT, TZ, NT, 0, RC>(a, sE, sG, i0, j0, k0, status);
@@ -383,7 +425,8 @@ __global__ void __launch_bounds__(NT, 1) stage_full_kernel(const StageArgs a) {
 
   const double tau = a.tau_frac * (a.dt_dev ? __longlong_as_double((long long)*a.dt_dev) : a.dt_host);
   const size_t ncell = (size_t)g.nr * g.nth * g.nz;
-  double dtmin = INFINITY;
+  constexpr int ND = NF > 5 ? (NF - 5) / 4 : 1;
+  double rate = 0.0;
   double sums[NF];
 #pragma unroll
   for (int f = 0; f < NF; ++f) sums[f] = 0.0;
@@ -398,13 +441,19 @@ __global__ void __launch_bounds__(NT, 1) stage_full_kernel(const StageArgs a) {
       U[f] = a.in[f][lin];
       G[f] = sG[f * NCORE + cidx];
     }
-    if (cell_nonphysical(g, U)) status |= STATUS_NONPHYSICAL;
-    if (g.geom == GEOM_CYL) {
-      double S[NF];
-      cell_sources<XT>(g, gi, gj, gk, U, S);
-      const double V = g.vol[gi];
+    {
+      double W[5], Vd[ND][2];
+      gas_prim(g.gamma, U, W);
+      bool bad = !positive(U[RHO]) || !positive(W[EN]);
 #pragma unroll
-      for (int f = 0; f < NF; ++f) G[f] += V * S[f];
+      for (int b = 5; b < NF; b += 4) {
+        bad |= !non_negative(U[b + 3]);
+        const int sidx = ((z + ZH) * BY + (y + 2)) * BX + (x + 2);  // the staged velocities
+        Vd[(b - 5) / 4][0] = sE[b * BOX + sidx];
+        Vd[(b - 5) / 4][1] = sE[(b + 1) * BOX + sidx];
+      }
+      if (bad) status |= STATUS_NONPHYSICAL;
+      if (g.geom == GEOM_CYL) add_sources<XT, NF>(g, gi, gj, gk, U, W, Vd, G);
     }
     if (g.r0) {
 #pragma unroll
@@ -412,7 +461,7 @@ __global__ void __launch_bounds__(NT, 1) stage_full_kernel(const StageArgs a) {
     }
     if (XT && g.damp_k) {  // wave-killing zones: the gas departures relax towards E0
       const double kd = g.damp_k[(size_t)gk * g.nr + gi];
-      if (kd != 0.0) {
+      if (positive(kd)) {
         const double V = g.vol[gi];
 #pragma unroll
         for (int f = 0; f < 5; ++f) G[f] -= V * kd * (U[f] - g.e0c[((size_t)f * g.nz + gk) * g.nr + gi]);
@@ -423,31 +472,28 @@ __global__ void __launch_bounds__(NT, 1) stage_full_kernel(const StageArgs a) {
       for (int f = 0; f < NF; ++f) a.gout[f * ncell + lin] = G[f];
       continue;
     }
-    const double iv = g.ivol[gi];
-    double E[NF];
+    const double tv = tau * g.ivol[gi];
+    double E[NF], ig = 0.0, id[ND];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) E[f] = a.base[f][lin] + tau * G[f] * iv;
-    if constexpr (NF > 5) apply_drag<XT, (NF - 5) / 4>(g, gi, E, tau, a.drag);
+    for (int f = 0; f < NF; ++f) E[f] = fma(tv, G[f], a.base[f][lin]);
+    if (NF > 5 || a.stage2) ig = recip(E[RHO]);
+#pragma unroll
+    for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = recip(E[b + 3]);
+    if constexpr (NF > 5) apply_drag<XT, ND>(g, gi, E, tau, a.drag, ig, id);
 #pragma unroll
     for (int f = 0; f < NF; ++f) a.out[f][lin] = E[f];
     if (a.stage2) {
-      dtmin = fmin(dtmin, cell_dt(g, gi, E));
-      if (cell_nonphysical(g, E)) status |= STATUS_NONPHYSICAL;
+      bool bad = false;
+      const double c = cell_rate<NF>(g, gi, E, ig, id, bad);
+      if (bad) status |= STATUS_NONPHYSICAL;
+      if (positive(c) && mag_less(rate, c)) rate = c;
       const double V = g.vol[gi];
 #pragma unroll
-      for (int f = 0; f < NF; ++f) sums[f] += V * E[f];
+      for (int f = 0; f < NF; ++f) sums[f] = fma(V, E[f], sums[f]);
     }
   }
-  if (a.mode == 0 && a.stage2) {
-    double* red = smem;  // the staged tile is no longer needed
-    const double m = block_min<NT>(dtmin, red);
-    if (threadIdx.x == 0) a.partials[(size_t)NF * gridDim.x + blockIdx.x] = m;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      const double s = block_sum<NT>(sums[f], red);
-      if (threadIdx.x == 0) a.partials[(size_t)f * gridDim.x + blockIdx.x] = s;
-    }
-  }
+  if (a.mode == 0 && a.stage2)  // a thread without a cell: rate 0, an infinite step
+    block_results<NT, NF>(sums, positive(rate) ? g.cfl / rate : INFINITY, smem, a.partials);
   if (status) atomicOr(a.status, status);
 }
 

@@ -29,6 +29,27 @@
 
 namespace rossbi {
 
+template <class T, int BOX, int S, bool UNI>
+__device__ __forceinline__ void dust_recon_cons(const T* sE, int sidx, int b, const T* w, T* wm, T* wp) {
+  T pm[4], p0[4], pp[4];
+  const T* r = sE + (b + 3) * BOX + sidx;
+  pm[3] = r[-S];
+  p0[3] = r[0];
+  pp[3] = r[S];
+  const T im = pm[3] > T(0) ? T(1) / pm[3] : T(0);
+  const T i0 = p0[3] > T(0) ? T(1) / p0[3] : T(0);
+  const T ip = pp[3] > T(0) ? T(1) / pp[3] : T(0);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const T* m = sE + (b + c) * BOX + sidx;
+    pm[c] = m[-S] * im;
+    p0[c] = m[0] * i0;
+    pp[c] = m[S] * ip;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) parabola<UNI>(pm[q], p0[q], pp[q], w, wm[q], wp[q]);
+}
+
 template <class T>
 struct PertTables {
   const T* cen;    // [8][nz][nr]   rho0, v0, p0, C_r, f_z, f_r + Omega^2 r, 2 v0/r + 2 Omega, 1/r
@@ -41,7 +62,7 @@ struct PertTables {
   const T* area_r;
   const T* area_t;
   const T* area_z;
-  const T* maxA;
+  const T* aov;    // largest face area over the volume
   const T* omk;    // Omega_K at the cell-centre radius (constant-St drag)
   unsigned long long* fallbacks;  // count of FP64 fallback Riemann faces
 };
@@ -552,18 +573,18 @@ __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* 
     const bool do_face = do_recon && c >= 0;
     const bool do_acc = line_ok && c >= 0 && c < TD && gd < nd;
     const int sidx = do_recon ? ((z + 2) * BY + (y + 2)) * BX + (x + 2) : (2 * BY + 2) * BX + 2;
-    T w[9];
-    parabola_weights<T, D>(a.t.rcoef, gi, g.nr, D == 1 ? a.dx1 : a.dx2, w);
+    constexpr bool UNI = D != 0;
+    T w[RCW];
+    parabola_weights<T, D>(a.t.rcoef, gi, g.nr, w);
     const int ci = clampi(gi, 0, g.nr - 1), ck = clampi(gk, 0, g.nz - 1);
     T area = T(0);
     if (do_face) area = D == 0 ? a.t.area_r[clampi(gi, 0, g.nr)] : (D == 1 ? a.t.area_t[ci] : a.t.area_z[ci]);
     {
       T qm[5], qp[5];
-      bool shaped = false;
 #pragma unroll
       for (int f = 0; f < 5; ++f) {
         const T* s = sE + f * BOX + sidx;
-        shaped |= parabola(s[-STRIDE], s[0], s[STRIDE], w, qm[f], qp[f]);
+        parabola<UNI>(s[-STRIDE], s[0], s[STRIDE], w, qm[f], qp[f]);
       }
       // both face states, used for the positivity check of Sect. 2.7's
       // reconstruction and then by the two faces' solvers
@@ -574,7 +595,7 @@ __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* 
       bool ok;
       if (RC == RECON_PRIM) {
         ok = pert_side<T, D>(gam, Wm, qm, has_eq, sm) & pert_side<T, D>(gam, Wp, qp, has_eq, sp);
-        if (!ok && shaped) {  // positivity fallback: flat reconstruction of the gas fields
+        if (!ok) {  // positivity fallback: flat reconstruction of the gas fields
 #pragma unroll
           for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + sidx];
           ok = pert_side<T, D>(gam, Wm, qm, has_eq, sm) & pert_side<T, D>(gam, Wp, qp, has_eq, sp);
@@ -586,7 +607,7 @@ __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* 
         face_prim<T>(gam, Wm.rho, v0m, qm, pm);
         face_prim<T>(gam, Wp.rho, v0p, qp, pp);
         ok = pert_side<T, D>(gam, Wm, pm, has_eq, sm) & pert_side<T, D>(gam, Wp, pp, has_eq, sp);
-        if (!ok && shaped) {  // positivity fallback: flat reconstruction of the gas fields
+        if (!ok) {  // positivity fallback: flat reconstruction of the gas fields
 #pragma unroll
           for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + sidx];
           face_prim<T>(gam, Wm.rho, v0m, qm, pm);
@@ -631,16 +652,14 @@ __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* 
 #pragma unroll 1
     for (int b = 5; b < NF; b += 4) {  // each dust species: primitive reconstruction, kinetic flux
       T qm[4], qp[4];
-      dust_recon<T, BOX, STRIDE>(sE, sidx, b, w, qm, qp);
+      dust_recon_cons<T, BOX, STRIDE, UNI>(sE, sidx, b, w, qm, qp);
       T F[4];
       {
         T WL[4];
 #pragma unroll
         for (int f = 0; f < 4; ++f) WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
         if (do_face) {
-          dust_kinetic_flux<D>(WL, qm, F);
-#pragma unroll
-          for (int f = 0; f < 4; ++f) F[f] *= area;
+          dust_kinetic_flux<D>(area, WL, qm, F);
         } else {
 #pragma unroll
           for (int f = 0; f < 4; ++f) F[f] = T(0);
@@ -870,13 +889,13 @@ __device__ __forceinline__ T pert_cell_dt(const PertArgs<T>& a, const PCell<T>& 
   const T v = c.v0 + dv;
   const T vel = Math<T>::sqrt_(du * du + v * v + dw * dw);
   const T cs = Math<T>::sqrt_(gam * p / rho);
-  const T V = t.vol[i], A = t.maxA[i], cfl = a.cfl;
-  T dt = cfl * V / ((vel + cs) * A);
+  const T aov = t.aov[i], cfl = a.cfl;
+  T dt = cfl / ((vel + cs) * aov);
 #pragma unroll
   for (int b = 5; b < NF; b += 4) {
     if (q[b + 3] > T(0)) {
       const T vd = Math<T>::sqrt_(q[b] * q[b] + q[b + 1] * q[b + 1] + q[b + 2] * q[b + 2]) / q[b + 3];
-      if (vd > T(0)) dt = fmin(dt, cfl * V / (vd * A));
+      if (vd > T(0)) dt = fmin(dt, cfl / (vd * aov));
     }
     bad |= !(q[b + 3] >= T(0));
   }
