@@ -394,10 +394,10 @@ __device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL
   if (star) {
     const double yl = s.d * s.ipl, yr = (s.d - dP) * s.ipr;
     const bool sl = !sign_bit(yl), sr = !sign_bit(yr);
-    const double tl = s.ircl * near_sum(C.tf, C.t, C.tt, sl, yl), tr = s.ircr * near_sum(C.tf, C.t, C.tt, sr, yr);
+    const double tl = s.ircl * near_sum(C.t, C.tt, sl, yl), tr = s.ircr * near_sum(C.t, C.tt, sr, yr);
     // rho* = rho_K (1 + x D(x)), x = p*/p_K - 1
     const double x = left ? yl : yr, ipk = left ? s.ipl : s.ipr;
-    const double hb = rb * rk * (near_sum(C.df, C.h, C.ht, left ? sl : sr, x) * ipk);
+    const double hb = rb * rk * (near_sum(C.h, C.ht, left ? sl : sr, x) * ipk);
     const double rkb = rb * (rho * recip(rk)), pkb = -hb * (1.0 + x);
     const double gu = 0.5 * ub;
     const double psb = pb + hb + gu * (tr - tl);
@@ -460,24 +460,18 @@ __device__ __forceinline__ void dust_flux_vjp(const double* WL, const double* WR
 }
 
 // ------------------------------------------------------------------ reconstruction adjoint
-// Limiter products of the axis-0 weights (w6 w0, w6 w1, w7 w0, w7 w1).
-__device__ __forceinline__ void limiter_weights(const double* w, double* lw) {
-  lw[0] = w[6] * w[0];
-  lw[1] = w[6] * w[1];
-  lw[2] = w[7] * w[0];
-  lw[3] = w[7] * w[1];
-}
 // Cotangents (bm, b0, bp) of the three cell deviations for cotangents gm, gp
 // on the face values, at the branches br that parabola_branches took: each
-// face value is e0 -/+ (alpha dm + beta dp) with the branch's two weights.
+// face value is e0 -/+ (alpha dm + beta dp) with the branch's two weights
+// (lw = {w6 w0, w6 w1}, the upper limiter's).
 template <bool UNI>
 __device__ __forceinline__ void parabola_vjp(unsigned br, const double* w, const double* lw, double gm, double gp,
                                              double& bm, double& b0, double& bp) {
   const bool live = br & 1, first = br & 2, A = br & 4, B = br & 8;
-  const double am = !live ? 0.0 : (A ? (UNI ? 0.375 : w[2]) : (first ? (UNI ? 1.0 : lw[0]) : 0.0));
-  const double ap = !live ? 0.0 : (A ? (UNI ? 0.125 : w[3]) : (first ? 0.0 : (UNI ? 1.0 : lw[1])));
-  const double cm = !live ? 0.0 : (B ? (UNI ? 0.125 : w[4]) : (first ? (UNI ? 1.0 : lw[2]) : 0.0));
-  const double cp = !live ? 0.0 : (B ? (UNI ? 0.375 : w[5]) : (first ? 0.0 : (UNI ? 1.0 : lw[3])));
+  const double am = !live ? 0.0 : (A ? (UNI ? 0.375 : w[2]) : (first ? (UNI ? 1.0 : w[0]) : 0.0));
+  const double ap = !live ? 0.0 : (A ? (UNI ? 0.125 : w[3]) : (first ? 0.0 : (UNI ? 1.0 : w[1])));
+  const double cm = !live ? 0.0 : (B ? (UNI ? 0.125 : w[4]) : (first ? (UNI ? 1.0 : lw[0]) : 0.0));
+  const double cp = !live ? 0.0 : (B ? (UNI ? 0.375 : w[5]) : (first ? 0.0 : (UNI ? 1.0 : lw[1])));
   const double dmb = fma(gp, cm, -(gm * am)), dpb = fma(gp, cp, -(gm * ap));
   bm = -dmb;
   bp = dpb;
@@ -708,7 +702,7 @@ constexpr size_t adj_flux_smem_doubles() {
 }
 
 template <int NF, int D, int L, int NL, int RC>
-__global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a) {
+__global__ void __launch_bounds__(L * NL, 2) adj_flux_kernel(const AdjFluxArgs a) {
   constexpr int T = L - 4;      // cells per line owned by a block
   constexpr int PE = T + 6;     // staged E': cells c0 - 3 .. c0 + T + 2
   constexpr int PM = T + 4;     // staged mu': cells c0 - 2 .. c0 + T + 1
@@ -806,7 +800,6 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
   auto sm = [&](int f, int q) -> double { return sM[((size_t)f * PM + q) * NLP + l]; };
   // equilibrium on a face: conservative, or primitive with RC = RECON_PRIM
   auto eq_face = [&](int f, int fd) -> double {
-    if (!g.has_eq) return 0.0;
     const double* tc = RC == RECON_PRIM ? g.w0c : g.e0c;
     const double* tr = RC == RECON_PRIM ? g.w0r : g.e0r;
     const double* tz = RC == RECON_PRIM ? g.w0z : g.e0z;
@@ -815,15 +808,18 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
     return tz[((size_t)f * (g.nz + 1) + clampi(fd, 0, g.nz)) * g.nr + ci];
   };
   constexpr bool UNI = D != 0;
-  double w[RCW], lw[4];
+  double w[RCW], lw[2];
   parabola_weights<double, D>(g.rcoef, gi, g.nr, w);
-  if (!UNI) limiter_weights(w, lw);
+  if (!UNI) {
+    lw[0] = w[6] * w[0];
+    lw[1] = w[6] * w[1];
+  }
 
   // ---- forward reconstruction of this lane's cell: the primitives of the
   // right state of its lower face (WR, 1 / rho irm) and of the left state of
   // its upper face (WP, irp), and the branches taken
   double WR[5], WP[5], irm = 0.0, irp = 0.0;
-  unsigned br[9];
+  unsigned br[5];
   bool fallback = false;
   {
     double qm[5], qp[5];
@@ -831,23 +827,24 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
     for (int f = 0; f < 5; ++f)
       br[f] = parabola_branches<UNI>(sv(f, p), sv(f, p + 1), sv(f, p + 2), w, qm[f], qp[f]);
     auto face_states = [&]() {
-      double Um[5], Up[5];
+      if (g.has_eq) {  // its radial and vertical velocities are zero
 #pragma unroll
-      for (int f = 0; f < 5; ++f) {
-        Um[f] = eq_face(f, c) + qm[f];
-        Up[f] = eq_face(f, c + 1) + qp[f];
+        for (int f : {MV, EN, RHO}) {
+          qm[f] += eq_face(f, c);
+          qp[f] += eq_face(f, c + 1);
+        }
       }
       if (RC == RECON_PRIM) {
 #pragma unroll
         for (int f = 0; f < 5; ++f) {
-          WR[f] = Um[f];
-          WP[f] = Up[f];
+          WR[f] = qm[f];
+          WP[f] = qp[f];
         }
       } else {
-        irm = gas_prim(gam, Um, WR);
-        irp = gas_prim(gam, Up, WP);
+        irm = gas_prim(gam, qm, WR);
+        irp = gas_prim(gam, qp, WP);
       }
-      return positive(Um[RHO]) && positive(Up[RHO]) && positive(WR[EN]) && positive(WP[EN]);
+      return positive(qm[RHO]) && positive(qp[RHO]) && positive(WR[EN]) && positive(WP[EN]);
     };
     if (!face_states() && line_ok) {  // the forward's positivity fallback: flat departures
       fallback = true;
@@ -856,48 +853,45 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
       face_states();
     }
   }
-  double dm[4], dp[4];
-  if (NF == 9) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      br[5 + q] = parabola_branches<UNI>(sv(5 + q, p), sv(5 + q, p + 1), sv(5 + q, p + 2), w, dm[q], dp[q]);
-  }
-
   // ---- the face below this cell: cotangents of its two states
   const bool has_face = line_ok && p >= 1;
   const double area = D == 0 ? g.area_r[clampi(c, 0, g.nr)] : (D == 1 ? g.area_t[ci] : g.area_z[ci]);
-  double Fb[9];
-#pragma unroll
-  for (int f = 0; f < NF; ++f) Fb[f] = has_face ? area * (sm(f, p) - sm(f, p > 0 ? p - 1 : 0)) : 0.0;
-  double ULb[5], URb[5];  // of the left state (the lane below's WP) and of this lane's WR
-  {
-    double WL[5];
-#pragma unroll
-    for (int f = 0; f < 5; ++f) WL[f] = __shfl_up_sync(FULL, WP[f], 1, L);
-    if (has_face) {
-      gas_flux_vjp<D>(g.near, WL, WR, Fb, ULb, URb, status);
-    } else {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) ULb[f] = URb[f] = 0.0;
+  auto flux_cot = [&](int f) -> double { return has_face ? area * (sm(f, p) - sm(f, p - 1)) : 0.0; };
+  const bool own = line_ok && p >= 2 && p < T + 2 && c < nd;
+  const size_t lin = ((size_t)cc[2] * g.nth + cc[1]) * g.nr + cc[0];
+  // what a cell receives of field cotangents tm, t0, tp on the cells c - 1, c,
+  // c + 1, the zero-gradient ghosts' folded into the edge cell they copy
+  const bool out_lo = g.bc_lo[D] == BC_OUTFLOW, out_hi = g.bc_hi[D] == BC_OUTFLOW;
+  auto gather = [&](double tm, double t0, double tp) -> double {
+    const double from_above = __shfl_down_sync(FULL, tm, 1, L);
+    const double from_below = __shfl_up_sync(FULL, tp, 1, L);
+    double tot = t0 + (p < L - 1 ? from_above : 0.0) + (p > 0 ? from_below : 0.0);
+    if (out_lo || out_hi) {
+      const double u1 = __shfl_up_sync(FULL, tot, 1, L), u2 = __shfl_up_sync(FULL, tot, 2, L);
+      const double d1 = __shfl_down_sync(FULL, tot, 1, L), d2 = __shfl_down_sync(FULL, tot, 2, L);
+      if (out_lo && c == 0 && p >= 2) tot += u1 + u2;
+      if (out_hi && c == nd - 1 && p + 2 < L) tot += d1 + d2;
     }
-  }
-  double WLb[4], WRb[4];
-  if (NF == 9) {
-    double WL[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) WL[q] = __shfl_up_sync(FULL, dp[q], 1, L);
-    if (has_face) {
-      dust_flux_vjp<D>(WL, dm, Fb + 5, WLb, WRb);
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) WLb[q] = WRb[q] = 0.0;
-    }
-  }
-
-  // ---- cotangents of this cell's face values: lower from its own face, upper from the lane above
-  double tm[9], t0[9], tp[9];  // contributions to cells c - 1, c, c + 1 (dust: of the primitives)
+    return tot;
+  };
   {
-    double gp[5];
+    double ULb[5], URb[5];  // of the left state (the lane below's WP) and of this lane's WR
+    {
+      double WL[5], Fb[5];
+#pragma unroll
+      for (int f = 0; f < 5; ++f) {
+        WL[f] = __shfl_up_sync(FULL, WP[f], 1, L);
+        Fb[f] = flux_cot(f);
+      }
+      if (has_face) {
+        gas_flux_vjp<D>(g.near, WL, WR, Fb, ULb, URb, status);
+      } else {
+#pragma unroll
+        for (int f = 0; f < 5; ++f) ULb[f] = URb[f] = 0.0;
+      }
+    }
+    // cotangents of this cell's face values: lower from its own face, upper from the lane above
+    double gp[5], tot[5];
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
       const double up = __shfl_down_sync(FULL, ULb[f], 1, L);
@@ -909,58 +903,62 @@ __global__ void __launch_bounds__(L * NL, 1) adj_flux_kernel(const AdjFluxArgs a
     }
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
+      double tm, t0, tp;
       if (fallback) {
-        tm[f] = tp[f] = 0.0;
-        t0[f] = URb[f] + gp[f];
+        tm = tp = 0.0;
+        t0 = URb[f] + gp[f];
       } else {
-        parabola_vjp<UNI>(br[f], w, lw, URb[f], gp[f], tm[f], t0[f], tp[f]);
+        parabola_vjp<UNI>(br[f], w, lw, URb[f], gp[f], tm, t0, tp);
+      }
+      tot[f] = gather(tm, t0, tp);
+    }
+    if (own) {
+      if (RC == RECON_PRIM) {  // primitive-deviation cotangents back to the conservative fields
+        double U[5], Ub[5];
+#pragma unroll
+        for (int f = 0; f < 5; ++f) U[f] = a.E[f][lin];
+        gas_prim_vjp(gam, U, tot, Ub);
+#pragma unroll
+        for (int f = 0; f < 5; ++f) a.lam[f][lin] += Ub[f];
+      } else {
+#pragma unroll
+        for (int f = 0; f < 5; ++f) a.lam[f][lin] += tot[f];
       }
     }
   }
-  if (NF == 9) {
+  if (NF == 9) {  // the dust, whose fluxes and sums share nothing with the gas's
+    double WLb[4], WRb[4], dm[4], dp[4], tot[4];
+    unsigned bd[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      bd[q] = parabola_branches<UNI>(sv(5 + q, p), sv(5 + q, p + 1), sv(5 + q, p + 2), w, dm[q], dp[q]);
+    {
+      double WL[4], Fb[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        WL[q] = __shfl_up_sync(FULL, dp[q], 1, L);
+        Fb[q] = flux_cot(5 + q);
+      }
+      if (has_face) {
+        dust_flux_vjp<D>(WL, dm, Fb, WLb, WRb);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) WLb[q] = WRb[q] = 0.0;
+      }
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const double up = __shfl_down_sync(FULL, WLb[q], 1, L);
-      parabola_vjp<UNI>(br[5 + q], w, lw, WRb[q], p < L - 1 ? up : 0.0, tm[5 + q], t0[5 + q], tp[5 + q]);
+      double tm, t0, tp;
+      parabola_vjp<UNI>(bd[q], w, lw, WRb[q], p < L - 1 ? up : 0.0, tm, t0, tp);
+      tot[q] = gather(tm, t0, tp);
     }
-  }
-  double tot[9];
-#pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    const double from_above = __shfl_down_sync(FULL, tm[f], 1, L);
-    const double from_below = __shfl_up_sync(FULL, tp[f], 1, L);
-    tot[f] = t0[f] + (p < L - 1 ? from_above : 0.0) + (p > 0 ? from_below : 0.0);
-  }
-  // zero-gradient ghosts copy the edge cell: fold their cotangents into it
-  const bool out_lo = g.bc_lo[D] == BC_OUTFLOW, out_hi = g.bc_hi[D] == BC_OUTFLOW;
-  if (out_lo || out_hi) {
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      const double u1 = __shfl_up_sync(FULL, tot[f], 1, L), u2 = __shfl_up_sync(FULL, tot[f], 2, L);
-      const double d1 = __shfl_down_sync(FULL, tot[f], 1, L), d2 = __shfl_down_sync(FULL, tot[f], 2, L);
-      if (out_lo && c == 0 && p >= 2) tot[f] += u1 + u2;
-      if (out_hi && c == nd - 1 && p + 2 < L) tot[f] += d1 + d2;
-    }
-  }
-  if (line_ok && p >= 2 && p < T + 2 && c < nd) {
-    const size_t lin = ((size_t)cc[2] * g.nth + cc[1]) * g.nr + cc[0];
-    if (RC == RECON_PRIM) {  // gas: primitive-deviation cotangents back to the conservative fields
-      double U[5], Ub[5];
-#pragma unroll
-      for (int f = 0; f < 5; ++f) U[f] = a.E[f][lin];
-      gas_prim_vjp(gam, U, tot, Ub);
-#pragma unroll
-      for (int f = 0; f < 5; ++f) a.lam[f][lin] += Ub[f];
-    } else {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) a.lam[f][lin] += tot[f];
-    }
-    if (NF == 9) {  // dust: the primitives' cotangents back to (rho_d u, rho_d v, rho_d w, rho_d)
+    if (own) {  // the primitives' cotangents back to (rho_d u, rho_d v, rho_d w, rho_d)
       const double rd = sv(8, p + 1), id = positive(rd) ? recip(rd) : 0.0;
-      double rb = tot[8];
+      double rb = tot[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const double m = tot[5 + q] * id;
+        const double m = tot[q] * id;
         a.lam[5 + q][lin] += m;
         rb = fma(-m, sv(5 + q, p + 1), rb);
       }

@@ -453,7 +453,7 @@ __device__ __forceinline__ void gas_face_flux(const NearCoef& C, double area, co
   F[n] = fma(m, u, pa);
   F[t1] = m * ut1;
   F[t2] = m * ut2;
-  F[EN] = fma(0.5 * m, fma(u, u, fma(ut1, ut1, ut2 * ut2)), C.g_gm1 * (pa * u));
+  F[EN] = fma(scale_down<1>(m), fma(u, u, fma(ut1, ut1, ut2 * ut2)), C.g_gm1 * (pa * u));
 }
 
 // Flux of the pressureless dust fluid (Sect. 2.9 "adapted" solver) by kinetic
@@ -478,12 +478,12 @@ __device__ __forceinline__ void dust_kinetic_flux(T area, const T* WL, const T* 
 // terms, stellar gravity (Sect. 2.1), the rotating-frame Coriolis /
 // centrifugal terms and, when switched on, the indirect gravity of Sect. 2.10
 // (force -grad Phi_ind on gas and dust, and its work on the gas); the Box has
-// none.  W: the cell's primitive gas state; Vd: the dust velocities (u, v) of
-// each species, zero where it has no mass.  XT = false compiles the optional
+// none.  W: the cell's primitive gas state; Vd: the azimuthal dust velocity
+// of each species, zero where it has no mass.  XT = false compiles the optional
 // terms out.
 template <bool XT, int NF>
 __device__ __forceinline__ void add_sources(const DevGrid& g, int i, int j, int k, const double* U, const double* W,
-                                            const double (*Vd)[2], double* G) {
+                                            const double* Vd, double* G) {
   const double V = g.vol[i], ir = g.ir[i], Om2 = 2.0 * g.omega;
   const size_t o = (size_t)k * g.nr + i;
   const double a1 = g.grav[o], fz = g.grav[(size_t)g.nz * g.nr + o];
@@ -505,7 +505,7 @@ __device__ __forceinline__ void add_sources(const DevGrid& g, int i, int j, int 
   G[EN] = fma(V, se, G[EN]);
 #pragma unroll
   for (int b = 5; b < NF; b += 4) {  // each dust species
-    const double v = Vd[(b - 5) / 4][1], rd = U[b + 3];
+    const double v = Vd[(b - 5) / 4], rd = U[b + 3];
     if (!positive(rd)) continue;
     G[b] = fma(V, fma(U[b + 1], fma(v, ir, Om2), rd * ar), G[b]);
     double sd = -U[b] * fma(v, ir, Om2);

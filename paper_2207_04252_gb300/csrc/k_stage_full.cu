@@ -14,12 +14,13 @@ template <int NF, int TT, int TZ, bool XT, int RC>
 cudaError_t launch(const StageArgs& a, int nblocks, cudaStream_t s) {
   constexpr int BOX = (F64_TR + 4) * (TT + 4) * (TZ == 1 ? 1 : TZ + 4);
   constexpr int NCORE = F64_TR * TT * TZ;
-  constexpr size_t smem = (size_t)NF * (BOX + NCORE) * sizeof(double);
-  auto kern = stage_full_kernel<NF, F64_TR, TT, TZ, F64_NT, XT, RC>;
+  constexpr size_t smem = (size_t)(5 * BOX + NF * NCORE) * sizeof(double);
+  constexpr int NT = TZ == 1 ? FLAT_NT : F64_NT, MINB = TZ == 1 ? 3 : 2;
+  auto kern = stage_full_kernel<NF, F64_TR, TT, TZ, NT, MINB, XT, RC>;
   static unsigned long long done = 0;
   cudaError_t e = set_smem_once(kern, smem, done);
   if (e != cudaSuccess) return e;
-  kern<<<nblocks, F64_NT, smem, s>>>(a);
+  kern<<<nblocks, NT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -29,8 +30,8 @@ cudaError_t launch_x(const StageArgs& a, int nblocks, cudaStream_t s, bool xt) {
     if (flat_grid(a.g.nz, a.g.bc_lo[2], a.g.bc_hi[2], NF))
       return xt ? launch<NF, FLAT_TT, 1, true, RC>(a, nblocks, s) : launch<NF, FLAT_TT, 1, false, RC>(a, nblocks, s);
   }
-  constexpr int TZ = tile_z(true, NF);
-  return xt ? launch<NF, F64_TT, TZ, true, RC>(a, nblocks, s) : launch<NF, F64_TT, TZ, false, RC>(a, nblocks, s);
+  return xt ? launch<NF, F64_TT, F64_TZ, true, RC>(a, nblocks, s)
+            : launch<NF, F64_TT, F64_TZ, false, RC>(a, nblocks, s);
 }
 
 }  // namespace

@@ -15,18 +15,18 @@ namespace rossbi {
 // Tiles of the stage kernels: 14 x 6 x 6 cells, lines of 16 / 8 / 8 lanes.
 constexpr int F64_TR = 14, F64_TT = 6, F64_TZ = 6, F64_NT = 192;
 constexpr int P32_TR = 14, P32_TT = 6, P32_TZ = 6, P32_NT = 256, P32_MINB = 2;
-// With more than one dust species the FP64-state kernels' staged 14 x 6 x 6
-// tile with its halo (18 x 10 x 10 cells) no longer fits in shared memory
-// (13 fields: 234 KB of the 227 KB a block may have): they take tiles two z
+// With more than one dust species the FP64 perturbation form's staged 14 x 6
+// x 6 tile with its halo (18 x 10 x 10 cells) no longer fits in shared memory
+// (13 fields: 234 KB of the 227 KB a block may have): it takes tiles two z
 // cells thick (lines of 4 lanes in z; 13 fields: 127 KB, 21: 205 KB).
 constexpr int THIN_TZ = 2;
-constexpr int tile_z(bool fp64_state, int nf) { return fp64_state && nf > 9 ? THIN_TZ : 6; }
+constexpr int tile_z(bool fp64_pert, int nf) { return fp64_pert && nf > 9 ? THIN_TZ : 6; }
 
 // The FP64 kernel's flat tile, 14 x 30 x 1 cells without a z halo or z
 // sweep, for grids one z cell thick whose z boundaries are periodic or
 // outflow (the cell's two z faces then carry the same flux), with at most
 // one dust species: the cylindrical explosion of Sect. 4.1 runs on it.
-constexpr int FLAT_TT = 30;
+constexpr int FLAT_TT = 30, FLAT_NT = 160;
 inline bool flat_grid(int nz, int bc_lo_z, int bc_hi_z, int nf) {
   return nz == 1 && bc_lo_z != BC_EQUILIBRIUM && bc_hi_z != BC_EQUILIBRIUM && nf <= 9;
 }
@@ -44,8 +44,9 @@ cudaError_t by_nf(int nf, F&& f) {
   }
   return cudaErrorInvalidValue;
 }
-// Adjoint flux kernel: lines of 16 lanes (12 owned cells), 16 lines per block.
-constexpr int ADJ_L = 16, ADJ_NL = 16;
+// Adjoint flux kernel: lines of 16 lanes (12 owned cells), 12 lines per block,
+// two blocks per SM.
+constexpr int ADJ_L = 16, ADJ_NL = 12;
 
 // Raises a kernel's dynamic shared-memory limit once per device (the
 // attribute belongs to the current device's context); `done` is the calling
@@ -62,34 +63,19 @@ cudaError_t set_smem_once(K kern, size_t smem, unsigned long long& done) {
   return e;
 }
 
-// Each launcher is instantiated per gas reconstruction mode RC in a
-// translation unit of its own (they compile in parallel).
-// One launch of the FP64 stage kernel over nblocks tiles; xt selects the
+// Each launcher is instantiated per gas reconstruction mode RC (and power form
+// P) in a translation unit of its own, which compile in parallel; the host
+// runtime selects one.  (A selecting inline function here would make every
+// such unit instantiate all of them.)
+// One launch of a stage kernel over nblocks tiles; xt selects the
 // instantiation with the optional terms (indirect gravity, damping zones,
 // Stokes drag regime).
 template <int RC>
 cudaError_t run_stage_full_rc(const StageArgs& a, int nblocks, cudaStream_t s, bool xt);
-inline cudaError_t run_stage_full(const StageArgs& a, int nblocks, cudaStream_t s, bool xt) {
-  return a.g.recon == RECON_PRIM ? run_stage_full_rc<RECON_PRIM>(a, nblocks, s, xt)
-                                 : run_stage_full_rc<RECON_CONS>(a, nblocks, s, xt);
-}
-// One launch of the perturbation-form stage kernel (float or double); g75
-// selects the gamma = 7/5 power forms of the float solver.
 template <class P, int RC>
 cudaError_t run_stage_pert_f32_rc(const PertArgs<float>& a, int nblocks, cudaStream_t s, bool xt);
-inline cudaError_t run_stage_pert_f32(const PertArgs<float>& a, int nblocks, cudaStream_t s, bool xt, bool g75) {
-  if (a.g.recon == RECON_PRIM)
-    return g75 ? run_stage_pert_f32_rc<PowG75, RECON_PRIM>(a, nblocks, s, xt)
-               : run_stage_pert_f32_rc<PowGeneric<float>, RECON_PRIM>(a, nblocks, s, xt);
-  return g75 ? run_stage_pert_f32_rc<PowG75, RECON_CONS>(a, nblocks, s, xt)
-             : run_stage_pert_f32_rc<PowGeneric<float>, RECON_CONS>(a, nblocks, s, xt);
-}
 template <int RC>
 cudaError_t run_stage_pert_f64_rc(const PertArgs<double>& a, int nblocks, cudaStream_t s, bool xt);
-inline cudaError_t run_stage_pert_f64(const PertArgs<double>& a, int nblocks, cudaStream_t s, bool xt) {
-  return a.g.recon == RECON_PRIM ? run_stage_pert_f64_rc<RECON_PRIM>(a, nblocks, s, xt)
-                                 : run_stage_pert_f64_rc<RECON_CONS>(a, nblocks, s, xt);
-}
 // One launch of the adjoint flux kernel along axis 0, 1 or 2.
 cudaError_t run_adj_flux(const AdjFluxArgs& a, int axis, cudaStream_t s);
 

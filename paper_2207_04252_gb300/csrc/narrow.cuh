@@ -41,6 +41,14 @@ __device__ __forceinline__ float neg_part(float x) { return fminf(x, 0.0f); }
 // The smaller of two values of one sign in magnitude.
 __device__ __forceinline__ double min_mag(double a, double b) { return mag_less(a, b) ? a : b; }
 
+// x / 2^K for normal results, by the exponent (0 below the normal range).
+template <int K>
+__device__ __forceinline__ double scale_down(double x) {
+  const int hi = __double2hiint(x);
+  const bool normal = (hi & 0x7ff00000) > (K << 20);
+  return __hiloint2double(normal ? hi - (K << 20) : (hi & 0x80000000), normal ? __double2loint(x) : 0);
+}
+
 // MinMod slope: 0 where the signs differ.
 __device__ __forceinline__ double minmod_bits(double a, double b) {
   const double m = min_mag(a, b);

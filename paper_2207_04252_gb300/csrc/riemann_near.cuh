@@ -1,6 +1,7 @@
 // Exact Riemann solution on the face (Sect. 2.6) where the star pressure is
-// close to both side pressures, |x_K| <= 1/32 with x_K = p*/p_K - 1: every
-// face of a smooth flow, and all but a few cells around a strong shock.
+// close to both side pressures, |x_K| <= 1/64 (float) or 1/128 (double) with
+// x_K = p*/p_K - 1: every face of a smooth flow, and all but a few cells
+// around a strong shock.
 //
 // There the pressure function of a side is f_K = x p_K / (rho_K c_K) S(x),
 // its derivative T(x) / (rho_K c_K) with T = (x S)', and the star density
@@ -15,11 +16,12 @@
 //
 // In double the Newton iteration runs in float and its result is corrected by
 // FP64 residuals: step = -F/F' with F in FP64 and the quotient in float.  A
-// step has a relative error of about 2^-21, so the iteration ends once it is
-// below 2^-32 p (one evaluation of F for |x| up to about 2^-11, two up to
-// 1/32) and p* is then exact to the last bits, as the FP64 iteration's is.
-// The series are summed in double to x^5, the rest (below 2^-30 of the sum)
-// in float.
+// step has a relative error of about 2^-22, so the iteration ends once it is
+// below 2^-31 p (one evaluation of F for |x| up to about 2^-9, two beyond)
+// and p* is then exact to the last bits, as the FP64 iteration's is.  The
+// series are summed in double to x^3, the rest (below 2^-30 of the sum at
+// |x| = 1/128) in float: 1/128 is where float's rounding of the tail reaches
+// 2^-54 of the sum; each power of two more takes another FP64 term per sum.
 //
 // What bounds the callers: in FP64 the two-lane FP64 pipe, which sees about
 // 55 operations here against 250 to 300 of the FP64 Newton iteration with its
@@ -29,17 +31,18 @@
 
 namespace rossbi {
 
-constexpr int NEAR_N = 6;  // FP64 terms of a series
+constexpr int NEAR_N = 4;  // FP64 terms of a series
 constexpr int NEAR_T = 5;  // float terms of its tail
-constexpr float NEAR_X = 0.03125f;
+constexpr float NEAR_XF = 0.015625f, NEAR_XD = 0.0078125f;
 
 // Series coefficients of one gamma, [0] rarefaction, [1] shock (built on the host).
 struct NearCoef {
   double s[2][NEAR_N], d[2][NEAR_N];
-  float st[2][NEAR_T], dt[2][NEAR_T];  // tails: the terms x^6 ... x^10
+  float st[2][NEAR_T], dt[2][NEAR_T];  // tails: the terms x^4 ... x^8
   double t[2][NEAR_N], h[2][NEAR_N];   // (x S)' and (x D)', for the adjoint
   float tt[2][NEAR_T], ht[2][NEAR_T];
-  float sf[2][5], tf[2][5], df[2][5];  // S, T, D to x^4 in float
+  float sf[2][5], tf[2][5], df[2][4];  // S, T, D in float
+  float t2m;                           // mean of the branches' T_2
   double gamma, g_gm1;  // gamma, gamma / (gamma - 1)
   float gammaf;
 };
@@ -66,7 +69,7 @@ inline NearCoef near_coef(double gamma) {
       if (k < 5) {
         c.sf[q][k] = (float)s[q];
         c.tf[q][k] = (float)((k + 1) * s[q]);
-        c.df[q][k] = (float)d[q];
+        if (k < 4) c.df[q][k] = (float)d[q];
       }
     }
     bb *= (beta - (k + 1)) / (k + 2);
@@ -78,6 +81,7 @@ inline NearCoef near_coef(double gamma) {
   c.gamma = gamma;
   c.g_gm1 = gamma / (gamma - 1.0);
   c.gammaf = (float)gamma;
+  c.t2m = 0.5f * (c.tf[0][2] + c.tf[1][2]);
   return c;
 }
 
@@ -88,12 +92,15 @@ __device__ __forceinline__ float near_sum_f(const float (&c)[2][5], bool shock, 
   for (int k = 3; k >= 2; --k) t = fmaf(t, x, shock ? c[1][k] : c[0][k]);
   return fmaf(fmaf(t, x, c[0][1]), x, c[0][0]);
 }
-__device__ __forceinline__ float near_sum(const float (&c)[2][5], const double (&)[2][NEAR_N],
-                                          const float (&)[2][NEAR_T], bool shock, float x) {
-  return near_sum_f(c, shock, x);
+// The same to x^3 (truncation below 2^-26 at |x| = 1/64).
+template <int N>
+__device__ __forceinline__ float near_cubic(const float (&c)[2][N], bool shock, float x) {
+  const float t = fmaf(shock ? c[1][3] : c[0][3], x, shock ? c[1][2] : c[0][2]);
+  return fmaf(fmaf(t, x, c[0][1]), x, c[0][0]);
 }
-__device__ __forceinline__ double near_sum(const float (&)[2][5], const double (&c)[2][NEAR_N],
-                                           const float (&ct)[2][NEAR_T], bool shock, double x) {
+// In double: NEAR_N terms in double, the tail in float.
+__device__ __forceinline__ double near_sum(const double (&c)[2][NEAR_N], const float (&ct)[2][NEAR_T], bool shock,
+                                           double x) {
   const float xf = narrow(x);
   float t = shock ? ct[1][NEAR_T - 1] : ct[0][NEAR_T - 1];
 #pragma unroll
@@ -120,15 +127,16 @@ struct NearStar {
 // flow being supersonic), NEAR_STAR_L / NEAR_STAR_R (the star state of that
 // side; s is set), or NEAR_GENERAL: not near, or within the sonic band where
 // a fan or a shock may sit on the face; the caller then takes the general
-// solver.  (rl, pl), (rr, pr): positive densities and pressures; dP = p_R -
+// solver.  (rl, pl), (rr, pr): densities and pressures (a float state that is
+// not positive comes back as NEAR_GENERAL; a double one is the caller's to sort out); dP = p_R -
 // p_L, ul, ur velocities about u0, dU = u_R - u_L; ulf, urf the full
 // velocities in float.
 template <class T>
 __device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl, T rr, T ur, T pr, T dP, T dU, T u0,
                                             bool has_u0, float ulf, float urf, NearStar<T>& s) {
   const float plf = narrow(pl), prf = narrow(pr), rlf = narrow(rl), rrf = narrow(rr);
-  // outside float's comfortable range: the general solver
-  if (!(fmaxf(fmaxf(plf, prf), fmaxf(rlf, rrf)) < 1e30f)) return NEAR_GENERAL;
+  // doubles beyond float's comfortable range: the general solver
+  if (sizeof(T) == 8 && !(fmaxf(fmaxf(plf, prf), fmaxf(rlf, rrf)) < 1e30f)) return NEAR_GENERAL;
   const float gl = C.gammaf * plf, gr = C.gammaf * prf;
   const float il = recip_sqrt(gl) * recip_sqrt(rlf), ir = recip_sqrt(gr) * recip_sqrt(rrf);  // 1 / (rho c)
   const float cl = gl * il, cr = gr * ir;
@@ -138,38 +146,41 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl,
   float d = (dPf * ir - dUf) * recip(il + ir);
   float xl = d * ipl, xr = (d - dPf) * ipr;
   float X = fabsf(xl) + fabsf(xr);
-  if (!(X <= NEAR_X)) return NEAR_GENERAL;  // NaN too
+  constexpr float XM = sizeof(T) == 4 ? NEAR_XF : NEAR_XD;
+  if (!(X <= 2.0f * NEAR_XF)) return NEAR_GENERAL;  // NaN too
   // supersonic by a margin that covers every wave speed at |x| <= 1/32
   if (ulf >= 1.1f * cl) return NEAR_LEFT;
   if (-urf >= 1.1f * cr) return NEAR_RIGHT;
-  float fl, fr, tl, tr;
+  if (!(X <= XM)) return NEAR_GENERAL;
   if constexpr (sizeof(T) == 4) {
-    // Newton in float: the error after a step is 0.43 step^2 / p at most
-    // ((gamma + 1)/(4 gamma) < 1/2), below the rounding of d once
-    // step^2 < 2^-23 |d| p
-    bool more = true;
-    for (int it = 0; it < 6 && more; ++it) {
-      const bool sl = d > 0.0f, sr = d > dPf;
+    // One Newton step from the acoustic value, whose error is below 0.45 x^2 p:
+    // what it leaves, below 0.1 x^4 p, is under the rounding of d for |x| <=
+    // 1/128, and a second step's beyond.  The slope needs three digits only
+    // (T to x^2 with the branches' mean T_2).
+    float fl, fr;
+    auto newton = [&]() {
+      const float dr = d - dPf;
       xl = d * ipl;
-      xr = (d - dPf) * ipr;
-      fl = d * il * near_sum_f(C.sf, sl, xl);
-      fr = (d - dPf) * ir * near_sum_f(C.sf, sr, xr);
-      tl = il * near_sum_f(C.tf, sl, xl);
-      tr = ir * near_sum_f(C.tf, sr, xr);
+      xr = dr * ipr;
+      const float tl = il * fmaf(fmaf(C.t2m, xl, C.tf[0][1]), xl, 1.0f);
+      const float tr = ir * fmaf(fmaf(C.t2m, xr, C.tf[0][1]), xr, 1.0f);
+      fl = d * il * near_cubic(C.sf, d > 0.0f, xl);
+      fr = dr * ir * near_cubic(C.sf, dr > 0.0f, xr);
       const float step = -(fl + fr + dUf) * recip(tl + tr);
       d += step;
-      fl += tl * step;
-      fr += tr * step;
-      const float scale = fabsf(d) + fabsf(d - dPf);
-      more = !(step * step <= 1.2e-7f * scale * fminf(plf, prf)) && fabsf(step) > 2.4e-7f * scale;
-    }
+      fl = fmaf(tl, step, fl);
+      fr = fmaf(tr, step, fr);
+    };
+    newton();
+    if (X > 0.0078125f) newton();
     s.d = d;
     s.fl = fl;
     s.fr = fr;
-    s.us = 0.5f * ((ul - fl) + (ur + fr));
+    s.us = ul - fl;
     s.ipl = ipl;
     s.ipr = ipr;
   } else {
+    float tl = 0.0f, tr = 0.0f;
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
       const bool sl = d > 0.0f, sr = d > dPf;
@@ -179,7 +190,7 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl,
       tr = ir * near_sum_f(C.tf, sr, xr);
       d -= (d * il * near_sum_f(C.sf, sl, xl) + (d - dPf) * ir * near_sum_f(C.sf, sr, xr) + dUf) * recip(tl + tr);
     }
-    const float iD = recip(tl + tr), small = 2.3e-10f * fminf(plf, prf);
+    const float iD = recip(tl + tr), small = 4.6e-10f * fminf(plf, prf);
     s.ircl = recip_sqrt(C.gamma * (pl * rl));
     s.ircr = recip_sqrt(C.gamma * (pr * rr));
     s.ipl = recip(pl);
@@ -191,8 +202,8 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl,
       const T dr = dd - dP;
       const T yl = dd * s.ipl, yr = dr * s.ipr;
       const bool sl = !sign_bit(yl), sr = !sign_bit(yr);
-      f1 = dd * s.ircl * near_sum(C.sf, C.s, C.st, sl, yl);
-      f2 = dr * s.ircr * near_sum(C.sf, C.s, C.st, sr, yr);
+      f1 = dd * s.ircl * near_sum(C.s, C.st, sl, yl);
+      f2 = dr * s.ircr * near_sum(C.s, C.st, sr, yr);
       step = -narrow(f1 + f2 + dU) * iD;
       dd += widen<T>(step);
       more = !(fabsf(step) <= small);
@@ -201,21 +212,19 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl,
     s.d = dd;
     s.fl = f1 + widen<T>(tl * step);
     s.fr = f2 + widen<T>(tr * step);
-    s.us = T(0.5) * ((ul - s.fl) + (ur + s.fr));
-    d = narrow(dd);
+    s.us = ul - s.fl;
   }
-  xl = d * ipl;
-  xr = (d - dPf) * ipr;
-  X = fabsf(xl) + fabsf(xr);
-  if (!(X <= 1.25f * NEAR_X)) return NEAR_GENERAL;
+  // u* = u_L - f_L = u_R + f_R: the side that the face lies on gives it
   const bool left = !sign_bit(has_u0 ? u0 + s.us : s.us);
+  if (!left) s.us = ur + s.fr;
   // the head of side K is at u_K -/+ c_K, its shock or tail within |x| c_K of
   // it: the side's own state beyond that band, the star state before it
-  const float v = left ? ulf : -urf, c = left ? cl : cr, band = c * (X + 1e-5f);
+  const float v = left ? ulf : -urf, c = left ? cl : cr, band = c * fmaf(1.25f, X, 1e-5f);
   if (v - c >= band) return left ? NEAR_LEFT : NEAR_RIGHT;
   if (!(c - v > band)) return NEAR_GENERAL;
   const T x = left ? s.d * s.ipl : (s.d - dP) * s.ipr;
-  s.drho = (left ? rl : rr) * (x * near_sum(C.df, C.d, C.dt, !sign_bit(x), x));
+  if constexpr (sizeof(T) == 4) s.drho = (left ? rl : rr) * (x * near_cubic(C.df, x > 0.0f, x));
+  else s.drho = (left ? rl : rr) * (x * near_sum(C.d, C.dt, !sign_bit(x), x));
   return left ? NEAR_STAR_L : NEAR_STAR_R;
 }
 

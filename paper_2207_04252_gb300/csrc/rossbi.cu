@@ -392,6 +392,25 @@ rossbi_status profile_drain(rossbi_grid* g) {
   return ROSSBI_OK;
 }
 
+// The launcher of a grid's reconstruction mode and, for the float form, of
+// the gamma = 7/5 integer powers or the general ones.
+cudaError_t run_stage_full(const StageArgs& a, int nblocks, cudaStream_t s, bool xt) {
+  return a.g.recon == RECON_PRIM ? run_stage_full_rc<RECON_PRIM>(a, nblocks, s, xt)
+                                 : run_stage_full_rc<RECON_CONS>(a, nblocks, s, xt);
+}
+cudaError_t run_stage_pert(const PertArgs<float>& a, int nblocks, cudaStream_t s, bool xt) {
+  const bool g75 = a.g.gamma == 1.4;
+  if (a.g.recon == RECON_PRIM)
+    return g75 ? run_stage_pert_f32_rc<PowG75, RECON_PRIM>(a, nblocks, s, xt)
+               : run_stage_pert_f32_rc<PowGeneric<float>, RECON_PRIM>(a, nblocks, s, xt);
+  return g75 ? run_stage_pert_f32_rc<PowG75, RECON_CONS>(a, nblocks, s, xt)
+             : run_stage_pert_f32_rc<PowGeneric<float>, RECON_CONS>(a, nblocks, s, xt);
+}
+cudaError_t run_stage_pert(const PertArgs<double>& a, int nblocks, cudaStream_t s, bool xt) {
+  return a.g.recon == RECON_PRIM ? run_stage_pert_f64_rc<RECON_PRIM>(a, nblocks, s, xt)
+                                 : run_stage_pert_f64_rc<RECON_CONS>(a, nblocks, s, xt);
+}
+
 rossbi_status launch_stage(rossbi_grid* g, const StageArgs& a, int nblocks) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (g->profiling && a.mode == 0) {
@@ -425,10 +444,7 @@ rossbi_status launch_pert(rossbi_grid* g, const PertArgs<T>& a, int nblocks) {
     CK(cudaEventRecord(e0, g->stream));
   }
   const bool xt = a.g.x_ind != 0.0 || a.g.damp_k != nullptr || a.drag.law == 2;  // optional terms on
-  if constexpr (sizeof(T) == 4)  // gamma = 7/5: integer-power forms of the float solver
-    CK(run_stage_pert_f32(a, nblocks, g->stream, xt, g->desc.gamma == 1.4));
-  else
-    CK(run_stage_pert_f64(a, nblocks, g->stream, xt));
+  CK(run_stage_pert(a, nblocks, g->stream, xt));
   if (e0) {
     CK(cudaEventRecord(e1, g->stream));
     g->ev_used++;
@@ -519,10 +535,22 @@ rossbi_status build_pert_tables(rossbi_grid* g, PertTables<T>& pt) {
   const rossbi_grid_desc& d = g->desc;
   const int nr = d.nr, nz = d.nz;
   const size_t ncen = (size_t)nz * nr, nfr = (size_t)nz * (nr + 1), nfz = (size_t)(nz + 1) * nr;
-  const size_t off_cen = 0, off_fr = off_cen + 8 * ncen, off_fz = off_fr + 5 * nfr, off_ft = off_fz + 5 * nfz;
-  const size_t off_rc = off_ft + 7 * ncen, off_vol = off_rc + (size_t)(nr + 2) * RCW, off_ivol = off_vol + nr;
-  const size_t off_ar = off_ivol + nr, off_at = off_ar + nr + 1, off_az = off_at + nr, off_ma = off_az + nr;
-  const size_t off_om = off_ma + nr, total = off_om + nr;
+  // offsets in elements, each a multiple of 8 (the kernels load 16 bytes at a time)
+  size_t total = 0;
+  auto room = [&](size_t n) {
+    const size_t at = total;
+    total += (n + 7) & ~(size_t)7;
+    return at;
+  };
+  const size_t off_cen = room(8 * ncen);
+  const size_t nface[3] = {nfr, ncen, nfz};
+  size_t off_face[3], off_wave[3];
+  for (int q = 0; q < 3; ++q) {
+    off_face[q] = room(4 * nface[q]);
+    off_wave[q] = room(4 * nface[q]);
+  }
+  const size_t off_rc = room((size_t)(nr + 2) * RCW), off_vol = room(nr), off_ivol = room(nr), off_ar = room(nr + 1);
+  const size_t off_at = room(nr), off_az = room(nr), off_ma = room(nr), off_om = room(nr);
   std::vector<double> h(total, 0.0);
   std::vector<double> v(nr), rcoef((size_t)(nr + 2) * RCW), ar(nr + 1), at(nr), az(nr), ma(nr), iv(nr);
   if (cudaMemcpy(v.data(), g->d_vol, nr * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
@@ -546,18 +574,15 @@ rossbi_status build_pert_tables(rossbi_grid* g, PertTables<T>& pt) {
   for (int i = 0; i <= nr; ++i) h[off_ar + i] = ar[i];
   if (g->has_disc) {
     const double dz = (d.x1[2] - d.x0[2]) / nz, Om = d.omega_frame, gam = d.gamma;
-    auto prim = [&](double r, double z, double* out, size_t stride, int nv) {
+    auto prim = [&](int axis, size_t at, double r, double z) {
       double rho, vth, p, dlnp;
       equilibrium_prim(d, g->disc, r, z, rho, vth, p, &dlnp);
-      const double v0 = vth - Om * r, c0 = std::sqrt(gam * p / rho);
-      out[0] = rho;
-      out[stride] = v0;
-      out[2 * stride] = p;
-      out[3 * stride] = c0;
-      out[4 * stride] = 0.5 * rho * v0 * v0 + gam * p / (gam - 1.0);
-      if (nv == 7) {
-        out[5 * stride] = v0 - c0;
-        out[6 * stride] = v0 + c0;
+      const double v0 = vth - Om * r, c0 = std::sqrt(gam * p / rho), un = axis == 1 ? v0 : 0.0;
+      const double f[4] = {rho, v0, p, 0.5 * rho * v0 * v0 + gam * p / (gam - 1.0)};
+      const double w[4] = {c0, un - c0, un + c0, 0.0};
+      for (int q = 0; q < 4; ++q) {
+        h[off_face[axis] + 4 * at + q] = f[q];
+        h[off_wave[axis] + 4 * at + q] = w[q];
       }
     };
     for (int k = 0; k < nz; ++k) {
@@ -568,22 +593,22 @@ rossbi_status build_pert_tables(rossbi_grid* g, PertTables<T>& pt) {
         equilibrium_prim(d, g->disc, r, z, rho, vth, p, &dlnp);
         const double v0 = vth - Om * r, R2 = r * r + z * z, R3 = R2 * std::sqrt(R2);
         const double cs2 = g->disc.T0 * std::pow(r, g->disc.beta_T);
-        double* c = &h[off_cen + (size_t)k * nr + i];
+        double* c = &h[off_cen + 8 * ((size_t)k * nr + i)];
         c[0] = rho;
-        c[ncen] = v0;
-        c[2 * ncen] = p;
-        c[3 * ncen] = cs2 * dlnp;                       // (1/rho0) dP0/dr
-        c[4 * ncen] = -d.gm * z / R3;                   // f_z
-        c[5 * ncen] = -d.gm * r / R3 + Om * Om * r;     // f_r + Omega^2 r
-        c[6 * ncen] = 2.0 * v0 / r + 2.0 * Om;
-        c[7 * ncen] = 1.0 / r;
-        prim(r, z, &h[off_ft + (size_t)k * nr + i], ncen, 7);
+        c[1] = v0;
+        c[2] = p;
+        c[3] = cs2 * dlnp;                       // (1/rho0) dP0/dr
+        c[4] = -d.gm * z / R3;                   // f_z
+        c[5] = -d.gm * r / R3 + Om * Om * r;     // f_r + Omega^2 r
+        c[6] = 2.0 * v0 / r + 2.0 * Om;
+        c[7] = 1.0 / r;
+        prim(1, (size_t)k * nr + i, r, z);
       }
-      for (int i = 0; i <= nr; ++i) prim(axis0_face(d, i), z, &h[off_fr + (size_t)k * (nr + 1) + i], nfr, 5);
+      for (int i = 0; i <= nr; ++i) prim(0, (size_t)k * (nr + 1) + i, axis0_face(d, i), z);
     }
     for (int k = 0; k <= nz; ++k) {
       const double z = d.x0[2] + k * dz;
-      for (int i = 0; i < nr; ++i) prim(axis0_centre(d, i), z, &h[off_fz + (size_t)k * nr + i], nfz, 5);
+      for (int i = 0; i < nr; ++i) prim(2, (size_t)k * nr + i, axis0_centre(d, i), z);
     }
   }
   std::vector<T> ht(total);
@@ -594,9 +619,10 @@ rossbi_status build_pert_tables(rossbi_grid* g, PertTables<T>& pt) {
   CK(cudaMemcpy(g->d_ptab, ht.data(), total * sizeof(T), cudaMemcpyHostToDevice));
   const T* b = (const T*)g->d_ptab;
   pt.cen = b + off_cen;
-  pt.fr = b + off_fr;
-  pt.fz = b + off_fz;
-  pt.ft = b + off_ft;
+  for (int q = 0; q < 3; ++q) {
+    pt.face[q] = b + off_face[q];
+    pt.wave[q] = b + off_wave[q];
+  }
   pt.rcoef = b + off_rc;
   pt.vol = b + off_vol;
   pt.ivol = b + off_ivol;
@@ -632,9 +658,8 @@ PertArgs<T> pert_args(rossbi_grid* g) {
   a.gam = (T)g->dg.gamma;
   a.om = (T)g->dg.omega;
   a.cfl = (T)g->dg.cfl;
-  a.dx1 = (T)g->dg.dx[1];
-  a.dx2 = (T)g->dg.dx[2];
-  for (int sp = 0; sp < ND_MAX; ++sp) a.st_factor[sp] = (T)g->dg.st_factor[sp];
+  a.gm1 = (T)(g->dg.gamma - 1.0);
+  a.g_gm1 = (T)g->dg.near.g_gm1;
   return a;
 }
 
@@ -642,9 +667,11 @@ PertArgs<T> pert_args(rossbi_grid* g) {
 template <class T>
 void set_pert_drag(PertArgs<T>& a, const DragArgs& drag) {
   a.drag = drag;
-  a.stokes = (T)drag.stokes;
-  a.rhos_rp = (T)drag.rhos_rp;
   a.kappa = (T)drag.kappa;
+  for (int sp = 0; sp < ND_MAX; ++sp) {
+    a.ist[sp] = (T)drag.ist[sp];
+    a.irr[sp] = (T)drag.irr[sp];
+  }
 }
 
 // Drag parameters of a step (Sect. 2.9 drag law; Epstein constant fixed so
@@ -1202,7 +1229,7 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   const bool pert = desc->precision != ROSSBI_FP64;  // tile of the form's stage kernel
   const bool flat = !pert && flat_grid(desc->nz, desc->bc_lo[2], desc->bc_hi[2], g->nf);
   const int tr = pert ? P32_TR : F64_TR, tt = pert ? P32_TT : (flat ? FLAT_TT : F64_TT);
-  const int tz = flat ? 1 : tile_z(desc->precision != ROSSBI_FP32_PERT, g->nf);
+  const int tz = flat ? 1 : tile_z(desc->precision == ROSSBI_FP64_PERT, g->nf);
   g->tile_tt = tt;
   g->tiles_r = (desc->nr + tr - 1) / tr;
   g->tiles_t = (desc->nth + tt - 1) / tt;
@@ -1222,14 +1249,14 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
     // x0, in the differences dm = e0 - em, dp = ep - e0:
     // q(x0 - hm) = e0 - (w2 dm + w3 dp), q(x0 + hp) = e0 + (w4 dm + w5 dp)
     const double hm = x0 - fm, hp = fp - x0, dl = x0 - xm, dr = xp - x0, dx = xp - xm;
-    w[0] = 1.0 / dl;
-    w[1] = 1.0 / dr;
+    const double lo = std::min(2.0 * hm, dl), up = std::min(2.0 * hp, dr);  // limiter reaches
+    w[0] = lo / dl;  // lower limit min(w0 dm, w1 dp), upper limit w6 times that
+    w[1] = lo / dr;
     w[2] = hm * (dr + hm) / (dl * dx);
     w[3] = hm * (dl - hm) / (dr * dx);
     w[4] = hp * (dr - hp) / (dl * dx);
     w[5] = hp * (dl + hp) / (dr * dx);
-    w[6] = std::min(2.0 * hm, dl);  // limiter reach on the lower side
-    w[7] = std::min(2.0 * hp, dr);  // and on the upper side
+    w[6] = up / lo;
   }
   std::vector<double> vol(nr), ivol(nr), ar(nr + 1), at(nr), az(nr), maxA(nr);
   if (d.geometry == ROSSBI_GEOM_CYL) {  // Sect. 2.2 finite volumes of the cylindrical mesh

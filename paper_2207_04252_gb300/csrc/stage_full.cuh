@@ -42,21 +42,22 @@ struct StageArgs {
 // dp = ep - e0 the parabola's face deviations are -(am dm + ap dp) and bm dm +
 // bp dp with positive weights (of the geometry alone, tabulated), so that
 // where dm and dp have one sign they have it too, and the limiter is a
-// minimum of magnitudes: w = {1/(x0-xm), 1/(xp-x0), am, ap, bm, bp, h-, h+}.
-// UNI: a uniform axis, where in units of the spacing am = bp = 3/8, ap = bm =
-// 1/8 and both reaches are 1.  8 (uniform) or 12 FP64 operations; forming the
-// slopes, the curvature and the limiter's products took 17 and four compares.
+// minimum of magnitudes: w = {lm, lp, am, ap, bm, bp, h+/h-}, the lower
+// limit min(lm dm, lp dp) being h- times the slope.  UNI: a uniform axis, where
+// in units of the spacing am = bp = 3/8, ap = bm = 1/8 and all limits 1.
+// 6 (uniform) or 11 FP64 operations; forming the slopes, the curvature and the
+// limiter's products took 17 and four compares.
 template <bool UNI>
 __device__ __forceinline__ void parabola(double em, double e0, double ep, const double* w, double& qm, double& qp) {
   const double dm = e0 - em, dp = ep - e0;
   if (UNI) {
-    const double s = minmod_bits(dm, dp), u = 0.125 * (dm + dp);
-    qm = e0 - min_mag(fma(0.25, dm, u), s);
-    qp = e0 + min_mag(fma(0.25, dp, u), s);
+    const double s = minmod_bits(dm, dp);
+    qm = e0 - min_mag(fma(0.375, dm, scale_down<3>(dp)), s);
+    qp = e0 + min_mag(fma(0.375, dp, scale_down<3>(dm)), s);
   } else {
     const double s = minmod_bits(dm * w[0], dp * w[1]);
-    qm = e0 - min_mag(fma(w[2], dm, w[3] * dp), w[6] * s);
-    qp = e0 + min_mag(fma(w[4], dm, w[5] * dp), w[7] * s);
+    qm = e0 - min_mag(fma(w[2], dm, w[3] * dp), s);
+    qp = e0 + min_mag(fma(w[4], dm, w[5] * dp), w[6] * s);
   }
 }
 template <bool UNI>
@@ -68,8 +69,8 @@ __device__ __forceinline__ void parabola(float em, float e0, float ep, const flo
     qp = e0 + min_xorsign(fmaf(0.25f, dp, u), s);
   } else {
     const float s = fmaxf(min_xorsign(dm * w[0], dp * w[1]), 0.0f);
-    qm = e0 - min_xorsign(fmaf(w[2], dm, w[3] * dp), w[6] * s);
-    qp = e0 + min_xorsign(fmaf(w[4], dm, w[5] * dp), w[7] * s);
+    qm = e0 - min_xorsign(fmaf(w[2], dm, w[3] * dp), s);
+    qp = e0 + min_xorsign(fmaf(w[4], dm, w[5] * dp), w[6] * s);
   }
 }
 
@@ -83,9 +84,8 @@ __device__ __forceinline__ unsigned parabola_branches(double em, double e0, doub
   const double dm = e0 - em, dp = ep - e0;
   double sm = dm, sp = dp, A, B, lo, up;
   if (UNI) {
-    const double u = 0.125 * (dm + dp);
-    A = fma(0.25, dm, u);
-    B = fma(0.25, dp, u);
+    A = fma(0.375, dm, scale_down<3>(dp));
+    B = fma(0.375, dp, scale_down<3>(dm));
   } else {
     sm = dm * w[0];
     sp = dp * w[1];
@@ -93,8 +93,8 @@ __device__ __forceinline__ unsigned parabola_branches(double em, double e0, doub
     B = fma(w[4], dm, w[5] * dp);
   }
   const double s = minmod_bits(sm, sp);
-  lo = UNI ? s : w[6] * s;
-  up = UNI ? s : w[7] * s;
+  lo = s;
+  up = UNI ? s : w[6] * s;
   const bool a = mag_less(A, lo), b = mag_less(B, up);
   qm = e0 - (a ? A : lo);
   qp = e0 + (b ? B : up);
@@ -145,26 +145,22 @@ __device__ __forceinline__ bool resolve_cell(const DevGrid& g, int c[3]) {
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
-template <int NF, int TR, int TT, int TZ, int NT, int D, int RC>
-__device__ __forceinline__ void sweep_full(const StageArgs& a, const double* sE, double* sG, int i0, int j0, int k0,
-                                           unsigned& status) {
-  constexpr int ZH = TZ == 1 ? 0 : 2;  // z halo (none in the flat one-z-cell tile)
-  constexpr int BX = TR + 4, BY = TT + 4, BZ = TZ + 2 * ZH, BOX = BX * BY * BZ, NCORE = TR * TT * TZ;
-  constexpr int TD = D == 0 ? TR : (D == 1 ? TT : TZ);
-  constexpr int L = pow2ceil(TD + 2);
+// One lane of a sweep along axis D of a TR x TT x TZ tile: its cell, and
+// what of it is inside the grid.
+template <int TR, int TT, int TZ, int D>
+struct SweepLane {
+  static constexpr int ZH = TZ == 1 ? 0 : 2;  // z halo (none in the flat one-z-cell tile)
+  static constexpr int BX = TR + 4, BY = TT + 4, BZ = TZ + 2 * ZH, BOX = BX * BY * BZ, NCORE = TR * TT * TZ;
+  static constexpr int TD = D == 0 ? TR : (D == 1 ? TT : TZ);
+  static constexpr int L = pow2ceil(TD + 2);
+  static constexpr int NA = D == 0 ? TT : TR;
+  static constexpr int NB = D == 2 ? TT : TZ;
+  static constexpr int ITEMS = NA * NB * L;
+  static constexpr int STRIDE = D == 0 ? 1 : (D == 1 ? BX : BX * BY);
   static_assert(L <= 32, "line does not fit a warp");
-  constexpr int NA = D == 0 ? TT : TR;
-  constexpr int NB = D == 2 ? TT : TZ;
-  constexpr int ITEMS = NA * NB * L;
-  constexpr int STRIDE = D == 0 ? 1 : (D == 1 ? BX : BX * BY);
-  constexpr int NW = NT / 32;
-  constexpr unsigned FULL = 0xffffffffu;
-  const DevGrid& g = a.g;
-  const double gam = g.gamma;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-
-  for (int base = warp * 32; base < ITEMS; base += NW * 32) {
-    const int item = base + lane;
+  int gi, gk, gd, sidx, core;
+  bool do_recon, do_face, do_acc;
+  __device__ __forceinline__ SweepLane(const DevGrid& g, int item, int i0, int j0, int k0) {
     const bool valid = item < ITEMS;
     const int line = valid ? item / L : 0;
     const int c = item % L - 1;
@@ -172,25 +168,57 @@ __device__ __forceinline__ void sweep_full(const StageArgs& a, const double* sE,
     const int x = D == 0 ? c : ta;
     const int y = D == 1 ? c : (D == 0 ? ta : tb);
     const int z = D == 2 ? c : tb;
-    const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
+    gi = i0 + x;
+    gk = k0 + z;
+    const int gj = j0 + y;
     const bool line_ok = valid && (D == 0 ? (gj < g.nth && gk < g.nz)
                                           : (D == 1 ? (gi < g.nr && gk < g.nz) : (gi < g.nr && gj < g.nth)));
-    const int gd = D == 0 ? gi : (D == 1 ? gj : gk);
+    gd = D == 0 ? gi : (D == 1 ? gj : gk);
     const int nd = D == 0 ? g.nr : (D == 1 ? g.nth : g.nz);
-    const bool do_recon = line_ok && c <= TD && gd <= nd;
-    const bool do_face = do_recon && c >= 0;
-    const bool do_acc = line_ok && c >= 0 && c < TD && gd < nd;
-    const int sidx = do_recon ? ((z + ZH) * BY + (y + 2)) * BX + (x + 2) : (ZH * BY + 2) * BX + 2;
+    do_recon = line_ok && c <= TD && gd <= nd;
+    do_face = do_recon && c >= 0;
+    do_acc = line_ok && c >= 0 && c < TD && gd < nd;
+    sidx = do_recon ? ((z + ZH) * BY + (y + 2)) * BX + (x + 2) : (ZH * BY + 2) * BX + 2;
+    core = (z * TT + y) * TR + x;
+  }
+};
 
-    constexpr bool UNI = D != 0;
+template <int D>
+__device__ __forceinline__ double face_area(const DevGrid& g, int gi, int ci) {
+  return D == 0 ? g.area_r[clampi(gi, 0, g.nr)] : (D == 1 ? g.area_t[ci] : g.area_z[ci]);
+}
+
+// Writes (D = 0) or adds the flux divergence F - (F of the lane above) of the
+// lane's cell to the field's accumulator.
+template <int D, int L>
+__device__ __forceinline__ void accumulate(double F, double* dst, bool own) {
+  const double Fu = __shfl_down_sync(0xffffffffu, F, 1, L);
+  if (own) {
+    if (D == 0) *dst = F - Fu;
+    else *dst += F - Fu;
+  }
+}
+
+// The gas sweep along axis D: sE holds the five staged gas departures.
+template <int TR, int TT, int TZ, int NT, int D, int RC>
+__device__ __forceinline__ void sweep_gas(const StageArgs& a, const double* sE, double* sG, int i0, int j0, int k0,
+                                          unsigned& status) {
+  using S = SweepLane<TR, TT, TZ, D>;
+  constexpr int BOX = S::BOX, STRIDE = S::STRIDE, L = S::L;
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr bool UNI = D != 0;
+  const DevGrid& g = a.g;
+  const double gam = g.gamma;
+  for (int base = threadIdx.x & ~31; base < S::ITEMS; base += NT) {
+    const S s(g, base + (threadIdx.x & 31), i0, j0, k0);
+    if (!__any_sync(FULL, s.do_face)) continue;  // a warp of lines beyond a ragged grid's edge
     double w[RCW];
-    parabola_weights<double, D>(g.rcoef, gi, g.nr, w);
+    parabola_weights<double, D>(g.rcoef, s.gi, g.nr, w);
     // equilibrium gas state (conservative, or primitive with RC = RECON_PRIM)
     // on the lower face of this cell (index along D = gd) and on its upper
-    // face; table indices clamped
-    const int ci = clampi(gi, 0, g.nr - 1), ck = clampi(gk, 0, g.nz - 1);
+    // face; table indices clamped.  Its radial and vertical velocities are zero.
+    const int ci = clampi(s.gi, 0, g.nr - 1), ck = clampi(s.gk, 0, g.nz - 1);
     auto eq_face = [&](int f, int fd) -> double {
-      if (!g.has_eq) return 0.0;
       const double* tc = RC == RECON_PRIM ? g.w0c : g.e0c;
       const double* tr = RC == RECON_PRIM ? g.w0r : g.e0r;
       const double* tz = RC == RECON_PRIM ? g.w0z : g.e0z;
@@ -198,93 +226,80 @@ __device__ __forceinline__ void sweep_full(const StageArgs& a, const double* sE,
       if (D == 1) return tc[((size_t)f * g.nz + ck) * g.nr + ci];
       return tz[((size_t)f * (g.nz + 1) + clampi(fd, 0, g.nz)) * g.nr + ci];
     };
-    double area = 0.0;
-    if (do_face) area = D == 0 ? g.area_r[clampi(gi, 0, g.nr)] : (D == 1 ? g.area_t[ci] : g.area_z[ci]);
-
-    // ---------------- gas: departures in slots 0..4
+    double WR[5], WP[5];  // primitives: right state of the lower face, left state of the upper face
     {
-      double WR[5], WP[5];  // primitives: right state of the lower face, left state of the upper face
-      {
-        double qm[5], qp[5];
-#pragma unroll
-        for (int f = 0; f < 5; ++f) {
-          const double* s = sE + f * BOX + sidx;
-          parabola<UNI>(s[-STRIDE], s[0], s[STRIDE], w, qm[f], qp[f]);
-        }
-        // face states E0 + q on both faces of this cell (Sect. 2.7); flat
-        // departures if either is not physical
-        auto face_states = [&]() {
-          double Um[5], Up[5];
-#pragma unroll
-          for (int f = 0; f < 5; ++f) {
-            Um[f] = eq_face(f, gd) + qm[f];
-            Up[f] = eq_face(f, gd + 1) + qp[f];
-          }
-          if (RC == RECON_PRIM) {
-#pragma unroll
-            for (int f = 0; f < 5; ++f) {
-              WR[f] = Um[f];
-              WP[f] = Up[f];
-            }
-          } else {
-            gas_prim(gam, Um, WR);
-            gas_prim(gam, Up, WP);
-          }
-          return positive(Um[RHO]) && positive(Up[RHO]) && positive(WR[EN]) && positive(WP[EN]);
-        };
-        if (!face_states() && do_recon) {
-#pragma unroll
-          for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + sidx];
-          face_states();
-        }
-      }
-      double F[5], WL[5];
-#pragma unroll
-      for (int f = 0; f < 5; ++f) WL[f] = __shfl_up_sync(FULL, WP[f], 1, L);
-      if (do_face) {
-        gas_face_flux<D>(g.near, area, WL, WR, F, status);
-      } else {
-#pragma unroll
-        for (int f = 0; f < 5; ++f) F[f] = 0.0;
-      }
+      double qm[5], qp[5];
 #pragma unroll
       for (int f = 0; f < 5; ++f) {
-        const double Fu = __shfl_down_sync(FULL, F[f], 1, L);
-        if (do_acc) {
-          double* dst = sG + f * NCORE + (z * TT + y) * TR + x;
-          if (D == 0) *dst = F[f] - Fu;
-          else *dst += F[f] - Fu;
-        }
+        const double* e = sE + f * BOX + s.sidx;
+        parabola<UNI>(e[-STRIDE], e[0], e[STRIDE], w, qm[f], qp[f]);
       }
-    }
-    // ---------------- dust: each species' fields b .. b + 3, primitive
-    // reconstruction, kinetic flux
-#pragma unroll 1
-    for (int b = 5; b < NF; b += 4) {
-      double qm[4], qp[4];
-      dust_recon<double, BOX, STRIDE, UNI>(sE, sidx, b, w, qm, qp);
-      double F[4];
-      {
-        double WL[4];
+      // face states E0 + q on both faces of this cell (Sect. 2.7); flat
+      // departures if either is not physical
+      auto face_states = [&]() {
+        if (g.has_eq) {
 #pragma unroll
-        for (int f = 0; f < 4; ++f) WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
-        if (do_face) {
-          dust_kinetic_flux<D>(area, WL, qm, F);
+          for (int f : {MV, EN, RHO}) {
+            qm[f] += eq_face(f, s.gd);
+            qp[f] += eq_face(f, s.gd + 1);
+          }
+        }
+        if (RC == RECON_PRIM) {
+#pragma unroll
+          for (int f = 0; f < 5; ++f) {
+            WR[f] = qm[f];
+            WP[f] = qp[f];
+          }
         } else {
-#pragma unroll
-          for (int f = 0; f < 4; ++f) F[f] = 0.0;
+          gas_prim(gam, qm, WR);
+          gas_prim(gam, qp, WP);
         }
-      }
+        return positive(qm[RHO]) && positive(qp[RHO]) && positive(WR[EN]) && positive(WP[EN]);
+      };
+      if (!face_states() && s.do_recon) {
 #pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        const double Fu = __shfl_down_sync(FULL, F[f], 1, L);
-        if (do_acc) {
-          double* dst = sG + (b + f) * NCORE + (z * TT + y) * TR + x;
-          if (D == 0) *dst = F[f] - Fu;
-          else *dst += F[f] - Fu;
-        }
+        for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + s.sidx];
+        face_states();
       }
     }
+    double F[5], WL[5];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) WL[f] = __shfl_up_sync(FULL, WP[f], 1, L);
+    if (s.do_face) {
+      gas_face_flux<D>(g.near, face_area<D>(g, s.gi, ci), WL, WR, F, status);
+    } else {
+#pragma unroll
+      for (int f = 0; f < 5; ++f) F[f] = 0.0;
+    }
+#pragma unroll
+    for (int f = 0; f < 5; ++f) accumulate<D, L>(F[f], sG + f * S::NCORE + s.core, s.do_acc);
+  }
+}
+
+// The sweep of one dust species along axis D: sE holds its staged primitives
+// (u, v, w, rho_d), sG its accumulators.
+template <int TR, int TT, int TZ, int NT, int D>
+__device__ __forceinline__ void sweep_dust(const StageArgs& a, const double* sE, double* sG, int i0, int j0, int k0) {
+  using S = SweepLane<TR, TT, TZ, D>;
+  constexpr int L = S::L;
+  constexpr unsigned FULL = 0xffffffffu;
+  const DevGrid& g = a.g;
+  for (int base = threadIdx.x & ~31; base < S::ITEMS; base += NT) {
+    const S s(g, base + (threadIdx.x & 31), i0, j0, k0);
+    if (!__any_sync(FULL, s.do_face)) continue;
+    double w[RCW], qm[4], qp[4], F[4], WL[4];
+    parabola_weights<double, D>(g.rcoef, s.gi, g.nr, w);
+    dust_recon<double, S::BOX, S::STRIDE, D != 0>(sE, s.sidx, 0, w, qm, qp);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
+    if (s.do_face) {
+      dust_kinetic_flux<D>(face_area<D>(g, s.gi, clampi(s.gi, 0, g.nr - 1)), WL, qm, F);
+    } else {
+#pragma unroll
+      for (int f = 0; f < 4; ++f) F[f] = 0.0;
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) accumulate<D, L>(F[f], sG + f * S::NCORE + s.core, s.do_acc);
   }
 }
 
@@ -360,13 +375,13 @@ __device__ __forceinline__ void block_results(const double* sums, double dtmin, 
 // periodic or outflow: both z ghosts of the cell are the cell itself, its two
 // z faces carry the same flux, and the z sweep, whose divergence is exactly
 // zero, is skipped (as is the z halo).
-template <int NF, int TR, int TT, int TZ, int NT, bool XT, int RC>
-__global__ void __launch_bounds__(NT, 1) stage_full_kernel(const StageArgs a) {
+template <int NF, int TR, int TT, int TZ, int NT, int MINB, bool XT, int RC>
+__global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a) {
   constexpr int ZH = TZ == 1 ? 0 : 2;
   constexpr int BX = TR + 4, BY = TT + 4, BZ = TZ + 2 * ZH, BOX = BX * BY * BZ, NCORE = TR * TT * TZ;
   extern __shared__ double smem[];
-  double* sE = smem;
-  double* sG = smem + NF * BOX;
+  double* sE = smem;             // [5][BOX] the gas departures, then the four primitives of one dust species at a time
+  double* sG = smem + 5 * BOX;   // [NF][NCORE] flux divergence
   const DevGrid& g = a.g;
   const int tile = blockIdx.x;
   // r fastest, then z, then theta: the tiles whose halos a tile re-reads
@@ -377,50 +392,77 @@ __global__ void __launch_bounds__(NT, 1) stage_full_kernel(const StageArgs a) {
   const int j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
   unsigned status = 0;
 
-  // tile + halo as deviations (corners are never read): the gas departures
-  // E' = E - E0 (or, with RC = RECON_PRIM, the primitive departures
-  // u', v', w', P', rho') in slots 0..4, the dust as it is
-  for (int idx = threadIdx.x; idx < BOX; idx += NT) {
-    const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - ZH;
-    const int outside = (x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ);
-    if (outside > 1) continue;
-    int c[3] = {i0 + x, j0 + y, k0 + z};
-    if (!resolve_cell(g, c)) {
+  // tile + halo (edges and corners are never read): put(idx, cell or null)
+  // for every staged cell, null for an equilibrium ghost
+  auto stage = [&](auto&& put) {
+    for (int idx = threadIdx.x; idx < BOX; idx += NT) {
+      const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - ZH;
+      const int outside = (x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ);
+      if (outside > 1) continue;
+      int c[3] = {i0 + x, j0 + y, k0 + z};
+      put(idx, resolve_cell(g, c) ? c : nullptr);
+    }
+  };
+  // the gas as deviations E' = E - E0 (or, with RC = RECON_PRIM, the primitive
+  // departures u', v', w', P', rho') in slots 0..4
+  stage([&](int idx, const int* c) {
+    if (!c) {
 #pragma unroll
-      for (int f = 0; f < NF; ++f) sE[f * BOX + idx] = 0.0;
-      continue;
+      for (int f = 0; f < 5; ++f) sE[f * BOX + idx] = 0.0;
+      return;
     }
     const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
     const size_t e0o = (size_t)c[2] * g.nr + c[0], e0s = (size_t)g.nz * g.nr;
-    if (RC == RECON_PRIM) {
-      double U[5], W[5];
+    double U[5], W[5];
 #pragma unroll
-      for (int f = 0; f < 5; ++f) U[f] = a.in[f][lin];
-      gas_prim(g.gamma, U, W);
+    for (int f = 0; f < 5; ++f) U[f] = a.in[f][lin];
+    if (RC == RECON_PRIM) gas_prim(g.gamma, U, W);
+    const double* e0 = RC == RECON_PRIM ? g.w0c : g.e0c;
 #pragma unroll
-      for (int f = 0; f < 5; ++f) sE[f * BOX + idx] = g.has_eq ? W[f] - g.w0c[f * e0s + e0o] : W[f];
-    } else {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) sE[f * BOX + idx] = g.has_eq ? a.in[f][lin] - g.e0c[f * e0s + e0o] : a.in[f][lin];
+    for (int f = 0; f < 5; ++f) {
+      double v = RC == RECON_PRIM ? W[f] : U[f];
+      if (g.has_eq && f != MU && f != MW) v -= e0[f * e0s + e0o];
+      sE[f * BOX + idx] = v;
     }
-    // the dust as primitives (u, v, w, rho_d): converted once per staged cell,
-    // not by every lane that reconstructs from it
-#pragma unroll
-    for (int b = 5; b < NF; b += 4) {
-      const double rd = a.in[b + 3][lin], id = positive(rd) ? recip(rd) : 0.0;
-#pragma unroll
-      for (int c3 = 0; c3 < 3; ++c3) sE[(b + c3) * BOX + idx] = a.in[b + c3][lin] * id;
-      sE[(b + 3) * BOX + idx] = rd;
-    }
-  }
+  });
   __syncthreads();
-  sweep_full<NF, TR, TT, TZ, NT, 0, RC>(a, sE, sG, i0, j0, k0, status);
+  sweep_gas<TR, TT, TZ, NT, 0, RC>(a, sE, sG, i0, j0, k0, status);
   __syncthreads();
-  sweep_full<NF, TR, TT, TZ, NT, 1, RC>(a, sE, sG, i0, j0, k0, status);
+  sweep_gas<TR, TT, TZ, NT, 1, RC>(a, sE, sG, i0, j0, k0, status);
   __syncthreads();
   if constexpr (TZ > 1) {
-    sweep_full<NF, TR, TT, TZ, NT, 2, RC>(a, sE, sG, i0, j0, k0, status);
+    sweep_gas<TR, TT, TZ, NT, 2, RC>(a, sE, sG, i0, j0, k0, status);
     __syncthreads();
+  }
+  // then each dust species through the same buffer, as primitives (u, v, w,
+  // rho_d) converted once per staged cell.  One species at a time keeps a
+  // nine-field block at 108 KB, two blocks to an SM, whose barriers and staging
+  // overlap (all fields staged at once: 166 KB, one block of six warps, FP64
+  // pipe 75 % busy), and lets every species count have the 14 x 6 x 6 tile.
+#pragma unroll 1
+  for (int b = 5; b < NF; b += 4) {
+    stage([&](int idx, const int* c) {
+      if (!c) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) sE[f * BOX + idx] = 0.0;
+        return;
+      }
+      const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
+      const double rd = a.in[b + 3][lin], id = positive(rd) ? recip(rd) : 0.0;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) sE[q * BOX + idx] = a.in[b + q][lin] * id;
+      sE[3 * BOX + idx] = rd;
+    });
+    __syncthreads();
+    double* sD = sG + b * NCORE;
+    sweep_dust<TR, TT, TZ, NT, 0>(a, sE, sD, i0, j0, k0);
+    __syncthreads();
+    sweep_dust<TR, TT, TZ, NT, 1>(a, sE, sD, i0, j0, k0);
+    __syncthreads();
+    if constexpr (TZ > 1) {
+      sweep_dust<TR, TT, TZ, NT, 2>(a, sE, sD, i0, j0, k0);
+      __syncthreads();
+    }
   }
 
   const double tau = a.tau_frac * (a.dt_dev ? __longlong_as_double((long long)*a.dt_dev) : a.dt_host);
@@ -442,15 +484,13 @@ __global__ void __launch_bounds__(NT, 1) stage_full_kernel(const StageArgs a) {
       G[f] = sG[f * NCORE + cidx];
     }
     {
-      double W[5], Vd[ND][2];
+      double W[5], Vd[ND];
       gas_prim(g.gamma, U, W);
       bool bad = !positive(U[RHO]) || !positive(W[EN]);
 #pragma unroll
       for (int b = 5; b < NF; b += 4) {
         bad |= !non_negative(U[b + 3]);
-        const int sidx = ((z + ZH) * BY + (y + 2)) * BX + (x + 2);  // the staged velocities
-        Vd[(b - 5) / 4][0] = sE[b * BOX + sidx];
-        Vd[(b - 5) / 4][1] = sE[(b + 1) * BOX + sidx];
+        Vd[(b - 5) / 4] = positive(U[b + 3]) ? U[b + 1] * recip(U[b + 3]) : 0.0;
       }
       if (bad) status |= STATUS_NONPHYSICAL;
       if (g.geom == GEOM_CYL) add_sources<XT, NF>(g, gi, gj, gk, U, W, Vd, G);

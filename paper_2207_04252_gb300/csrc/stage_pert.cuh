@@ -13,8 +13,10 @@
 //     dP = (gamma-1)(E' - [rho' |u0|^2/2 + rho u0.du + rho |du|^2/2]);
 //     with RC = RECON_PRIM the same conversion is applied to each cell and
 //     the parabola acts on the primitive perturbations instead;
-//   - the exact Riemann solver (Sect. 2.6) iterates on dp* = p* - p0 with
-//     the pressure functions written in p/p_K - 1 (log1p / expm1 for the
+//   - the exact Riemann solution (Sect. 2.6) comes from the series near p_K
+//     (riemann_near.cuh) in the differences of the two side perturbations;
+//     where they do not reach, a solver out of line iterates on dp* = p* - p0
+//     with the pressure functions written in p/p_K - 1 (log1p / expm1 for the
 //     rarefaction powers), samples the wave pattern on full values and returns
 //     the face-state perturbation; near-sonic fans use the FP64-derived
 //     u0 -/+ c0 of the face;
@@ -29,33 +31,15 @@
 
 namespace rossbi {
 
-template <class T, int BOX, int S, bool UNI>
-__device__ __forceinline__ void dust_recon_cons(const T* sE, int sidx, int b, const T* w, T* wm, T* wp) {
-  T pm[4], p0[4], pp[4];
-  const T* r = sE + (b + 3) * BOX + sidx;
-  pm[3] = r[-S];
-  p0[3] = r[0];
-  pp[3] = r[S];
-  const T im = pm[3] > T(0) ? T(1) / pm[3] : T(0);
-  const T i0 = p0[3] > T(0) ? T(1) / p0[3] : T(0);
-  const T ip = pp[3] > T(0) ? T(1) / pp[3] : T(0);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const T* m = sE + (b + c) * BOX + sidx;
-    pm[c] = m[-S] * im;
-    p0[c] = m[0] * i0;
-    pp[c] = m[S] * ip;
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) parabola<UNI>(pm[q], p0[q], pp[q], w, wm[q], wp[q]);
-}
-
+// Equilibrium and metric tables in the state precision.  A cell's or a face's
+// values are adjacent, so that a lane takes them in 16-byte loads from one
+// address.
 template <class T>
 struct PertTables {
-  const T* cen;    // [8][nz][nr]   rho0, v0, p0, C_r, f_z, f_r + Omega^2 r, 2 v0/r + 2 Omega, 1/r
-  const T* fr;     // [5][nz][nr+1] rho0, v0, p0, c0, h0 on r faces   (h0 = E0 + p0)
-  const T* fz;     // [5][nz+1][nr] same on z faces
-  const T* ft;     // [7][nz][nr]   same on theta faces (= centres), then v0 - c0, v0 + c0
+  const T* cen;      // [nz][nr][8] rho0, v0, p0, C_r, f_z, f_r + Omega^2 r, 2 v0/r + 2 Omega, 1/r
+  const T* face[3];  // [..][4] rho0, v0, p0, h0 (= E0 + p0) on r faces [nz][nr+1], theta faces (= centres)
+                     // [nz][nr] and z faces [nz+1][nr]
+  const T* wave[3];  // [..][4] c0, u0 - c0, u0 + c0 (u0 normal to the face), for the general solver
   const T* rcoef;  // axis-0 parabola weights, RCW per cell as DevGrid::rcoef
   const T* vol;
   const T* ivol;
@@ -166,43 +150,31 @@ struct PowG75 {
   }
 };
 
-// Face equilibrium in the frame of a face normal to axis D.
+// Face equilibrium as the general solver takes it, in the frame of the face's normal.
 template <class T>
 struct PFace {
-  T rho, un, ut1, ut2, p, c, h, un_mc, un_pc;
+  T rho, un, p, c, un_mc, un_pc;
 };
 
 // Perturbation of one side of a face, with the full values the wave pattern needs.
 template <class T>
 struct PSide {
-  T drho, dun, dut1, dut2, dp;  // perturbations
-  T rho, un, p, c, dc;          // full values and c - c0
+  T drho, dun, dp;      // perturbations
+  T rho, un, p, c, dc;  // full values and c - c0
 };
 
-// Face primitive perturbations (du, dv, dw, dP, drho in the field slots MU,
-// MV, MW, EN, RHO) about the face equilibrium, in the frame of axis D, with
-// the full values the wave pattern needs.  Returns false if the full state is
-// not physical.
-template <class T, int D>
-__device__ __forceinline__ bool pert_side(T g, const PFace<T>& W0, const T* q, bool has_eq, PSide<T>& s) {
-  const T dur = q[MU], dvt = q[MV], dwz = q[MW], dp = q[EN];
-  const T rho = W0.rho + q[RHO];
-  s.drho = q[RHO];
+template <class T>
+__device__ __forceinline__ PSide<T> pert_side(T g, const PFace<T>& W0, T drho, T dun, T dp, bool has_eq) {
+  PSide<T> s;
+  s.drho = drho;
+  s.dun = dun;
   s.dp = dp;
-  s.dun = D == 0 ? dur : (D == 1 ? dvt : dwz);
-  s.dut1 = D == 0 ? dvt : dur;
-  s.dut2 = D == 2 ? dvt : dwz;
-  s.rho = rho;
+  s.rho = W0.rho + drho;
   s.p = W0.p + dp;
-  s.un = W0.un + s.dun;
-  if (!(rho > T(0)) || !(s.p > T(0))) return false;
-  s.c = Math<T>::sqrt_(g * s.p / rho);
-  if (has_eq) {
-    s.dc = W0.c * sqrt1pm1((dp * W0.rho - W0.p * q[RHO]) / (W0.p * rho));
-  } else {
-    s.dc = s.c;
-  }
-  return true;
+  s.un = W0.un + dun;
+  s.c = Math<T>::sqrt_(g * s.p / s.rho);
+  s.dc = has_eq ? W0.c * sqrt1pm1((dp * W0.rho - W0.p * drho) / (W0.p * s.rho)) : s.c;
+  return s;
 }
 
 // Reciprocals of a side that the series form of its pressure function uses.
@@ -357,21 +329,44 @@ __device__ __forceinline__ int pert_riemann(T g, const PFace<T>& W0, const PSide
   return 0;
 }
 
-// F(W0 + dW) - F(W0) through a face (App. B flux components, energy flux
-// (E + P) u_n), written without forming the equilibrium flux.  F is in face
-// order: mass, normal momentum, transverse momenta t1, t2, energy.
+// Equilibrium of a face: density, azimuthal velocity, pressure and E0 + p0.
 template <class T>
-__device__ __forceinline__ void pert_flux(T g, const PFace<T>& W0, T drho, T dun, T dut1, T dut2, T dp, T* F) {
-  const T un = W0.un + dun, ut1 = W0.ut1 + dut1, ut2 = W0.ut2 + dut2;
-  const T dmass = drho * un + W0.rho * dun;
-  const T m0 = W0.rho * W0.un;
-  F[0] = dmass;
-  F[1] = dmass * un + m0 * dun + dp;
-  F[2] = dmass * ut1 + m0 * dut1;
-  F[3] = dmass * ut2 + m0 * dut2;
-  const T du2 = dun * (T(2) * W0.un + dun) + dut1 * (T(2) * W0.ut1 + dut1) + dut2 * (T(2) * W0.ut2 + dut2);
-  const T dh = T(0.5) * drho * (un * un + ut1 * ut1 + ut2 * ut2) + T(0.5) * W0.rho * du2 + g / (g - T(1)) * dp;
-  F[4] = dh * un + W0.h * dun;
+struct PEq {
+  T rho, v, p, h;
+};
+__device__ __forceinline__ PEq<float> load_eq(const float* t) {
+  const float4 q = *reinterpret_cast<const float4*>(t);
+  return {q.x, q.y, q.z, q.w};
+}
+__device__ __forceinline__ PEq<double> load_eq(const double* t) {
+  const double2 q = reinterpret_cast<const double2*>(t)[0], r = reinterpret_cast<const double2*>(t)[1];
+  return {q.x, q.y, r.x, r.y};
+}
+
+// A (F(W0 + dW) - F(W0)) through a face of area A (App. B flux components,
+// energy flux (E + P) u_n), written without forming the equilibrium flux: the
+// face state differs from the equilibrium by drho, dp and the velocity
+// departures d[MU], d[MV], d[MW].  F in the field slots.
+template <class T, int D>
+__device__ __forceinline__ void pert_flux(T g_gm1, T area, const PEq<T>& W0, T drho, const T* d, T dp, T* F) {
+  constexpr int n = Axes<D>::n;
+  T v[3] = {d[MU], W0.v + d[MV], d[MW]};
+  const T un = v[n];
+  const T dm = drho * un + W0.rho * d[n];  // of the mass flux
+  const T du2 = d[MU] * d[MU] + d[MV] * (W0.v + v[MV]) + d[MW] * d[MW];
+  const T q2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+  const T dh = T(0.5) * (drho * q2 + W0.rho * du2) + g_gm1 * dp;
+  const T dmA = area * dm;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) F[q] = dmA * v[q];
+  if (D == 1) {  // the equilibrium mass flux rho0 v0 carries the velocity departures
+    const T m0 = area * (W0.rho * W0.v);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) F[q] += m0 * d[q];
+  }
+  F[n] += area * dp;
+  F[EN] = area * (dh * un + W0.h * d[n]);
+  F[RHO] = dmA;
 }
 
 // Face state perturbation of a Riemann solve, the side whose transverse
@@ -380,7 +375,7 @@ template <class T>
 struct PStar {
   T drho, dun, dp;
   int side;
-  unsigned status;
+  unsigned status, fallback;  // fallback: the FP64 solver took the face
 };
 
 // FP64 full-state solver on W0 + dW for the faces the perturbation solver
@@ -394,7 +389,7 @@ __device__ __noinline__ PStar<T> pert_fallback_fp64(T g, const PFace<T> W0, cons
   const double pl = (double)W0.p + (double)L.dp, pr = (double)W0.p + (double)R.dp;
   double rho, u, p;
   PStar<T> o;
-  o.status = 0;
+  o.status = o.fallback = 0;
   o.side = riemann_face((double)g, rl, ul, pl, rr, ur, pr, rho, u, p, o.status);
   o.drho = (T)(rho - (double)W0.rho);
   o.dun = (T)(u - (double)W0.un);
@@ -402,51 +397,25 @@ __device__ __noinline__ PStar<T> pert_fallback_fp64(T g, const PFace<T> W0, cons
   return o;
 }
 
-// Face-order gas flux perturbation (as pert_flux), status bits and whether
-// the FP64 fallback solved the face.
-template <class T>
-struct PFlux {
-  T F[5];
-  unsigned status, fallback;
-};
-
-// Gas flux perturbation through a face from the primitive perturbations of
-// its two reconstructed states (already checked physical).  One out-of-line
-// copy serves the three sweep directions; arguments and result by value.
+// The general solver of a face: near a strong wave or in the sonic band.  One
+// out-of-line copy serves the three sweep directions; arguments and result by
+// value.
 template <class T, class P>
-__device__ __noinline__ PFlux<T> pert_face_flux(T g, const PFace<T> W0, const PSide<T> L, const PSide<T> R) {
-  PFlux<T> o;
-  o.status = 0;
-  o.fallback = 0;
-  PStar<T> st;
-  st.side = 0;
-  if (pert_riemann<T, P>(g, W0, L, R, st.drho, st.dun, st.dp, st.side) != 0) {
-    o.fallback = 1;
-    st = pert_fallback_fp64(g, W0, L, R);
-    o.status = st.status;
+__device__ __noinline__ PStar<T> pert_general(T g, const PFace<T> W0, T lr, T lu, T lp, T rr, T ru, T rp,
+                                              bool has_eq) {
+  PStar<T> o;
+  o.side = 0;
+  o.status = o.fallback = 0;
+  o.drho = o.dun = o.dp = T(0);
+  if (!(W0.rho + lr > T(0)) || !(W0.rho + rr > T(0)) || !(W0.p + lp > T(0)) || !(W0.p + rp > T(0))) {
+    o.status = STATUS_NONPHYSICAL;
+    return o;
   }
-  T dut1 = T(0), dut2 = T(0);
-  if (st.side < 0) { dut1 = L.dut1; dut2 = L.dut2; }
-  else if (st.side > 0) { dut1 = R.dut1; dut2 = R.dut2; }
-  else { dut1 = -W0.ut1; dut2 = -W0.ut2; }  // vacuum: no transverse motion
-  pert_flux<T>(g, W0, st.drho, st.dun, dut1, dut2, st.dp, o.F);
-  return o;
-}
-
-template <class T>
-__device__ __forceinline__ PSide<T> shfl_up_side(const PSide<T>& s, int width) {
-  constexpr unsigned FULL = 0xffffffffu;
-  PSide<T> o;
-  o.drho = __shfl_up_sync(FULL, s.drho, 1, width);
-  o.dun = __shfl_up_sync(FULL, s.dun, 1, width);
-  o.dut1 = __shfl_up_sync(FULL, s.dut1, 1, width);
-  o.dut2 = __shfl_up_sync(FULL, s.dut2, 1, width);
-  o.dp = __shfl_up_sync(FULL, s.dp, 1, width);
-  o.rho = __shfl_up_sync(FULL, s.rho, 1, width);
-  o.un = __shfl_up_sync(FULL, s.un, 1, width);
-  o.p = __shfl_up_sync(FULL, s.p, 1, width);
-  o.c = __shfl_up_sync(FULL, s.c, 1, width);
-  o.dc = __shfl_up_sync(FULL, s.dc, 1, width);
+  const PSide<T> L = pert_side(g, W0, lr, lu, lp, has_eq), R = pert_side(g, W0, rr, ru, rp, has_eq);
+  if (pert_riemann<T, P>(g, W0, L, R, o.drho, o.dun, o.dp, o.side) != 0) {
+    o = pert_fallback_fp64(g, W0, L, R);
+    o.fallback = 1;
+  }
   return o;
 }
 
@@ -468,8 +437,8 @@ struct PertArgs {
   // the grid's and the drag's parameters in the state precision, converted
   // once on the host (GB300's FP64 pipe is narrow: per-use conversions of the
   // double originals cost latency in the float kernel)
-  T gam, om, cfl, dx1, dx2, stokes, rhos_rp, kappa;
-  T st_factor[ND_MAX];  // Stokes-number factor of each dust species
+  T gam, gm1, g_gm1, om, cfl, kappa;
+  T ist[ND_MAX], irr[ND_MAX];  // 1 / (St x factor), 1 / (rho_s r_p x factor) of each dust species
 };
 
 // Primitive perturbations (du, dv, dw, dP, drho in the field slots MU, MV,
@@ -477,220 +446,173 @@ struct PertArgs {
 // density rho0 and azimuthal velocity v0 (r and z velocities zero):
 // rho = rho0 + rho', du = (m' - rho' u0)/rho,
 // dP = (gamma-1)(E' - [rho' |u0|^2/2 + rho u0.du + rho |du|^2/2]).
+// Returns 1 / rho.
 template <class T>
-__device__ __forceinline__ void face_prim(T g, T rho0, T v0, const T* q, T* w) {
-  const T rho = rho0 + q[RHO];
-  const T ir = T(1) / rho;
-  const T du = q[MU] * ir, dv = (q[MV] - q[RHO] * v0) * ir, dw = q[MW] * ir;
-  const T dke = T(0.5) * q[RHO] * v0 * v0 + rho * v0 * dv + T(0.5) * rho * (du * du + dv * dv + dw * dw);
-  w[MU] = du;
-  w[MV] = dv;
-  w[MW] = dw;
-  w[EN] = (g - T(1)) * (q[EN] - dke);
+__device__ __forceinline__ T face_prim(T gm1, T rho0, T v0, const T* q, T* w) {
+  const T ir = recip(rho0 + q[RHO]);
+  const T m1 = q[MV] - q[RHO] * v0;  // rho dv
+  w[MU] = q[MU] * ir;
+  w[MV] = m1 * ir;
+  w[MW] = q[MW] * ir;
+  const T ke = q[MU] * w[MU] + m1 * w[MV] + q[MW] * w[MW];
+  w[EN] = gm1 * (q[EN] - (v0 * (T(0.5) * q[RHO] * v0 + m1) + T(0.5) * ke));
   w[RHO] = q[RHO];
-}
-
-template <class T, int D>
-__device__ __forceinline__ PFace<T> face_eq(const PertTables<T>& t, const DevGrid& g, int ci, int ck, int fd,
-                                            T& v0) {
-  PFace<T> W;
-  if (!g.has_eq) {
-    W.rho = W.un = W.ut1 = W.ut2 = W.p = W.c = W.h = W.un_mc = W.un_pc = T(0);
-    v0 = T(0);
-    return W;
-  }
-  if (D == 1) {
-    const size_t s = (size_t)g.nz * g.nr, o = (size_t)ck * g.nr + ci;
-    W.rho = t.ft[o];
-    v0 = t.ft[s + o];
-    W.p = t.ft[2 * s + o];
-    W.c = t.ft[3 * s + o];
-    W.h = t.ft[4 * s + o];
-    W.un_mc = t.ft[5 * s + o];
-    W.un_pc = t.ft[6 * s + o];
-    W.un = v0;
-    W.ut1 = W.ut2 = T(0);
-    return W;
-  }
-  const T* tab;
-  size_t s, o;
-  if (D == 0) {
-    tab = t.fr;
-    s = (size_t)g.nz * (g.nr + 1);
-    o = (size_t)ck * (g.nr + 1) + clampi(fd, 0, g.nr);
-  } else {
-    tab = t.fz;
-    s = (size_t)(g.nz + 1) * g.nr;
-    o = (size_t)clampi(fd, 0, g.nz) * g.nr + ci;
-  }
-  W.rho = tab[o];
-  v0 = tab[s + o];
-  W.p = tab[2 * s + o];
-  W.c = tab[3 * s + o];
-  W.h = tab[4 * s + o];
-  W.un = T(0);
-  W.un_mc = -W.c;
-  W.un_pc = W.c;
-  W.ut1 = D == 0 ? v0 : T(0);  // r face: t1 = theta;  z face: t1 = r, t2 = theta
-  W.ut2 = D == 2 ? v0 : T(0);
-  return W;
+  return ir;
 }
 
 // One 32-lane chunk of the sweep along axis D: items base .. base + 31 (whole
-// lines of L lanes).  The flux divergence of the chunk's cells is written to
-// sG (ACC: added to it).
-template <class T, int NF, int TR, int TT, int TZ, int NT, int D, class P, int RC, bool ACC>
+// lines of L lanes).  sE holds the gas departures (conservative, or primitive
+// with RC = RECON_PRIM) and the dust primitives.  The flux divergence of the
+// chunk's cells is written to sG (ACC: added to it).
+template <class T, int NF, int TR, int TT, int TZ, int D, class P, int RC, bool ACC>
 __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* sE, T* sG, int i0, int j0, int k0,
                                                  int base, unsigned& status, unsigned& nfallback) {
-  constexpr int BX = TR + 4, BY = TT + 4, BZ = TZ + 4, BOX = BX * BY * BZ, NCORE = TR * TT * TZ;
-  constexpr int TD = D == 0 ? TR : (D == 1 ? TT : TZ);
-  constexpr int L = pow2ceil(TD + 2);
-  static_assert(L <= 32, "line does not fit a warp");
-  constexpr int NA = D == 0 ? TT : TR;
-  constexpr int NB = D == 2 ? TT : TZ;
-  constexpr int ITEMS = NA * NB * L;
-  constexpr int STRIDE = D == 0 ? 1 : (D == 1 ? BX : BX * BY);
+  using S = SweepLane<TR, TT, TZ, D>;
+  constexpr int BOX = S::BOX, NCORE = S::NCORE, L = S::L, STRIDE = S::STRIDE;
   constexpr unsigned FULL = 0xffffffffu;
+  constexpr bool UNI = D != 0;
+  constexpr int n = Axes<D>::n;
   const DevGrid& g = a.g;
-  const T gam = a.gam;
-  const bool has_eq = g.has_eq != 0;
-  const int lane = threadIdx.x & 31;
+  const S s(g, base + (threadIdx.x & 31), i0, j0, k0);
+  if (!__any_sync(FULL, s.do_face)) return;  // a warp of lines beyond a ragged grid's edge
+  T w[RCW];
+  parabola_weights<T, D>(a.t.rcoef, s.gi, g.nr, w);
+  const int ci = clampi(s.gi, 0, g.nr - 1), ck = clampi(s.gk, 0, g.nz - 1);
+  T area = T(0);
+  if (s.do_face) area = D == 0 ? a.t.area_r[s.gi] : (D == 1 ? a.t.area_t[ci] : a.t.area_z[ci]);
   {
-    const int item = base + lane;
-    const bool valid = item < ITEMS;
-    const int line = valid ? item / L : 0;
-    const int c = item % L - 1;
-    const int ta = line % NA, tb = line / NA;
-    const int x = D == 0 ? c : ta;
-    const int y = D == 1 ? c : (D == 0 ? ta : tb);
-    const int z = D == 2 ? c : tb;
-    const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
-    const bool line_ok = valid && (D == 0 ? (gj < g.nth && gk < g.nz)
-                                          : (D == 1 ? (gi < g.nr && gk < g.nz) : (gi < g.nr && gj < g.nth)));
-    const int gd = D == 0 ? gi : (D == 1 ? gj : gk);
-    const int nd = D == 0 ? g.nr : (D == 1 ? g.nth : g.nz);
-    const bool do_recon = line_ok && c <= TD && gd <= nd;
-    const bool do_face = do_recon && c >= 0;
-    const bool do_acc = line_ok && c >= 0 && c < TD && gd < nd;
-    const int sidx = do_recon ? ((z + 2) * BY + (y + 2)) * BX + (x + 2) : (2 * BY + 2) * BX + 2;
-    constexpr bool UNI = D != 0;
-    T w[RCW];
-    parabola_weights<T, D>(a.t.rcoef, gi, g.nr, w);
-    const int ci = clampi(gi, 0, g.nr - 1), ck = clampi(gk, 0, g.nz - 1);
-    T area = T(0);
-    if (do_face) area = D == 0 ? a.t.area_r[clampi(gi, 0, g.nr)] : (D == 1 ? a.t.area_t[ci] : a.t.area_z[ci]);
+    // the equilibrium of this cell's lower and upper face (clamped; one face
+    // for a theta line, whose cells share the radius and height)
+    PEq<T> Em{T(0), T(0), T(0), T(0)}, Ep{T(0), T(0), T(0), T(0)};
+    int of = 0;
+    if (g.has_eq) {
+      const T* f = a.t.face[D];
+      if (D == 0) {
+        of = ck * (g.nr + 1) + clampi(s.gd, 0, g.nr);
+        Em = load_eq(f + 4 * (size_t)of);
+        Ep = load_eq(f + 4 * (size_t)(ck * (g.nr + 1) + clampi(s.gd + 1, 0, g.nr)));
+      } else if (D == 1) {
+        of = ck * g.nr + ci;
+        Em = Ep = load_eq(f + 4 * (size_t)of);
+      } else {
+        of = clampi(s.gd, 0, g.nz) * g.nr + ci;
+        Em = load_eq(f + 4 * (size_t)of);
+        Ep = load_eq(f + 4 * (size_t)(clampi(s.gd + 1, 0, g.nz) * g.nr + ci));
+      }
+    }
+    T wm[5], wp[5];  // primitive perturbations: right state of the lower face, left state of the upper face
     {
       T qm[5], qp[5];
 #pragma unroll
       for (int f = 0; f < 5; ++f) {
-        const T* s = sE + f * BOX + sidx;
-        parabola<UNI>(s[-STRIDE], s[0], s[STRIDE], w, qm[f], qp[f]);
+        const T* e = sE + f * BOX + s.sidx;
+        parabola<UNI>(e[-STRIDE], e[0], e[STRIDE], w, qm[f], qp[f]);
       }
-      // both face states, used for the positivity check of Sect. 2.7's
-      // reconstruction and then by the two faces' solvers
-      T v0m, v0p;
-      const PFace<T> Wm = face_eq<T, D>(a.t, g, ci, ck, gd, v0m);
-      const PFace<T> Wp = face_eq<T, D>(a.t, g, ci, ck, gd + 1, v0p);
-      PSide<T> sm, sp;
-      bool ok;
-      if (RC == RECON_PRIM) {
-        ok = pert_side<T, D>(gam, Wm, qm, has_eq, sm) & pert_side<T, D>(gam, Wp, qp, has_eq, sp);
-        if (!ok) {  // positivity fallback: flat reconstruction of the gas fields
+      auto face_states = [&]() {
+        if (RC == RECON_PRIM) {
 #pragma unroll
-          for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + sidx];
-          ok = pert_side<T, D>(gam, Wm, qm, has_eq, sm) & pert_side<T, D>(gam, Wp, qp, has_eq, sp);
-        }
-      } else {
-        // conservative face departures -> primitive perturbations about the
-        // face equilibrium (rho0, v0 of that face)
-        T pm[5], pp[5];
-        face_prim<T>(gam, Wm.rho, v0m, qm, pm);
-        face_prim<T>(gam, Wp.rho, v0p, qp, pp);
-        ok = pert_side<T, D>(gam, Wm, pm, has_eq, sm) & pert_side<T, D>(gam, Wp, pp, has_eq, sp);
-        if (!ok) {  // positivity fallback: flat reconstruction of the gas fields
-#pragma unroll
-          for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + sidx];
-          face_prim<T>(gam, Wm.rho, v0m, qm, pm);
-          face_prim<T>(gam, Wp.rho, v0p, qp, pp);
-          ok = pert_side<T, D>(gam, Wm, pm, has_eq, sm) & pert_side<T, D>(gam, Wp, pp, has_eq, sp);
-        }
-      }
-      T F[5];
-      {
-        const PSide<T> sl = shfl_up_side(sp, L);  // upper face state of the lower neighbour
-        const bool okl = __shfl_up_sync(FULL, ok ? 1 : 0, 1, L) != 0;
-        if (do_face) {
-          if (ok && okl) {
-            const PFlux<T> ff = pert_face_flux<T, P>(gam, Wm, sl, sm);
-            status |= ff.status;
-            nfallback += ff.fallback;
-            F[RHO] = ff.F[0] * area;
-            F[Axes<D>::n] = ff.F[1] * area;
-            F[Axes<D>::t1] = ff.F[2] * area;
-            F[Axes<D>::t2] = ff.F[3] * area;
-            F[EN] = ff.F[4] * area;
-          } else {
-            status |= STATUS_NONPHYSICAL;
-#pragma unroll
-            for (int f = 0; f < 5; ++f) F[f] = T(0);
+          for (int f = 0; f < 5; ++f) {
+            wm[f] = qm[f];
+            wp[f] = qp[f];
           }
         } else {
-#pragma unroll
-          for (int f = 0; f < 5; ++f) F[f] = T(0);
+          face_prim(a.gm1, Em.rho, Em.v, qm, wm);
+          face_prim(a.gm1, Ep.rho, Ep.v, qp, wp);
         }
-      }
+        return positive(Em.rho + wm[RHO]) && positive(Ep.rho + wp[RHO]) && positive(Em.p + wm[EN]) &&
+               positive(Ep.p + wp[EN]);
+      };
+      if (!face_states()) {  // positivity fallback: flat reconstruction of the gas fields
 #pragma unroll
-      for (int f = 0; f < 5; ++f) {
-        const T Fu = __shfl_down_sync(FULL, F[f], 1, L);
-        if (do_acc) {
-          T* dst = sG + f * NCORE + (z * TT + y) * TR + x;
-          if (ACC) *dst += F[f] - Fu;
-          else *dst = F[f] - Fu;
-        }
+        for (int f = 0; f < 5; ++f) qm[f] = qp[f] = sE[f * BOX + s.sidx];
+        face_states();
       }
     }
-#pragma unroll 1
-    for (int b = 5; b < NF; b += 4) {  // each dust species: primitive reconstruction, kinetic flux
-      T qm[4], qp[4];
-      dust_recon_cons<T, BOX, STRIDE, UNI>(sE, sidx, b, w, qm, qp);
-      T F[4];
-      {
-        T WL[4];
+    T F[5], wl[5];
 #pragma unroll
-        for (int f = 0; f < 4; ++f) WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
-        if (do_face) {
-          dust_kinetic_flux<D>(area, WL, qm, F);
-        } else {
+    for (int f = 0; f < 5; ++f) {
+      wl[f] = __shfl_up_sync(FULL, wp[f], 1, L);  // upper face state of the lower neighbour
+      F[f] = T(0);
+    }
+    if (s.do_face) {
+      const T un0 = D == 1 ? Em.v : T(0);
+      const T rl = Em.rho + wl[RHO], pl = Em.p + wl[EN], rr = Em.rho + wm[RHO], pr = Em.p + wm[EN];
+      NearStar<T> st;
+      int kind = NEAR_GENERAL;
+      if (sizeof(T) == 4 || (positive(rl) && positive(rr) && positive(pl) && positive(pr)))
+        kind = near_riemann<T>(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
+                               narrow(un0 + wl[n]), narrow(un0 + wm[n]), st);
+      const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
+      T d[3], drho = left ? wl[RHO] : wm[RHO], dp = left ? wl[EN] : wm[EN];
 #pragma unroll
-          for (int f = 0; f < 4; ++f) F[f] = T(0);
-        }
+      for (int q = 0; q < 3; ++q) d[q] = left ? wl[q] : wm[q];
+      if (kind >= NEAR_STAR_L) {
+        drho += st.drho;
+        d[n] = st.us;
+        dp = wl[EN] + st.d;
       }
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        const T Fu = __shfl_down_sync(FULL, F[f], 1, L);
-        if (do_acc) {
-          T* dst = sG + (b + f) * NCORE + (z * TT + y) * TR + x;
-          if (ACC) *dst += F[f] - Fu;
-          else *dst = F[f] - Fu;
+      bool ok = true;
+      if (kind == NEAR_GENERAL) {
+        PFace<T> W0{Em.rho, un0, Em.p, T(0), T(0), T(0)};
+        if (g.has_eq) {
+          const T* wv = a.t.wave[D] + 4 * (size_t)of;
+          W0.c = wv[0];
+          W0.un_mc = wv[1];
+          W0.un_pc = wv[2];
         }
+        const PStar<T> o = pert_general<T, P>(a.gam, W0, wl[RHO], wl[n], wl[EN], wm[RHO], wm[n], wm[EN],
+                                              g.has_eq != 0);
+        status |= o.status;
+        nfallback += o.fallback;
+        ok = !(o.status & STATUS_NONPHYSICAL);
+        // the transverse velocity of the side that the face lies on; a vacuum has none
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          d[q] = o.side < 0 ? wl[q] : (o.side > 0 ? wm[q] : (q == MV ? -Em.v : T(0)));
+        drho = o.drho;
+        d[n] = o.dun;
+        dp = o.dp;
+      }
+      if (ok) pert_flux<T, D>(a.g_gm1, area, Em, drho, d, dp, F);
+    }
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+      const T Fu = __shfl_down_sync(FULL, F[f], 1, L);
+      if (s.do_acc) {
+        T* dst = sG + f * NCORE + s.core;
+        if (ACC) *dst += F[f] - Fu;
+        else *dst = F[f] - Fu;
       }
     }
   }
-}
-
-// Items (lanes) of the sweep along axis D of a TR x TT x TZ tile.
-template <int TR, int TT, int TZ, int D>
-__host__ __device__ constexpr int sweep_items() {
-  return (D == 0 ? TT * TZ : (D == 1 ? TR * TZ : TR * TT)) * pow2ceil((D == 0 ? TR : (D == 1 ? TT : TZ)) + 2);
+#pragma unroll 1
+  for (int b = 5; b < NF; b += 4) {  // each dust species: primitive reconstruction, kinetic flux
+    T qm[4], qp[4], F[4], WL[4];
+    dust_recon<T, BOX, STRIDE, UNI>(sE, s.sidx, b, w, qm, qp);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
+      F[f] = T(0);
+    }
+    if (s.do_face) dust_kinetic_flux<D>(area, WL, qm, F);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const T Fu = __shfl_down_sync(FULL, F[f], 1, L);
+      if (s.do_acc) {
+        T* dst = sG + (b + f) * NCORE + s.core;
+        if (ACC) *dst += F[f] - Fu;
+        else *dst = F[f] - Fu;
+      }
+    }
+  }
 }
 
 // The whole sweep along axis D, chunks spread over the block's warps.
 template <class T, int NF, int TR, int TT, int TZ, int NT, int D, class P, int RC, bool ACC>
 __device__ __forceinline__ void sweep_pert(const PertArgs<T>& a, const T* sE, T* sG, int i0, int j0, int k0,
                                            unsigned& status, unsigned& nfallback) {
-  constexpr int CH = (sweep_items<TR, TT, TZ, D>() + 31) / 32;
-  for (int ch = threadIdx.x >> 5; ch < CH; ch += NT / 32)
-    sweep_pert_chunk<T, NF, TR, TT, TZ, NT, D, P, RC, ACC>(a, sE, sG, i0, j0, k0, ch * 32, status, nfallback);
+  for (int base = threadIdx.x & ~31; base < SweepLane<TR, TT, TZ, D>::ITEMS; base += NT)
+    sweep_pert_chunk<T, NF, TR, TT, TZ, D, P, RC, ACC>(a, sE, sG, i0, j0, k0, base, status, nfallback);
 }
 
 // Dynamic shared memory of stage_pert_kernel: the staged tile and halo, and
@@ -711,69 +633,36 @@ struct PCell {
 
 template <class T>
 __device__ __forceinline__ PCell<T> cell_eq(const PertTables<T>& t, const DevGrid& g, int i, int k) {
-  PCell<T> c;
-  if (!g.has_eq) {
-    c.rho0 = c.v0 = c.p0 = c.Cr = c.fz = c.gr = c.cor = c.ir = T(0);
-    return c;
-  }
-  const size_t s = (size_t)g.nz * g.nr, o = (size_t)k * g.nr + i;
-  c.rho0 = t.cen[o];
-  c.v0 = t.cen[s + o];
-  c.p0 = t.cen[2 * s + o];
-  c.Cr = t.cen[3 * s + o];
-  c.fz = t.cen[4 * s + o];
-  c.gr = t.cen[5 * s + o];
-  c.cor = t.cen[6 * s + o];
-  c.ir = t.cen[7 * s + o];
+  PCell<T> c{};
+  if (!g.has_eq) return c;
+  const T* q = t.cen + 8 * ((size_t)k * g.nr + i);
+  const PEq<T> lo = load_eq(q), hi = load_eq(q + 4);
+  c.rho0 = lo.rho;
+  c.v0 = lo.v;
+  c.p0 = lo.p;
+  c.Cr = lo.h;
+  c.fz = hi.rho;
+  c.gr = hi.v;
+  c.cor = hi.p;
+  c.ir = hi.h;
   return c;
 }
 
-// Primitive perturbations at a cell centre: rho, (du, dv, dw), dp.
-template <class T>
-__device__ __forceinline__ void cell_prim(T g, const PCell<T>& c, const T* q, T& rho, T& du, T& dv, T& dw, T& dp) {
-  rho = c.rho0 + q[RHO];
-  const T ir = T(1) / rho;
-  du = q[MU] * ir;
-  dv = (q[MV] - q[RHO] * c.v0) * ir;
-  dw = q[MW] * ir;
-  const T dke = T(0.5) * q[RHO] * c.v0 * c.v0 + rho * c.v0 * dv + T(0.5) * rho * (du * du + dv * dv + dw * dw);
-  dp = (g - T(1)) * (q[EN] - dke);
-}
-
-// Source perturbation S(E0 + E') - S(E0) per unit volume (App. B sources,
-// stellar gravity, rotating frame), cylindrical geometry, plus the whole
-// indirect-gravity source of Sect. 2.10 when it is on (the equilibrium's
-// residual carries none).
-// q: the staged cell, primitive gas perturbations (du, dv, dw, dP, drho) in
-// slots 0..4 and the conservative dust fields in slots 5..8.
+// G += V (S(E0 + E') - S(E0)) (App. B sources, stellar gravity, rotating
+// frame), cylindrical geometry, plus the whole indirect-gravity source of
+// Sect. 2.10 when it is on (the equilibrium's residual carries none).
+// w: the cell's primitive gas perturbations; rd, vd: density and velocity
+// (u, v, w) of each dust species, zero without mass.
 template <class T, int NF, bool XT>
-__device__ __forceinline__ void pert_sources(const PertArgs<T>& a, const PCell<T>& c, int j, const T* q, T* S) {
+__device__ __forceinline__ void pert_sources(const PertArgs<T>& a, const PCell<T>& c, int j, T V, const T* w,
+                                             const T (*dust)[4], T* G) {
   const DevGrid& g = a.g;
-  const T Om = a.om;
-  const T rho = c.rho0 + q[RHO], du = q[MU], dv = q[MV], dw = q[MW], dp = q[EN];
-  const T v = c.v0 + dv;
-  S[MU] = q[RHO] * c.Cr + rho * dv * c.cor + rho * dv * dv * c.ir + dp * c.ir;
-  S[MV] = -rho * du * (v * c.ir + T(2) * Om);
-  S[MW] = q[RHO] * c.fz;
-  S[EN] = rho * du * c.gr + rho * dw * c.fz;
-  S[RHO] = T(0);
-#pragma unroll
-  for (int b = 5; b < NF; b += 4) {  // each dust species
-    const T rd = q[b + 3];
-    if (rd > T(0)) {
-      const T ird = T(1) / rd;
-      const T dvd = (q[b + 1] - rd * c.v0) * ird;  // v_d - v0
-      const T vd = c.v0 + dvd;
-      S[b] = rd * (c.Cr + dvd * c.cor + dvd * dvd * c.ir);
-      S[b + 1] = -q[b] * (vd * c.ir + T(2) * Om);
-      S[b + 2] = rd * c.fz;
-    } else {
-      S[b] = S[b + 1] = S[b + 2] = T(0);
-    }
-    S[b + 3] = T(0);
-  }
-  if (XT && g.x_ind != 0.0) {
-    T gr, gt;  // grad Phi_ind, (r, theta), tabulated per axis-1 index in the state precision
+  const T Om2 = T(2) * a.om;
+  const T rho = c.rho0 + w[RHO], du = w[MU], dv = w[MV], dw = w[MW], dp = w[EN];
+  const T v = c.v0 + dv, rv = rho * dv;
+  T gr = T(0), gt = T(0);  // grad Phi_ind, (r, theta), tabulated per axis-1 index in the state precision
+  const bool ind = XT && g.x_ind != 0.0;
+  if (ind) {
     if constexpr (sizeof(T) == 4) {
       gr = g.ind_gf[j];
       gt = g.ind_gf[g.nth + j];
@@ -781,34 +670,46 @@ __device__ __forceinline__ void pert_sources(const PertArgs<T>& a, const PCell<T
       gr = g.ind_g[j];
       gt = g.ind_g[g.nth + j];
     }
-    S[MU] -= rho * gr;
-    S[MV] -= rho * gt;
-    S[EN] -= rho * (du * gr + v * gt);
+  }
+  T sr = w[RHO] * c.Cr + rv * (c.cor + dv * c.ir) + dp * c.ir;
+  T st = -rho * du * (v * c.ir + Om2);
+  T se = rho * (du * c.gr + dw * c.fz);
+  if (ind) {
+    sr -= rho * gr;
+    st -= rho * gt;
+    se -= rho * (du * gr + v * gt);
+  }
+  G[MU] += V * sr;
+  G[MV] += V * st;
+  G[MW] += V * (w[RHO] * c.fz);
+  G[EN] += V * se;
 #pragma unroll
-    for (int b = 5; b < NF; b += 4) {
-      if (q[b + 3] > T(0)) {
-        S[b] -= q[b + 3] * gr;
-        S[b + 1] -= q[b + 3] * gt;
-      }
+  for (int b = 5; b < NF; b += 4) {  // each dust species
+    const T* d = dust[(b - 5) / 4];
+    const T Vr = positive(d[3]) ? V * d[3] : T(0);
+    const T dvd = d[1] - c.v0;  // v_d - v0
+    T s0 = c.Cr + dvd * (c.cor + dvd * c.ir), s1 = -d[0] * (d[1] * c.ir + Om2);
+    if (ind) {
+      s0 -= gr;
+      s1 -= gt;
     }
+    G[b] += Vr * s0;
+    G[b + 1] += Vr * s1;
+    G[b + 2] += Vr * c.fz;
   }
 }
 
-// Stopping time of dust species s in a perturbation-form cell (as
-// stopping_time of the full-state kernel; gas density rg, pressure p0 + dp).
+// 1 / t_s of dust species s in a perturbation-form cell (as inv_stopping_time
+// of the full-state kernel; gas density rg, pressure p).
 template <class T, bool XT>
-__device__ __forceinline__ T pert_stopping_time(const PertArgs<T>& a, const PCell<T>& c, int i, T rg, T dp, int s) {
-  if (a.drag.law == 0) {
-    const T st = a.stokes * a.st_factor[s];
-    return a.g.geom == GEOM_CYL ? st / a.t.omk[i] : st;
-  }
-  const T cs = Math<T>::sqrt_(a.gam * (c.p0 + dp) / rg);
-  T ts = a.rhos_rp * a.st_factor[s] / (rg * cs);
+__device__ __forceinline__ T pert_inv_stopping_time(const PertArgs<T>& a, int i, T rg, T p, int s) {
+  if (a.drag.law == 0) return a.t.omk[i] * a.ist[s];
+  T it = root(a.gam * p * rg) * a.irr[s];
   if (XT && a.drag.law == 2) {  // Stokes regime of Sect. 2.9 above r_p = 9 lambda / 4
     const T x = a.kappa * rg;
-    if (x > T(2.25)) ts = ts * (T(4.0 / 9.0) * x);
+    if (positive(x - T(2.25))) it *= T(2.25) * recip(x);
   }
-  return ts;
+  return it;
 }
 
 // Semi-implicit drag on a perturbation-form cell state (the closed forms of
@@ -816,90 +717,91 @@ __device__ __forceinline__ T pert_stopping_time(const PertArgs<T>& a, const PCel
 // velocity moves by D = sum rho_k w_k (v_k - v_g) / (rho_g + sum rho_k w_k)
 // and species k by w_k (D - (v_k - v_g)), w_k = a_k / (1 + a_k), every
 // quantity a difference of velocities, never the large u0 itself.
+// ig = 1 / rho_g, id = 1 / rho_d of each species (any value without mass).
 template <class T, int NF, bool XT>
-__device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& c, int i, T* q, T tau) {
-  const T gam = a.gam;
-  T rg, du, dv, dw, dp;
-  cell_prim(gam, c, q, rg, du, dv, dw, dp);
+__device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& c, int i, T* q, T tau, T ig,
+                                          const T* id) {
+  const T rg = c.rho0 + q[RHO];
+  if (!positive(rg)) return;
+  const T m1 = q[MV] - q[RHO] * c.v0;
   const T u0[3] = {T(0), c.v0, T(0)};
-  const T dug[3] = {du, dv, dw};
-  if constexpr (NF == 9) {
-    const T rd = q[DRHO];
-    if (!(rd > T(0)) || !(rg > T(0))) return;
-    const T ts = pert_stopping_time<T, XT>(a, c, i, rg, dp, 0);
-    const T kk = tau * (T(1) + rd / rg) / ts;
-    const T mu = rg * rd / (rg + rd);
-    const T relax = kk / (T(1) + kk);
-    const T ird = T(1) / rd;
-    T dE = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const T dvd = (q[DMU + k] - rd * u0[k]) * ird;  // v_d - u0
-      const T X = mu * (dvd - dug[k]) * relax;
-      const T vg_ex = u0[k] + dug[k];
-      q[MU + k] += X;
-      q[DMU + k] -= X;
-      dE += T(0.5) * X * (T(2) * vg_ex + X / rg);
-    }
-    q[EN] += dE;
-  } else {
-  constexpr int ND = (NF - 5) / 4;
-  if (!(rg > T(0))) return;
-  T wk[ND], den = rg, num[3] = {T(0), T(0), T(0)};
-#pragma unroll
-  for (int s = 0; s < ND; ++s) {
-    const int b = 5 + 4 * s;
-    wk[s] = T(0);
-    const T rd = q[b + 3];
-    if (!(rd > T(0))) continue;
-    const T ak = tau / pert_stopping_time<T, XT>(a, c, i, rg, dp, s);
-    wk[s] = ak / (T(1) + ak);
-    den += rd * wk[s];
-    const T ird = T(1) / rd;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) num[k] += rd * wk[s] * ((q[b + k] - rd * u0[k]) * ird - dug[k]);
+  const T dug[3] = {q[MU] * ig, m1 * ig, q[MW] * ig};
+  T p = T(0);
+  if (a.drag.law != 0) {
+    const T ke = q[MU] * dug[0] + m1 * dug[1] + q[MW] * dug[2];
+    p = c.p0 + a.gm1 * (q[EN] - (c.v0 * (T(0.5) * q[RHO] * c.v0 + m1) + T(0.5) * ke));
   }
   T dE = T(0);
+  if constexpr (NF == 9) {
+    const T rd = q[DRHO];
+    if (!positive(rd)) return;
+    const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, p, 0);
+    const T K = rd * ak * recip(T(1) + ak * (T(1) + rd * ig));
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const T D = num[k] / den;  // v_g' - v_g
+    for (int k = 0; k < 3; ++k) {
+      const T vd = (q[DMU + k] - rd * u0[k]) * id[0];  // v_d - u0
+      const T X = K * (vd - dug[k]);
+      q[MU + k] += X;
+      q[DMU + k] -= X;
+      dE += X * ((u0[k] + dug[k]) + T(0.5) * ig * X);
+    }
+  } else {
+    constexpr int ND = (NF - 5) / 4;
+    T wk[ND], den = rg, num[3] = {T(0), T(0), T(0)};
 #pragma unroll
     for (int s = 0; s < ND; ++s) {
       const int b = 5 + 4 * s;
       const T rd = q[b + 3];
-      if (!(rd > T(0))) continue;
-      const T rel = (q[b + k] - rd * u0[k]) / rd - dug[k];  // v_k - v_g
-      q[b + k] += rd * wk[s] * (D - rel);
+      wk[s] = T(0);
+      if (!positive(rd)) continue;
+      const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, p, s);
+      wk[s] = ak * recip(T(1) + ak);
+      den += rd * wk[s];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) num[k] += rd * wk[s] * ((q[b + k] - rd * u0[k]) * id[s] - dug[k]);
     }
-    q[MU + k] += rg * D;
-    dE += T(0.5) * rg * D * (T(2) * (u0[k] + dug[k]) + D);
+    const T iden = recip(den);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const T D = num[k] * iden;  // v_g' - v_g
+#pragma unroll
+      for (int s = 0; s < ND; ++s) {
+        const int b = 5 + 4 * s;
+        const T rd = q[b + 3];
+        if (!positive(rd)) continue;
+        const T rel = (q[b + k] - rd * u0[k]) * id[s] - dug[k];  // v_k - v_g
+        q[b + k] += rd * wk[s] * (D - rel);
+      }
+      q[MU + k] += rg * D;
+      dE += T(0.5) * rg * D * (T(2) * (u0[k] + dug[k]) + D);
+    }
   }
   q[EN] += dE;
-  }
 }
 
+// The largest (|v| + c) A / V and |v_d| A / V of a cell (the CFL step is N_CFL
+// over their maximum) and whether the cell is not physical.  ig, id: as pert_drag.
 template <class T, int NF>
-__device__ __forceinline__ T pert_cell_dt(const PertArgs<T>& a, const PCell<T>& c, int i, const T* q, bool& bad) {
-  const PertTables<T>& t = a.t;
-  const T gam = a.gam;
-  T rho, du, dv, dw, dp;
-  cell_prim(gam, c, q, rho, du, dv, dw, dp);
-  const T p = c.p0 + dp;
-  bad = !(rho > T(0)) || !(p > T(0));
-  const T v = c.v0 + dv;
-  const T vel = Math<T>::sqrt_(du * du + v * v + dw * dw);
-  const T cs = Math<T>::sqrt_(gam * p / rho);
-  const T aov = t.aov[i], cfl = a.cfl;
-  T dt = cfl / ((vel + cs) * aov);
+__device__ __forceinline__ T pert_cell_rate(const PertArgs<T>& a, const PCell<T>& c, int i, const T* q, T ig,
+                                            const T* id, bool& bad) {
+  const T rho = c.rho0 + q[RHO], m1 = q[MV] - q[RHO] * c.v0;
+  const T du = q[MU] * ig, dv = m1 * ig, dw = q[MW] * ig, v = c.v0 + dv;
+  const T ke = q[MU] * du + m1 * dv + q[MW] * dw;
+  const T p = c.p0 + a.gm1 * (q[EN] - (c.v0 * (T(0.5) * q[RHO] * c.v0 + m1) + T(0.5) * ke));
+  bad = !positive(rho) || !positive(p);
+  const T v2 = du * du + v * v + dw * dw;
+  T rate = root(a.gam * p * ig) + (positive(v2) ? root(v2) : T(0));
 #pragma unroll
   for (int b = 5; b < NF; b += 4) {
-    if (q[b + 3] > T(0)) {
-      const T vd = Math<T>::sqrt_(q[b] * q[b] + q[b + 1] * q[b + 1] + q[b + 2] * q[b + 2]) / q[b + 3];
-      if (vd > T(0)) dt = fmin(dt, cfl / (vd * aov));
+    const T j = id[(b - 5) / 4], ud = q[b] * j, vd = q[b + 1] * j, wd = q[b + 2] * j;
+    const T d2 = ud * ud + vd * vd + wd * wd;
+    if (positive(q[b + 3]) && positive(d2)) {
+      const T vel = root(d2);
+      if (!(vel <= rate)) rate = vel;
     }
-    bad |= !(q[b + 3] >= T(0));
+    bad |= !non_negative(q[b + 3]);
   }
-  return dt;
+  return rate * a.t.aov[i];
 }
 
 // XT: the optional terms (indirect gravity, wave-killing zones) are compiled
@@ -920,86 +822,53 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> 
   const int j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
   unsigned status = 0, nfallback = 0;
 
-  if constexpr (RC == RECON_CONS) {
-    // the conservative departures are staged as they are stored: each cell's
-    // fields go global -> shared by asynchronous copies (cp.async, no
-    // registers), all of a thread's cells in flight at once; equilibrium
-    // ghosts are zero departures
+  // each cell's fields go global -> shared by asynchronous copies (cp.async, no
+  // registers), all of a thread's cells in flight at once; equilibrium ghosts
+  // are zero departures.  A thread then converts the cells it copied: the dust
+  // to primitives (u, v, w, rho_d), which every reconstruction of the three
+  // sweeps reads, and with RC = RECON_PRIM the gas to primitive departures.
+  auto stage = [&](auto&& put) {
     for (int idx = threadIdx.x; idx < BOX; idx += NT) {
       const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - 2;
       const int outside = (x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ);
       if (outside > 1) continue;  // edge and corner cells of the box: no sweep reads them
       int c[3] = {i0 + x, j0 + y, k0 + z};
-      if (!resolve_cell(g, c)) {
-#pragma unroll
-        for (int f = 0; f < NF; ++f) sE[f * BOX + idx] = T(0);
-      } else {
-        const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) cp_async_elem<T>(sE + f * BOX + idx, a.in[f] + lin);
-      }
+      const bool in = resolve_cell(g, c);
+      put(idx, c, in);
     }
-    cp_async_wait_all();
-  } else {
-  // staging in batches of CH cells per thread: every load of a batch is
-  // issued before any of them is used (memory-level parallelism)
-    constexpr int NIT = (BOX + NT - 1) / NT;
-    constexpr int CH = 2;
-    for (int it0 = 0; it0 < NIT; it0 += CH) {
-      T v[CH][NF], e0[CH][3];
-      int st[CH];  // 0: nothing, 1: equilibrium ghost (zero), 2: loaded
+  };
+  stage([&](int idx, const int* c, bool in) {
+    if (!in) {
 #pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        const int idx = threadIdx.x + (it0 + u) * NT;
-        st[u] = 0;
-        if (it0 + u < NIT && idx < BOX) {
-          const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - 2;
-          const int outside = (x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ);
-          if (outside <= 1) {
-            int c[3] = {i0 + x, j0 + y, k0 + z};
-            if (!resolve_cell(g, c)) {
-              st[u] = 1;
-            } else {
-              st[u] = 2;
-              const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
+      for (int f = 0; f < NF; ++f) sE[f * BOX + idx] = T(0);
+      return;
+    }
+    const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
 #pragma unroll
-              for (int f = 0; f < NF; ++f) v[u][f] = a.in[f][lin];
-              if (RC == RECON_PRIM && g.has_eq) {
-                const size_t sz = (size_t)g.nz * g.nr, o = (size_t)c[2] * g.nr + c[0];
-                e0[u][0] = a.t.cen[o];
-                e0[u][1] = a.t.cen[sz + o];
-                e0[u][2] = a.t.cen[2 * sz + o];
-              } else {
-                e0[u][0] = e0[u][1] = e0[u][2] = T(0);
-              }
-            }
-          }
+    for (int f = 0; f < NF; ++f) cp_async_elem<T>(sE + f * BOX + idx, a.in[f] + lin);
+  });
+  cp_async_wait_all();
+  if (NF > 5 || RC == RECON_PRIM) {
+    for (int idx = threadIdx.x; idx < BOX; idx += NT) {
+      const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - 2;
+      if ((x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ) > 1) continue;
+      if (RC == RECON_PRIM) {
+        int c[3] = {i0 + x, j0 + y, k0 + z};
+        if (resolve_cell(g, c)) {
+          const PEq<T> e = g.has_eq ? load_eq(a.t.cen + 8 * ((size_t)c[2] * g.nr + c[0])) : PEq<T>{};
+          T q[5], w[5];
+#pragma unroll
+          for (int f = 0; f < 5; ++f) q[f] = sE[f * BOX + idx];
+          face_prim(a.gm1, e.rho, e.v, q, w);
+#pragma unroll
+          for (int f = 0; f < 4; ++f) sE[f * BOX + idx] = w[f];
         }
       }
 #pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        const int idx = threadIdx.x + (it0 + u) * NT;
-        if (st[u] == 1) {
+      for (int b = 5; b < NF; b += 4) {
+        const T rd = sE[(b + 3) * BOX + idx], id = positive(rd) ? recip(rd) : T(0);
 #pragma unroll
-          for (int f = 0; f < NF; ++f) sE[f * BOX + idx] = T(0);
-        } else if (st[u] == 2 && RC == RECON_CONS) {  // the state is E' itself
-#pragma unroll
-          for (int f = 0; f < NF; ++f) sE[f * BOX + idx] = v[u][f];
-        } else if (st[u] == 2) {
-          PCell<T> ce;
-          ce.rho0 = e0[u][0];
-          ce.v0 = e0[u][1];
-          ce.p0 = e0[u][2];
-          T rho, du, dv, dw, dp;
-          cell_prim(a.gam, ce, v[u], rho, du, dv, dw, dp);
-          sE[MU * BOX + idx] = du;
-          sE[MV * BOX + idx] = dv;
-          sE[MW * BOX + idx] = dw;
-          sE[EN * BOX + idx] = dp;
-          sE[RHO * BOX + idx] = v[u][RHO];
-#pragma unroll
-          for (int f = 5; f < NF; ++f) sE[f * BOX + idx] = v[u][f];
-        }
+        for (int q = 0; q < 3; ++q) sE[(b + q) * BOX + idx] *= id;
       }
     }
   }
@@ -1012,7 +881,8 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> 
   __syncthreads();
 
   const T tau = (T)(a.tau_frac * (a.dt_dev ? __longlong_as_double((long long)*a.dt_dev) : a.dt_host));
-  T dtmin = T(INFINITY);
+  constexpr int ND = NF > 5 ? (NF - 5) / 4 : 1;
+  T rate = T(0);
   double sums[NF];  // the conservation partials of V E', in FP64 from the first product
 #pragma unroll
   for (int f = 0; f < NF; ++f) sums[f] = 0.0;
@@ -1023,94 +893,61 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> 
     const size_t lin = ((size_t)gk * g.nth + gj) * g.nr + gi;
     const PCell<T> ce = cell_eq(a.t, g, gi, gk);
     const int sidx = ((z + 2) * BY + (y + 2)) * BX + (x + 2);
-    T q[NF], G[NF];  // q: primitive gas perturbations, conservative dust
+    T e[5], w[5], dust[ND][4], G[NF];  // staged gas, its primitive perturbations, the dust's primitives
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      q[f] = sE[f * BOX + sidx];
-      G[f] = sG[f * NCORE + cidx];
-    }
-    if (RC == RECON_CONS) {  // the staged gas departures are conservative
-      T qc[5];
+    for (int f = 0; f < 5; ++f) e[f] = sE[f * BOX + sidx];
 #pragma unroll
-      for (int f = 0; f < 5; ++f) qc[f] = q[f];
-      face_prim<T>(a.gam, ce.rho0, ce.v0, qc, q);
-    }
-    if (g.geom == GEOM_CYL) {
-      T S[NF];
-      pert_sources<T, NF, XT>(a, ce, gj, q, S);
-      const T V = a.t.vol[gi];
+    for (int f = 5; f < NF; ++f) dust[(f - 5) / 4][(f - 5) % 4] = sE[f * BOX + sidx];
 #pragma unroll
-      for (int f = 0; f < NF; ++f) G[f] += V * S[f];
+    for (int f = 0; f < NF; ++f) G[f] = sG[f * NCORE + cidx];
+    if (RC == RECON_CONS) {
+      face_prim(a.gm1, ce.rho0, ce.v0, e, w);
+    } else {
+#pragma unroll
+      for (int f = 0; f < 5; ++f) w[f] = e[f];
     }
+    if (g.geom == GEOM_CYL) pert_sources<T, NF, XT>(a, ce, gj, a.t.vol[gi], w, dust, G);
     if (XT && g.damp_k) {  // wave-killing zones: the gas departures E' relax towards 0
       T kd;
       if constexpr (sizeof(T) == 4) kd = g.damp_kf[(size_t)gk * g.nr + gi];
       else kd = g.damp_k[(size_t)gk * g.nr + gi];
-      if (kd != T(0)) {
+      if (positive(kd)) {
         const T V = a.t.vol[gi];
 #pragma unroll
         for (int f = 0; f < 5; ++f) G[f] -= V * kd * a.in[f][lin];
       }
     }
-    const T iv = a.t.ivol[gi];
-    T E[NF];
+    const T tv = tau * a.t.ivol[gi];
+    T E[NF], ig = T(0), id[ND];
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      // stage 1 updates its own input, whose raw values are staged
-      const T b = !a.stage2 && (RC == RECON_CONS || f >= 5) ? sE[f * BOX + sidx] : a.base[f][lin];
-      E[f] = b + tau * G[f] * iv;
+      // stage 1 updates its own input, whose gas is staged as it is stored
+      const T b = !a.stage2 && RC == RECON_CONS && f < 5 ? e[f] : a.base[f][lin];
+      E[f] = b + tv * G[f];
     }
-    if constexpr (NF > 5) pert_drag<T, NF, XT>(a, ce, gi, E, tau);
+    if (NF > 5 || a.stage2) ig = recip(ce.rho0 + E[RHO]);
+#pragma unroll
+    for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = recip(E[b + 3]);
+    if constexpr (NF > 5) pert_drag<T, NF, XT>(a, ce, gi, E, tau, ig, id);
 #pragma unroll
     for (int f = 0; f < NF; ++f) a.out[f][lin] = E[f];
-    bool bad_in = false;
+    bool bad = false;
     if (a.stage2) {
-      bool bad = false;
-      dtmin = fmin(dtmin, pert_cell_dt<T, NF>(a, ce, gi, E, bad));
-      if (bad) status |= STATUS_NONPHYSICAL;
+      const T c = pert_cell_rate<T, NF>(a, ce, gi, E, ig, id, bad);
+      if (positive(c) && !(c <= rate)) rate = c;
       const double V = g.vol[gi];
 #pragma unroll
       for (int f = 0; f < NF; ++f) sums[f] += V * (double)E[f];
     } else {
-      bad_in = !(ce.rho0 + q[RHO] > T(0)) || !(ce.p0 + q[EN] > T(0));
+      bad = !positive(ce.rho0 + w[RHO]) || !positive(ce.p0 + w[EN]);
 #pragma unroll
-      for (int b = 5; b < NF; b += 4) bad_in |= !(q[b + 3] >= T(0));
-      if (bad_in) status |= STATUS_NONPHYSICAL;
+      for (int s = 0; s < (NF - 5) / 4; ++s) bad |= !non_negative(dust[s][3]);
     }
+    if (bad) status |= STATUS_NONPHYSICAL;
   }
-  if (a.stage2) {
-    // the block's sums in FP64: each thread's partials to shared memory (the
-    // staging area, free once every thread is past the epilogue), then NF x 8
-    // threads add 32 of them each and 8-lane shuffles finish; the CFL minimum,
-    // exact in any precision, stays in the state's
-    constexpr int NW = NT / 32, SEG = NT / 8;
-    static_assert(NT % 8 == 0 && NF * 8 <= NT, "reduction layout");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dtmin = fmin(dtmin, __shfl_xor_sync(0xffffffffu, dtmin, o));
-    __syncthreads();
-    double* red = reinterpret_cast<double*>(smem_raw);  // [NF][NT] partials, then [NW] minima
-#pragma unroll
-    for (int f = 0; f < NF; ++f) red[f * NT + threadIdx.x] = sums[f];
-    if (lane == 0) red[NF * NT + warp] = (double)dtmin;
-    __syncthreads();
-    if (threadIdx.x < NF * 8) {
-      const int f = threadIdx.x >> 3, seg = threadIdx.x & 7;
-      const double* src = red + f * NT + seg * SEG;
-      double acc = 0.0;
-#pragma unroll 8
-      for (int u = 0; u < SEG; ++u) acc += src[u];
-      const unsigned grp = 0xffu << (lane & 24);  // this 8-lane group (all of it active)
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) acc += __shfl_down_sync(grp, acc, o, 8);
-      if (seg == 0) a.partials[(size_t)f * gridDim.x + blockIdx.x] = acc;
-    }
-    if (threadIdx.x == NT - 1) {
-      double m = red[NF * NT];
-      for (int w = 1; w < NW; ++w) m = fmin(m, red[NF * NT + w]);
-      a.partials[(size_t)NF * gridDim.x + blockIdx.x] = m;
-    }
-  }
+  if (a.stage2)  // a thread without a cell: rate 0, an infinite step
+    block_results<NT, NF>(sums, positive(rate) ? (double)(a.cfl / rate) : INFINITY,
+                          reinterpret_cast<double*>(smem_raw), a.partials);
   if (status) atomicOr(a.status, status);
   if (nfallback) atomicAdd(a.t.fallbacks, (unsigned long long)nfallback);
 }
@@ -1121,18 +958,22 @@ __global__ void pert_cfl_kernel(const PertArgs<T> a, unsigned long long* slot) {
   __shared__ double red[256 / 32];
   const DevGrid& g = a.g;
   const size_t ncell = (size_t)g.nr * g.nth * g.nz;
-  double m = INFINITY;
+  T rate = T(0);
   unsigned status = 0;
   for (size_t lin = blockIdx.x * (size_t)256 + threadIdx.x; lin < ncell; lin += (size_t)gridDim.x * 256) {
-    T q[NF];
+    T q[NF], id[NF > 5 ? (NF - 5) / 4 : 1];
 #pragma unroll
     for (int f = 0; f < NF; ++f) q[f] = a.in[f][lin];
+#pragma unroll
+    for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = recip(q[b + 3]);
     const int i = (int)(lin % g.nr), k = (int)(lin / ((size_t)g.nr * g.nth));
+    const PCell<T> ce = cell_eq(a.t, g, i, k);
     bool bad = false;
-    m = fmin(m, (double)pert_cell_dt<T, NF>(a, cell_eq(a.t, g, i, k), i, q, bad));
+    const T c = pert_cell_rate<T, NF>(a, ce, i, q, recip(ce.rho0 + q[RHO]), id, bad);
+    if (positive(c) && !(c <= rate)) rate = c;
     if (bad) status |= STATUS_NONPHYSICAL;
   }
-  m = block_min<256>(m, red);
+  const double m = block_min<256>(positive(rate) ? (double)(a.cfl / rate) : INFINITY, red);
   if (threadIdx.x == 0) atomic_min_pos_double(slot, m);
   if (status) atomicOr(a.status, status);
 }
