@@ -313,7 +313,7 @@ rossbi_status rossbi_step_host(rossbi_grid* g, void* const* host_state, double d
  * allocator at start-up, or loops that cannot accept the device-wide
  * synchronisation a cudaMalloc or cudaFree may cause.
  * Same arguments and result as rossbi_step with scratch == NULL, except that
- * the intermediate state E* and the reduction partials live in a fixed
+ * the intermediate state E* lives in a fixed
  * 64 MiB (67,108,864-byte) array inside the library, allocated with the
  * library image on every GPU that loads it and held until the process exits.
  * Limit: nfields * (cells * element size, rounded up to 256 bytes) plus

@@ -638,10 +638,4 @@ __device__ __forceinline__ double cell_rate(const DevGrid& g, int i, const doubl
   return rate * g.aov[i];
 }
 
-// Positive doubles order like their bit patterns, so a 64-bit integer
-// atomicMin of the bits is an exact, order-independent minimum.
-__device__ __forceinline__ void atomic_min_pos_double(unsigned long long* slot, double v) {
-  atomicMin(slot, (unsigned long long)__double_as_longlong(v));
-}
-
 }  // namespace rossbi

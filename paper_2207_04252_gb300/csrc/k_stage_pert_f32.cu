@@ -14,15 +14,27 @@
 namespace rossbi {
 namespace {
 
-template <int NF, class P, bool XT, int RC>
-cudaError_t launch(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
+template <int NF, int NT, int MINB, class P, bool XT, int RC>
+cudaError_t launch_nt(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
   constexpr size_t smem = pert_smem_bytes<float, NF, P32_TR, P32_TT, P32_TZ>();
-  auto kern = stage_pert_kernel<float, NF, P32_TR, P32_TT, P32_TZ, P32_NT, P32_MINB, P, XT, RC>;
+  auto kern = stage_pert_kernel<float, NF, P32_TR, P32_TT, P32_TZ, NT, MINB, P, XT, RC>;
   static unsigned long long done = 0;
   cudaError_t e = set_smem_once(kern, smem, done);
   if (e != cudaSuccess) return e;
-  kern<<<nblocks, P32_NT, smem, s>>>(a);
+  kern<<<nblocks, NT, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+// Two blocks of 8 warps share an SM where their shared memory allows it (up to
+// nine fields) and there are tiles for them; otherwise one block of 16 warps
+// takes the SM: more fields (120 KB and up), or a grid of at most one tile per
+// SM (32 x 48 x 32: 207 -> 153 us for four steps).
+template <int NF, class P, bool XT, int RC>
+cudaError_t launch(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
+  if constexpr (NF <= 9) {
+    if (nblocks > a.sms) return launch_nt<NF, P32_NT, P32_MINB, P, XT, RC>(a, nblocks, s);
+  }
+  return launch_nt<NF, P32_WIDE_NT, 1, P, XT, RC>(a, nblocks, s);
 }
 
 }  // namespace

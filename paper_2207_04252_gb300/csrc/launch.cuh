@@ -14,7 +14,7 @@ namespace rossbi {
 
 // Tiles of the stage kernels: 14 x 6 x 6 cells, lines of 16 / 8 / 8 lanes.
 constexpr int F64_TR = 14, F64_TT = 6, F64_TZ = 6, F64_NT = 192;
-constexpr int P32_TR = 14, P32_TT = 6, P32_TZ = 6, P32_NT = 256, P32_MINB = 2;
+constexpr int P32_TR = 14, P32_TT = 6, P32_TZ = 6, P32_NT = 256, P32_MINB = 2, P32_WIDE_NT = 512;
 // With more than one dust species the FP64 perturbation form's staged 14 x 6
 // x 6 tile with its halo (18 x 10 x 10 cells) no longer fits in shared memory
 // (13 fields: 234 KB of the 227 KB a block may have): it takes tiles two z

@@ -27,6 +27,7 @@ struct rossbi_grid {
   rossbi_grid_desc desc{};
   cudaStream_t stream = nullptr;
   int device = -1;                     // the device current at rossbi_init_grid
+  int sms = 1;                         // its SM count
   int nf = 5;
   size_t ncell = 0;
   DevGrid dg{};
@@ -41,8 +42,8 @@ struct rossbi_grid {
   double* d_w0 = nullptr;              // primitive equilibrium tables (centres, r faces, z faces)
   std::vector<double> h_e0c;
   // reductions and status
-  unsigned long long* d_dt = nullptr;  // [3]: step ping-pong slots 0/1, standalone CFL slot 2
-  int dt_slot = 0;                     // slot holding the step length of the next step
+  unsigned long long* d_dt = nullptr;  // [2]: ping-pong slots of the largest CFL rate (the step is N_CFL over it)
+  int dt_slot = 0;                     // slot holding the rate of the next step
   bool dt_on_device = false;
   double* d_partials = nullptr;
   size_t partials_cap = 0;
@@ -187,10 +188,18 @@ rossbi_status sync_and_status(rossbi_grid* g) {
   return status_from_word(w);
 }
 
+// The step length N_CFL / rate of a rate slot, on the host (no cell with a
+// rate: infinite).  Synchronises.
+rossbi_status read_dt(rossbi_grid* g, int slot, double* dt) {
+  CK(cudaMemcpyAsync(g->h_pinned, g->d_dt + slot, sizeof(double), cudaMemcpyDeviceToHost, g->stream));
+  const rossbi_status st = sync_and_status(g);
+  *dt = g->desc.cfl / g->h_pinned[0];
+  return st;
+}
+
 // ---------------------------------------------------------------- kernels
 template <int NF>
 __global__ void cfl_kernel(DevGrid g, StageArgs a, unsigned long long* slot) {
-  __shared__ double red[CFL_NT / 32];
   const size_t ncell = (size_t)g.nr * g.nth * g.nz;
   double rate = 0.0;
   unsigned status = 0;
@@ -205,12 +214,9 @@ __global__ void cfl_kernel(DevGrid g, StageArgs a, unsigned long long* slot) {
     if (bad) status |= STATUS_NONPHYSICAL;
     if (positive(c) && mag_less(rate, c)) rate = c;
   }
-  const double m = block_min<CFL_NT>(positive(rate) ? g.cfl / rate : INFINITY, red);
-  if (threadIdx.x == 0) atomic_min_pos_double(slot, m);
+  raise_rate(slot, rate);
   if (status) atomicOr(a.status, status);
 }
-
-__global__ void set_slot_kernel(unsigned long long* slot, unsigned long long v) { *slot = v; }
 
 // Primitive equilibrium table from a conservative one ([5][n] each), with the
 // conversion the stage kernels apply to the state, so that the deviations of
@@ -239,25 +245,17 @@ __global__ void sums_kernel(DevGrid g, StageArgs a, double* partials) {
   }
 }
 
-// Reduces the per-block partials row by row in a fixed order (so the result
-// does not depend on scheduling): rows 0..nf-1 are summed into sums[], row nf
-// (when dt_slot is set) is minimised into the step-length slot.
+// Sums the per-block partials row by row in a fixed order (so the result
+// does not depend on scheduling) into sums[].
 constexpr int RED_NT = 512;
-__global__ void __launch_bounds__(RED_NT) reduce_partials_kernel(const double* partials, int nblocks, int nf,
-                                                                 double* sums, unsigned long long* dt_slot) {
+__global__ void __launch_bounds__(RED_NT) reduce_partials_kernel(const double* partials, int nblocks, double* sums) {
   __shared__ double red[RED_NT / 32];
   const int row = blockIdx.x;
   const double* p = partials + (size_t)row * nblocks;
-  const bool is_min = row == nf;
-  double v = is_min ? INFINITY : 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += RED_NT) v = is_min ? fmin(v, p[b]) : v + p[b];
-  if (is_min) {
-    v = block_min<RED_NT>(v, red);
-    if (threadIdx.x == 0) *dt_slot = (unsigned long long)__double_as_longlong(v);
-  } else {
-    v = block_sum<RED_NT>(v, red);
-    if (threadIdx.x == 0) sums[row] = v;
-  }
+  double v = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += RED_NT) v += p[b];
+  v = block_sum<RED_NT>(v, red);
+  if (threadIdx.x == 0) sums[row] = v;
 }
 
 // Dust densities of every species (null beyond n).
@@ -655,6 +653,7 @@ PertArgs<T> pert_args(rossbi_grid* g) {
   a.status = g->d_status;
   a.tiles_r = g->tiles_r;
   a.tiles_z = g->tiles_z;
+  a.sms = g->sms;
   a.gam = (T)g->dg.gamma;
   a.om = (T)g->dg.omega;
   a.cfl = (T)g->dg.cfl;
@@ -725,8 +724,6 @@ rossbi_status prepare_step(rossbi_grid* g, void* const* state, void* const* scra
     if (st != ROSSBI_OK) return st;
     for (int f = 0; f < g->nf; ++f) sc[f] = (char*)g->d_scratch + (size_t)f * g->ncell * elem_size(g);
   }
-  rossbi_status st = ensure_partials(g, n_tiles(g));
-  if (st != ROSSBI_OK) return st;
   return drag_args(g, dust, drag);
 }
 
@@ -824,32 +821,23 @@ rossbi_status indirect_moments(rossbi_grid* g, void* const* state) {
   return ROSSBI_OK;
 }
 
-rossbi_status finish_step(rossbi_grid* g, const double* partials, int nxt, double* next_dt) {
-  reduce_partials_kernel<<<g->nf + 1, RED_NT, 0, g->stream>>>(partials, n_tiles(g), g->nf, g->d_sums,
-                                                               g->d_dt + nxt);
-  CK(cudaGetLastError());
+rossbi_status finish_step(rossbi_grid* g, int nxt, double* next_dt) {
   g->dt_slot = nxt;
   g->dt_on_device = true;
-  if (next_dt) {
-    CK(cudaMemcpyAsync(g->h_pinned, g->d_dt + nxt, sizeof(double), cudaMemcpyDeviceToHost, g->stream));
-    const rossbi_status st = sync_and_status(g);
-    *next_dt = g->h_pinned[0];
-    return st;
-  }
-  return ROSSBI_OK;
+  return next_dt ? read_dt(g, nxt, next_dt) : ROSSBI_OK;
 }
 
-// The two stages of one step (Sect. 2.5) with E* in sc and the stage-2
-// block partials in `partials`; with the indirect gravity on, the disc
+// The two stages of one step (Sect. 2.5) with E* in sc; with the indirect gravity on, the disc
 // moments of each stage's input are summed before it.  Allocates nothing.
-rossbi_status step_full(rossbi_grid* g, void* const* state, void* const* sc, double* partials, double dt,
+rossbi_status step_full(rossbi_grid* g, void* const* state, void* const* sc, double dt,
                         const DragArgs& drag, double* next_dt) {
   const int nblocks = n_tiles(g);
   const int cur = g->dt_slot, nxt = 1 - g->dt_slot;
   StageArgs a = base_args(g);
   a.drag = drag;
   a.dt_host = dt;
-  a.dt_dev = dt == 0.0 ? g->d_dt + cur : nullptr;
+  a.rate_in = dt == 0.0 ? g->d_dt + cur : nullptr;
+  a.rate_out = g->d_dt + nxt;
   // stage 1: E* = E^n + dt/2 (G(E^n) - R0)/V, then drag
   for (int f = 0; f < g->nf; ++f) {
     a.in[f] = (const double*)state[f];
@@ -870,21 +858,21 @@ rossbi_status step_full(rossbi_grid* g, void* const* state, void* const* sc, dou
   }
   a.tau_frac = 1.0;
   a.stage2 = 1;
-  a.partials = partials;
   st = launch_stage(g, a, nblocks);
   if (st != ROSSBI_OK) return st;
-  return finish_step(g, partials, nxt, next_dt);
+  return finish_step(g, nxt, next_dt);
 }
 
 template <class T>
-rossbi_status step_pert(rossbi_grid* g, void* const* state, void* const* sc, double* partials, double dt,
+rossbi_status step_pert(rossbi_grid* g, void* const* state, void* const* sc, double dt,
                         const DragArgs& drag, double* next_dt) {
   const int nblocks = n_tiles(g);
   const int cur = g->dt_slot, nxt = 1 - g->dt_slot;
   PertArgs<T> a = pert_args<T>(g);
   set_pert_drag(a, drag);
   a.dt_host = dt;
-  a.dt_dev = dt == 0.0 ? g->d_dt + cur : nullptr;
+  a.rate_in = dt == 0.0 ? g->d_dt + cur : nullptr;
+  a.rate_out = g->d_dt + nxt;
   for (int f = 0; f < g->nf; ++f) {
     a.in[f] = (const T*)state[f];
     a.base[f] = (const T*)state[f];
@@ -903,18 +891,17 @@ rossbi_status step_pert(rossbi_grid* g, void* const* state, void* const* sc, dou
   }
   a.tau_frac = 1.0;
   a.stage2 = 1;
-  a.partials = partials;
   st = launch_pert<T>(g, a, nblocks);
   if (st != ROSSBI_OK) return st;
-  return finish_step(g, partials, nxt, next_dt);
+  return finish_step(g, nxt, next_dt);
 }
 
-rossbi_status step_form(rossbi_grid* g, void* const* state, void* const* sc, double* partials, double dt,
+rossbi_status step_form(rossbi_grid* g, void* const* state, void* const* sc, double dt,
                         const DragArgs& drag, double* next_dt) {
   switch (g->desc.precision) {
-    case ROSSBI_FP64: return step_full(g, state, sc, partials, dt, drag, next_dt);
-    case ROSSBI_FP32_PERT: return step_pert<float>(g, state, sc, partials, dt, drag, next_dt);
-    default: return step_pert<double>(g, state, sc, partials, dt, drag, next_dt);
+    case ROSSBI_FP64: return step_full(g, state, sc, dt, drag, next_dt);
+    case ROSSBI_FP32_PERT: return step_pert<float>(g, state, sc, dt, drag, next_dt);
+    default: return step_pert<double>(g, state, sc, dt, drag, next_dt);
   }
 }
 
@@ -965,7 +952,7 @@ rossbi_status adjoint_reverse(rossbi_grid* g, void* const* state, double dt, con
   adj_point_kernel<NF><<<nb, ADJ_PT_NT, 0, g->stream>>>(p);
   CK(cudaGetLastError());
   if (ind) {
-    reduce_partials_kernel<<<2, RED_NT, 0, g->stream>>>(ind_part, nb, 2, ind_dab, nullptr);
+    reduce_partials_kernel<<<2, RED_NT, 0, g->stream>>>(ind_part, nb, ind_dab);
     CK(cudaGetLastError());
     adj_indirect_bcast_kernel<<<nb, ADJ_PT_NT, 0, g->stream>>>(g->dg, g->d_ind + L.w, ind_dab, LamS[RHO],
                                                                 NF == 9 ? LamS[DRHO] : nullptr);
@@ -991,7 +978,7 @@ rossbi_status adjoint_reverse(rossbi_grid* g, void* const* state, double dt, con
   adj_point_kernel<NF><<<nb, ADJ_PT_NT, 0, g->stream>>>(p);
   CK(cudaGetLastError());
   if (ind) {
-    reduce_partials_kernel<<<2, RED_NT, 0, g->stream>>>(ind_part + 2 * (size_t)nb, nb, 2, ind_dab + 2, nullptr);
+    reduce_partials_kernel<<<2, RED_NT, 0, g->stream>>>(ind_part + 2 * (size_t)nb, nb, ind_dab + 2);
     CK(cudaGetLastError());
     adj_indirect_bcast_kernel<<<nb, ADJ_PT_NT, 0, g->stream>>>(g->dg, g->d_ind + L.w, ind_dab + 2,
                                                                 (double*)lam_n[RHO],
@@ -1113,7 +1100,7 @@ rossbi_status step_device(rossbi_grid* g, void* const* state, void* const* scrat
   DragArgs drag;
   rossbi_status st = prepare_step(g, state, scratch, dt, dust, sc, drag);
   if (st != ROSSBI_OK) return st;
-  return step_form(g, state, sc, g->d_partials, dt, drag, next_dt);
+  return step_form(g, state, sc, dt, drag, next_dt);
 }
 
 }  // namespace
@@ -1220,7 +1207,8 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   if (!g) return ROSSBI_ERR_OOM;
   g->desc = *desc;
   g->stream = (cudaStream_t)cuda_stream;
-  if (cudaGetDevice(&g->device) != cudaSuccess) {
+  if (cudaGetDevice(&g->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess) {
     delete g;
     return ROSSBI_ERR_CUDA;
   }
@@ -1306,7 +1294,7 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
     if ((st = upload(&g->d_ir, ir, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_omk, omk, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_grav, grav, g->stream)) != ROSSBI_OK) break;
-    if (cudaMalloc(&g->d_dt, 3 * sizeof(unsigned long long)) != cudaSuccess) { st = ROSSBI_ERR_OOM; break; }
+    if (cudaMalloc(&g->d_dt, 2 * sizeof(unsigned long long)) != cudaSuccess) { st = ROSSBI_ERR_OOM; break; }
     if (cudaMalloc(&g->d_sums, NF_MAX * sizeof(double)) != cudaSuccess) { st = ROSSBI_ERR_OOM; break; }
     if (cudaMalloc(&g->d_status, sizeof(unsigned)) != cudaSuccess) { st = ROSSBI_ERR_OOM; break; }
     if (cudaMemsetAsync(g->d_status, 0, sizeof(unsigned), g->stream) != cudaSuccess) { st = ROSSBI_ERR_CUDA; break; }
@@ -1442,8 +1430,7 @@ rossbi_status rossbi_cfl_dt(rossbi_grid* g, const void* const* state, double* dt
   for (int f = 0; f < g->nf; ++f)
     if (!state[f]) return ROSSBI_ERR_ARG;
   unsigned long long* slot = g->d_dt + g->dt_slot;
-  set_slot_kernel<<<1, 1, 0, g->stream>>>(slot, 0x7ff0000000000000ull);
-  CK(cudaGetLastError());
+  CK(cudaMemsetAsync(slot, 0, sizeof(*slot), g->stream));
   const int blocks = (int)std::min<size_t>((g->ncell + CFL_NT - 1) / CFL_NT, 152 * 8);
   const int prec = g->desc.precision;
   if (prec == ROSSBI_FP64) {
@@ -1469,11 +1456,8 @@ rossbi_status rossbi_cfl_dt(rossbi_grid* g, const void* const* state, double* dt
     }));
   }
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(g->h_pinned, slot, sizeof(double), cudaMemcpyDeviceToHost, g->stream));
-  const rossbi_status st = sync_and_status(g);
-  *dt_out = g->h_pinned[0];
   g->dt_on_device = true;
-  return st;
+  return read_dt(g, g->dt_slot, dt_out);
 }
 
 rossbi_status rossbi_step(rossbi_grid* g, void* const* state, void* const* scratch, double dt,
@@ -1532,7 +1516,7 @@ rossbi_status rossbi_conservation_sums(rossbi_grid* g, const void* const* state,
     }));
   }
   CK(cudaGetLastError());
-  reduce_partials_kernel<<<g->nf, RED_NT, 0, g->stream>>>(g->d_partials, blocks, g->nf, g->d_sums, nullptr);
+  reduce_partials_kernel<<<g->nf, RED_NT, 0, g->stream>>>(g->d_partials, blocks, g->d_sums);
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(g->h_pinned, g->d_sums, g->nf * sizeof(double), cudaMemcpyDeviceToHost, g->stream));
   st = sync_and_status(g);
@@ -1764,9 +1748,8 @@ rossbi_status rossbi_take_status(rossbi_grid* g) {
 // ---------------------------------------------------------------------------
 // Step without device allocation.
 //
-// rossbi_step takes its stage scratch (the intermediate state E* and the
-// per-block reduction partials) from a buffer it cudaMallocs on first use, or
-// from caller-passed buffers.  Some callers can allocate neither: host codes
+// rossbi_step takes its stage scratch (the intermediate state E*) from a
+// buffer it cudaMallocs on first use, or from caller-passed buffers.  Some callers can allocate neither: host codes
 // that hand all device memory to their own pool at start-up and forbid any
 // later cudaMalloc, or loops that cannot afford the implicit device
 // synchronisation a cudaMalloc/cudaFree may cause.  rossbi_step_noalloc runs
@@ -1780,8 +1763,7 @@ rossbi_status rossbi_take_status(rossbi_grid* g) {
 // rossbi_step_noalloc call made on that device.  That first call should
 // therefore come before any stream capture.  All calls share the array and it
 // keeps the last call's contents; nothing in it needs to start at zero
-// (stage 1 writes every E* cell stage 2 reads, and each stage-2 block writes
-// its own partials).  Calls whose work overlaps on the GPU (other streams,
+// (stage 1 writes every E* cell stage 2 reads).  Calls whose work overlaps on the GPU (other streams,
 // other grids, other threads) race on the array and must be serialised by the
 // caller.
 // ---------------------------------------------------------------------------
@@ -1823,9 +1805,16 @@ extern "C" rossbi_status rossbi_step_noalloc(rossbi_grid* g, void* const* state,
   int dev = -1;
   CK(cudaGetDevice(&dev));
   if (dev != g->device) return ROSSBI_ERR_ARG;
-  const int nblocks = n_tiles(g);
   const size_t field_bytes = align256(g->ncell * elem_size(g));
-  const size_t partial_bytes = (size_t)(g->nf + 1) * nblocks * sizeof(double);
+  // the documented limit: beside the fields, nf + 1 doubles per tile (14 x 6 x 6
+  // cells; two z cells in the FP64-state forms of two and more species, 14 x 30 x
+  // 1 on a flat FP64 grid), whatever the launches use
+  const rossbi_grid_desc& d = g->desc;
+  const bool f64 = d.precision != ROSSBI_FP32_PERT;
+  const bool flat = d.precision == ROSSBI_FP64 && flat_grid(d.nz, d.bc_lo[2], d.bc_hi[2], g->nf);
+  auto tiles = [](int n, int t) { return (size_t)((n + t - 1) / t); };
+  const size_t ntiles = tiles(d.nr, 14) * tiles(d.nth, flat ? 30 : 6) * tiles(d.nz, flat ? 1 : (f64 && g->nf > 9 ? 2 : 6));
+  const size_t partial_bytes = (size_t)(g->nf + 1) * ntiles * sizeof(double);
   if ((size_t)g->nf * field_bytes + partial_bytes > NOALLOC_SCRATCH_BYTES) return ROSSBI_ERR_ARG;
   DragArgs drag;
   rossbi_status st = drag_args(g, dust, drag);
@@ -1835,8 +1824,7 @@ extern "C" rossbi_status rossbi_step_noalloc(rossbi_grid* g, void* const* state,
   if (st != ROSSBI_OK) return st;
   void* sc[NF_MAX];
   for (int f = 0; f < g->nf; ++f) sc[f] = (char*)base + (size_t)f * field_bytes;
-  double* partials = (double*)((char*)base + (size_t)g->nf * field_bytes);
   // the same two stages as rossbi_step (with the indirect gravity's moments
   // in the grid's own tables, set up by rossbi_set_indirect)
-  return step_form(g, state, sc, partials, dt, drag, next_dt);
+  return step_form(g, state, sc, dt, drag, next_dt);
 }

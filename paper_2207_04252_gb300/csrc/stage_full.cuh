@@ -13,7 +13,7 @@
 // is accumulated in shared memory; the epilogue adds the sources (App. B),
 // subtracts the balanced residual R0 (Sect. 2.8), applies the RK stage update
 // (Sect. 2.5) and the semi-implicit drag (Sect. 2.9), and in stage 2 fuses the
-// CFL minimum and the FP64 conservation partial sums of the new state.
+// CFL rate of the new state.
 #pragma once
 #include "device_common.cuh"
 
@@ -26,11 +26,11 @@ struct StageArgs {
   double* out[NF_MAX];         // updated state
   double* gout;            // mode 1: G(E) - R0 written here, [nf][ncell]
   double dt_host;
-  const unsigned long long* dt_dev;  // if set, dt is read from this device slot
-  double tau_frac;                   // 0.5 (stage 1) or 1.0 (stage 2)
+  const unsigned long long* rate_in;  // if set, dt = N_CFL / (the rate in this device slot)
+  unsigned long long* rate_out;       // the largest CFL rate of the output: cleared by stage 1, raised by stage 2
+  double tau_frac;                    // 0.5 (stage 1) or 1.0 (stage 2)
   DragArgs drag;
-  int stage2;                        // fuse CFL of the output and conservation partials
-  double* partials;                  // stage 2: [nf + 1][gridDim.x] block sums of V*E, then block dt minima
+  int stage2;                         // fuse the CFL rate of the output
   unsigned* status;
   int mode;                          // 0 update, 1 residual only (empty run)
   int tiles_r, tiles_z;  // tile counts along r and z (block -> tile: r fastest, then z, then theta)
@@ -124,23 +124,23 @@ __device__ __forceinline__ void dust_recon(const T* sE, int sidx, int b, const T
   }
 }
 
-// Ghost rule of Sect. 2.4 for a cell index possibly outside the domain.
-// Returns false for an equilibrium ghost (E' = 0).
-__device__ __forceinline__ bool resolve_cell(const DevGrid& g, int c[3]) {
-  const int n[3] = {g.nr, g.nth, g.nz};
-#pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-    if (c[ax] >= 0 && c[ax] < n[ax]) continue;
-    const int bc = c[ax] < 0 ? g.bc_lo[ax] : g.bc_hi[ax];
-    if (bc == BC_EQUILIBRIUM) return false;
-    if (bc == BC_PERIODIC) {
-      c[ax] %= n[ax];
-      if (c[ax] < 0) c[ax] += n[ax];
-    } else {
-      c[ax] = c[ax] < 0 ? 0 : n[ax] - 1;
-    }
+// Ghost rule of Sect. 2.4 for a cell index of one axis, possibly outside the
+// domain.  Returns false for an equilibrium ghost (E' = 0).
+__device__ __forceinline__ bool resolve_axis(const DevGrid& g, int ax, int& c) {
+  const int n = ax == 0 ? g.nr : (ax == 1 ? g.nth : g.nz);
+  if (c >= 0 && c < n) return true;
+  const int bc = c < 0 ? g.bc_lo[ax] : g.bc_hi[ax];
+  if (bc == BC_EQUILIBRIUM) return false;
+  if (bc == BC_PERIODIC) {
+    c %= n;
+    if (c < 0) c += n;
+  } else {
+    c = c < 0 ? 0 : n - 1;
   }
   return true;
+}
+__device__ __forceinline__ bool resolve_cell(const DevGrid& g, int c[3]) {
+  return resolve_axis(g, 0, c[0]) && resolve_axis(g, 1, c[1]) && resolve_axis(g, 2, c[2]);
 }
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
@@ -330,43 +330,31 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;
 }
 
-// The block's stage-2 results: the sums in FP64 in a fixed order (each thread's
-// partials to shared memory, then NF x 8 threads add NT / 8 of them each and
-// 8-lane shuffles finish; a five-level butterfly in every lane cost the FP64
-// pipe ten times that), and the smallest step length.  smem: NF NT + NT / 32
-// doubles, free once every thread is here.
-template <int NT, int NF>
-__device__ __forceinline__ void block_results(const double* sums, double dtmin, double* red, double* partials) {
-  constexpr int NW = NT / 32, SEG = NT / 8;
-  static_assert(NT % 8 == 0 && NF * 8 <= NT, "reduction layout");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// The stage's length tau, formed by one thread (an FP64 division is worth
+// eight operations of the two-lane pipe) for all to read after a barrier.
+__device__ __forceinline__ void publish_tau(double* tau, double frac, double dt_host, const unsigned long long* rate_in,
+                                            double cfl) {
+  if (threadIdx.x == 0) *tau = frac * (rate_in ? cfl / __longlong_as_double((long long)*rate_in) : dt_host);
+}
+// Stage 1 clears the slot that stage 2 of the step raises.
+__device__ __forceinline__ void clear_rate(unsigned long long* rate_out) {
+  if (rate_out && blockIdx.x == 0 && threadIdx.x == 0) *rate_out = 0;
+}
+// Raises the slot to the warp's largest rate (non-negative values order like
+// their bits: exact and independent of the order).  The CFL step is N_CFL over
+// the maximum, so that no block divides and no launch reduces partials.
+__device__ __forceinline__ void raise_rate(unsigned long long* rate_out, float rate) {
+  const float m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rate)));
+  if ((threadIdx.x & 31) == 0 && positive(m))
+    atomicMax(rate_out, (unsigned long long)__double_as_longlong((double)m));
+}
+__device__ __forceinline__ void raise_rate(unsigned long long* rate_out, double rate) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const double other = __shfl_xor_sync(0xffffffffu, dtmin, o);
-    if (mag_less(other, dtmin)) dtmin = other;
+    const double other = __shfl_xor_sync(0xffffffffu, rate, o);
+    if (mag_less(rate, other)) rate = other;
   }
-  __syncthreads();
-#pragma unroll
-  for (int f = 0; f < NF; ++f) red[f * NT + threadIdx.x] = sums[f];
-  if (lane == 0) red[NF * NT + warp] = dtmin;
-  __syncthreads();
-  if (threadIdx.x < NF * 8) {
-    const int f = threadIdx.x >> 3, seg = threadIdx.x & 7;
-    const double* src = red + f * NT + seg * SEG;
-    double acc = 0.0;
-#pragma unroll 8
-    for (int u = 0; u < SEG; ++u) acc += src[u];
-    const unsigned grp = 0xffu << (lane & 24);  // this 8-lane group (all of it active)
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) acc += __shfl_down_sync(grp, acc, o, 8);
-    if (seg == 0) partials[(size_t)f * gridDim.x + blockIdx.x] = acc;
-  }
-  if (threadIdx.x == NT - 1) {
-    double m = red[NF * NT];
-    for (int w = 1; w < NW; ++w)
-      if (mag_less(red[NF * NT + w], m)) m = red[NF * NT + w];
-    partials[(size_t)NF * gridDim.x + blockIdx.x] = m;
-  }
+  if ((threadIdx.x & 31) == 0 && positive(rate)) atomicMax(rate_out, (unsigned long long)__double_as_longlong(rate));
 }
 
 // XT: the optional terms (indirect gravity, wave-killing zones) are compiled
@@ -391,6 +379,9 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
   const int k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
   const int j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
   unsigned status = 0;
+  __shared__ double s_tau;
+  publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, g.cfl);
+  if (!a.stage2) clear_rate(a.rate_out);
 
   // tile + halo (edges and corners are never read): put(idx, cell or null)
   // for every staged cell, null for an equilibrium ghost
@@ -465,13 +456,10 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
     }
   }
 
-  const double tau = a.tau_frac * (a.dt_dev ? __longlong_as_double((long long)*a.dt_dev) : a.dt_host);
+  const double tau = s_tau;
   const size_t ncell = (size_t)g.nr * g.nth * g.nz;
   constexpr int ND = NF > 5 ? (NF - 5) / 4 : 1;
   double rate = 0.0;
-  double sums[NF];
-#pragma unroll
-  for (int f = 0; f < NF; ++f) sums[f] = 0.0;
   for (int cidx = threadIdx.x; cidx < NCORE; cidx += NT) {
     const int x = cidx % TR, y = (cidx / TR) % TT, z = cidx / (TR * TT);
     const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
@@ -527,13 +515,9 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
       const double c = cell_rate<NF>(g, gi, E, ig, id, bad);
       if (bad) status |= STATUS_NONPHYSICAL;
       if (positive(c) && mag_less(rate, c)) rate = c;
-      const double V = g.vol[gi];
-#pragma unroll
-      for (int f = 0; f < NF; ++f) sums[f] = fma(V, E[f], sums[f]);
     }
   }
-  if (a.mode == 0 && a.stage2)  // a thread without a cell: rate 0, an infinite step
-    block_results<NT, NF>(sums, positive(rate) ? g.cfl / rate : INFINITY, smem, a.partials);
+  if (a.mode == 0 && a.stage2) raise_rate(a.rate_out, rate);
   if (status) atomicOr(a.status, status);
 }
 

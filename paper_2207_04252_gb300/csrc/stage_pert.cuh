@@ -427,13 +427,14 @@ struct PertArgs {
   const T* base[NF_MAX];
   T* out[NF_MAX];
   double dt_host;
-  const unsigned long long* dt_dev;
+  const unsigned long long* rate_in;  // as StageArgs
+  unsigned long long* rate_out;
   double tau_frac;
   DragArgs drag;
   int stage2;
-  double* partials;  // stage 2: [nf + 1][gridDim.x] block sums of V*E', then block dt minima
   unsigned* status;
-  int tiles_r, tiles_z;  // tile counts along r and z (block -> tile: r fastest, then z, then theta)
+  int tiles_r, tiles_z;  // tile counts along r and z (tile number: r fastest, then z, then theta)
+  int sms;               // SMs of the device
   // the grid's and the drag's parameters in the state precision, converted
   // once on the host (GB300's FP64 pipe is narrow: per-use conversions of the
   // double originals cost latency in the float kernel)
@@ -616,10 +617,7 @@ __device__ __forceinline__ void sweep_pert(const PertArgs<T>& a, const T* sE, T*
 }
 
 // Dynamic shared memory of stage_pert_kernel: the staged tile and halo, and
-// the accumulator of the flux divergence.  (A second accumulator, which let
-// the r and theta sweeps share one pool of chunks without a barrier between
-// them, measured 15 % slower on the FP32 bench grid: 101 KB per block leaves
-// two blocks per SM too little L1 for the face solver's stack.)
+// the accumulator of the flux divergence.
 template <class T, int NF, int TR, int TT, int TZ>
 __host__ __device__ constexpr size_t pert_smem_bytes() {
   return (size_t)NF * ((TR + 4) * (TT + 4) * (TZ + 4) + TR * TT * TZ) * sizeof(T);
@@ -804,102 +802,115 @@ __device__ __forceinline__ T pert_cell_rate(const PertArgs<T>& a, const PCell<T>
   return rate * a.t.aov[i];
 }
 
-// XT: the optional terms (indirect gravity, wave-killing zones) are compiled
-// in; the plain instantiation carries none of their code.
-template <class T, int NF, int TR, int TT, int TZ, int NT, int MINB, class P, bool XT, int RC>
-__global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> a) {
-  constexpr int BX = TR + 4, BY = TT + 4, BZ = TZ + 4, BOX = BX * BY * BZ, NCORE = TR * TT * TZ;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sE = reinterpret_cast<T*>(smem_raw);
-  T* sG = sE + NF * BOX;
-  const DevGrid& g = a.g;
-  const int tile = blockIdx.x;
-  // r fastest, then z, then theta: the tiles whose halos a tile re-reads
-  // (its r, z and theta neighbours) run at most tiles_r x tiles_z blocks
-  // apart, so the re-reads hit in L2
-  const int i0 = (tile % a.tiles_r) * TR;
-  const int k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
-  const int j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
-  unsigned status = 0, nfallback = 0;
+// The box of a TR x TT x TZ tile: staging and the per-cell epilogue.
+template <class T, int NF, int TR, int TT, int TZ, int NT, int RC>
+struct PertTile {
+  static constexpr int BX = TR + 4, BY = TT + 4, BZ = TZ + 4, PLANE = BX * BY, BOX = PLANE * BZ, NCORE = TR * TT * TZ;
+  // Each thread owns one (r, theta) position of the box and walks its z planes
+  // (half of them where the block has two threads per position), so that an
+  // index costs one addition (a division into three indices for each of the
+  // box's 1,800 cells made staging a sixth of the kernel's instructions).
+  static constexpr int HALVES = NT >= 2 * PLANE ? 2 : 1;
+  static_assert(PLANE <= NT && BZ % 2 == 0, "a thread per (r, theta) position of the box");
+  int i0, j0, k0;
 
-  // each cell's fields go global -> shared by asynchronous copies (cp.async, no
+  __device__ __forceinline__ PertTile(const PertArgs<T>& a, int tile) {
+    // r fastest, then z, then theta: the tiles whose halos a tile re-reads
+    // (its r, z and theta neighbours) run at most tiles_r x tiles_z blocks
+    // apart, so the re-reads hit in L2
+    i0 = (tile % a.tiles_r) * TR;
+    k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
+    j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
+  }
+
+  // walk(position, z plane, cell indices ci, cj, ck, inside) over this thread's cells
+  template <class F>
+  __device__ __forceinline__ void walk(const DevGrid& g, F&& put) const {
+    if (threadIdx.x >= HALVES * PLANE) return;
+    const int half = HALVES == 2 && threadIdx.x >= PLANE ? 1 : 0, pos = (int)threadIdx.x - half * PLANE;
+    const int x = pos % BX - 2, y = pos / BX - 2;
+    const bool side = x < 0 || x >= TR, end = y < 0 || y >= TT;
+    if (side && end) return;  // no sweep reads the box's edges and corners
+    int ci = i0 + x, cj = j0 + y;
+    const bool in = resolve_axis(g, 0, ci) && resolve_axis(g, 1, cj);
+    int z0 = side || end ? 2 : 0, z1 = side || end ? TZ + 2 : BZ;
+    if (HALVES == 2) {
+      if (half) z0 = BZ / 2;
+      else z1 = BZ / 2;
+    }
+#pragma unroll 2
+    for (int z = z0; z < z1; ++z) {
+      int ck = k0 + z - 2;
+      const bool inside = resolve_axis(g, 2, ck) && in;
+      put(z * PLANE + pos, ci, cj, ck, inside);
+    }
+  }
+
+  // The fields global -> shared by asynchronous copies (cp.async, no
   // registers), all of a thread's cells in flight at once; equilibrium ghosts
-  // are zero departures.  A thread then converts the cells it copied: the dust
+  // are zero departures.
+  __device__ __forceinline__ void copy(const PertArgs<T>& a, T* sE) const {
+    walk(a.g, [&](int idx, int ci, int cj, int ck, bool inside) {
+      T* dst = sE + idx;
+      if (inside) {
+        const size_t lin = ((size_t)ck * a.g.nth + cj) * a.g.nr + ci;
+#pragma unroll
+        for (int f = 0; f < NF; ++f) cp_async_elem<T>(dst + f * BOX, a.in[f] + lin);
+      } else {
+#pragma unroll
+        for (int f = 0; f < NF; ++f) dst[f * BOX] = T(0);
+      }
+    });
+  }
+
+  // Waits for this thread's copies and converts the cells it copied: the dust
   // to primitives (u, v, w, rho_d), which every reconstruction of the three
   // sweeps reads, and with RC = RECON_PRIM the gas to primitive departures.
-  auto stage = [&](auto&& put) {
-    for (int idx = threadIdx.x; idx < BOX; idx += NT) {
-      const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - 2;
-      const int outside = (x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ);
-      if (outside > 1) continue;  // edge and corner cells of the box: no sweep reads them
-      int c[3] = {i0 + x, j0 + y, k0 + z};
-      const bool in = resolve_cell(g, c);
-      put(idx, c, in);
-    }
-  };
-  stage([&](int idx, const int* c, bool in) {
-    if (!in) {
+  __device__ __forceinline__ void convert(const PertArgs<T>& a, T* sE) const {
+    cp_async_wait_all();
+    if (NF == 5 && RC != RECON_PRIM) return;
+    walk(a.g, [&](int idx, int ci, int, int ck, bool inside) {
+      T* e = sE + idx;
+      if (RC == RECON_PRIM && inside) {
+        const PEq<T> eq = a.g.has_eq ? load_eq(a.t.cen + 8 * ((size_t)ck * a.g.nr + ci)) : PEq<T>{};
+        T q[5], w[5];
 #pragma unroll
-      for (int f = 0; f < NF; ++f) sE[f * BOX + idx] = T(0);
-      return;
-    }
-    const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
+        for (int f = 0; f < 5; ++f) q[f] = e[f * BOX];
+        face_prim(a.gm1, eq.rho, eq.v, q, w);
 #pragma unroll
-    for (int f = 0; f < NF; ++f) cp_async_elem<T>(sE + f * BOX + idx, a.in[f] + lin);
-  });
-  cp_async_wait_all();
-  if (NF > 5 || RC == RECON_PRIM) {
-    for (int idx = threadIdx.x; idx < BOX; idx += NT) {
-      const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - 2;
-      if ((x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ) > 1) continue;
-      if (RC == RECON_PRIM) {
-        int c[3] = {i0 + x, j0 + y, k0 + z};
-        if (resolve_cell(g, c)) {
-          const PEq<T> e = g.has_eq ? load_eq(a.t.cen + 8 * ((size_t)c[2] * g.nr + c[0])) : PEq<T>{};
-          T q[5], w[5];
-#pragma unroll
-          for (int f = 0; f < 5; ++f) q[f] = sE[f * BOX + idx];
-          face_prim(a.gm1, e.rho, e.v, q, w);
-#pragma unroll
-          for (int f = 0; f < 4; ++f) sE[f * BOX + idx] = w[f];
-        }
+        for (int f = 0; f < 4; ++f) e[f * BOX] = w[f];
       }
 #pragma unroll
       for (int b = 5; b < NF; b += 4) {
-        const T rd = sE[(b + 3) * BOX + idx], id = positive(rd) ? recip(rd) : T(0);
+        const T rd = e[(b + 3) * BOX], id = positive(rd) ? recip(rd) : T(0);
 #pragma unroll
-        for (int q = 0; q < 3; ++q) sE[(b + q) * BOX + idx] *= id;
+        for (int q = 0; q < 3; ++q) e[(b + q) * BOX] *= id;
       }
-    }
+    });
   }
-  __syncthreads();
-  sweep_pert<T, NF, TR, TT, TZ, NT, 0, P, RC, false>(a, sE, sG, i0, j0, k0, status, nfallback);
-  __syncthreads();
-  sweep_pert<T, NF, TR, TT, TZ, NT, 1, P, RC, true>(a, sE, sG, i0, j0, k0, status, nfallback);
-  __syncthreads();
-  sweep_pert<T, NF, TR, TT, TZ, NT, 2, P, RC, true>(a, sE, sG, i0, j0, k0, status, nfallback);
-  __syncthreads();
 
-  const T tau = (T)(a.tau_frac * (a.dt_dev ? __longlong_as_double((long long)*a.dt_dev) : a.dt_host));
-  constexpr int ND = NF > 5 ? (NF - 5) / 4 : 1;
-  T rate = T(0);
-  double sums[NF];  // the conservation partials of V E', in FP64 from the first product
-#pragma unroll
-  for (int f = 0; f < NF; ++f) sums[f] = 0.0;
-  for (int cidx = threadIdx.x; cidx < NCORE; cidx += NT) {
+  // The stage update of core cell cidx from the staged cell and its flux
+  // divergence div(f), raising the thread's CFL rate.  XT: the optional terms
+  // (indirect gravity, wave-killing zones) are compiled in; the plain
+  // instantiation carries none of their code.
+  template <bool XT, class F>
+  __device__ __forceinline__ void update(const PertArgs<T>& a, const T* sE, F&& div, int cidx, T tau, T& rate,
+                                         unsigned& status) const {
+    constexpr int ND = NF > 5 ? (NF - 5) / 4 : 1;
+    const DevGrid& g = a.g;
     const int x = cidx % TR, y = (cidx / TR) % TT, z = cidx / (TR * TT);
     const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
-    if (gi >= g.nr || gj >= g.nth || gk >= g.nz) continue;
+    if (gi >= g.nr || gj >= g.nth || gk >= g.nz) return;
     const size_t lin = ((size_t)gk * g.nth + gj) * g.nr + gi;
     const PCell<T> ce = cell_eq(a.t, g, gi, gk);
-    const int sidx = ((z + 2) * BY + (y + 2)) * BX + (x + 2);
+    const int sidx = (z + 2) * PLANE + (y + 2) * BX + (x + 2);
     T e[5], w[5], dust[ND][4], G[NF];  // staged gas, its primitive perturbations, the dust's primitives
 #pragma unroll
     for (int f = 0; f < 5; ++f) e[f] = sE[f * BOX + sidx];
 #pragma unroll
     for (int f = 5; f < NF; ++f) dust[(f - 5) / 4][(f - 5) % 4] = sE[f * BOX + sidx];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) G[f] = sG[f * NCORE + cidx];
+    for (int f = 0; f < NF; ++f) G[f] = div(f);
     if (RC == RECON_CONS) {
       face_prim(a.gm1, ce.rho0, ce.v0, e, w);
     } else {
@@ -935,9 +946,6 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> 
     if (a.stage2) {
       const T c = pert_cell_rate<T, NF>(a, ce, gi, E, ig, id, bad);
       if (positive(c) && !(c <= rate)) rate = c;
-      const double V = g.vol[gi];
-#pragma unroll
-      for (int f = 0; f < NF; ++f) sums[f] += V * (double)E[f];
     } else {
       bad = !positive(ce.rho0 + w[RHO]) || !positive(ce.p0 + w[EN]);
 #pragma unroll
@@ -945,17 +953,41 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> 
     }
     if (bad) status |= STATUS_NONPHYSICAL;
   }
-  if (a.stage2)  // a thread without a cell: rate 0, an infinite step
-    block_results<NT, NF>(sums, positive(rate) ? (double)(a.cfl / rate) : INFINITY,
-                          reinterpret_cast<double*>(smem_raw), a.partials);
+};
+
+// One RK stage of one tile per block.
+template <class T, int NF, int TR, int TT, int TZ, int NT, int MINB, class P, bool XT, int RC>
+__global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> a) {
+  using Tile = PertTile<T, NF, TR, TT, TZ, NT, RC>;
+  constexpr int NCORE = Tile::NCORE;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* sE = reinterpret_cast<T*>(smem_raw);
+  T* sG = sE + NF * Tile::BOX;
+  const Tile t(a, blockIdx.x);
+  unsigned status = 0, nfallback = 0;
+  __shared__ double s_tau;
+  publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, a.g.cfl);
+  if (!a.stage2) clear_rate(a.rate_out);
+  t.copy(a, sE);
+  t.convert(a, sE);
+  __syncthreads();
+  sweep_pert<T, NF, TR, TT, TZ, NT, 0, P, RC, false>(a, sE, sG, t.i0, t.j0, t.k0, status, nfallback);
+  __syncthreads();
+  sweep_pert<T, NF, TR, TT, TZ, NT, 1, P, RC, true>(a, sE, sG, t.i0, t.j0, t.k0, status, nfallback);
+  __syncthreads();
+  sweep_pert<T, NF, TR, TT, TZ, NT, 2, P, RC, true>(a, sE, sG, t.i0, t.j0, t.k0, status, nfallback);
+  __syncthreads();
+  T rate = T(0);
+  for (int cidx = threadIdx.x; cidx < NCORE; cidx += NT)
+    t.template update<XT>(a, sE, [&](int f) { return sG[f * NCORE + cidx]; }, cidx, (T)s_tau, rate, status);
+  if (a.stage2) raise_rate(a.rate_out, rate);
   if (status) atomicOr(a.status, status);
   if (nfallback) atomicAdd(a.t.fallbacks, (unsigned long long)nfallback);
 }
 
-// CFL of a perturbation-form state (Sect. 2.5), block minimum into *slot.
+// Largest CFL rate of a perturbation-form state (Sect. 2.5) into *slot.
 template <class T, int NF>
 __global__ void pert_cfl_kernel(const PertArgs<T> a, unsigned long long* slot) {
-  __shared__ double red[256 / 32];
   const DevGrid& g = a.g;
   const size_t ncell = (size_t)g.nr * g.nth * g.nz;
   T rate = T(0);
@@ -973,8 +1005,7 @@ __global__ void pert_cfl_kernel(const PertArgs<T> a, unsigned long long* slot) {
     if (positive(c) && !(c <= rate)) rate = c;
     if (bad) status |= STATUS_NONPHYSICAL;
   }
-  const double m = block_min<256>(positive(rate) ? (double)(a.cfl / rate) : INFINITY, red);
-  if (threadIdx.x == 0) atomic_min_pos_double(slot, m);
+  raise_rate(slot, rate);
   if (status) atomicOr(a.status, status);
 }
 
