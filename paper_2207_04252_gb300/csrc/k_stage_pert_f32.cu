@@ -1,8 +1,9 @@
-// Launcher of the FP32 perturbation-form stage kernel (stage_pert.cuh) for
+// Launcher of the FP32 perturbation-form stage kernel (stage_f32.cuh) for
 // one power form of the solver (ROSSBI_POW: the gamma = 7/5 integer powers
 // unless the including translation unit chose the general ones) and one gas
 // reconstruction mode (ROSSBI_RC, conservative unless chosen otherwise).
 #include "launch.cuh"
+#include "stage_f32.cuh"
 
 #ifndef ROSSBI_RC
 #define ROSSBI_RC RECON_CONS
@@ -16,8 +17,8 @@ namespace {
 
 template <int NF, int NT, int MINB, class P, bool XT, int RC>
 cudaError_t launch_nt(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
-  constexpr size_t smem = pert_smem_bytes<float, NF, P32_TR, P32_TT, P32_TZ>();
-  auto kern = stage_pert_kernel<float, NF, P32_TR, P32_TT, P32_TZ, NT, MINB, P, XT, RC>;
+  constexpr size_t smem = F32Smem<NF, P32_TR, P32_TT, P32_TZ>::bytes;
+  auto kern = stage_f32_kernel<NF, P32_TR, P32_TT, P32_TZ, NT, MINB, P, XT, RC>;
   static unsigned long long done = 0;
   cudaError_t e = set_smem_once(kern, smem, done);
   if (e != cudaSuccess) return e;

@@ -1,0 +1,436 @@
+// Fused RK2 stage kernel of the FP32 perturbation form.
+//
+// The physics is that of stage_pert.cuh (its face solver, flux, sources, drag
+// and update are called from here); the layout is made for the issue slots,
+// which bound this kernel (a face's work is a few hundred FP32 instructions
+// against nine loads of its state):
+//   - the staged box and the accumulators hold quads, {rho u', rho v', rho w',
+//     E'} of the gas and {u, v, w, rho_d} of a dust species, so that a
+//     reconstruction reads its nine fields at three cells with nine loads
+//     instead of 27, and works on two fields per instruction (the packed f32x2
+//     arithmetic of sm_100 and later);
+//   - row and plane strides are odd numbers of quads, so that the lanes of a
+//     line along any axis fall into different banks;
+//   - the equilibrium of the tile's faces, the parabola weights and the face
+//     areas are copied to shared memory with the box: the sweeps load nothing
+//     from global memory and form no 64-bit address.
+#pragma once
+#include "stage_pert.cuh"
+
+namespace rossbi {
+
+// ---------------------------------------------------------------- two floats at a time
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack2(-1.0f, -1.0f), a); }
+// min(|a|, |b|) with the sign of a b, and the MinMod slope, of both halves
+__device__ __forceinline__ f32x2 min_xorsign2(f32x2 a, f32x2 b) {
+  float a0, a1, b0, b1;
+  unpack2(a, a0, a1);
+  unpack2(b, b0, b1);
+  return pack2(min_xorsign(a0, b0), min_xorsign(a1, b1));
+}
+__device__ __forceinline__ f32x2 minmod2(f32x2 a, f32x2 b) {
+  float a0, a1, b0, b1;
+  unpack2(a, a0, a1);
+  unpack2(b, b0, b1);
+  return pack2(fmaxf(min_xorsign(a0, b0), 0.0f), fmaxf(min_xorsign(a1, b1), 0.0f));
+}
+
+// parabola() of two fields.
+template <bool UNI>
+__device__ __forceinline__ void parabola2(f32x2 em, f32x2 e0, f32x2 ep, const float* w, f32x2& qm, f32x2& qp) {
+  const f32x2 dm = sub2(e0, em), dp = sub2(ep, e0);
+  if (UNI) {
+    const f32x2 c3 = pack2(0.375f, 0.375f), c1 = pack2(0.125f, 0.125f), s = minmod2(dm, dp);
+    qm = sub2(e0, min_xorsign2(fma2(c3, dm, mul2(c1, dp)), s));
+    qp = add2(e0, min_xorsign2(fma2(c3, dp, mul2(c1, dm)), s));
+  } else {
+    auto two = [&](int q) { return pack2(w[q], w[q]); };
+    const f32x2 s = minmod2(mul2(dm, two(0)), mul2(dp, two(1)));
+    qm = sub2(e0, min_xorsign2(fma2(two(2), dm, mul2(two(3), dp)), s));
+    qp = add2(e0, min_xorsign2(fma2(two(4), dm, mul2(two(5), dp)), mul2(two(6), s)));
+  }
+}
+
+// ---------------------------------------------------------------- shared memory
+// Offsets in floats of a block's arrays; quads on 16-byte boundaries.
+template <int NF, int TR, int TT, int TZ>
+struct F32Smem {
+  static constexpr int ND = (NF - 5) / 4, NQ = 1 + ND;  // quads per cell: the gas's, then each dust species'
+  static constexpr int BX = TR + 4, BY = TT + 4, BZ = TZ + 4;
+  static constexpr int ROW = BX | 1, PLANE = (ROW * BY) | 1, BOX = PLANE * BZ;  // staged box, in cells
+  static constexpr int CROW = TR | 1, CPLANE = (CROW * TT) | 1, CORE = CPLANE * TZ;  // accumulators
+  __host__ __device__ static constexpr int up4(int n) { return (n + 3) & ~3; }
+  __host__ __device__ static constexpr int quad(int q) { return 4 * BOX * q; }             // [BOX] quads
+  static constexpr int rho = 4 * BOX * NQ;                             // [BOX] rho'
+  static constexpr int acc0 = up4(rho + BOX);
+  __host__ __device__ static constexpr int acc(int q) { return acc0 + 4 * CORE * q; }      // [CORE] quads
+  static constexpr int acc_rho = acc0 + 4 * CORE * NQ;                 // [CORE]
+  static constexpr int face0 = up4(acc_rho + CORE);                    // r faces -1 .. TR + 1 of each z: [TZ][TR + 3]
+  static constexpr int face1 = face0 + 4 * (TR + 3) * TZ;              // theta faces: [TZ][TR]
+  static constexpr int face2 = face1 + 4 * TR * TZ;                    // z faces -1 .. TZ + 1: [TZ + 3][TR]
+  static constexpr int wgt = face2 + 4 * TR * (TZ + 3);                // [TR + 2][RCW] weights of cells -1 .. TR
+  static constexpr int area = wgt + RCW * (TR + 2);                    // areas: TR + 1 r faces, TR theta, TR z
+  static constexpr int total = up4(area + 3 * TR + 1);
+  static constexpr size_t bytes = (size_t)total * sizeof(float);
+  __host__ __device__ static constexpr int face(int axis) { return axis == 0 ? face0 : (axis == 1 ? face1 : face2); }
+};
+
+template <int NF, int TR, int TT, int TZ, int NT, int RC>
+struct F32Tile {
+  using M = F32Smem<NF, TR, TT, TZ>;
+  int i0, j0, k0;
+  __device__ __forceinline__ F32Tile(const PertArgs<float>& a, int tile) {
+    // r fastest, then z, then theta: the tiles whose halos a tile re-reads run
+    // at most tiles_r x tiles_z blocks apart, so the re-reads hit in L2
+    i0 = (tile % a.tiles_r) * TR;
+    k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
+    j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
+  }
+
+  // The tile and its halo as deviations: the gas as conservative departures (or,
+  // with RC = RECON_PRIM, primitive ones), the dust as primitives, converted
+  // once here.  Each thread owns one (r, theta) position of the box and walks
+  // its z planes (half of them where the block has two threads per position),
+  // so that an index costs one addition; the loads of a batch of planes are all
+  // in flight before the first is used.  Equilibrium ghosts are zero departures.
+  __device__ __forceinline__ void stage(const PertArgs<float>& a, float* sm) const {
+    constexpr int COLS = M::BX * M::BY, HALVES = NT >= 2 * COLS ? 2 : 1, NB = NF <= 9 ? 5 : 2;
+    static_assert(COLS <= NT && M::BZ % 2 == 0, "a thread per (r, theta) position of the box");
+    const DevGrid& g = a.g;
+    if (threadIdx.x >= HALVES * COLS) return;
+    const int half = HALVES == 2 && threadIdx.x >= COLS ? 1 : 0, pos = (int)threadIdx.x - half * COLS;
+    const int x = pos % M::BX - 2, y = pos / M::BX - 2;
+    const bool side = x < 0 || x >= TR, end = y < 0 || y >= TT;
+    if (side && end) return;  // no sweep reads the box's edges and corners
+    int ci = i0 + x, cj = j0 + y;
+    const bool in = resolve_axis(g, 0, ci) && resolve_axis(g, 1, cj);
+    const int first = side || end ? 2 : 0, last = side || end ? TZ + 2 : M::BZ;
+    const int z0 = HALVES == 2 && half ? M::BZ / 2 : 0, z1 = HALVES == 2 && !half ? M::BZ / 2 : M::BZ;
+    const size_t plane = (size_t)g.nth * g.nr, row = (size_t)cj * g.nr + ci;
+    const int at = (y + 2) * M::ROW + (x + 2);
+#pragma unroll 1
+    for (int zb = z0; zb < z1; zb += NB) {
+      float v[NB][NF], eq[NB][2];
+      bool use[NB], inside[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        const int z = zb + u;
+        int ck = k0 + z - 2;
+        use[u] = z < z1 && z >= first && z < last;
+        inside[u] = use[u] && resolve_axis(g, 2, ck) && in;
+        if (inside[u]) {
+          const size_t lin = (size_t)ck * plane + row;
+#pragma unroll
+          for (int f = 0; f < NF; ++f) v[u][f] = a.in[f][lin];
+          if (RC == RECON_PRIM) {
+            const float* c = a.t.cen + 8 * ((size_t)ck * g.nr + ci);
+            eq[u][0] = g.has_eq ? c[0] : 0.0f;
+            eq[u][1] = g.has_eq ? c[1] : 0.0f;
+          }
+        } else {
+#pragma unroll
+          for (int f = 0; f < NF; ++f) v[u][f] = 0.0f;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        if (!use[u]) continue;
+        const int s = (zb + u) * M::PLANE + at;
+        if (RC == RECON_PRIM && inside[u]) {
+          float w[5];
+          face_prim(a.gm1, eq[u][0], eq[u][1], v[u], w);
+#pragma unroll
+          for (int f = 0; f < 4; ++f) v[u][f] = w[f];
+        }
+        reinterpret_cast<float4*>(sm)[s] = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
+        sm[M::rho + s] = v[u][RHO];
+#pragma unroll
+        for (int b = 5; b < NF; b += 4) {
+          const float rd = v[u][b + 3], id = positive(rd) ? recip(rd) : 0.0f;
+          reinterpret_cast<float4*>(sm + M::quad((b - 1) / 4))[s] =
+              make_float4(v[u][b] * id, v[u][b + 1] * id, v[u][b + 2] * id, rd);
+        }
+      }
+    }
+  }
+
+  // The tables of the tile's faces and cells, indices clamped to the grid.
+  __device__ __forceinline__ void tables(const PertArgs<float>& a, float* sm) const {
+    const DevGrid& g = a.g;
+    constexpr int N0 = (TR + 3) * TZ, N1 = N0 + TR * TZ, N2 = N1 + TR * (TZ + 3);
+    for (int q = threadIdx.x; q < N2; q += NT) {
+      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (g.has_eq) {
+        size_t o;
+        const float* t;
+        if (q < N0) {
+          const int f = clampi(i0 - 1 + q % (TR + 3), 0, g.nr), k = clampi(k0 + q / (TR + 3), 0, g.nz - 1);
+          t = a.t.face[0];
+          o = (size_t)k * (g.nr + 1) + f;
+        } else if (q < N1) {
+          const int c = q - N0, i = clampi(i0 + c % TR, 0, g.nr - 1), k = clampi(k0 + c / TR, 0, g.nz - 1);
+          t = a.t.face[1];
+          o = (size_t)k * g.nr + i;
+        } else {
+          const int c = q - N1, i = clampi(i0 + c % TR, 0, g.nr - 1), f = clampi(k0 - 1 + c / TR, 0, g.nz);
+          t = a.t.face[2];
+          o = (size_t)f * g.nr + i;
+        }
+        v = reinterpret_cast<const float4*>(t)[o];
+      }
+      reinterpret_cast<float4*>(sm + M::face0)[q] = v;
+    }
+    constexpr int W = RCW * (TR + 2);
+    for (int q = threadIdx.x; q < W + 3 * TR + 1; q += NT) {
+      float v;
+      if (q < W) {
+        const int c = i0 - 1 + q / RCW;  // weights of cells -1 .. nr are tabulated
+        v = a.t.rcoef[(size_t)((c > g.nr ? g.nr : c) + 1) * RCW + q % RCW];
+      } else if (q < W + TR + 1) {
+        v = a.t.area_r[clampi(i0 + q - W, 0, g.nr)];
+      } else if (q < W + 2 * TR + 1) {
+        v = a.t.area_t[clampi(i0 + q - W - TR - 1, 0, g.nr - 1)];
+      } else {
+        v = a.t.area_z[clampi(i0 + q - W - 2 * TR - 1, 0, g.nr - 1)];
+      }
+      sm[M::wgt + q] = v;
+    }
+  }
+
+  // One 32-lane chunk of the sweep along axis D: items base .. base + 31 (whole
+  // lines of L lanes).  Lane p of a line reconstructs cell p - 1, takes the
+  // upper face state of its lower neighbour by a shuffle, solves its lower
+  // face and takes the flux of its upper face by a second shuffle.
+  template <int D, class P>
+  __device__ __forceinline__ void chunk(const PertArgs<float>& a, float* sm, int base, unsigned& status,
+                                        unsigned& nfallback) const {
+    constexpr int TD = D == 0 ? TR : (D == 1 ? TT : TZ), L = pow2ceil(TD + 2);
+    constexpr int NA = D == 0 ? TT : TR;
+    constexpr int ITEMS = items<D>();
+    constexpr int ST = D == 0 ? 1 : (D == 1 ? M::ROW : M::PLANE);
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr bool UNI = D != 0;
+    static_assert(L <= 32, "line does not fit a warp");
+    const DevGrid& g = a.g;
+    const int item = base + (threadIdx.x & 31);
+    const int line = item / L, c = item % L - 1;
+    const int ta = line % NA, tb = line / NA;
+    const int x = D == 0 ? c : ta, y = D == 1 ? c : (D == 0 ? ta : tb), z = D == 2 ? c : tb;
+    const bool line_ok = item < ITEMS && (D == 0 ? (j0 + y < g.nth && k0 + z < g.nz)
+                                                 : (D == 1 ? (i0 + x < g.nr && k0 + z < g.nz)
+                                                           : (i0 + x < g.nr && j0 + y < g.nth)));
+    const int gd = D == 0 ? i0 + x : (D == 1 ? j0 + y : k0 + z), nd = D == 0 ? g.nr : (D == 1 ? g.nth : g.nz);
+    const bool do_recon = line_ok && c <= TD && gd <= nd, do_face = do_recon && c >= 0;
+    const bool do_acc = do_face && c < TD && gd < nd;
+    if (!__any_sync(FULL, do_face)) return;  // a warp of lines beyond a ragged grid's edge
+    // idle lanes read a cell that exists
+    const int s = do_recon ? (z + 2) * M::PLANE + (y + 2) * M::ROW + (x + 2) : 2 * M::PLANE + 2 * M::ROW + 2;
+    const int fx = do_recon ? (D == 0 ? z * (TR + 3) + x + 1 : (D == 1 ? z * TR + x : (z + 1) * TR + x)) : 0;
+    const int ax = do_face ? x : 0;
+    const int core = do_acc ? z * M::CPLANE + y * M::CROW + x : 0;
+    float w[RCW];
+    if (!UNI) {
+      const float4* q = reinterpret_cast<const float4*>(sm + M::wgt) + 2 * (do_recon ? x + 1 : 0);
+      const float4 q0 = q[0], q1 = q[1];
+      w[0] = q0.x; w[1] = q0.y; w[2] = q0.z; w[3] = q0.w;
+      w[4] = q1.x; w[5] = q1.y; w[6] = q1.z;
+    }
+    const float area = sm[M::area + (D == 0 ? 0 : (D == 1 ? TR + 1 : 2 * TR + 1)) + ax];
+    {
+      const float4* ft = reinterpret_cast<const float4*>(sm + M::face(D)) + fx;
+      constexpr int FS = D == 0 ? 1 : (D == 1 ? 0 : TR);  // to the upper face (theta: the same)
+      const float4 fm = ft[0], fp = ft[FS];
+      const PEq<float> Em{fm.x, fm.y, fm.z, fm.w};
+      float wm[5], wp[5];  // primitive perturbations: right state of the lower face, left state of the upper face
+      {
+        float qm[5], qp[5];
+        {
+          const ulonglong2* e = reinterpret_cast<const ulonglong2*>(sm) + s;
+          const ulonglong2 em = e[-ST], e0 = e[0], ep = e[ST];
+          const float* r = sm + M::rho + s;
+          f32x2 lo[2], up[2];
+          parabola2<UNI>(em.x, e0.x, ep.x, w, lo[0], up[0]);
+          parabola2<UNI>(em.y, e0.y, ep.y, w, lo[1], up[1]);
+          parabola<UNI>(r[-ST], r[0], r[ST], w, qm[RHO], qp[RHO]);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            unpack2(lo[q], qm[2 * q], qm[2 * q + 1]);
+            unpack2(up[q], qp[2 * q], qp[2 * q + 1]);
+          }
+        }
+        auto face_states = [&]() {
+          if (RC == RECON_PRIM) {
+#pragma unroll
+            for (int f = 0; f < 5; ++f) {
+              wm[f] = qm[f];
+              wp[f] = qp[f];
+            }
+          } else {
+            face_prim(a.gm1, Em.rho, Em.v, qm, wm);
+            face_prim(a.gm1, fp.x, fp.y, qp, wp);
+          }
+          return positive(fminf(Em.rho + wm[RHO], fp.x + wp[RHO])) && positive(fminf(Em.p + wm[EN], fp.z + wp[EN]));
+        };
+        if (!face_states()) {  // positivity fallback: flat reconstruction of the gas fields
+          const float4 e = reinterpret_cast<const float4*>(sm)[s];
+          qm[0] = qp[0] = e.x;
+          qm[1] = qp[1] = e.y;
+          qm[2] = qp[2] = e.z;
+          qm[3] = qp[3] = e.w;
+          qm[RHO] = qp[RHO] = sm[M::rho + s];
+          face_states();
+        }
+      }
+      float F[5], wl[5];
+#pragma unroll
+      for (int f = 0; f < 5; ++f) {
+        wl[f] = __shfl_up_sync(FULL, wp[f], 1, L);  // upper face state of the lower neighbour
+        F[f] = 0.0f;
+      }
+      if (do_face)
+        pert_face<float, D, P>(
+            a, Em, area, wl, wm,
+            [&]() {
+              const int k = k0 + (D == 2 ? 0 : z);  // in the grid: do_face
+              return D == 0 ? k * (g.nr + 1) + gd : (D == 1 ? k * g.nr + i0 + x : gd * g.nr + i0 + x);
+            },
+            F, status, nfallback);
+      add_divergence<D, L>(F, sm + M::acc0, core, do_acc);
+      const float Fu = __shfl_down_sync(FULL, F[RHO], 1, L);
+      if (do_acc) {
+        float* d = sm + M::acc_rho + core;
+        *d = D == 0 ? F[RHO] - Fu : *d + (F[RHO] - Fu);
+      }
+    }
+#pragma unroll 1
+    for (int q = 1; q < M::NQ; ++q) {  // each dust species: primitive reconstruction, kinetic flux
+      const ulonglong2* e = reinterpret_cast<const ulonglong2*>(sm + M::quad(q)) + s;
+      const ulonglong2 em = e[-ST], e0 = e[0], ep = e[ST];
+      f32x2 lo[2], up[2];
+      parabola2<UNI>(em.x, e0.x, ep.x, w, lo[0], up[0]);
+      parabola2<UNI>(em.y, e0.y, ep.y, w, lo[1], up[1]);
+      float qm[4], qp[4], F[4], WL[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        unpack2(lo[h], qm[2 * h], qm[2 * h + 1]);
+        unpack2(up[h], qp[2 * h], qp[2 * h + 1]);
+      }
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
+        F[f] = 0.0f;
+      }
+      if (do_face) dust_kinetic_flux<D>(area, WL, qm, F);
+      add_divergence<D, L>(F, sm + M::acc(q), core, do_acc);
+    }
+  }
+
+  // Writes (D = 0) or adds the divergence F - (F of the lane above) of a quad.
+  template <int D, int L>
+  __device__ __forceinline__ static void add_divergence(const float* F, float* acc, int core, bool own) {
+    float u[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) u[f] = __shfl_down_sync(0xffffffffu, F[f], 1, L);
+    if (own) {
+      ulonglong2* d = reinterpret_cast<ulonglong2*>(acc) + core;
+      ulonglong2 v;
+      v.x = sub2(pack2(F[0], F[1]), pack2(u[0], u[1]));
+      v.y = sub2(pack2(F[2], F[3]), pack2(u[2], u[3]));
+      if (D != 0) {
+        const ulonglong2 o = *d;
+        v.x = add2(o.x, v.x);
+        v.y = add2(o.y, v.y);
+      }
+      *d = v;
+    }
+  }
+
+  template <int D>
+  static __host__ __device__ constexpr int items() {
+    return (D == 0 ? TT * TZ : (D == 1 ? TR * TZ : TR * TT)) * pow2ceil((D == 0 ? TR : (D == 1 ? TT : TZ)) + 2);
+  }
+  template <int D, class P>
+  __device__ __forceinline__ void sweep(const PertArgs<float>& a, float* sm, unsigned& status,
+                                        unsigned& nfallback) const {
+    for (int base = threadIdx.x & ~31; base < items<D>(); base += NT) chunk<D, P>(a, sm, base, status, nfallback);
+  }
+
+  template <bool XT>
+  __device__ __forceinline__ void update(const PertArgs<float>& a, const float* sm, int cidx, float tau, float& rate,
+                                         unsigned& status) const {
+    const int x = cidx % TR, y = (cidx / TR) % TT, z = cidx / (TR * TT);
+    const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
+    if (gi >= a.g.nr || gj >= a.g.nth || gk >= a.g.nz) return;
+    const int s = (z + 2) * M::PLANE + (y + 2) * M::ROW + (x + 2), core = z * M::CPLANE + y * M::CROW + x;
+    float e[5], dust[NF > 5 ? M::ND : 1][4], G[NF];
+    auto quad = [&](int at, float* q) {
+      const float4 v = reinterpret_cast<const float4*>(sm)[at];
+      q[0] = v.x;
+      q[1] = v.y;
+      q[2] = v.z;
+      q[3] = v.w;
+    };
+    quad(s, e);
+    e[RHO] = sm[M::rho + s];
+    quad(M::acc(0) / 4 + core, G);
+    G[RHO] = sm[M::acc_rho + core];
+#pragma unroll
+    for (int q = 1; q < M::NQ; ++q) {
+      quad(M::quad(q) / 4 + s, dust[q - 1]);
+      quad(M::acc(q) / 4 + core, G + 1 + 4 * q);
+    }
+    pert_update<float, NF, RC, XT>(a, gi, gj, gk, e, dust, G, tau, rate, status);
+  }
+};
+
+// One RK stage of one tile per block.
+template <int NF, int TR, int TT, int TZ, int NT, int MINB, class P, bool XT, int RC>
+__global__ void __launch_bounds__(NT, MINB) stage_f32_kernel(const PertArgs<float> a) {
+  extern __shared__ __align__(16) float sm[];
+  const F32Tile<NF, TR, TT, TZ, NT, RC> t(a, blockIdx.x);
+  unsigned status = 0, nfallback = 0;
+  __shared__ double s_tau;
+  publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, a.g.cfl);
+  if (!a.stage2) clear_rate(a.rate_out);
+  t.tables(a, sm);
+  t.stage(a, sm);
+  __syncthreads();
+  t.template sweep<0, P>(a, sm, status, nfallback);
+  __syncthreads();
+  t.template sweep<1, P>(a, sm, status, nfallback);
+  __syncthreads();
+  t.template sweep<2, P>(a, sm, status, nfallback);
+  __syncthreads();
+  float rate = 0.0f;
+  for (int cidx = threadIdx.x; cidx < TR * TT * TZ; cidx += NT)
+    t.template update<XT>(a, sm, cidx, (float)s_tau, rate, status);
+  if (a.stage2) raise_rate(a.rate_out, rate);
+  if (status) atomicOr(a.status, status);
+  if (nfallback) atomicAdd(a.t.fallbacks, (unsigned long long)nfallback);
+}
+
+}  // namespace rossbi

@@ -461,6 +461,53 @@ __device__ __forceinline__ T face_prim(T gm1, T rho0, T v0, const T* q, T* w) {
   return ir;
 }
 
+// Area times the gas flux perturbation through a face normal to axis D of
+// equilibrium Em, from the primitive perturbations wl, wm of its left and right
+// states; wave_at(): the face's place in the table of wave speeds.
+template <class T, int D, class P, class W>
+__device__ __forceinline__ void pert_face(const PertArgs<T>& a, const PEq<T>& Em, T area, const T* wl, const T* wm,
+                                          W&& wave_at, T* F, unsigned& status, unsigned& nfallback) {
+  constexpr int n = Axes<D>::n;
+  const DevGrid& g = a.g;
+  const T un0 = D == 1 ? Em.v : T(0);
+  const T rl = Em.rho + wl[RHO], pl = Em.p + wl[EN], rr = Em.rho + wm[RHO], pr = Em.p + wm[EN];
+  NearStar<T> st;
+  int kind = NEAR_GENERAL;
+  if (sizeof(T) == 4 || (positive(rl) && positive(rr) && positive(pl) && positive(pr)))
+    kind = near_riemann<T>(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
+                           narrow(un0 + wl[n]), narrow(un0 + wm[n]), st);
+  const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
+  T d[3], drho = left ? wl[RHO] : wm[RHO], dp = left ? wl[EN] : wm[EN];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) d[q] = left ? wl[q] : wm[q];
+  if (kind >= NEAR_STAR_L) {
+    drho += st.drho;
+    d[n] = st.us;
+    dp = wl[EN] + st.d;
+  }
+  bool ok = true;
+  if (kind == NEAR_GENERAL) {
+    PFace<T> W0{Em.rho, un0, Em.p, T(0), T(0), T(0)};
+    if (g.has_eq) {
+      const T* wv = a.t.wave[D] + 4 * (size_t)wave_at();
+      W0.c = wv[0];
+      W0.un_mc = wv[1];
+      W0.un_pc = wv[2];
+    }
+    const PStar<T> o = pert_general<T, P>(a.gam, W0, wl[RHO], wl[n], wl[EN], wm[RHO], wm[n], wm[EN], g.has_eq != 0);
+    status |= o.status;
+    nfallback += o.fallback;
+    ok = !(o.status & STATUS_NONPHYSICAL);
+    // the transverse velocity of the side that the face lies on; a vacuum has none
+#pragma unroll
+    for (int q = 0; q < 3; ++q) d[q] = o.side < 0 ? wl[q] : (o.side > 0 ? wm[q] : (q == MV ? -Em.v : T(0)));
+    drho = o.drho;
+    d[n] = o.dun;
+    dp = o.dp;
+  }
+  if (ok) pert_flux<T, D>(a.g_gm1, area, Em, drho, d, dp, F);
+}
+
 // One 32-lane chunk of the sweep along axis D: items base .. base + 31 (whole
 // lines of L lanes).  sE holds the gas departures (conservative, or primitive
 // with RC = RECON_PRIM) and the dust primitives.  The flux divergence of the
@@ -472,7 +519,6 @@ __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* 
   constexpr int BOX = S::BOX, NCORE = S::NCORE, L = S::L, STRIDE = S::STRIDE;
   constexpr unsigned FULL = 0xffffffffu;
   constexpr bool UNI = D != 0;
-  constexpr int n = Axes<D>::n;
   const DevGrid& g = a.g;
   const S s(g, base + (threadIdx.x & 31), i0, j0, k0);
   if (!__any_sync(FULL, s.do_face)) return;  // a warp of lines beyond a ragged grid's edge
@@ -535,47 +581,7 @@ __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* 
       wl[f] = __shfl_up_sync(FULL, wp[f], 1, L);  // upper face state of the lower neighbour
       F[f] = T(0);
     }
-    if (s.do_face) {
-      const T un0 = D == 1 ? Em.v : T(0);
-      const T rl = Em.rho + wl[RHO], pl = Em.p + wl[EN], rr = Em.rho + wm[RHO], pr = Em.p + wm[EN];
-      NearStar<T> st;
-      int kind = NEAR_GENERAL;
-      if (sizeof(T) == 4 || (positive(rl) && positive(rr) && positive(pl) && positive(pr)))
-        kind = near_riemann<T>(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
-                               narrow(un0 + wl[n]), narrow(un0 + wm[n]), st);
-      const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
-      T d[3], drho = left ? wl[RHO] : wm[RHO], dp = left ? wl[EN] : wm[EN];
-#pragma unroll
-      for (int q = 0; q < 3; ++q) d[q] = left ? wl[q] : wm[q];
-      if (kind >= NEAR_STAR_L) {
-        drho += st.drho;
-        d[n] = st.us;
-        dp = wl[EN] + st.d;
-      }
-      bool ok = true;
-      if (kind == NEAR_GENERAL) {
-        PFace<T> W0{Em.rho, un0, Em.p, T(0), T(0), T(0)};
-        if (g.has_eq) {
-          const T* wv = a.t.wave[D] + 4 * (size_t)of;
-          W0.c = wv[0];
-          W0.un_mc = wv[1];
-          W0.un_pc = wv[2];
-        }
-        const PStar<T> o = pert_general<T, P>(a.gam, W0, wl[RHO], wl[n], wl[EN], wm[RHO], wm[n], wm[EN],
-                                              g.has_eq != 0);
-        status |= o.status;
-        nfallback += o.fallback;
-        ok = !(o.status & STATUS_NONPHYSICAL);
-        // the transverse velocity of the side that the face lies on; a vacuum has none
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-          d[q] = o.side < 0 ? wl[q] : (o.side > 0 ? wm[q] : (q == MV ? -Em.v : T(0)));
-        drho = o.drho;
-        d[n] = o.dun;
-        dp = o.dp;
-      }
-      if (ok) pert_flux<T, D>(a.g_gm1, area, Em, drho, d, dp, F);
-    }
+    if (s.do_face) pert_face<T, D, P>(a, Em, area, wl, wm, [&]() { return of; }, F, status, nfallback);
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
       const T Fu = __shfl_down_sync(FULL, F[f], 1, L);
@@ -802,6 +808,62 @@ __device__ __forceinline__ T pert_cell_rate(const PertArgs<T>& a, const PCell<T>
   return rate * a.t.aov[i];
 }
 
+// The stage update of cell (gi, gj, gk) from its staged gas e (conservative
+// departures, or primitive ones with RC = RECON_PRIM), the primitives of its
+// dust and its flux divergence G, raising the thread's CFL rate.  XT: the
+// optional terms (indirect gravity, wave-killing zones) are compiled in; the
+// plain instantiation carries none of their code.
+template <class T, int NF, int RC, bool XT>
+__device__ __forceinline__ void pert_update(const PertArgs<T>& a, int gi, int gj, int gk, const T* e,
+                                            const T (*dust)[4], T* G, T tau, T& rate, unsigned& status) {
+  constexpr int ND = NF > 5 ? (NF - 5) / 4 : 1;
+  const DevGrid& g = a.g;
+  const size_t lin = ((size_t)gk * g.nth + gj) * g.nr + gi;
+  const PCell<T> ce = cell_eq(a.t, g, gi, gk);
+  T w[5];  // primitive perturbations
+  if (RC == RECON_CONS) {
+    face_prim(a.gm1, ce.rho0, ce.v0, e, w);
+  } else {
+#pragma unroll
+    for (int f = 0; f < 5; ++f) w[f] = e[f];
+  }
+  if (g.geom == GEOM_CYL) pert_sources<T, NF, XT>(a, ce, gj, a.t.vol[gi], w, dust, G);
+  if (XT && g.damp_k) {  // wave-killing zones: the gas departures E' relax towards 0
+    T kd;
+    if constexpr (sizeof(T) == 4) kd = g.damp_kf[(size_t)gk * g.nr + gi];
+    else kd = g.damp_k[(size_t)gk * g.nr + gi];
+    if (positive(kd)) {
+      const T V = a.t.vol[gi];
+#pragma unroll
+      for (int f = 0; f < 5; ++f) G[f] -= V * kd * a.in[f][lin];
+    }
+  }
+  const T tv = tau * a.t.ivol[gi];
+  T E[NF], ig = T(0), id[ND];
+#pragma unroll
+  for (int f = 0; f < NF; ++f) {
+    // stage 1 updates its own input, whose gas is staged as it is stored
+    const T b = !a.stage2 && RC == RECON_CONS && f < 5 ? e[f] : a.base[f][lin];
+    E[f] = b + tv * G[f];
+  }
+  if (NF > 5 || a.stage2) ig = recip(ce.rho0 + E[RHO]);
+#pragma unroll
+  for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = recip(E[b + 3]);
+  if constexpr (NF > 5) pert_drag<T, NF, XT>(a, ce, gi, E, tau, ig, id);
+#pragma unroll
+  for (int f = 0; f < NF; ++f) a.out[f][lin] = E[f];
+  bool bad = false;
+  if (a.stage2) {
+    const T c = pert_cell_rate<T, NF>(a, ce, gi, E, ig, id, bad);
+    if (positive(c) && !(c <= rate)) rate = c;
+  } else {
+    bad = !positive(ce.rho0 + w[RHO]) || !positive(ce.p0 + w[EN]);
+#pragma unroll
+    for (int s = 0; s < (NF - 5) / 4; ++s) bad |= !non_negative(dust[s][3]);
+  }
+  if (bad) status |= STATUS_NONPHYSICAL;
+}
+
 // The box of a TR x TT x TZ tile: staging and the per-cell epilogue.
 template <class T, int NF, int TR, int TT, int TZ, int NT, int RC>
 struct PertTile {
@@ -889,69 +951,22 @@ struct PertTile {
     });
   }
 
-  // The stage update of core cell cidx from the staged cell and its flux
-  // divergence div(f), raising the thread's CFL rate.  XT: the optional terms
-  // (indirect gravity, wave-killing zones) are compiled in; the plain
-  // instantiation carries none of their code.
-  template <bool XT, class F>
-  __device__ __forceinline__ void update(const PertArgs<T>& a, const T* sE, F&& div, int cidx, T tau, T& rate,
+  // The update of core cell cidx from the staged fields and accumulators.
+  template <bool XT>
+  __device__ __forceinline__ void update(const PertArgs<T>& a, const T* sE, const T* sG, int cidx, T tau, T& rate,
                                          unsigned& status) const {
-    constexpr int ND = NF > 5 ? (NF - 5) / 4 : 1;
-    const DevGrid& g = a.g;
     const int x = cidx % TR, y = (cidx / TR) % TT, z = cidx / (TR * TT);
     const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
-    if (gi >= g.nr || gj >= g.nth || gk >= g.nz) return;
-    const size_t lin = ((size_t)gk * g.nth + gj) * g.nr + gi;
-    const PCell<T> ce = cell_eq(a.t, g, gi, gk);
+    if (gi >= a.g.nr || gj >= a.g.nth || gk >= a.g.nz) return;
     const int sidx = (z + 2) * PLANE + (y + 2) * BX + (x + 2);
-    T e[5], w[5], dust[ND][4], G[NF];  // staged gas, its primitive perturbations, the dust's primitives
+    T e[5], dust[NF > 5 ? (NF - 5) / 4 : 1][4], G[NF];
 #pragma unroll
     for (int f = 0; f < 5; ++f) e[f] = sE[f * BOX + sidx];
 #pragma unroll
     for (int f = 5; f < NF; ++f) dust[(f - 5) / 4][(f - 5) % 4] = sE[f * BOX + sidx];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) G[f] = div(f);
-    if (RC == RECON_CONS) {
-      face_prim(a.gm1, ce.rho0, ce.v0, e, w);
-    } else {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) w[f] = e[f];
-    }
-    if (g.geom == GEOM_CYL) pert_sources<T, NF, XT>(a, ce, gj, a.t.vol[gi], w, dust, G);
-    if (XT && g.damp_k) {  // wave-killing zones: the gas departures E' relax towards 0
-      T kd;
-      if constexpr (sizeof(T) == 4) kd = g.damp_kf[(size_t)gk * g.nr + gi];
-      else kd = g.damp_k[(size_t)gk * g.nr + gi];
-      if (positive(kd)) {
-        const T V = a.t.vol[gi];
-#pragma unroll
-        for (int f = 0; f < 5; ++f) G[f] -= V * kd * a.in[f][lin];
-      }
-    }
-    const T tv = tau * a.t.ivol[gi];
-    T E[NF], ig = T(0), id[ND];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      // stage 1 updates its own input, whose gas is staged as it is stored
-      const T b = !a.stage2 && RC == RECON_CONS && f < 5 ? e[f] : a.base[f][lin];
-      E[f] = b + tv * G[f];
-    }
-    if (NF > 5 || a.stage2) ig = recip(ce.rho0 + E[RHO]);
-#pragma unroll
-    for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = recip(E[b + 3]);
-    if constexpr (NF > 5) pert_drag<T, NF, XT>(a, ce, gi, E, tau, ig, id);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) a.out[f][lin] = E[f];
-    bool bad = false;
-    if (a.stage2) {
-      const T c = pert_cell_rate<T, NF>(a, ce, gi, E, ig, id, bad);
-      if (positive(c) && !(c <= rate)) rate = c;
-    } else {
-      bad = !positive(ce.rho0 + w[RHO]) || !positive(ce.p0 + w[EN]);
-#pragma unroll
-      for (int s = 0; s < (NF - 5) / 4; ++s) bad |= !non_negative(dust[s][3]);
-    }
-    if (bad) status |= STATUS_NONPHYSICAL;
+    for (int f = 0; f < NF; ++f) G[f] = sG[f * NCORE + cidx];
+    pert_update<T, NF, RC, XT>(a, gi, gj, gk, e, dust, G, tau, rate, status);
   }
 };
 
@@ -979,7 +994,7 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> 
   __syncthreads();
   T rate = T(0);
   for (int cidx = threadIdx.x; cidx < NCORE; cidx += NT)
-    t.template update<XT>(a, sE, [&](int f) { return sG[f * NCORE + cidx]; }, cidx, (T)s_tau, rate, status);
+    t.template update<XT>(a, sE, sG, cidx, (T)s_tau, rate, status);
   if (a.stage2) raise_rate(a.rate_out, rate);
   if (status) atomicOr(a.status, status);
   if (nfallback) atomicAdd(a.t.fallbacks, (unsigned long long)nfallback);
