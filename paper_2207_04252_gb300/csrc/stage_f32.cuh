@@ -260,6 +260,28 @@ struct F32Tile {
       w[4] = q1.x; w[5] = q1.y; w[6] = q1.z;
     }
     const float area = sm[M::area + (D == 0 ? 0 : (D == 1 ? TR + 1 : 2 * TR + 1)) + ax];
+    // the divergence of dust species q: primitive reconstruction, kinetic flux
+    auto dust_flux = [&](int q, float* F) {
+      const ulonglong2* e = reinterpret_cast<const ulonglong2*>(sm + M::quad(q)) + s;
+      const ulonglong2 em = e[-ST], e0 = e[0], ep = e[ST];
+      f32x2 lo[2], up[2];
+      parabola2<UNI>(em.x, e0.x, ep.x, w, lo[0], up[0]);
+      parabola2<UNI>(em.y, e0.y, ep.y, w, lo[1], up[1]);
+      float qm[4], qp[4], WL[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        unpack2(lo[h], qm[2 * h], qm[2 * h + 1]);
+        unpack2(up[h], qp[2 * h], qp[2 * h + 1]);
+      }
+#pragma unroll
+      for (int f = 0; f < 4; ++f) WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
+      dust_kinetic_flux<D>(do_face ? area : 0.0f, WL, qm, F);
+    };
+    // The first species' flux has no branch and nothing in common with the
+    // gas's: here its instructions fill the latencies of the gas's
+    // reconstruction.
+    float Fd[4];
+    if constexpr (M::NQ > 1) dust_flux(1, Fd);
     {
       const float4* ft = reinterpret_cast<const float4*>(sm + M::face(D)) + fx;
       constexpr int FS = D == 0 ? 1 : (D == 1 ? 0 : TR);  // to the upper face (theta: the same)
@@ -326,26 +348,13 @@ struct F32Tile {
         *d = D == 0 ? F[RHO] - Fu : *d + (F[RHO] - Fu);
       }
     }
+    if constexpr (M::NQ > 1) {
+      add_divergence<D, L>(Fd, sm + M::acc(1), core, do_acc);
 #pragma unroll 1
-    for (int q = 1; q < M::NQ; ++q) {  // each dust species: primitive reconstruction, kinetic flux
-      const ulonglong2* e = reinterpret_cast<const ulonglong2*>(sm + M::quad(q)) + s;
-      const ulonglong2 em = e[-ST], e0 = e[0], ep = e[ST];
-      f32x2 lo[2], up[2];
-      parabola2<UNI>(em.x, e0.x, ep.x, w, lo[0], up[0]);
-      parabola2<UNI>(em.y, e0.y, ep.y, w, lo[1], up[1]);
-      float qm[4], qp[4], F[4], WL[4];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        unpack2(lo[h], qm[2 * h], qm[2 * h + 1]);
-        unpack2(up[h], qp[2 * h], qp[2 * h + 1]);
+      for (int q = 2; q < M::NQ; ++q) {
+        dust_flux(q, Fd);
+        add_divergence<D, L>(Fd, sm + M::acc(q), core, do_acc);
       }
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
-        F[f] = 0.0f;
-      }
-      if (do_face) dust_kinetic_flux<D>(area, WL, qm, F);
-      add_divergence<D, L>(F, sm + M::acc(q), core, do_acc);
     }
   }
 
