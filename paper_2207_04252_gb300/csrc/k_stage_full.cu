@@ -10,28 +10,25 @@
 namespace rossbi {
 namespace {
 
-template <int NF, int TT, int TZ, bool XT, int RC>
+template <int NF, class T, bool XT, int RC>
 cudaError_t launch(const StageArgs& a, int nblocks, cudaStream_t s) {
-  constexpr int BOX = (F64_TR + 4) * (TT + 4) * (TZ == 1 ? 1 : TZ + 4);
-  constexpr int NCORE = F64_TR * TT * TZ;
-  constexpr size_t smem = (size_t)(5 * BOX + NF * NCORE) * sizeof(double);
-  constexpr int NT = TZ == 1 ? FLAT_NT : F64_NT, MINB = TZ == 1 ? 3 : 2;
-  auto kern = stage_full_kernel<NF, F64_TR, TT, TZ, NT, MINB, XT, RC>;
+  constexpr size_t smem = (size_t)(5 * SweepLane<T::TR, T::TT, T::TZ, 0>::BOX + NF * T::TR * T::TT * T::TZ) * sizeof(double);
+  auto kern = stage_full_kernel<NF, T::TR, T::TT, T::TZ, T::NT, T::MINB, XT, RC>;
   static unsigned long long done = 0;
   cudaError_t e = set_smem_once(kern, smem, done);
   if (e != cudaSuccess) return e;
-  kern<<<nblocks, NT, smem, s>>>(a);
+  kern<<<nblocks, T::NT, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <int NF, int RC>
 cudaError_t launch_x(const StageArgs& a, int nblocks, cudaStream_t s, bool xt) {
-  if constexpr (NF <= 9) {
-    if (flat_grid(a.g.nz, a.g.bc_lo[2], a.g.bc_hi[2], NF))
-      return xt ? launch<NF, FLAT_TT, 1, true, RC>(a, nblocks, s) : launch<NF, FLAT_TT, 1, false, RC>(a, nblocks, s);
-  }
-  return xt ? launch<NF, F64_TT, F64_TZ, true, RC>(a, nblocks, s)
-            : launch<NF, F64_TT, F64_TZ, false, RC>(a, nblocks, s);
+  auto go = [&](auto tile) {
+    using T = decltype(tile);
+    return xt ? launch<NF, T, true, RC>(a, nblocks, s) : launch<NF, T, false, RC>(a, nblocks, s);
+  };
+  if constexpr (NF <= 9) return by_tile(a.tile, go);
+  else return go(TileMain{});
 }
 
 }  // namespace

@@ -10,26 +10,35 @@
 namespace rossbi {
 namespace {
 
-template <int NF, int TZ, bool XT, int RC>
+template <int NF, class T, bool XT, int RC>
 cudaError_t launch(const PertArgs<double>& a, int nblocks, cudaStream_t s) {
-  constexpr size_t smem = pert_smem_bytes<double, NF, P32_TR, P32_TT, TZ>();
-  auto kern = stage_pert_kernel<double, NF, P32_TR, P32_TT, TZ, P32_NT, 1, PowGeneric<double>, XT, RC>;
+  constexpr size_t smem = (size_t)(5 * SweepLane<T::TR, T::TT, T::TZ, 0>::BOX + NF * T::TR * T::TT * T::TZ) * sizeof(double);
+  auto kern = stage_pert_kernel<NF, T::TR, T::TT, T::TZ, T::NT, T::MINB, PowGeneric<double>, XT, RC>;
   static unsigned long long done = 0;
   cudaError_t e = set_smem_once(kern, smem, done);
   if (e != cudaSuccess) return e;
-  kern<<<nblocks, P32_NT, smem, s>>>(a);
+  kern<<<nblocks, T::NT, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+template <int NF, int RC>
+cudaError_t launch_x(const PertArgs<double>& a, int nblocks, cudaStream_t s, bool xt) {
+  auto go = [&](auto tile) {
+    using T = decltype(tile);
+    return xt ? launch<NF, T, true, RC>(a, nblocks, s) : launch<NF, T, false, RC>(a, nblocks, s);
+  };
+  if constexpr (NF <= 9) {
+    if (a.tile == TILE_MID) return go(TileMid{});
+    if (a.tile == TILE_SMALL) return go(TileSmall{});
+  }
+  return go(TileMain{});
 }
 
 }  // namespace
 
 template <int RC>
 cudaError_t run_stage_pert_f64_rc(const PertArgs<double>& a, int nblocks, cudaStream_t s, bool xt) {
-  return by_nf(a.g.nf, [&](auto nf) {
-    constexpr int NF = decltype(nf)::value;
-    constexpr int TZ = tile_z(true, NF);
-    return xt ? launch<NF, TZ, true, RC>(a, nblocks, s) : launch<NF, TZ, false, RC>(a, nblocks, s);
-  });
+  return by_nf(a.g.nf, [&](auto nf) { return launch_x<decltype(nf)::value, RC>(a, nblocks, s, xt); });
 }
 
 template cudaError_t run_stage_pert_f64_rc<ROSSBI_RC>(const PertArgs<double>&, int, cudaStream_t, bool);

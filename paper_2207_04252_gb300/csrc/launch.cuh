@@ -12,21 +12,68 @@
 
 namespace rossbi {
 
-// Tiles of the stage kernels: 14 x 6 x 6 cells, lines of 16 / 8 / 8 lanes.
-constexpr int F64_TR = 14, F64_TT = 6, F64_TZ = 6, F64_NT = 192;
+// Tiles of the float stage kernel: 14 x 6 x 6 cells, lines of 16 / 8 / 8 lanes.
 constexpr int P32_TR = 14, P32_TT = 6, P32_TZ = 6, P32_NT = 256, P32_MINB = 2, P32_WIDE_NT = 512;
-// With more than one dust species the FP64 perturbation form's staged 14 x 6
-// x 6 tile with its halo (18 x 10 x 10 cells) no longer fits in shared memory
-// (13 fields: 234 KB of the 227 KB a block may have): it takes tiles two z
-// cells thick (lines of 4 lanes in z; 13 fields: 127 KB, 21: 205 KB).
-constexpr int THIN_TZ = 2;
-constexpr int tile_z(bool fp64_pert, int nf) { return fp64_pert && nf > 9 ? THIN_TZ : 6; }
 
-// The FP64 kernel's flat tile, 14 x 30 x 1 cells without a z halo or z
-// sweep, for grids one z cell thick whose z boundaries are periodic or
-// outflow (the cell's two z faces then carry the same flux), with at most
-// one dust species: the cylindrical explosion of Sect. 4.1 runs on it.
-constexpr int FLAT_TT = 30, FLAT_NT = 160;
+// Tiles of the double stage kernels (both forms), with threads per block and
+// blocks per SM.  TILE_MAIN wastes the fewest lanes on halos (1.27 of the
+// cells); the thinner ones spread a small grid over the SMs; the flat ones,
+// without a z halo or z sweep, are for full-state grids one z cell thick whose z
+// boundaries are periodic or outflow (the cell's two z faces then carry the same
+// flux): the cylindrical explosion of Sect. 4.1.
+template <int R, int T, int Z, int N, int B>
+struct Tile {
+  static constexpr int TR = R, TT = T, TZ = Z, NT = N, MINB = B;
+};
+using TileMain = Tile<14, 6, 6, 192, 2>;
+using TileMid = Tile<6, 6, 2, 128, 4>;
+using TileSmall = Tile<6, 2, 2, 128, 4>;
+using TileFlat = Tile<14, 30, 1, 160, 3>;
+using TileFlatSmall = Tile<14, 6, 1, 128, 4>;
+enum { TILE_MAIN = 0, TILE_MID = 1, TILE_SMALL = 2, TILE_FLAT = 3, TILE_FLAT_SMALL = 4 };
+
+// Calls f(Tile{}) for tile number t.
+template <class F>
+auto by_tile(int t, F&& f) {
+  switch (t) {
+    case TILE_MID: return f(TileMid{});
+    case TILE_SMALL: return f(TileSmall{});
+    case TILE_FLAT: return f(TileFlat{});
+    case TILE_FLAT_SMALL: return f(TileFlatSmall{});
+    default: return f(TileMain{});
+  }
+}
+
+// The tile of a double grid: the one with the least work on the busiest SM,
+// in 32-lane chunks of its sweeps (60 for a main tile, whose sweeps have 18, 21
+// and 21), as the FP64 pipe, which bounds these kernels, takes chunks at one
+// rate.  Grids of some thousand main tiles keep the main tile; at 19 main
+// tiles (the Sod tube, 256 x 4 x 4) 15 % of the SMs had all the work: 240 us per
+// step against 30 with the small tile.  More than one dust species: the main
+// tile only (the others are not instantiated).
+template <class T>
+constexpr long tile_chunks() {
+  auto sweep = [](int lines, int cells) { return (long)(lines * pow2ceil(cells + 2) + 31) / 32; };
+  return sweep(T::TT * T::TZ, T::TR) + sweep(T::TR * T::TZ, T::TT) + (T::TZ > 1 ? sweep(T::TR * T::TT, T::TZ) : 0);
+}
+inline int choose_tile(int nr, int nth, int nz, bool flat, int nf, int sms) {
+  if (nf > 9) return TILE_MAIN;
+  const int from = flat ? TILE_FLAT : TILE_MAIN, to = flat ? TILE_FLAT_SMALL : TILE_SMALL;
+  int best = from;
+  long least = 0;
+  for (int t = from; t <= to; ++t) {
+    const long work = by_tile(t, [&](auto tile) {
+      using T = decltype(tile);
+      const long n = (long)((nr + T::TR - 1) / T::TR) * ((nth + T::TT - 1) / T::TT) * ((nz + T::TZ - 1) / T::TZ);
+      return (n + sms - 1) / sms * tile_chunks<T>();
+    });
+    if (t == from || work < least) {
+      best = t;
+      least = work;
+    }
+  }
+  return best;
+}
 inline bool flat_grid(int nz, int bc_lo_z, int bc_hi_z, int nf) {
   return nz == 1 && bc_lo_z != BC_EQUILIBRIUM && bc_hi_z != BC_EQUILIBRIUM && nf <= 9;
 }

@@ -55,6 +55,7 @@ struct rossbi_grid {
   void* d_hoststate = nullptr;         // device copy for rossbi_step_host
   int tiles_r = 0, tiles_t = 0, tiles_z = 0;
   int tile_tt = 6;                     // theta extent of a stage-kernel tile
+  int tile = TILE_MAIN;                // double forms: which tile
   // perturbation forms: equilibrium and metric tables in the state precision
   void* d_ptab = nullptr;              // one allocation holding every table below
   PertTables<float> pt_f{};
@@ -469,6 +470,7 @@ StageArgs base_args(rossbi_grid* g) {
   a.status = g->d_status;
   a.tiles_r = g->tiles_r;
   a.tiles_z = g->tiles_z;
+  a.tile = g->tile;
   return a;
 }
 
@@ -654,6 +656,7 @@ PertArgs<T> pert_args(rossbi_grid* g) {
   a.tiles_r = g->tiles_r;
   a.tiles_z = g->tiles_z;
   a.sms = g->sms;
+  a.tile = g->tile;
   a.gam = (T)g->dg.gamma;
   a.om = (T)g->dg.omega;
   a.cfl = (T)g->dg.cfl;
@@ -1214,14 +1217,24 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   }
   g->nf = 5 + 4 * desc->n_dust;
   g->ncell = (size_t)desc->nr * desc->nth * desc->nz;
-  const bool pert = desc->precision != ROSSBI_FP64;  // tile of the form's stage kernel
-  const bool flat = !pert && flat_grid(desc->nz, desc->bc_lo[2], desc->bc_hi[2], g->nf);
-  const int tr = pert ? P32_TR : F64_TR, tt = pert ? P32_TT : (flat ? FLAT_TT : F64_TT);
-  const int tz = flat ? 1 : tile_z(desc->precision == ROSSBI_FP64_PERT, g->nf);
-  g->tile_tt = tt;
-  g->tiles_r = (desc->nr + tr - 1) / tr;
-  g->tiles_t = (desc->nth + tt - 1) / tt;
-  g->tiles_z = (desc->nz + tz - 1) / tz;
+  // the tile of the form's stage kernel
+  auto set_tiles = [&](int tr, int tt, int tz) {
+    g->tile_tt = tt;
+    g->tiles_r = (desc->nr + tr - 1) / tr;
+    g->tiles_t = (desc->nth + tt - 1) / tt;
+    g->tiles_z = (desc->nz + tz - 1) / tz;
+  };
+  if (desc->precision == ROSSBI_FP32_PERT) {
+    set_tiles(P32_TR, P32_TT, P32_TZ);
+  } else {
+    const bool flat = desc->precision == ROSSBI_FP64 && flat_grid(desc->nz, desc->bc_lo[2], desc->bc_hi[2], g->nf);
+    g->tile = choose_tile(desc->nr, desc->nth, desc->nz, flat, g->nf, g->sms);
+    by_tile(g->tile, [&](auto t) {
+      using T = decltype(t);
+      set_tiles(T::TR, T::TT, T::TZ);
+      return 0;
+    });
+  }
   const rossbi_grid_desc& d = *desc;
   const int nr = d.nr;
   const double dy = (d.x1[1] - d.x0[1]) / d.nth;

@@ -21,6 +21,7 @@ namespace rossbi {
 
 struct StageArgs {
   DevGrid g;
+  int tile;                    // TILE_*, chosen by the host
   const double* in[NF_MAX];    // stage input (stencil) state
   const double* base[NF_MAX];  // E^n, base of the update
   double* out[NF_MAX];         // updated state
@@ -279,11 +280,10 @@ __device__ __forceinline__ void sweep_gas(const StageArgs& a, const double* sE, 
 // The sweep of one dust species along axis D: sE holds its staged primitives
 // (u, v, w, rho_d), sG its accumulators.
 template <int TR, int TT, int TZ, int NT, int D>
-__device__ __forceinline__ void sweep_dust(const StageArgs& a, const double* sE, double* sG, int i0, int j0, int k0) {
+__device__ __forceinline__ void sweep_dust(const DevGrid& g, const double* sE, double* sG, int i0, int j0, int k0) {
   using S = SweepLane<TR, TT, TZ, D>;
   constexpr int L = S::L;
   constexpr unsigned FULL = 0xffffffffu;
-  const DevGrid& g = a.g;
   for (int base = threadIdx.x & ~31; base < S::ITEMS; base += NT) {
     const S s(g, base + (threadIdx.x & 31), i0, j0, k0);
     if (!__any_sync(FULL, s.do_face)) continue;
@@ -303,17 +303,57 @@ __device__ __forceinline__ void sweep_dust(const StageArgs& a, const double* sE,
   }
 }
 
-template <int NT>
-__device__ __forceinline__ double block_min(double v, double* red) {
+// Every dust species of a tile through the gas's staging buffer sE, as
+// primitives (u, v, w, rho_d) converted once per staged cell, into its
+// accumulators in sG; `stage` walks the box (put(idx, cell or null)).  One
+// species at a time keeps a nine-field block at 108 KB, two blocks to an SM,
+// whose barriers and staging overlap (all fields staged at once: 166 KB, one
+// block of six warps, FP64 pipe 75 % busy), and lets every species count have
+// the 14 x 6 x 6 tile.
+template <int NF, int TR, int TT, int TZ, int NT, class Stage>
+__device__ __forceinline__ void dust_species(const DevGrid& g, const double* const* in, double* sE, double* sG,
+                                             Stage& stage, int i0, int j0, int k0) {
+  constexpr int BOX = SweepLane<TR, TT, TZ, 0>::BOX, NCORE = TR * TT * TZ;
+#pragma unroll 1
+  for (int b = 5; b < NF; b += 4) {
+    stage([&](int idx, const int* c) {
+      if (!c) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  double m = red[0];
-  for (int q = 1; q < NT / 32; ++q) m = fmin(m, red[q]);
-  __syncthreads();
-  return m;
+        for (int f = 0; f < 4; ++f) sE[f * BOX + idx] = 0.0;
+        return;
+      }
+      const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
+      const double rd = in[b + 3][lin], id = positive(rd) ? recip(rd) : 0.0;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) sE[q * BOX + idx] = in[b + q][lin] * id;
+      sE[3 * BOX + idx] = rd;
+    });
+    __syncthreads();
+    double* sD = sG + b * NCORE;
+    sweep_dust<TR, TT, TZ, NT, 0>(g, sE, sD, i0, j0, k0);
+    __syncthreads();
+    sweep_dust<TR, TT, TZ, NT, 1>(g, sE, sD, i0, j0, k0);
+    __syncthreads();
+    if constexpr (TZ > 1) {
+      sweep_dust<TR, TT, TZ, NT, 2>(g, sE, sD, i0, j0, k0);
+      __syncthreads();
+    }
+  }
+}
+
+// Walks the staged box of a tile: put(idx, cell or null) for every cell that
+// a sweep reads (tile and halo without edges and corners), null for an
+// equilibrium ghost.
+template <int TR, int TT, int TZ, int NT, class F>
+__device__ __forceinline__ void walk_box(const DevGrid& g, int i0, int j0, int k0, F&& put) {
+  constexpr int ZH = TZ == 1 ? 0 : 2, BX = TR + 4, BY = TT + 4, BOX = BX * BY * (TZ + 2 * ZH);
+  for (int idx = threadIdx.x; idx < BOX; idx += NT) {
+    const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - ZH;
+    const int outside = (x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ);
+    if (outside > 1) continue;
+    int c[3] = {i0 + x, j0 + y, k0 + z};
+    put(idx, resolve_cell(g, c) ? c : nullptr);
+  }
 }
 
 // Fixed-order block sum (deterministic for a fixed launch shape).
@@ -383,17 +423,7 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
   publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, g.cfl);
   if (!a.stage2) clear_rate(a.rate_out);
 
-  // tile + halo (edges and corners are never read): put(idx, cell or null)
-  // for every staged cell, null for an equilibrium ghost
-  auto stage = [&](auto&& put) {
-    for (int idx = threadIdx.x; idx < BOX; idx += NT) {
-      const int x = idx % BX - 2, y = (idx / BX) % BY - 2, z = idx / (BX * BY) - ZH;
-      const int outside = (x < 0 || x >= TR) + (y < 0 || y >= TT) + (z < 0 || z >= TZ);
-      if (outside > 1) continue;
-      int c[3] = {i0 + x, j0 + y, k0 + z};
-      put(idx, resolve_cell(g, c) ? c : nullptr);
-    }
-  };
+  auto stage = [&](auto&& put) { walk_box<TR, TT, TZ, NT>(g, i0, j0, k0, put); };
   // the gas as deviations E' = E - E0 (or, with RC = RECON_PRIM, the primitive
   // departures u', v', w', P', rho') in slots 0..4
   stage([&](int idx, const int* c) {
@@ -425,36 +455,7 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
     sweep_gas<TR, TT, TZ, NT, 2, RC>(a, sE, sG, i0, j0, k0, status);
     __syncthreads();
   }
-  // then each dust species through the same buffer, as primitives (u, v, w,
-  // rho_d) converted once per staged cell.  One species at a time keeps a
-  // nine-field block at 108 KB, two blocks to an SM, whose barriers and staging
-  // overlap (all fields staged at once: 166 KB, one block of six warps, FP64
-  // pipe 75 % busy), and lets every species count have the 14 x 6 x 6 tile.
-#pragma unroll 1
-  for (int b = 5; b < NF; b += 4) {
-    stage([&](int idx, const int* c) {
-      if (!c) {
-#pragma unroll
-        for (int f = 0; f < 4; ++f) sE[f * BOX + idx] = 0.0;
-        return;
-      }
-      const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
-      const double rd = a.in[b + 3][lin], id = positive(rd) ? recip(rd) : 0.0;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) sE[q * BOX + idx] = a.in[b + q][lin] * id;
-      sE[3 * BOX + idx] = rd;
-    });
-    __syncthreads();
-    double* sD = sG + b * NCORE;
-    sweep_dust<TR, TT, TZ, NT, 0>(a, sE, sD, i0, j0, k0);
-    __syncthreads();
-    sweep_dust<TR, TT, TZ, NT, 1>(a, sE, sD, i0, j0, k0);
-    __syncthreads();
-    if constexpr (TZ > 1) {
-      sweep_dust<TR, TT, TZ, NT, 2>(a, sE, sD, i0, j0, k0);
-      __syncthreads();
-    }
-  }
+  dust_species<NF, TR, TT, TZ, NT>(g, a.in, sE, sG, stage, i0, j0, k0);
 
   const double tau = s_tau;
   const size_t ncell = (size_t)g.nr * g.nth * g.nz;

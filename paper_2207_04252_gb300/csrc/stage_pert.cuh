@@ -1,4 +1,5 @@
-// Fused RK2 stage kernel of the perturbation forms (state E' = E - E0).
+// The physics of the perturbation forms (state E' = E - E0) and the RK2 stage
+// kernel of the double one (the float one has stage_f32.cuh).
 //
 // Same tiling and sweeps as the FP64 full-state kernel, but every quantity is
 // formed as an exact algebraic difference from the equilibrium state E0
@@ -50,23 +51,6 @@ struct PertTables {
   const T* omk;    // Omega_K at the cell-centre radius (constant-St drag)
   unsigned long long* fallbacks;  // count of FP64 fallback Riemann faces
 };
-
-// One state element global -> shared by an asynchronous copy (cp.async with
-// the L1-allocating .ca policy: the halo cells are read again by the
-// neighbouring tiles), and the wait for all of a thread's copies.
-template <class T>
-__device__ __forceinline__ void cp_async_elem(T* smem, const T* gmem) {
-  static_assert(sizeof(T) == 4 || sizeof(T) == 8, "4- or 8-byte elements");
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  if constexpr (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-}
 
 template <class T> struct Math;
 template <> struct Math<float> {
@@ -435,6 +419,7 @@ struct PertArgs {
   unsigned* status;
   int tiles_r, tiles_z;  // tile counts along r and z (tile number: r fastest, then z, then theta)
   int sms;               // SMs of the device
+  int tile;              // double form: TILE_*, chosen by the host
   // the grid's and the drag's parameters in the state precision, converted
   // once on the host (GB300's FP64 pipe is narrow: per-use conversions of the
   // double originals cost latency in the float kernel)
@@ -508,32 +493,28 @@ __device__ __forceinline__ void pert_face(const PertArgs<T>& a, const PEq<T>& Em
   if (ok) pert_flux<T, D>(a.g_gm1, area, Em, drho, d, dp, F);
 }
 
-// One 32-lane chunk of the sweep along axis D: items base .. base + 31 (whole
-// lines of L lanes).  sE holds the gas departures (conservative, or primitive
-// with RC = RECON_PRIM) and the dust primitives.  The flux divergence of the
-// chunk's cells is written to sG (ACC: added to it).
-template <class T, int NF, int TR, int TT, int TZ, int D, class P, int RC, bool ACC>
-__device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* sE, T* sG, int i0, int j0, int k0,
-                                                 int base, unsigned& status, unsigned& nfallback) {
+// The gas sweep along axis D of the double form: sE holds the staged gas
+// departures (conservative, or primitive with RC = RECON_PRIM).
+template <int TR, int TT, int TZ, int NT, int D, class P, int RC>
+__device__ __forceinline__ void sweep_pert_gas(const PertArgs<double>& a, const double* sE, double* sG, int i0, int j0,
+                                               int k0, unsigned& status, unsigned& nfallback) {
   using S = SweepLane<TR, TT, TZ, D>;
-  constexpr int BOX = S::BOX, NCORE = S::NCORE, L = S::L, STRIDE = S::STRIDE;
+  constexpr int BOX = S::BOX, L = S::L, STRIDE = S::STRIDE;
   constexpr unsigned FULL = 0xffffffffu;
   constexpr bool UNI = D != 0;
   const DevGrid& g = a.g;
-  const S s(g, base + (threadIdx.x & 31), i0, j0, k0);
-  if (!__any_sync(FULL, s.do_face)) return;  // a warp of lines beyond a ragged grid's edge
-  T w[RCW];
-  parabola_weights<T, D>(a.t.rcoef, s.gi, g.nr, w);
-  const int ci = clampi(s.gi, 0, g.nr - 1), ck = clampi(s.gk, 0, g.nz - 1);
-  T area = T(0);
-  if (s.do_face) area = D == 0 ? a.t.area_r[s.gi] : (D == 1 ? a.t.area_t[ci] : a.t.area_z[ci]);
-  {
+  for (int base = threadIdx.x & ~31; base < S::ITEMS; base += NT) {
+    const S s(g, base + (threadIdx.x & 31), i0, j0, k0);
+    if (!__any_sync(FULL, s.do_face)) continue;  // a warp of lines beyond a ragged grid's edge
+    double w[RCW];
+    parabola_weights<double, D>(g.rcoef, s.gi, g.nr, w);
+    const int ci = clampi(s.gi, 0, g.nr - 1), ck = clampi(s.gk, 0, g.nz - 1);
     // the equilibrium of this cell's lower and upper face (clamped; one face
     // for a theta line, whose cells share the radius and height)
-    PEq<T> Em{T(0), T(0), T(0), T(0)}, Ep{T(0), T(0), T(0), T(0)};
+    PEq<double> Em{0.0, 0.0, 0.0, 0.0}, Ep{0.0, 0.0, 0.0, 0.0};
     int of = 0;
     if (g.has_eq) {
-      const T* f = a.t.face[D];
+      const double* f = a.t.face[D];
       if (D == 0) {
         of = ck * (g.nr + 1) + clampi(s.gd, 0, g.nr);
         Em = load_eq(f + 4 * (size_t)of);
@@ -547,12 +528,12 @@ __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* 
         Ep = load_eq(f + 4 * (size_t)(clampi(s.gd + 1, 0, g.nz) * g.nr + ci));
       }
     }
-    T wm[5], wp[5];  // primitive perturbations: right state of the lower face, left state of the upper face
+    double wm[5], wp[5];  // primitive perturbations: right state of the lower face, left state of the upper face
     {
-      T qm[5], qp[5];
+      double qm[5], qp[5];
 #pragma unroll
       for (int f = 0; f < 5; ++f) {
-        const T* e = sE + f * BOX + s.sidx;
+        const double* e = sE + f * BOX + s.sidx;
         parabola<UNI>(e[-STRIDE], e[0], e[STRIDE], w, qm[f], qp[f]);
       }
       auto face_states = [&]() {
@@ -575,58 +556,17 @@ __device__ __forceinline__ void sweep_pert_chunk(const PertArgs<T>& a, const T* 
         face_states();
       }
     }
-    T F[5], wl[5];
+    double F[5], wl[5];
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
       wl[f] = __shfl_up_sync(FULL, wp[f], 1, L);  // upper face state of the lower neighbour
-      F[f] = T(0);
+      F[f] = 0.0;
     }
-    if (s.do_face) pert_face<T, D, P>(a, Em, area, wl, wm, [&]() { return of; }, F, status, nfallback);
+    if (s.do_face)
+      pert_face<double, D, P>(a, Em, face_area<D>(g, s.gi, ci), wl, wm, [&]() { return of; }, F, status, nfallback);
 #pragma unroll
-    for (int f = 0; f < 5; ++f) {
-      const T Fu = __shfl_down_sync(FULL, F[f], 1, L);
-      if (s.do_acc) {
-        T* dst = sG + f * NCORE + s.core;
-        if (ACC) *dst += F[f] - Fu;
-        else *dst = F[f] - Fu;
-      }
-    }
+    for (int f = 0; f < 5; ++f) accumulate<D, L>(F[f], sG + f * S::NCORE + s.core, s.do_acc);
   }
-#pragma unroll 1
-  for (int b = 5; b < NF; b += 4) {  // each dust species: primitive reconstruction, kinetic flux
-    T qm[4], qp[4], F[4], WL[4];
-    dust_recon<T, BOX, STRIDE, UNI>(sE, s.sidx, b, w, qm, qp);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
-      F[f] = T(0);
-    }
-    if (s.do_face) dust_kinetic_flux<D>(area, WL, qm, F);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      const T Fu = __shfl_down_sync(FULL, F[f], 1, L);
-      if (s.do_acc) {
-        T* dst = sG + (b + f) * NCORE + s.core;
-        if (ACC) *dst += F[f] - Fu;
-        else *dst = F[f] - Fu;
-      }
-    }
-  }
-}
-
-// The whole sweep along axis D, chunks spread over the block's warps.
-template <class T, int NF, int TR, int TT, int TZ, int NT, int D, class P, int RC, bool ACC>
-__device__ __forceinline__ void sweep_pert(const PertArgs<T>& a, const T* sE, T* sG, int i0, int j0, int k0,
-                                           unsigned& status, unsigned& nfallback) {
-  for (int base = threadIdx.x & ~31; base < SweepLane<TR, TT, TZ, D>::ITEMS; base += NT)
-    sweep_pert_chunk<T, NF, TR, TT, TZ, D, P, RC, ACC>(a, sE, sG, i0, j0, k0, base, status, nfallback);
-}
-
-// Dynamic shared memory of stage_pert_kernel: the staged tile and halo, and
-// the accumulator of the flux divergence.
-template <class T, int NF, int TR, int TT, int TZ>
-__host__ __device__ constexpr size_t pert_smem_bytes() {
-  return (size_t)NF * ((TR + 4) * (TT + 4) * (TZ + 4) + TR * TT * TZ) * sizeof(T);
 }
 
 // Cell-centre equilibrium coefficients.
@@ -864,137 +804,72 @@ __device__ __forceinline__ void pert_update(const PertArgs<T>& a, int gi, int gj
   if (bad) status |= STATUS_NONPHYSICAL;
 }
 
-// The box of a TR x TT x TZ tile: staging and the per-cell epilogue.
-template <class T, int NF, int TR, int TT, int TZ, int NT, int RC>
-struct PertTile {
-  static constexpr int BX = TR + 4, BY = TT + 4, BZ = TZ + 4, PLANE = BX * BY, BOX = PLANE * BZ, NCORE = TR * TT * TZ;
-  // Each thread owns one (r, theta) position of the box and walks its z planes
-  // (half of them where the block has two threads per position), so that an
-  // index costs one addition (a division into three indices for each of the
-  // box's 1,800 cells made staging a sixth of the kernel's instructions).
-  static constexpr int HALVES = NT >= 2 * PLANE ? 2 : 1;
-  static_assert(PLANE <= NT && BZ % 2 == 0, "a thread per (r, theta) position of the box");
-  int i0, j0, k0;
-
-  __device__ __forceinline__ PertTile(const PertArgs<T>& a, int tile) {
-    // r fastest, then z, then theta: the tiles whose halos a tile re-reads
-    // (its r, z and theta neighbours) run at most tiles_r x tiles_z blocks
-    // apart, so the re-reads hit in L2
-    i0 = (tile % a.tiles_r) * TR;
-    k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
-    j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
-  }
-
-  // walk(position, z plane, cell indices ci, cj, ck, inside) over this thread's cells
-  template <class F>
-  __device__ __forceinline__ void walk(const DevGrid& g, F&& put) const {
-    if (threadIdx.x >= HALVES * PLANE) return;
-    const int half = HALVES == 2 && threadIdx.x >= PLANE ? 1 : 0, pos = (int)threadIdx.x - half * PLANE;
-    const int x = pos % BX - 2, y = pos / BX - 2;
-    const bool side = x < 0 || x >= TR, end = y < 0 || y >= TT;
-    if (side && end) return;  // no sweep reads the box's edges and corners
-    int ci = i0 + x, cj = j0 + y;
-    const bool in = resolve_axis(g, 0, ci) && resolve_axis(g, 1, cj);
-    int z0 = side || end ? 2 : 0, z1 = side || end ? TZ + 2 : BZ;
-    if (HALVES == 2) {
-      if (half) z0 = BZ / 2;
-      else z1 = BZ / 2;
-    }
-#pragma unroll 2
-    for (int z = z0; z < z1; ++z) {
-      int ck = k0 + z - 2;
-      const bool inside = resolve_axis(g, 2, ck) && in;
-      put(z * PLANE + pos, ci, cj, ck, inside);
-    }
-  }
-
-  // The fields global -> shared by asynchronous copies (cp.async, no
-  // registers), all of a thread's cells in flight at once; equilibrium ghosts
-  // are zero departures.
-  __device__ __forceinline__ void copy(const PertArgs<T>& a, T* sE) const {
-    walk(a.g, [&](int idx, int ci, int cj, int ck, bool inside) {
-      T* dst = sE + idx;
-      if (inside) {
-        const size_t lin = ((size_t)ck * a.g.nth + cj) * a.g.nr + ci;
-#pragma unroll
-        for (int f = 0; f < NF; ++f) cp_async_elem<T>(dst + f * BOX, a.in[f] + lin);
-      } else {
-#pragma unroll
-        for (int f = 0; f < NF; ++f) dst[f * BOX] = T(0);
-      }
-    });
-  }
-
-  // Waits for this thread's copies and converts the cells it copied: the dust
-  // to primitives (u, v, w, rho_d), which every reconstruction of the three
-  // sweeps reads, and with RC = RECON_PRIM the gas to primitive departures.
-  __device__ __forceinline__ void convert(const PertArgs<T>& a, T* sE) const {
-    cp_async_wait_all();
-    if (NF == 5 && RC != RECON_PRIM) return;
-    walk(a.g, [&](int idx, int ci, int, int ck, bool inside) {
-      T* e = sE + idx;
-      if (RC == RECON_PRIM && inside) {
-        const PEq<T> eq = a.g.has_eq ? load_eq(a.t.cen + 8 * ((size_t)ck * a.g.nr + ci)) : PEq<T>{};
-        T q[5], w[5];
-#pragma unroll
-        for (int f = 0; f < 5; ++f) q[f] = e[f * BOX];
-        face_prim(a.gm1, eq.rho, eq.v, q, w);
-#pragma unroll
-        for (int f = 0; f < 4; ++f) e[f * BOX] = w[f];
-      }
-#pragma unroll
-      for (int b = 5; b < NF; b += 4) {
-        const T rd = e[(b + 3) * BOX], id = positive(rd) ? recip(rd) : T(0);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) e[(b + q) * BOX] *= id;
-      }
-    });
-  }
-
-  // The update of core cell cidx from the staged fields and accumulators.
-  template <bool XT>
-  __device__ __forceinline__ void update(const PertArgs<T>& a, const T* sE, const T* sG, int cidx, T tau, T& rate,
-                                         unsigned& status) const {
-    const int x = cidx % TR, y = (cidx / TR) % TT, z = cidx / (TR * TT);
-    const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
-    if (gi >= a.g.nr || gj >= a.g.nth || gk >= a.g.nz) return;
-    const int sidx = (z + 2) * PLANE + (y + 2) * BX + (x + 2);
-    T e[5], dust[NF > 5 ? (NF - 5) / 4 : 1][4], G[NF];
-#pragma unroll
-    for (int f = 0; f < 5; ++f) e[f] = sE[f * BOX + sidx];
-#pragma unroll
-    for (int f = 5; f < NF; ++f) dust[(f - 5) / 4][(f - 5) % 4] = sE[f * BOX + sidx];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) G[f] = sG[f * NCORE + cidx];
-    pert_update<T, NF, RC, XT>(a, gi, gj, gk, e, dust, G, tau, rate, status);
-  }
-};
-
-// One RK stage of one tile per block.
-template <class T, int NF, int TR, int TT, int TZ, int NT, int MINB, class P, bool XT, int RC>
-__global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<T> a) {
-  using Tile = PertTile<T, NF, TR, TT, TZ, NT, RC>;
-  constexpr int NCORE = Tile::NCORE;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sE = reinterpret_cast<T*>(smem_raw);
-  T* sG = sE + NF * Tile::BOX;
-  const Tile t(a, blockIdx.x);
+// One RK stage of one tile per block (double form).
+template <int NF, int TR, int TT, int TZ, int NT, int MINB, class P, bool XT, int RC>
+__global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<double> a) {
+  using S = SweepLane<TR, TT, TZ, 0>;
+  constexpr int BOX = S::BOX, NCORE = S::NCORE, ND = NF > 5 ? (NF - 5) / 4 : 1;
+  extern __shared__ double smem[];
+  double* sE = smem;             // [5][BOX] the gas departures, then the four primitives of one dust species at a time
+  double* sG = smem + 5 * BOX;   // [NF][NCORE] flux divergence
+  const DevGrid& g = a.g;
+  // tiles r fastest, then z, then theta, as in the full-state kernel
+  const int tile = blockIdx.x;
+  const int i0 = (tile % a.tiles_r) * TR;
+  const int k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
+  const int j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
   unsigned status = 0, nfallback = 0;
   __shared__ double s_tau;
-  publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, a.g.cfl);
+  publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, g.cfl);
   if (!a.stage2) clear_rate(a.rate_out);
-  t.copy(a, sE);
-  t.convert(a, sE);
+  auto stage = [&](auto&& put) { walk_box<TR, TT, TZ, NT>(g, i0, j0, k0, put); };
+  stage([&](int idx, const int* c) {
+    double q[5], w[5];
+    if (!c) {
+#pragma unroll
+      for (int f = 0; f < 5; ++f) sE[f * BOX + idx] = 0.0;
+      return;
+    }
+    const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) q[f] = a.in[f][lin];
+    if (RC == RECON_PRIM) {
+      const PEq<double> eq = g.has_eq ? load_eq(a.t.cen + 8 * ((size_t)c[2] * g.nr + c[0])) : PEq<double>{};
+      face_prim(a.gm1, eq.rho, eq.v, q, w);
+    }
+#pragma unroll
+    for (int f = 0; f < 5; ++f) sE[f * BOX + idx] = RC == RECON_PRIM ? w[f] : q[f];
+  });
   __syncthreads();
-  sweep_pert<T, NF, TR, TT, TZ, NT, 0, P, RC, false>(a, sE, sG, t.i0, t.j0, t.k0, status, nfallback);
+  sweep_pert_gas<TR, TT, TZ, NT, 0, P, RC>(a, sE, sG, i0, j0, k0, status, nfallback);
   __syncthreads();
-  sweep_pert<T, NF, TR, TT, TZ, NT, 1, P, RC, true>(a, sE, sG, t.i0, t.j0, t.k0, status, nfallback);
+  sweep_pert_gas<TR, TT, TZ, NT, 1, P, RC>(a, sE, sG, i0, j0, k0, status, nfallback);
   __syncthreads();
-  sweep_pert<T, NF, TR, TT, TZ, NT, 2, P, RC, true>(a, sE, sG, t.i0, t.j0, t.k0, status, nfallback);
+  sweep_pert_gas<TR, TT, TZ, NT, 2, P, RC>(a, sE, sG, i0, j0, k0, status, nfallback);
   __syncthreads();
-  T rate = T(0);
-  for (int cidx = threadIdx.x; cidx < NCORE; cidx += NT)
-    t.template update<XT>(a, sE, sG, cidx, (T)s_tau, rate, status);
+  dust_species<NF, TR, TT, TZ, NT>(g, a.in, sE, sG, stage, i0, j0, k0);
+  double rate = 0.0;
+  for (int cidx = threadIdx.x; cidx < NCORE; cidx += NT) {
+    const int x = cidx % TR, y = (cidx / TR) % TT, z = cidx / (TR * TT);
+    const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
+    if (gi >= g.nr || gj >= g.nth || gk >= g.nz) continue;
+    const size_t lin = ((size_t)gk * g.nth + gj) * g.nr + gi;
+    double e[5], dust[ND][4], G[NF];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) e[f] = a.in[f][lin];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) G[f] = sG[f * NCORE + cidx];
+#pragma unroll
+    for (int b = 5; b < NF; b += 4) {
+      double* d = dust[(b - 5) / 4];
+      d[3] = a.in[b + 3][lin];
+      const double id = positive(d[3]) ? recip(d[3]) : 0.0;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) d[q] = a.in[b + q][lin] * id;
+    }
+    // e is the state as it is stored, whatever the sweeps reconstructed from
+    pert_update<double, NF, RECON_CONS, XT>(a, gi, gj, gk, e, dust, G, s_tau, rate, status);
+  }
   if (a.stage2) raise_rate(a.rate_out, rate);
   if (status) atomicOr(a.status, status);
   if (nfallback) atomicAdd(a.t.fallbacks, (unsigned long long)nfallback);
