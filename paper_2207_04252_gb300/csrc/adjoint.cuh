@@ -363,7 +363,7 @@ __device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL
   const FluxCot F{Fb[RHO], Fb[n], Fb[t1], Fb[t2], Fb[EN]};
   const double dP = pr - pl;
   NearStar<double> s;
-  const int kind = near_riemann<double>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, narrow(WL[n]),
+  const int kind = near_riemann<true>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, narrow(WL[n]),
                                         narrow(WR[n]), s);
   if (kind == NEAR_GENERAL) {
     const RFaceVjp o = riemann_vjp_general(C.gamma, rl, WL[n], pl, WL[t1], WL[t2], rr, WR[n], pr, WR[t1], WR[t2], F);

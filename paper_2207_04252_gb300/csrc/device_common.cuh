@@ -429,7 +429,7 @@ __device__ __forceinline__ void gas_face_flux(const NearCoef& C, double area, co
     return;
   }
   NearStar<double> s;
-  const int kind = near_riemann<double>(C, WL[RHO], WL[n], WL[EN], WR[RHO], WR[n], WR[EN], WR[EN] - WL[EN],
+  const int kind = near_riemann(C, WL[RHO], WL[n], WL[EN], WR[RHO], WR[n], WR[EN], WR[EN] - WL[EN],
                                         WR[n] - WL[n], 0.0, false, narrow(WL[n]), narrow(WR[n]), s);
   const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
   double rho = left ? WL[RHO] : WR[RHO], u = left ? WL[n] : WR[n], p = left ? WL[EN] : WR[EN];
@@ -465,6 +465,22 @@ __device__ __forceinline__ void gas_face_flux(const NearCoef& C, double area, co
 template <int D, class T>
 __device__ __forceinline__ void dust_kinetic_flux(T area, const T* WL, const T* WR, T* F) {
   constexpr int n = Axes<D>::n, t1 = Axes<D>::t1, t2 = Axes<D>::t2;  // 0..2 in the dust block
+  if constexpr (sizeof(T) == 8) {
+    // one of the two parts is zero unless the streams collide (u_L > 0 > u_R):
+    // five FP64 operations for the upwind side instead of eleven for both
+    const bool fromL = positive(WL[n]);
+    const T rho = fromL ? WL[3] : WR[3], un = fromL ? WL[n] : neg_part(WR[n]);
+    F[3] = area * (rho * un);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) F[q] = F[3] * (fromL ? WL[q] : WR[q]);
+    if (fromL && sign_bit(WR[n])) {
+      const T mr = area * (WR[3] * WR[n]);
+      F[3] += mr;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) F[q] = fma(mr, WR[q], F[q]);
+    }
+    return;
+  }
   const T ml = area * (WL[3] * pos_part(WL[n]));
   const T mr = area * (WR[3] * neg_part(WR[n]));
   F[3] = ml + mr;

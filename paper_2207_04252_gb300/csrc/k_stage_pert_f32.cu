@@ -26,9 +26,9 @@ cudaError_t launch_nt(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Two blocks of 8 warps share an SM where their shared memory allows it (up to
-// nine fields) and there are tiles for them; otherwise one block of 16 warps
-// takes the SM: more fields (120 KB and up), or a grid of at most one tile per
+// Two blocks of 12 warps share an SM where their shared memory allows it (up to
+// nine fields) and there are tiles for them; otherwise one block
+// takes the SM, of 24 warps: more fields (133 KB and up), or a grid of at most one tile per
 // SM (32 x 48 x 32: 207 -> 153 us for four steps).
 template <int NF, class P, bool XT, int RC>
 cudaError_t launch(const PertArgs<float>& a, int nblocks, cudaStream_t s) {

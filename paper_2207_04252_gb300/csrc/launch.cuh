@@ -13,7 +13,7 @@
 namespace rossbi {
 
 // Tiles of the float stage kernel: 14 x 6 x 6 cells, lines of 16 / 8 / 8 lanes.
-constexpr int P32_TR = 14, P32_TT = 6, P32_TZ = 6, P32_NT = 256, P32_MINB = 2, P32_WIDE_NT = 512;
+constexpr int P32_TR = 14, P32_TT = 6, P32_TZ = 6, P32_NT = 384, P32_MINB = 2, P32_WIDE_NT = 768;
 
 // Tiles of the double stage kernels (both forms), with threads per block and
 // blocks per SM.  TILE_MAIN wastes the fewest lanes on halos (1.27 of the

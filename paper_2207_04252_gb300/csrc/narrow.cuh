@@ -109,6 +109,11 @@ __device__ __forceinline__ float recip_sqrt(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// One Newton step of 1/x and x^-1/2 from y (error squared: 2^-22 -> 2^-43).
+__device__ __forceinline__ double refine_recip(double x, double y) { return fma(y, fma(-x, y, 1.0), y); }
+__device__ __forceinline__ double refine_recip_sqrt(double x, double y) {
+  return fma(scale_down<1>(y), fma(-(x * y), y, 1.0), y);
+}
 // sqrt(x), x > 0
 __device__ __forceinline__ double root(double x) {
   double y;
@@ -118,4 +123,30 @@ __device__ __forceinline__ double root(double x) {
 }
 __device__ __forceinline__ float root(float x) { return x * recip_sqrt(x); }
 
+// ---------------------------------------------------------------- two floats at a time (the packed arithmetic of sm_100 and later)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack2(-1.0f, -1.0f), a); }
 }  // namespace rossbi

@@ -27,6 +27,8 @@
 // 55 operations here against 250 to 300 of the FP64 Newton iteration with its
 // two branches; in float the issue slots.
 #pragma once
+#include <cstring>
+
 #include "narrow.cuh"
 
 namespace rossbi {
@@ -42,7 +44,7 @@ struct NearCoef {
   double t[2][NEAR_N], h[2][NEAR_N];   // (x S)' and (x D)', for the adjoint
   float tt[2][NEAR_T], ht[2][NEAR_T];
   float sf[2][5], tf[2][5], df[2][4];  // S, T, D in float
-  float t2m;                           // mean of the branches' T_2
+  f32x2 g2, t22, t12, s12;             // twice gamma, the mean of the branches' T_2, T_1 and S_1
   double gamma, g_gm1;  // gamma, gamma / (gamma - 1)
   float gammaf;
 };
@@ -81,7 +83,16 @@ inline NearCoef near_coef(double gamma) {
   c.gamma = gamma;
   c.g_gm1 = gamma / (gamma - 1.0);
   c.gammaf = (float)gamma;
-  c.t2m = 0.5f * (c.tf[0][2] + c.tf[1][2]);
+  auto twice = [](float v) {
+    f32x2 r;
+    const float two[2] = {v, v};
+    std::memcpy(&r, two, sizeof(r));
+    return r;
+  };
+  c.g2 = twice(c.gammaf);
+  c.t22 = twice(0.5f * (c.tf[0][2] + c.tf[1][2]));
+  c.t12 = twice(c.tf[0][1]);
+  c.s12 = twice(c.sf[0][1]);
   return c;
 }
 
@@ -131,12 +142,18 @@ struct NearStar {
 // not positive comes back as NEAR_GENERAL; a double one is the caller's to sort out); dP = p_R -
 // p_L, ul, ur velocities about u0, dU = u_R - u_L; ulf, urf the full
 // velocities in float.
-template <class T>
-__device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl, T rr, T ur, T pr, T dP, T dU, T u0,
-                                            bool has_u0, float ulf, float urf, NearStar<T>& s) {
+// EXACT_INV: s.irc and s.ip rounded to the last bits (the adjoint's use of
+// them). The solution itself takes them to about 2^-43: they multiply p* - p_K,
+// at most 2^-7 p, so the star state keeps its last bits; one Newton step each
+// from the float values, five and two FP64 operations instead of seven and three.
+template <bool EXACT_INV = false>
+__device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double ul, double pl, double rr, double ur,
+                                            double pr, double dP, double dU, double u0, bool has_u0, float ulf,
+                                            float urf, NearStar<double>& s) {
+  using T = double;
   const float plf = narrow(pl), prf = narrow(pr), rlf = narrow(rl), rrf = narrow(rr);
   // doubles beyond float's comfortable range: the general solver
-  if (sizeof(T) == 8 && !(fmaxf(fmaxf(plf, prf), fmaxf(rlf, rrf)) < 1e30f)) return NEAR_GENERAL;
+  if (!(fmaxf(fmaxf(plf, prf), fmaxf(rlf, rrf)) < 1e30f)) return NEAR_GENERAL;
   const float gl = C.gammaf * plf, gr = C.gammaf * prf;
   const float il = recip_sqrt(gl) * recip_sqrt(rlf), ir = recip_sqrt(gr) * recip_sqrt(rrf);  // 1 / (rho c)
   const float cl = gl * il, cr = gr * ir;
@@ -146,40 +163,12 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl,
   float d = (dPf * ir - dUf) * recip(il + ir);
   float xl = d * ipl, xr = (d - dPf) * ipr;
   float X = fabsf(xl) + fabsf(xr);
-  constexpr float XM = sizeof(T) == 4 ? NEAR_XF : NEAR_XD;
   if (!(X <= 2.0f * NEAR_XF)) return NEAR_GENERAL;  // NaN too
   // supersonic by a margin that covers every wave speed at |x| <= 1/32
   if (ulf >= 1.1f * cl) return NEAR_LEFT;
   if (-urf >= 1.1f * cr) return NEAR_RIGHT;
-  if (!(X <= XM)) return NEAR_GENERAL;
-  if constexpr (sizeof(T) == 4) {
-    // One Newton step from the acoustic value, whose error is below 0.45 x^2 p:
-    // what it leaves, below 0.1 x^4 p, is under the rounding of d for |x| <=
-    // 1/128, and a second step's beyond.  The slope needs three digits only
-    // (T to x^2 with the branches' mean T_2).
-    float fl, fr;
-    auto newton = [&]() {
-      const float dr = d - dPf;
-      xl = d * ipl;
-      xr = dr * ipr;
-      const float tl = il * fmaf(fmaf(C.t2m, xl, C.tf[0][1]), xl, 1.0f);
-      const float tr = ir * fmaf(fmaf(C.t2m, xr, C.tf[0][1]), xr, 1.0f);
-      fl = d * il * near_cubic(C.sf, d > 0.0f, xl);
-      fr = dr * ir * near_cubic(C.sf, dr > 0.0f, xr);
-      const float step = -(fl + fr + dUf) * recip(tl + tr);
-      d += step;
-      fl = fmaf(tl, step, fl);
-      fr = fmaf(tr, step, fr);
-    };
-    newton();
-    if (X > 0.0078125f) newton();
-    s.d = d;
-    s.fl = fl;
-    s.fr = fr;
-    s.us = ul - fl;
-    s.ipl = ipl;
-    s.ipr = ipr;
-  } else {
+  if (!(X <= NEAR_XD)) return NEAR_GENERAL;
+  {
     float tl = 0.0f, tr = 0.0f;
 #pragma unroll
     for (int it = 0; it < 2; ++it) {
@@ -191,10 +180,17 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl,
       d -= (d * il * near_sum_f(C.sf, sl, xl) + (d - dPf) * ir * near_sum_f(C.sf, sr, xr) + dUf) * recip(tl + tr);
     }
     const float iD = recip(tl + tr), small = 4.6e-10f * fminf(plf, prf);
-    s.ircl = recip_sqrt(C.gamma * (pl * rl));
-    s.ircr = recip_sqrt(C.gamma * (pr * rr));
-    s.ipl = recip(pl);
-    s.ipr = recip(pr);
+    if constexpr (EXACT_INV) {
+      s.ircl = recip_sqrt(C.gamma * (pl * rl));
+      s.ircr = recip_sqrt(C.gamma * (pr * rr));
+      s.ipl = recip(pl);
+      s.ipr = recip(pr);
+    } else {
+      s.ircl = refine_recip_sqrt(C.gamma * (pl * rl), widen<T>(il));
+      s.ircr = refine_recip_sqrt(C.gamma * (pr * rr), widen<T>(ir));
+      s.ipl = refine_recip(pl, widen<T>(ipl));
+      s.ipr = refine_recip(pr, widen<T>(ipr));
+    }
     T dd = widen<T>(d), f1 = T(0), f2 = T(0);
     float step = 0.0f;
     bool more = true;
@@ -223,8 +219,64 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, T rl, T ul, T pl,
   if (v - c >= band) return left ? NEAR_LEFT : NEAR_RIGHT;
   if (!(c - v > band)) return NEAR_GENERAL;
   const T x = left ? s.d * s.ipl : (s.d - dP) * s.ipr;
-  if constexpr (sizeof(T) == 4) s.drho = (left ? rl : rr) * (x * near_cubic(C.df, x > 0.0f, x));
-  else s.drho = (left ? rl : rr) * (x * near_sum(C.d, C.dt, !sign_bit(x), x));
+  s.drho = (left ? rl : rr) * (x * near_sum(C.d, C.dt, !sign_bit(x), x));
+  return left ? NEAR_STAR_L : NEAR_STAR_R;
+}
+
+// The same in float, the two sides in the halves of packed values (they take
+// the same operations).
+__device__ __forceinline__ int near_riemann(const NearCoef& C, float rl, float ul, float pl, float rr, float ur,
+                                            float pr, float dP, float dU, float u0, bool has_u0, float ulf, float urf,
+                                            NearStar<float>& s) {
+  const f32x2 one = pack2(1.0f, 1.0f), g2 = mul2(C.g2, pack2(pl, pr));
+  float gl, gr, il, ir, cl, cr, xl, xr, fl, fr, tl, tr;
+  unpack2(g2, gl, gr);
+  const f32x2 i2 = mul2(pack2(recip_sqrt(gl), recip_sqrt(gr)), pack2(recip_sqrt(rl), recip_sqrt(rr)));  // 1 / (rho c)
+  unpack2(i2, il, ir);
+  unpack2(mul2(g2, i2), cl, cr);
+  s.ipl = recip(pl);
+  s.ipr = recip(pr);
+  const f32x2 ip2 = pack2(s.ipl, s.ipr);
+  // linear (acoustic) star pressure d = p* - p_L
+  float d = (dP * ir - dU) * recip(il + ir);
+  unpack2(mul2(pack2(d, d - dP), ip2), xl, xr);
+  const float X = fabsf(xl) + fabsf(xr);
+  if (!(X <= 2.0f * NEAR_XF)) return NEAR_GENERAL;  // NaN too: a state that is not positive
+  if (ulf >= 1.1f * cl) return NEAR_LEFT;
+  if (-urf >= 1.1f * cr) return NEAR_RIGHT;
+  if (!(X <= NEAR_XF)) return NEAR_GENERAL;
+  // One Newton step from the acoustic value, whose error is below 0.45 x^2 p:
+  // what it leaves, below 0.1 x^4 p, is under the rounding of d for |x| <=
+  // 1/128, and a second step's beyond.  The slope needs three digits only
+  // (T to x^2 with the branches' mean T_2).
+  auto newton = [&]() {
+    const float dr = d - dP;
+    const f32x2 d2 = pack2(d, dr), x2 = mul2(d2, ip2);
+    const f32x2 t2 = mul2(i2, fma2(fma2(C.t22, x2, C.t12), x2, one));
+    const bool sl = d > 0.0f, sr = dr > 0.0f;  // shock branches
+    f32x2 S = fma2(pack2(sl ? C.sf[1][3] : C.sf[0][3], sr ? C.sf[1][3] : C.sf[0][3]), x2,
+                   pack2(sl ? C.sf[1][2] : C.sf[0][2], sr ? C.sf[1][2] : C.sf[0][2]));
+    S = fma2(fma2(S, x2, C.s12), x2, one);
+    f32x2 f2 = mul2(mul2(d2, i2), S);
+    unpack2(f2, fl, fr);
+    unpack2(t2, tl, tr);
+    const float step = -(fl + fr + dU) * recip(tl + tr);
+    d += step;
+    unpack2(fma2(t2, pack2(step, step), f2), fl, fr);
+  };
+  newton();
+  if (X > 0.0078125f) newton();
+  s.d = d;
+  s.fl = fl;
+  s.fr = fr;
+  s.us = ul - fl;
+  const bool left = !sign_bit(has_u0 ? u0 + s.us : s.us);
+  if (!left) s.us = ur + fr;
+  const float v = left ? ulf : -urf, c = left ? cl : cr, band = c * fmaf(1.25f, X, 1e-5f);
+  if (v - c >= band) return left ? NEAR_LEFT : NEAR_RIGHT;
+  if (!(c - v > band)) return NEAR_GENERAL;
+  const float x = left ? d * s.ipl : (d - dP) * s.ipr;
+  s.drho = (left ? rl : rr) * (x * near_cubic(C.df, x > 0.0f, x));
   return left ? NEAR_STAR_L : NEAR_STAR_R;
 }
 

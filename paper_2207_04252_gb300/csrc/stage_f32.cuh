@@ -19,32 +19,7 @@
 
 namespace rossbi {
 
-// ---------------------------------------------------------------- two floats at a time
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack2(-1.0f, -1.0f), a); }
+// ---------------------------------------------------------------- two fields at a time
 // min(|a|, |b|) with the sign of a b, and the MinMod slope, of both halves
 __device__ __forceinline__ f32x2 min_xorsign2(f32x2 a, f32x2 b) {
   float a0, a1, b0, b1;
@@ -76,6 +51,13 @@ __device__ __forceinline__ void parabola2(f32x2 em, f32x2 e0, f32x2 ep, const fl
 }
 
 // ---------------------------------------------------------------- shared memory
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* smem, const void* gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gmem), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
 // Offsets in floats of a block's arrays; quads on 16-byte boundaries.
 template <int NF, int TR, int TT, int TZ>
 struct F32Smem {
@@ -103,12 +85,14 @@ template <int NF, int TR, int TT, int TZ, int NT, int RC>
 struct F32Tile {
   using M = F32Smem<NF, TR, TT, TZ>;
   int i0, j0, k0;
+  bool full;  // the tile lies within the grid
   __device__ __forceinline__ F32Tile(const PertArgs<float>& a, int tile) {
     // r fastest, then z, then theta: the tiles whose halos a tile re-reads run
     // at most tiles_r x tiles_z blocks apart, so the re-reads hit in L2
     i0 = (tile % a.tiles_r) * TR;
     k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
     j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
+    full = i0 + TR <= a.g.nr && j0 + TT <= a.g.nth && k0 + TZ <= a.g.nz;
   }
 
   // The tile and its halo as deviations: the gas as conservative departures (or,
@@ -178,13 +162,16 @@ struct F32Tile {
     }
   }
 
-  // The tables of the tile's faces and cells, indices clamped to the grid.
+  // The tables of the tile's faces and cells, indices clamped to the grid, by
+  // asynchronous copies (in flight while the box is staged).
   __device__ __forceinline__ void tables(const PertArgs<float>& a, float* sm) const {
     const DevGrid& g = a.g;
     constexpr int N0 = (TR + 3) * TZ, N1 = N0 + TR * TZ, N2 = N1 + TR * (TZ + 3);
     for (int q = threadIdx.x; q < N2; q += NT) {
-      float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (g.has_eq) {
+      float4* dst = reinterpret_cast<float4*>(sm + M::face0) + q;
+      if (!g.has_eq) {
+        *dst = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      } else {
         size_t o;
         const float* t;
         if (q < N0) {
@@ -200,24 +187,21 @@ struct F32Tile {
           t = a.t.face[2];
           o = (size_t)f * g.nr + i;
         }
-        v = reinterpret_cast<const float4*>(t)[o];
+        copy_async<16>(dst, t + 4 * o);
       }
-      reinterpret_cast<float4*>(sm + M::face0)[q] = v;
     }
-    constexpr int W = RCW * (TR + 2);
+    constexpr int W = RCW / 4 * (TR + 2);  // 16-byte pieces of the weights, then the areas one by one
     for (int q = threadIdx.x; q < W + 3 * TR + 1; q += NT) {
-      float v;
       if (q < W) {
-        const int c = i0 - 1 + q / RCW;  // weights of cells -1 .. nr are tabulated
-        v = a.t.rcoef[(size_t)((c > g.nr ? g.nr : c) + 1) * RCW + q % RCW];
-      } else if (q < W + TR + 1) {
-        v = a.t.area_r[clampi(i0 + q - W, 0, g.nr)];
-      } else if (q < W + 2 * TR + 1) {
-        v = a.t.area_t[clampi(i0 + q - W - TR - 1, 0, g.nr - 1)];
+        const int c = i0 - 1 + q / (RCW / 4);  // weights of cells -1 .. nr are tabulated
+        copy_async<16>(sm + M::wgt + 4 * q, a.t.rcoef + (size_t)((c > g.nr ? g.nr : c) + 1) * RCW + 4 * (q % (RCW / 4)));
       } else {
-        v = a.t.area_z[clampi(i0 + q - W - 2 * TR - 1, 0, g.nr - 1)];
+        const int n = q - W;
+        const float* t = n < TR + 1 ? a.t.area_r + clampi(i0 + n, 0, g.nr)
+                                    : (n < 2 * TR + 1 ? a.t.area_t + clampi(i0 + n - TR - 1, 0, g.nr - 1)
+                                                      : a.t.area_z + clampi(i0 + n - 2 * TR - 1, 0, g.nr - 1));
+        copy_async<4>(sm + M::area + n, t);
       }
-      sm[M::wgt + q] = v;
     }
   }
 
@@ -225,8 +209,11 @@ struct F32Tile {
   // lines of L lanes).  Lane p of a line reconstructs cell p - 1, takes the
   // upper face state of its lower neighbour by a shuffle, solves its lower
   // face and takes the flux of its upper face by a second shuffle.
-  template <int D, class P>
-  __device__ __forceinline__ void chunk(const PertArgs<float>& a, float* sm, int base, unsigned& status,
+  // Returns whether the lane's face needs the general solver; its flux then
+  // counts as zero until the chunk is taken again with REDO, which solves the
+  // faces of the `again` lanes and adds their fluxes.
+  template <int D, class P, bool REDO>
+  __device__ __forceinline__ bool chunk(const PertArgs<float>& a, float* sm, int base, bool again, unsigned& status,
                                         unsigned& nfallback) const {
     constexpr int TD = D == 0 ? TR : (D == 1 ? TT : TZ), L = pow2ceil(TD + 2);
     constexpr int NA = D == 0 ? TT : TR;
@@ -235,31 +222,35 @@ struct F32Tile {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr bool UNI = D != 0;
     static_assert(L <= 32, "line does not fit a warp");
+    static_assert(ITEMS % 32 == 0, "whole chunks");
     const DevGrid& g = a.g;
     const int item = base + (threadIdx.x & 31);
     const int line = item / L, c = item % L - 1;
     const int ta = line % NA, tb = line / NA;
     const int x = D == 0 ? c : ta, y = D == 1 ? c : (D == 0 ? ta : tb), z = D == 2 ? c : tb;
-    const bool line_ok = item < ITEMS && (D == 0 ? (j0 + y < g.nth && k0 + z < g.nz)
-                                                 : (D == 1 ? (i0 + x < g.nr && k0 + z < g.nz)
-                                                           : (i0 + x < g.nr && j0 + y < g.nth)));
-    const int gd = D == 0 ? i0 + x : (D == 1 ? j0 + y : k0 + z), nd = D == 0 ? g.nr : (D == 1 ? g.nth : g.nz);
-    const bool do_recon = line_ok && c <= TD && gd <= nd, do_face = do_recon && c >= 0;
-    const bool do_acc = do_face && c < TD && gd < nd;
-    if (!__any_sync(FULL, do_face)) return;  // a warp of lines beyond a ragged grid's edge
-    // idle lanes read a cell that exists
-    const int s = do_recon ? (z + 2) * M::PLANE + (y + 2) * M::ROW + (x + 2) : 2 * M::PLANE + 2 * M::ROW + 2;
-    const int fx = do_recon ? (D == 0 ? z * (TR + 3) + x + 1 : (D == 1 ? z * TR + x : (z + 1) * TR + x)) : 0;
-    const int ax = do_face ? x : 0;
-    const int core = do_acc ? z * M::CPLANE + y * M::CROW + x : 0;
+    // Every cell -1 .. TD of every line is staged, also beyond the grid's edge,
+    // so that only what a lane contributes needs conditions; none in a tile
+    // within the grid.
+    bool do_face = c >= 0, do_acc = c >= 0 && c < TD;
+    if (!full) {
+      const bool line_ok = D == 0 ? (j0 + y < g.nth && k0 + z < g.nz)
+                                  : (D == 1 ? (i0 + x < g.nr && k0 + z < g.nz) : (i0 + x < g.nr && j0 + y < g.nth));
+      const int gd = D == 0 ? i0 + x : (D == 1 ? j0 + y : k0 + z), nd = D == 0 ? g.nr : (D == 1 ? g.nth : g.nz);
+      do_face = do_face && line_ok && gd <= nd;
+      do_acc = do_acc && line_ok && gd < nd;
+      if (!__any_sync(FULL, do_face)) return false;  // a warp of lines beyond the edge
+    }
+    const int s = (z + 2) * M::PLANE + (y + 2) * M::ROW + (x + 2);
+    const int fx = D == 0 ? z * (TR + 3) + x + 1 : (D == 1 ? z * TR + x : (z + 1) * TR + x);
+    const int core = z * M::CPLANE + y * M::CROW + x;
     float w[RCW];
     if (!UNI) {
-      const float4* q = reinterpret_cast<const float4*>(sm + M::wgt) + 2 * (do_recon ? x + 1 : 0);
+      const float4* q = reinterpret_cast<const float4*>(sm + M::wgt) + 2 * (x + 1);
       const float4 q0 = q[0], q1 = q[1];
       w[0] = q0.x; w[1] = q0.y; w[2] = q0.z; w[3] = q0.w;
       w[4] = q1.x; w[5] = q1.y; w[6] = q1.z;
     }
-    const float area = sm[M::area + (D == 0 ? 0 : (D == 1 ? TR + 1 : 2 * TR + 1)) + ax];
+    const float area = sm[M::area + (D == 0 ? 0 : (D == 1 ? TR + 1 : 2 * TR + 1)) + x];
     // the divergence of dust species q: primitive reconstruction, kinetic flux
     auto dust_flux = [&](int q, float* F) {
       const ulonglong2* e = reinterpret_cast<const ulonglong2*>(sm + M::quad(q)) + s;
@@ -275,13 +266,13 @@ struct F32Tile {
       }
 #pragma unroll
       for (int f = 0; f < 4; ++f) WL[f] = __shfl_up_sync(FULL, qp[f], 1, L);
-      dust_kinetic_flux<D>(do_face ? area : 0.0f, WL, qm, F);
+      dust_kinetic_flux<D>(area, WL, qm, F);
     };
     // The first species' flux has no branch and nothing in common with the
     // gas's: here its instructions fill the latencies of the gas's
     // reconstruction.
     float Fd[4];
-    if constexpr (M::NQ > 1) dust_flux(1, Fd);
+    if constexpr (M::NQ > 1 && !REDO) dust_flux(1, Fd);
     {
       const float4* ft = reinterpret_cast<const float4*>(sm + M::face(D)) + fx;
       constexpr int FS = D == 0 ? 1 : (D == 1 ? 0 : TR);  // to the upper face (theta: the same)
@@ -333,33 +324,36 @@ struct F32Tile {
         wl[f] = __shfl_up_sync(FULL, wp[f], 1, L);  // upper face state of the lower neighbour
         F[f] = 0.0f;
       }
-      if (do_face)
-        pert_face<float, D, P>(
+      bool general = false;
+      if (do_face && (!REDO || again))
+        general = pert_face<float, D, P, REDO>(
             a, Em, area, wl, wm,
             [&]() {
-              const int k = k0 + (D == 2 ? 0 : z);  // in the grid: do_face
-              return D == 0 ? k * (g.nr + 1) + gd : (D == 1 ? k * g.nr + i0 + x : gd * g.nr + i0 + x);
+              const int k = k0 + z;  // in the grid: do_face
+              return (size_t)k * (D == 0 ? g.nr + 1 : g.nr) + i0 + x;
             },
             F, status, nfallback);
-      add_divergence<D, L>(F, sm + M::acc0, core, do_acc);
+      constexpr bool WRITE = D == 0 && !REDO;
+      add_divergence<WRITE, L>(F, sm + M::acc0, core, do_acc);
       const float Fu = __shfl_down_sync(FULL, F[RHO], 1, L);
       if (do_acc) {
         float* d = sm + M::acc_rho + core;
-        *d = D == 0 ? F[RHO] - Fu : *d + (F[RHO] - Fu);
+        *d = WRITE ? F[RHO] - Fu : *d + (F[RHO] - Fu);
       }
-    }
-    if constexpr (M::NQ > 1) {
-      add_divergence<D, L>(Fd, sm + M::acc(1), core, do_acc);
+      if constexpr (M::NQ > 1 && !REDO) {
+        add_divergence<D == 0, L>(Fd, sm + M::acc(1), core, do_acc);
 #pragma unroll 1
-      for (int q = 2; q < M::NQ; ++q) {
-        dust_flux(q, Fd);
-        add_divergence<D, L>(Fd, sm + M::acc(q), core, do_acc);
+        for (int q = 2; q < M::NQ; ++q) {
+          dust_flux(q, Fd);
+          add_divergence<D == 0, L>(Fd, sm + M::acc(q), core, do_acc);
+        }
       }
+      return general;
     }
   }
 
-  // Writes (D = 0) or adds the divergence F - (F of the lane above) of a quad.
-  template <int D, int L>
+  // Writes or adds the divergence F - (F of the lane above) of a quad.
+  template <bool WRITE, int L>
   __device__ __forceinline__ static void add_divergence(const float* F, float* acc, int core, bool own) {
     float u[4];
 #pragma unroll
@@ -369,7 +363,7 @@ struct F32Tile {
       ulonglong2 v;
       v.x = sub2(pack2(F[0], F[1]), pack2(u[0], u[1]));
       v.y = sub2(pack2(F[2], F[3]), pack2(u[2], u[3]));
-      if (D != 0) {
+      if (!WRITE) {
         const ulonglong2 o = *d;
         v.x = add2(o.x, v.x);
         v.y = add2(o.y, v.y);
@@ -382,10 +376,43 @@ struct F32Tile {
   static __host__ __device__ constexpr int items() {
     return (D == 0 ? TT * TZ : (D == 1 ? TR * TZ : TR * TT)) * pow2ceil((D == 0 ? TR : (D == 1 ? TT : TZ)) + 2);
   }
+  // The sweep along axis D, chunks spread over the warps; sets bit BITS D + n of
+  // `left` where the lane's face of the warp's n-th chunk is left to redo().
+  static constexpr int BITS = 10;
   template <int D, class P>
-  __device__ __forceinline__ void sweep(const PertArgs<float>& a, float* sm, unsigned& status,
-                                        unsigned& nfallback) const {
-    for (int base = threadIdx.x & ~31; base < items<D>(); base += NT) chunk<D, P>(a, sm, base, status, nfallback);
+  __device__ __forceinline__ void sweep(const PertArgs<float>& a, float* sm, unsigned& left) const {
+    static_assert((items<D>() + NT - 1) / NT <= BITS, "a bit per chunk");
+    unsigned bit = 1u << (BITS * D), status = 0, nfallback = 0;
+#pragma unroll 1
+    for (int base = threadIdx.x & ~31; base < items<D>(); base += NT, bit <<= 1)
+      if (chunk<D, P, false>(a, sm, base, false, status, nfallback)) left |= bit;
+  }
+  template <int D, class P>
+  __device__ __forceinline__ void resweep(const PertArgs<float>& a, float* sm, unsigned left, unsigned& status,
+                                          unsigned& nfallback) const {
+    unsigned bit = 1u << (BITS * D);
+#pragma unroll 1
+    for (int base = threadIdx.x & ~31; base < items<D>(); base += NT, bit <<= 1)
+      if (__any_sync(0xffffffffu, left & bit)) chunk<D, P, true>(a, sm, base, left & bit, status, nfallback);
+    __syncthreads();
+  }
+
+  // The faces for the general solver (near a strong wave or in the sonic band)
+  // of all three sweeps, for blocks that have any; sweep by sweep, so that every
+  // sum has one order.  Out of line and after the sweeps: with no call in their
+  // loops the kernel takes 80 registers and 24 warps share an SM; with the
+  // solver called from the loops it took 128 (16 warps), and spilled at fewer.
+  struct Word2 {
+    unsigned status, nfallback;
+  };
+  template <class P>
+  static __device__ __noinline__ Word2 redo(const PertArgs<float>& a, float* sm, unsigned left) {
+    const F32Tile t(a, blockIdx.x);
+    Word2 w{0, 0};
+    t.template resweep<0, P>(a, sm, left, w.status, w.nfallback);
+    t.template resweep<1, P>(a, sm, left, w.status, w.nfallback);
+    t.template resweep<2, P>(a, sm, left, w.status, w.nfallback);
+    return w;
   }
 
   template <bool XT>
@@ -418,28 +445,33 @@ struct F32Tile {
 
 // One RK stage of one tile per block.
 template <int NF, int TR, int TT, int TZ, int NT, int MINB, class P, bool XT, int RC>
-__global__ void __launch_bounds__(NT, MINB) stage_f32_kernel(const PertArgs<float> a) {
+__global__ void __launch_bounds__(NT, MINB) stage_f32_kernel(const __grid_constant__ PertArgs<float> a) {
   extern __shared__ __align__(16) float sm[];
-  const F32Tile<NF, TR, TT, TZ, NT, RC> t(a, blockIdx.x);
-  unsigned status = 0, nfallback = 0;
+  using Tile = F32Tile<NF, TR, TT, TZ, NT, RC>;
+  const Tile t(a, blockIdx.x);
+  unsigned status = 0, left = 0;
   __shared__ double s_tau;
   publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, a.g.cfl);
   if (!a.stage2) clear_rate(a.rate_out);
   t.tables(a, sm);
   t.stage(a, sm);
+  copy_async_wait();
   __syncthreads();
-  t.template sweep<0, P>(a, sm, status, nfallback);
+  t.template sweep<0, P>(a, sm, left);
   __syncthreads();
-  t.template sweep<1, P>(a, sm, status, nfallback);
+  t.template sweep<1, P>(a, sm, left);
   __syncthreads();
-  t.template sweep<2, P>(a, sm, status, nfallback);
-  __syncthreads();
+  t.template sweep<2, P>(a, sm, left);
+  if (__syncthreads_or(left)) {
+    const typename Tile::Word2 w = Tile::template redo<P>(a, sm, left);
+    status = w.status;
+    if (w.nfallback) atomicAdd(a.t.fallbacks, (unsigned long long)w.nfallback);
+  }
   float rate = 0.0f;
   for (int cidx = threadIdx.x; cidx < TR * TT * TZ; cidx += NT)
     t.template update<XT>(a, sm, cidx, (float)s_tau, rate, status);
   if (a.stage2) raise_rate(a.rate_out, rate);
   if (status) atomicOr(a.status, status);
-  if (nfallback) atomicAdd(a.t.fallbacks, (unsigned long long)nfallback);
 }
 
 }  // namespace rossbi

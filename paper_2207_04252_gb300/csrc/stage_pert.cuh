@@ -448,9 +448,11 @@ __device__ __forceinline__ T face_prim(T gm1, T rho0, T v0, const T* q, T* w) {
 
 // Area times the gas flux perturbation through a face normal to axis D of
 // equilibrium Em, from the primitive perturbations wl, wm of its left and right
-// states; wave_at(): the face's place in the table of wave speeds.
-template <class T, int D, class P, class W>
-__device__ __forceinline__ void pert_face(const PertArgs<T>& a, const PEq<T>& Em, T area, const T* wl, const T* wm,
+// states; wave_at(): the face's place in the table of wave speeds.  Returns
+// whether the face needs the general solver; with GENERAL = false F is then
+// left as it is.
+template <class T, int D, class P, bool GENERAL, class W>
+__device__ __forceinline__ bool pert_face(const PertArgs<T>& a, const PEq<T>& Em, T area, const T* wl, const T* wm,
                                           W&& wave_at, T* F, unsigned& status, unsigned& nfallback) {
   constexpr int n = Axes<D>::n;
   const DevGrid& g = a.g;
@@ -459,8 +461,9 @@ __device__ __forceinline__ void pert_face(const PertArgs<T>& a, const PEq<T>& Em
   NearStar<T> st;
   int kind = NEAR_GENERAL;
   if (sizeof(T) == 4 || (positive(rl) && positive(rr) && positive(pl) && positive(pr)))
-    kind = near_riemann<T>(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
+    kind = near_riemann(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
                            narrow(un0 + wl[n]), narrow(un0 + wm[n]), st);
+  if (!GENERAL && kind == NEAR_GENERAL) return true;
   const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
   T d[3], drho = left ? wl[RHO] : wm[RHO], dp = left ? wl[EN] : wm[EN];
 #pragma unroll
@@ -471,7 +474,7 @@ __device__ __forceinline__ void pert_face(const PertArgs<T>& a, const PEq<T>& Em
     dp = wl[EN] + st.d;
   }
   bool ok = true;
-  if (kind == NEAR_GENERAL) {
+  if (GENERAL && kind == NEAR_GENERAL) {
     PFace<T> W0{Em.rho, un0, Em.p, T(0), T(0), T(0)};
     if (g.has_eq) {
       const T* wv = a.t.wave[D] + 4 * (size_t)wave_at();
@@ -491,6 +494,7 @@ __device__ __forceinline__ void pert_face(const PertArgs<T>& a, const PEq<T>& Em
     dp = o.dp;
   }
   if (ok) pert_flux<T, D>(a.g_gm1, area, Em, drho, d, dp, F);
+  return kind == NEAR_GENERAL;
 }
 
 // The gas sweep along axis D of the double form: sE holds the staged gas
@@ -563,7 +567,7 @@ __device__ __forceinline__ void sweep_pert_gas(const PertArgs<double>& a, const 
       F[f] = 0.0;
     }
     if (s.do_face)
-      pert_face<double, D, P>(a, Em, face_area<D>(g, s.gi, ci), wl, wm, [&]() { return of; }, F, status, nfallback);
+      pert_face<double, D, P, true>(a, Em, face_area<D>(g, s.gi, ci), wl, wm, [&]() { return of; }, F, status, nfallback);
 #pragma unroll
     for (int f = 0; f < 5; ++f) accumulate<D, L>(F[f], sG + f * S::NCORE + s.core, s.do_acc);
   }
