@@ -70,6 +70,32 @@ struct DevGrid {
   NearCoef near;         // series of the exact Riemann solution near p_K
 };
 
+// Division of 0 <= n < 2^31 by a divisor fixed on the host (multiplication by
+// a rounded-up reciprocal; Granlund & Montgomery 1994): three instructions
+// where a division takes about 25, in every warp of every block.
+struct FastDiv {
+  unsigned d, mul, shift;
+  __device__ __forceinline__ int operator()(int n) const { return (int)((__umulhi((unsigned)n, mul) + (unsigned)n) >> shift); }
+};
+inline FastDiv fast_div(unsigned d) {
+  FastDiv f{d, 0, 0};
+  while ((1ull << f.shift) < d) ++f.shift;
+  f.mul = (unsigned)(((1ull << 32) * ((1ull << f.shift) - d)) / d + 1);
+  return f;
+}
+// Tile numbers run r fastest, then z, then theta: the tiles whose halos a tile
+// re-reads (its r, z and theta neighbours) run at most tiles_r x tiles_z
+// blocks apart, so the re-reads hit in L2.
+struct TileOrder {
+  FastDiv r, z;  // tiles along r and z
+  __device__ __forceinline__ void origin(int tile, int tr, int tt, int tz, int& i0, int& j0, int& k0) const {
+    const int rest = r(tile), t = z(rest);
+    i0 = (tile - rest * (int)r.d) * tr;
+    k0 = (rest - t * (int)z.d) * tz;
+    j0 = t * tt;
+  }
+};
+
 __host__ __device__ constexpr int pow2ceil(int v) {
   int p = 1;
   while (p < v) p <<= 1;

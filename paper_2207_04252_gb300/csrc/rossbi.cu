@@ -468,8 +468,7 @@ StageArgs base_args(rossbi_grid* g) {
   std::memset(&a, 0, sizeof(a));
   a.g = g->dg;
   a.status = g->d_status;
-  a.tiles_r = g->tiles_r;
-  a.tiles_z = g->tiles_z;
+  a.order = TileOrder{fast_div(g->tiles_r), fast_div(g->tiles_z)};
   a.tile = g->tile;
   return a;
 }
@@ -653,8 +652,7 @@ PertArgs<T> pert_args(rossbi_grid* g) {
   if constexpr (sizeof(T) == 4) a.t = g->pt_f;
   else a.t = g->pt_d;
   a.status = g->d_status;
-  a.tiles_r = g->tiles_r;
-  a.tiles_z = g->tiles_z;
+  a.order = TileOrder{fast_div(g->tiles_r), fast_div(g->tiles_z)};
   a.sms = g->sms;
   a.tile = g->tile;
   a.gam = (T)g->dg.gamma;

@@ -87,11 +87,7 @@ struct F32Tile {
   int i0, j0, k0;
   bool full;  // the tile lies within the grid
   __device__ __forceinline__ F32Tile(const PertArgs<float>& a, int tile) {
-    // r fastest, then z, then theta: the tiles whose halos a tile re-reads run
-    // at most tiles_r x tiles_z blocks apart, so the re-reads hit in L2
-    i0 = (tile % a.tiles_r) * TR;
-    k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
-    j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
+    a.order.origin(tile, TR, TT, TZ, i0, j0, k0);
     full = i0 + TR <= a.g.nr && j0 + TT <= a.g.nth && k0 + TZ <= a.g.nz;
   }
 

@@ -34,7 +34,7 @@ struct StageArgs {
   int stage2;                         // fuse the CFL rate of the output
   unsigned* status;
   int mode;                          // 0 update, 1 residual only (empty run)
-  int tiles_r, tiles_z;  // tile counts along r and z (block -> tile: r fastest, then z, then theta)
+  TileOrder order;
 };
 
 // Parabola through three deviations (Sect. 2.7) with the MinMod limiter: each
@@ -411,13 +411,8 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
   double* sE = smem;             // [5][BOX] the gas departures, then the four primitives of one dust species at a time
   double* sG = smem + 5 * BOX;   // [NF][NCORE] flux divergence
   const DevGrid& g = a.g;
-  const int tile = blockIdx.x;
-  // r fastest, then z, then theta: the tiles whose halos a tile re-reads
-  // (its r, z and theta neighbours) run at most tiles_r x tiles_z blocks
-  // apart, so the re-reads hit in L2
-  const int i0 = (tile % a.tiles_r) * TR;
-  const int k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
-  const int j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
+  int i0, j0, k0;
+  a.order.origin(blockIdx.x, TR, TT, TZ, i0, j0, k0);
   unsigned status = 0;
   __shared__ double s_tau;
   publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, g.cfl);

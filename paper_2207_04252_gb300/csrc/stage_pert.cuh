@@ -417,7 +417,7 @@ struct PertArgs {
   DragArgs drag;
   int stage2;
   unsigned* status;
-  int tiles_r, tiles_z;  // tile counts along r and z (tile number: r fastest, then z, then theta)
+  TileOrder order;
   int sms;               // SMs of the device
   int tile;              // double form: TILE_*, chosen by the host
   // the grid's and the drag's parameters in the state precision, converted
@@ -817,11 +817,8 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<dou
   double* sE = smem;             // [5][BOX] the gas departures, then the four primitives of one dust species at a time
   double* sG = smem + 5 * BOX;   // [NF][NCORE] flux divergence
   const DevGrid& g = a.g;
-  // tiles r fastest, then z, then theta, as in the full-state kernel
-  const int tile = blockIdx.x;
-  const int i0 = (tile % a.tiles_r) * TR;
-  const int k0 = ((tile / a.tiles_r) % a.tiles_z) * TZ;
-  const int j0 = (tile / (a.tiles_r * a.tiles_z)) * TT;
+  int i0, j0, k0;
+  a.order.origin(blockIdx.x, TR, TT, TZ, i0, j0, k0);
   unsigned status = 0, nfallback = 0;
   __shared__ double s_tau;
   publish_tau(&s_tau, a.tau_frac, a.dt_host, a.rate_in, g.cfl);
