@@ -9,8 +9,9 @@
 //     reconstruction reads its nine fields at three cells with nine loads
 //     instead of 27, and works on two fields per instruction (the packed f32x2
 //     arithmetic of sm_100 and later);
-//   - row and plane strides are odd numbers of quads, so that the lanes of a
-//     line along any axis fall into different banks;
+//   - row and plane strides are odd numbers of quads (an odd number times four
+//     for single floats), so that the eight lanes of a quarter warp's quads, or
+//     four lines of eight lanes, fall into different banks along any axis;
 //   - the equilibrium of the tile's faces, the parabola weights and the face
 //     areas are copied to shared memory with the box: the sweeps load nothing
 //     from global memory and form no 64-bit address.
@@ -66,15 +67,19 @@ struct F32Smem {
   static constexpr int ROW = BX | 1, PLANE = (ROW * BY) | 1, BOX = PLANE * BZ;  // staged box, in cells
   static constexpr int CROW = TR | 1, CPLANE = (CROW * TT) | 1, CORE = CPLANE * TZ;  // accumulators
   __host__ __device__ static constexpr int up4(int n) { return (n + 3) & ~3; }
+  __host__ __device__ static constexpr int up_odd4(int n) { return (n + 3) / 4 % 2 ? up4(n) : up4(n) + 4; }
+  static constexpr int RROW = up_odd4(BX), RPLANE = up_odd4(RROW * BY);      // staged rho'
+  static constexpr int CRROW = up_odd4(TR), CRPLANE = up_odd4(CRROW * TT);  // its accumulator
+  static constexpr int ZROW = TR | 1;                                       // z faces, in quads
   __host__ __device__ static constexpr int quad(int q) { return 4 * BOX * q; }             // [BOX] quads
-  static constexpr int rho = 4 * BOX * NQ;                             // [BOX] rho'
-  static constexpr int acc0 = up4(rho + BOX);
+  static constexpr int rho = 4 * BOX * NQ;                             // [RPLANE BZ] rho'
+  static constexpr int acc0 = up4(rho + RPLANE * BZ);
   __host__ __device__ static constexpr int acc(int q) { return acc0 + 4 * CORE * q; }      // [CORE] quads
-  static constexpr int acc_rho = acc0 + 4 * CORE * NQ;                 // [CORE]
-  static constexpr int face0 = up4(acc_rho + CORE);                    // r faces -1 .. TR + 1 of each z: [TZ][TR + 3]
+  static constexpr int acc_rho = acc0 + 4 * CORE * NQ;                 // [CRPLANE TZ]
+  static constexpr int face0 = up4(acc_rho + CRPLANE * TZ);                    // r faces -1 .. TR + 1 of each z: [TZ][TR + 3]
   static constexpr int face1 = face0 + 4 * (TR + 3) * TZ;              // theta faces: [TZ][TR]
-  static constexpr int face2 = face1 + 4 * TR * TZ;                    // z faces -1 .. TZ + 1: [TZ + 3][TR]
-  static constexpr int wgt = face2 + 4 * TR * (TZ + 3);                // [TR + 2][RCW] weights of cells -1 .. TR
+  static constexpr int face2 = face1 + 4 * TR * TZ;                    // z faces -1 .. TZ + 1: [TZ + 3][ZROW]
+  static constexpr int wgt = face2 + 4 * ZROW * (TZ + 3);              // [2][TR + 2] quads: weights of cells -1 .. TR
   static constexpr int area = wgt + RCW * (TR + 2);                    // areas: TR + 1 r faces, TR theta, TR z
   static constexpr int total = up4(area + 3 * TR + 1);
   static constexpr size_t bytes = (size_t)total * sizeof(float);
@@ -147,7 +152,7 @@ struct F32Tile {
           for (int f = 0; f < 4; ++f) v[u][f] = w[f];
         }
         reinterpret_cast<float4*>(sm)[s] = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
-        sm[M::rho + s] = v[u][RHO];
+        sm[M::rho + (zb + u) * M::RPLANE + (y + 2) * M::RROW + (x + 2)] = v[u][RHO];
 #pragma unroll
         for (int b = 5; b < NF; b += 4) {
           const float rd = v[u][b + 3], id = positive(rd) ? recip(rd) : 0.0f;
@@ -164,7 +169,8 @@ struct F32Tile {
     const DevGrid& g = a.g;
     constexpr int N0 = (TR + 3) * TZ, N1 = N0 + TR * TZ, N2 = N1 + TR * (TZ + 3);
     for (int q = threadIdx.x; q < N2; q += NT) {
-      float4* dst = reinterpret_cast<float4*>(sm + M::face0) + q;
+      const int at = q < N1 ? q : N1 + (q - N1) / TR * M::ZROW + (q - N1) % TR;
+      float4* dst = reinterpret_cast<float4*>(sm + M::face0) + at;
       if (!g.has_eq) {
         *dst = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       } else {
@@ -190,7 +196,7 @@ struct F32Tile {
     for (int q = threadIdx.x; q < W + 3 * TR + 1; q += NT) {
       if (q < W) {
         const int c = i0 - 1 + q / (RCW / 4);  // weights of cells -1 .. nr are tabulated
-        copy_async<16>(sm + M::wgt + 4 * q, a.t.rcoef + (size_t)((c > g.nr ? g.nr : c) + 1) * RCW + 4 * (q % (RCW / 4)));
+        copy_async<16>(sm + M::wgt + 4 * (q % (RCW / 4) * (TR + 2) + q / (RCW / 4)), a.t.rcoef + (size_t)((c > g.nr ? g.nr : c) + 1) * RCW + 4 * (q % (RCW / 4)));
       } else {
         const int n = q - W;
         const float* t = n < TR + 1 ? a.t.area_r + clampi(i0 + n, 0, g.nr)
@@ -237,12 +243,13 @@ struct F32Tile {
       if (!__any_sync(FULL, do_face)) return false;  // a warp of lines beyond the edge
     }
     const int s = (z + 2) * M::PLANE + (y + 2) * M::ROW + (x + 2);
-    const int fx = D == 0 ? z * (TR + 3) + x + 1 : (D == 1 ? z * TR + x : (z + 1) * TR + x);
+    const int sr = (z + 2) * M::RPLANE + (y + 2) * M::RROW + (x + 2);
+    const int fx = D == 0 ? z * (TR + 3) + x + 1 : (D == 1 ? z * TR + x : (z + 1) * M::ZROW + x);
     const int core = z * M::CPLANE + y * M::CROW + x;
     float w[RCW];
     if (!UNI) {
-      const float4* q = reinterpret_cast<const float4*>(sm + M::wgt) + 2 * (x + 1);
-      const float4 q0 = q[0], q1 = q[1];
+      const float4* q = reinterpret_cast<const float4*>(sm + M::wgt) + (x + 1);
+      const float4 q0 = q[0], q1 = q[TR + 2];
       w[0] = q0.x; w[1] = q0.y; w[2] = q0.z; w[3] = q0.w;
       w[4] = q1.x; w[5] = q1.y; w[6] = q1.z;
     }
@@ -271,7 +278,7 @@ struct F32Tile {
     if constexpr (M::NQ > 1 && !REDO) dust_flux(1, Fd);
     {
       const float4* ft = reinterpret_cast<const float4*>(sm + M::face(D)) + fx;
-      constexpr int FS = D == 0 ? 1 : (D == 1 ? 0 : TR);  // to the upper face (theta: the same)
+      constexpr int FS = D == 0 ? 1 : (D == 1 ? 0 : M::ZROW);  // to the upper face (theta: the same)
       const float4 fm = ft[0], fp = ft[FS];
       const PEq<float> Em{fm.x, fm.y, fm.z, fm.w};
       float wm[5], wp[5];  // primitive perturbations: right state of the lower face, left state of the upper face
@@ -280,11 +287,12 @@ struct F32Tile {
         {
           const ulonglong2* e = reinterpret_cast<const ulonglong2*>(sm) + s;
           const ulonglong2 em = e[-ST], e0 = e[0], ep = e[ST];
-          const float* r = sm + M::rho + s;
+          constexpr int SR = D == 0 ? 1 : (D == 1 ? M::RROW : M::RPLANE);
+          const float* r = sm + M::rho + sr;
           f32x2 lo[2], up[2];
           parabola2<UNI>(em.x, e0.x, ep.x, w, lo[0], up[0]);
           parabola2<UNI>(em.y, e0.y, ep.y, w, lo[1], up[1]);
-          parabola<UNI>(r[-ST], r[0], r[ST], w, qm[RHO], qp[RHO]);
+          parabola<UNI>(r[-SR], r[0], r[SR], w, qm[RHO], qp[RHO]);
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             unpack2(lo[q], qm[2 * q], qm[2 * q + 1]);
@@ -310,7 +318,7 @@ struct F32Tile {
           qm[1] = qp[1] = e.y;
           qm[2] = qp[2] = e.z;
           qm[3] = qp[3] = e.w;
-          qm[RHO] = qp[RHO] = sm[M::rho + s];
+          qm[RHO] = qp[RHO] = sm[M::rho + sr];
           face_states();
         }
       }
@@ -333,7 +341,7 @@ struct F32Tile {
       add_divergence<WRITE, L>(F, sm + M::acc0, core, do_acc);
       const float Fu = __shfl_down_sync(FULL, F[RHO], 1, L);
       if (do_acc) {
-        float* d = sm + M::acc_rho + core;
+        float* d = sm + M::acc_rho + z * M::CRPLANE + y * M::CRROW + x;
         *d = WRITE ? F[RHO] - Fu : *d + (F[RHO] - Fu);
       }
       if constexpr (M::NQ > 1 && !REDO) {
@@ -427,9 +435,9 @@ struct F32Tile {
       q[3] = v.w;
     };
     quad(s, e);
-    e[RHO] = sm[M::rho + s];
+    e[RHO] = sm[M::rho + (z + 2) * M::RPLANE + (y + 2) * M::RROW + (x + 2)];
     quad(M::acc(0) / 4 + core, G);
-    G[RHO] = sm[M::acc_rho + core];
+    G[RHO] = sm[M::acc_rho + z * M::CRPLANE + y * M::CRROW + x];
 #pragma unroll
     for (int q = 1; q < M::NQ; ++q) {
       quad(M::quad(q) / 4 + s, dust[q - 1]);
