@@ -88,10 +88,11 @@ inline FastDiv fast_div(unsigned d) {
 // blocks apart, so the re-reads hit in L2.
 struct TileOrder {
   FastDiv r, z;  // tiles along r and z
+  int k_first;   // first z index of the tiles (0, or a slab's)
   __device__ __forceinline__ void origin(int tile, int tr, int tt, int tz, int& i0, int& j0, int& k0) const {
     const int rest = r(tile), t = z(rest);
     i0 = (tile - rest * (int)r.d) * tr;
-    k0 = (rest - t * (int)z.d) * tz;
+    k0 = k_first + (rest - t * (int)z.d) * tz;
     j0 = t * tt;
   }
 };

@@ -53,8 +53,10 @@ struct rossbi_grid {
   // library-owned buffers
   void* d_scratch = nullptr;           // E* when the caller passes none
   void* d_hoststate = nullptr;         // device copy for rossbi_step_host
+  cudaStream_t s_in = nullptr, s_out = nullptr;  // its copies, one stream per direction
+  cudaEvent_t host_ev[17] = {};        // slabs copied in [0..7], slabs stepped [8..15], start
   int tiles_r = 0, tiles_t = 0, tiles_z = 0;
-  int tile_tt = 6;                     // theta extent of a stage-kernel tile
+  int tile_tt = 6, tile_tz = 6;        // theta and z extents of a stage-kernel tile
   int tile = TILE_MAIN;                // double forms: which tile
   // perturbation forms: equilibrium and metric tables in the state precision
   void* d_ptab = nullptr;              // one allocation holding every table below
@@ -410,30 +412,19 @@ cudaError_t run_stage_pert(const PertArgs<double>& a, int nblocks, cudaStream_t 
                                  : run_stage_pert_f64_rc<RECON_CONS>(a, nblocks, s, xt);
 }
 
-rossbi_status launch_stage(rossbi_grid* g, const StageArgs& a, int nblocks) {
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (g->profiling && a.mode == 0) {
-    if (g->ev_used == PROFILE_PAIRS) {
-      rossbi_status st = profile_drain(g);
-      if (st != ROSSBI_OK) return st;
-    }
-    e0 = g->ev[2 * g->ev_used];
-    e1 = g->ev[2 * g->ev_used + 1];
-    CK(cudaEventRecord(e0, g->stream));
-  }
-  const bool xt = a.g.x_ind != 0.0 || a.g.damp_k != nullptr || a.drag.law == 2;  // optional terms on
-  CK(run_stage_full(a, nblocks, g->stream, xt));
-  if (e0) {
-    CK(cudaEventRecord(e1, g->stream));
-    g->ev_used++;
-  }
-  return ROSSBI_OK;
+cudaError_t run_stage(const StageArgs& a, int nblocks, cudaStream_t s, bool xt) {
+  return run_stage_full(a, nblocks, s, xt);
+}
+template <class T>
+cudaError_t run_stage(const PertArgs<T>& a, int nblocks, cudaStream_t s, bool xt) {
+  return run_stage_pert(a, nblocks, s, xt);
 }
 
-template <class T>
-rossbi_status launch_pert(rossbi_grid* g, const PertArgs<T>& a, int nblocks) {
+// One launch of the form's stage kernel over nblocks tiles, timed where asked.
+template <class Args>
+rossbi_status launch_stage(rossbi_grid* g, const Args& a, int nblocks, bool timed = true) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (g->profiling) {
+  if (g->profiling && timed) {
     if (g->ev_used == PROFILE_PAIRS) {
       rossbi_status st = profile_drain(g);
       if (st != ROSSBI_OK) return st;
@@ -443,7 +434,7 @@ rossbi_status launch_pert(rossbi_grid* g, const PertArgs<T>& a, int nblocks) {
     CK(cudaEventRecord(e0, g->stream));
   }
   const bool xt = a.g.x_ind != 0.0 || a.g.damp_k != nullptr || a.drag.law == 2;  // optional terms on
-  CK(run_stage_pert(a, nblocks, g->stream, xt));
+  CK(run_stage(a, nblocks, g->stream, xt));
   if (e0) {
     CK(cudaEventRecord(e1, g->stream));
     g->ev_used++;
@@ -468,7 +459,7 @@ StageArgs base_args(rossbi_grid* g) {
   std::memset(&a, 0, sizeof(a));
   a.g = g->dg;
   a.status = g->d_status;
-  a.order = TileOrder{fast_div(g->tiles_r), fast_div(g->tiles_z)};
+  a.order = TileOrder{fast_div(g->tiles_r), fast_div(g->tiles_z), 0};
   a.tile = g->tile;
   return a;
 }
@@ -502,7 +493,7 @@ rossbi_status empty_run(rossbi_grid* g) {
     a.gout = dG;
     a.mode = 1;
     const int nblocks = g->tiles_r * 1 * g->tiles_z;  // one tile along theta
-    st = launch_stage(g, a, nblocks);
+    st = launch_stage(g, a, nblocks, false);
     if (st != ROSSBI_OK) break;
     std::vector<double> G(E0.size());
     if (cudaMemcpyAsync(G.data(), dG, G.size() * sizeof(double), cudaMemcpyDeviceToHost, g->stream) !=
@@ -652,7 +643,7 @@ PertArgs<T> pert_args(rossbi_grid* g) {
   if constexpr (sizeof(T) == 4) a.t = g->pt_f;
   else a.t = g->pt_d;
   a.status = g->d_status;
-  a.order = TileOrder{fast_div(g->tiles_r), fast_div(g->tiles_z)};
+  a.order = TileOrder{fast_div(g->tiles_r), fast_div(g->tiles_z), 0};
   a.sms = g->sms;
   a.tile = g->tile;
   a.gam = (T)g->dg.gamma;
@@ -828,82 +819,137 @@ rossbi_status finish_step(rossbi_grid* g, int nxt, double* next_dt) {
   return next_dt ? read_dt(g, nxt, next_dt) : ROSSBI_OK;
 }
 
-// The two stages of one step (Sect. 2.5) with E* in sc; with the indirect gravity on, the disc
-// moments of each stage's input are summed before it.  Allocates nothing.
-rossbi_status step_full(rossbi_grid* g, void* const* state, void* const* sc, double dt,
-                        const DragArgs& drag, double* next_dt) {
-  const int nblocks = n_tiles(g);
-  const int cur = g->dt_slot, nxt = 1 - g->dt_slot;
-  StageArgs a = base_args(g);
-  a.drag = drag;
+// The arguments of stage `stage2` of a step from `state` in place with E* in
+// sc: stage 1 E* = E^n + dt/2 (G(E^n) - R0)/V, stage 2 E^{n+1} = E^n +
+// dt (G(E*) - R0)/V with the CFL rate fused, each followed by the drag.
+template <class T, class Args>
+void set_stage(rossbi_grid* g, Args& a, void* const* state, void* const* sc, double dt, bool stage2) {
   a.dt_host = dt;
-  a.rate_in = dt == 0.0 ? g->d_dt + cur : nullptr;
-  a.rate_out = g->d_dt + nxt;
-  // stage 1: E* = E^n + dt/2 (G(E^n) - R0)/V, then drag
+  a.rate_in = dt == 0.0 ? g->d_dt + g->dt_slot : nullptr;
+  a.rate_out = g->d_dt + (1 - g->dt_slot);
   for (int f = 0; f < g->nf; ++f) {
-    a.in[f] = (const double*)state[f];
-    a.base[f] = (const double*)state[f];
-    a.out[f] = (double*)sc[f];
+    a.in[f] = (const T*)(stage2 ? sc[f] : state[f]);
+    a.base[f] = (const T*)state[f];
+    a.out[f] = (T*)(stage2 ? state[f] : sc[f]);
   }
-  a.tau_frac = 0.5;
-  a.stage2 = 0;
-  rossbi_status st = g->dg.x_ind != 0.0 ? indirect_moments(g, state) : ROSSBI_OK;
-  if (st == ROSSBI_OK) st = launch_stage(g, a, nblocks);
-  if (st != ROSSBI_OK) return st;
-  if (g->dg.x_ind != 0.0 && (st = indirect_moments(g, sc)) != ROSSBI_OK) return st;
-  // stage 2: E^{n+1} = E^n + dt (G(E*) - R0)/V, then drag; fused CFL and sums
-  for (int f = 0; f < g->nf; ++f) {
-    a.in[f] = (const double*)sc[f];
-    a.base[f] = (const double*)state[f];
-    a.out[f] = (double*)state[f];
-  }
-  a.tau_frac = 1.0;
-  a.stage2 = 1;
-  st = launch_stage(g, a, nblocks);
-  if (st != ROSSBI_OK) return st;
-  return finish_step(g, nxt, next_dt);
+  a.tau_frac = stage2 ? 1.0 : 0.5;
+  a.stage2 = stage2;
 }
 
-template <class T>
-rossbi_status step_pert(rossbi_grid* g, void* const* state, void* const* sc, double dt,
-                        const DragArgs& drag, double* next_dt) {
-  const int nblocks = n_tiles(g);
-  const int cur = g->dt_slot, nxt = 1 - g->dt_slot;
-  PertArgs<T> a = pert_args<T>(g);
-  set_pert_drag(a, drag);
-  a.dt_host = dt;
-  a.rate_in = dt == 0.0 ? g->d_dt + cur : nullptr;
-  a.rate_out = g->d_dt + nxt;
-  for (int f = 0; f < g->nf; ++f) {
-    a.in[f] = (const T*)state[f];
-    a.base[f] = (const T*)state[f];
-    a.out[f] = (T*)sc[f];
-  }
-  a.tau_frac = 0.5;
-  a.stage2 = 0;
-  rossbi_status st = g->dg.x_ind != 0.0 ? indirect_moments(g, state) : ROSSBI_OK;
-  if (st == ROSSBI_OK) st = launch_pert<T>(g, a, nblocks);
-  if (st != ROSSBI_OK) return st;
-  if (g->dg.x_ind != 0.0 && (st = indirect_moments(g, sc)) != ROSSBI_OK) return st;
-  for (int f = 0; f < g->nf; ++f) {
-    a.in[f] = (const T*)sc[f];
-    a.base[f] = (const T*)state[f];
-    a.out[f] = (T*)state[f];
-  }
-  a.tau_frac = 1.0;
-  a.stage2 = 1;
-  st = launch_pert<T>(g, a, nblocks);
-  if (st != ROSSBI_OK) return st;
-  return finish_step(g, nxt, next_dt);
+// Host copies of a step on host buffers.
+struct HostState {
+  void* const* host;
+  void* const* dev;
+};
+
+// The two stages of one step (Sect. 2.5); with the indirect gravity on, the
+// disc moments of each stage's input are summed before it.  Allocates nothing.
+template <class Args>
+rossbi_status run_stages(rossbi_grid* g, const Args& a1, const Args& a2, void* const* state, void* const* sc) {
+  const bool ind = g->dg.x_ind != 0.0;
+  rossbi_status st = ind ? indirect_moments(g, state) : ROSSBI_OK;
+  if (st == ROSSBI_OK) st = launch_stage(g, a1, n_tiles(g));
+  if (st == ROSSBI_OK && ind) st = indirect_moments(g, sc);
+  if (st == ROSSBI_OK) st = launch_stage(g, a2, n_tiles(g));
+  return st;
 }
 
-rossbi_status step_form(rossbi_grid* g, void* const* state, void* const* sc, double dt,
-                        const DragArgs& drag, double* next_dt) {
-  switch (g->desc.precision) {
-    case ROSSBI_FP64: return step_full(g, state, sc, dt, drag, next_dt);
-    case ROSSBI_FP32_PERT: return step_pert<float>(g, state, sc, dt, drag, next_dt);
-    default: return step_pert<double>(g, state, sc, dt, drag, next_dt);
+// Slabs of whole tile layers along z that a host step is cut into: at most 8,
+// each of at least four tiles per SM (fewer leave the last wave of every launch
+// too empty).  One where the layers depend on one another otherwise (periodic
+// in z, the moments of the indirect gravity) or launches are timed.
+int host_slabs(const rossbi_grid* g) {
+  if (g->desc.bc_lo[2] == ROSSBI_BC_PERIODIC || g->dg.x_ind != 0.0 || g->profiling) return 1;
+  return std::max(1, std::min({8, g->tiles_z, n_tiles(g) / (4 * g->sms)}));
+}
+
+rossbi_status ensure_host_streams(rossbi_grid* g) {
+  if (g->s_in) return ROSSBI_OK;
+  for (cudaEvent_t& e : g->host_ev) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  CK(cudaStreamCreateWithFlags(&g->s_out, cudaStreamNonBlocking));
+  CK(cudaStreamCreateWithFlags(&g->s_in, cudaStreamNonBlocking));
+  return ROSSBI_OK;
+}
+
+// The same in slabs along z, each copied in, stepped and copied out on three
+// streams, so that the two directions of the link and the kernels work at the
+// same time (one after the other the copies of a 127 MB state took 1.3 of 2.0
+// ms).  Stage 1 of a slab waits for the next slab's planes (its halo), stage 2
+// of a slab follows stage 1 of the next one, which is also the last to read E^n
+// of this slab.
+template <class Args>
+rossbi_status run_slabs(rossbi_grid* g, const Args& a1, const Args& a2, const HostState& h, int slabs) {
+  const int tz = g->tile_tz, nz = g->desc.nz;
+  const size_t plane = (size_t)g->desc.nr * g->desc.nth * elem_size(g);
+  auto layer = [&](int s) { return (int)((long)g->tiles_z * s / slabs); };
+  auto copy = [&](int s, bool in) -> rossbi_status {
+    const size_t k0 = (size_t)layer(s) * tz, k1 = std::min<size_t>((size_t)layer(s + 1) * tz, nz);
+    for (int f = 0; f < g->nf; ++f) {
+      char* d = (char*)h.dev[f] + k0 * plane;
+      char* c = (char*)h.host[f] + k0 * plane;
+      CK(in ? cudaMemcpyAsync(d, c, (k1 - k0) * plane, cudaMemcpyHostToDevice, g->s_in)
+            : cudaMemcpyAsync(c, d, (k1 - k0) * plane, cudaMemcpyDeviceToHost, g->s_out));
+    }
+    return ROSSBI_OK;
+  };
+  auto stage = [&](Args a, int s) -> rossbi_status {
+    const int layers = layer(s + 1) - layer(s);
+    a.order.z = fast_div(layers);
+    a.order.k_first = layer(s) * tz;
+    if (!a.stage2 && s > 0) a.rate_out = nullptr;  // cleared once
+    return launch_stage(g, a, g->tiles_r * g->tiles_t * layers);
+  };
+  auto finish = [&](int s) -> rossbi_status {  // stage 2 of a slab and its way home
+    rossbi_status st = stage(a2, s);
+    if (st != ROSSBI_OK) return st;
+    CK(cudaEventRecord(g->host_ev[8 + s], g->stream));
+    CK(cudaStreamWaitEvent(g->s_out, g->host_ev[8 + s], 0));
+    return copy(s, false);
+  };
+  CK(cudaEventRecord(g->host_ev[16], g->stream));  // after what the caller's stream holds
+  CK(cudaStreamWaitEvent(g->s_in, g->host_ev[16], 0));
+  rossbi_status st = ROSSBI_OK;
+  for (int s = 0; s < slabs && st == ROSSBI_OK; ++s) {
+    st = copy(s, true);
+    if (st == ROSSBI_OK) CK(cudaEventRecord(g->host_ev[s], g->s_in));
   }
+  for (int s = 0; s < slabs && st == ROSSBI_OK; ++s) {
+    CK(cudaStreamWaitEvent(g->stream, g->host_ev[std::min(s + 1, slabs - 1)], 0));
+    st = stage(a1, s);
+    if (st == ROSSBI_OK && s > 0) st = finish(s - 1);
+  }
+  if (st == ROSSBI_OK) st = finish(slabs - 1);
+  return st;
+}
+
+// One step of the grid's form; h: the state's host copies, to be read before
+// and written after it, or null.
+rossbi_status step_form(rossbi_grid* g, void* const* state, void* const* sc, double dt, const DragArgs& drag,
+                        double* next_dt, const HostState* h = nullptr, int slabs = 1) {
+  const int nxt = 1 - g->dt_slot;
+  auto run = [&](auto a1, auto tag) {
+    using T = decltype(tag);
+    auto a2 = a1;
+    set_stage<T>(g, a1, state, sc, dt, false);
+    set_stage<T>(g, a2, state, sc, dt, true);
+    return h ? run_slabs(g, a1, a2, *h, slabs) : run_stages(g, a1, a2, state, sc);
+  };
+  auto pert = [&](auto tag) {
+    PertArgs<decltype(tag)> a = pert_args<decltype(tag)>(g);
+    set_pert_drag(a, drag);
+    return run(a, tag);
+  };
+  rossbi_status st;
+  if (g->desc.precision == ROSSBI_FP64) {
+    StageArgs a = base_args(g);
+    a.drag = drag;
+    st = run(a, double{});
+  } else if (g->desc.precision == ROSSBI_FP32_PERT) {
+    st = pert(float{});
+  } else {
+    st = pert(double{});
+  }
+  return st == ROSSBI_OK ? finish_step(g, nxt, next_dt) : st;
 }
 
 // ---------------------------------------------------------------- adjoint
@@ -1196,6 +1242,10 @@ void rossbi_destroy(rossbi_grid* g) {
   if (g->d_damp) cudaFree(g->d_damp);
   if (g->h_pinned) cudaFreeHost(g->h_pinned);
   for (cudaEvent_t e : g->ev) cudaEventDestroy(e);
+  for (cudaEvent_t e : g->host_ev)
+    if (e) cudaEventDestroy(e);
+  if (g->s_in) cudaStreamDestroy(g->s_in);
+  if (g->s_out) cudaStreamDestroy(g->s_out);
   delete g;
 }
 
@@ -1218,6 +1268,7 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   // the tile of the form's stage kernel
   auto set_tiles = [&](int tr, int tt, int tz) {
     g->tile_tt = tt;
+    g->tile_tz = tz;
     g->tiles_r = (desc->nr + tr - 1) / tr;
     g->tiles_t = (desc->nth + tt - 1) / tt;
     g->tiles_z = (desc->nz + tz - 1) / tz;
@@ -1486,11 +1537,26 @@ rossbi_status rossbi_step_host(rossbi_grid* g, void* const* host_state, double d
   if (st != ROSSBI_OK) return st;
   const size_t bytes = g->ncell * elem_size(g);
   void* dev[NF_MAX];
-  for (int f = 0; f < g->nf; ++f) {
-    dev[f] = (char*)g->d_hoststate + (size_t)f * bytes;
-    CK(cudaMemcpyAsync(dev[f], host_state[f], bytes, cudaMemcpyHostToDevice, g->stream));
-  }
+  for (int f = 0; f < g->nf; ++f) dev[f] = (char*)g->d_hoststate + (size_t)f * bytes;
   double ndt = 0.0;
+  const int slabs = host_slabs(g);
+  if (slabs > 1) {
+    void* sc[NF_MAX];
+    DragArgs drag;
+    st = prepare_step(g, dev, nullptr, dt, dust, sc, drag);
+    if (st == ROSSBI_OK) st = ensure_host_streams(g);
+    if (st != ROSSBI_OK) return st;
+    const HostState h{host_state, dev};
+    st = step_form(g, dev, sc, dt, drag, &ndt, &h, slabs);
+    // the host buffers are the caller's again, whatever happened
+    const cudaError_t e1 = cudaStreamSynchronize(g->s_in), e2 = cudaStreamSynchronize(g->s_out);
+    CK(e1);
+    CK(e2);
+    if (next_dt) *next_dt = ndt;
+    return st;
+  }
+  for (int f = 0; f < g->nf; ++f)
+    CK(cudaMemcpyAsync(dev[f], host_state[f], bytes, cudaMemcpyHostToDevice, g->stream));
   st = step_device(g, dev, nullptr, dt, dust, &ndt);
   for (int f = 0; f < g->nf; ++f)
     CK(cudaMemcpyAsync(host_state[f], dev[f], bytes, cudaMemcpyDeviceToHost, g->stream));

@@ -376,7 +376,8 @@ __device__ __forceinline__ void publish_tau(double* tau, double frac, double dt_
                                             double cfl) {
   if (threadIdx.x == 0) *tau = frac * (rate_in ? cfl / __longlong_as_double((long long)*rate_in) : dt_host);
 }
-// Stage 1 clears the slot that stage 2 of the step raises.
+// Stage 1 clears the slot that stage 2 of the step raises (in slabs: the first
+// launch does; the host passes no slot to the others of stage 1).
 __device__ __forceinline__ void clear_rate(unsigned long long* rate_out) {
   if (rate_out && blockIdx.x == 0 && threadIdx.x == 0) *rate_out = 0;
 }
