@@ -744,7 +744,7 @@ __global__ void __launch_bounds__(L * NL, 2) adj_flux_kernel(const AdjFluxArgs a
     double U[5], W[5];
 #pragma unroll
     for (int f = 0; f < 5; ++f) U[f] = a.E[f][lin];
-    if (RC == RECON_PRIM) gas_prim(g.gamma, U, W);
+    if (RC == RECON_PRIM) cell_prim_rounded(g.gamma, U, W);
     const double* e0 = RC == RECON_PRIM ? g.w0c : g.e0c;
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
@@ -826,6 +826,12 @@ __global__ void __launch_bounds__(L * NL, 2) adj_flux_kernel(const AdjFluxArgs a
 #pragma unroll
     for (int f = 0; f < 5; ++f)
       br[f] = parabola_branches<UNI>(sv(f, p), sv(f, p + 1), sv(f, p + 2), w, qm[f], qp[f]);
+    if (RC == RECON_PRIM) {
+      double v[9];
+      slope_weights<D>(g, gi, v);
+#pragma unroll
+      for (int f = 0; f < 5; ++f) br[f] = slope_branches(sv(f, p), sv(f, p + 1), sv(f, p + 2), v);
+    }
     auto face_states = [&]() {
       if (g.has_eq) {  // its radial and vertical velocities are zero
 #pragma unroll

@@ -36,6 +36,7 @@ struct DevGrid {
   const double* rc;      // axis-0 cell centres,  index i + GH, i in [-GH, nr + GH)
   const double* rf;      // axis-0 lower faces,   index i + GH, i in [-GH, nr + GH]
   const double* rcoef;   // axis-0 parabola weights for cells i in [-1, nr]: RCW per cell at (i + 1) * RCW
+  const double* rslope;  // axis-0 slopes and distances for slope_branches: 9 per cell at (i + 1) * 9
   const double* vol;     // V(i)
   const double* ivol;    // 1 / V(i)
   const double* area_r;  // A of the axis-0 face i - 1/2, i in [0, nr]
@@ -413,6 +414,20 @@ __device__ __forceinline__ double gas_prim(double g, const double* U, double* W)
   W[EN] = (g - 1.0) * fma(-0.5, fma(U[MU], W[MU], fma(U[MV], W[MV], U[MW] * W[MW])), U[EN]);
   W[RHO] = U[RHO];
   return ir;
+}
+
+// The conversion of a cell that the primitive option takes its departures
+// from, with a rounded division.  Departures can be nothing but this rounding
+// (an isobaric density perturbation has no pressure departure), and then the
+// limiter's branches, which the adjoint differentiates, are decided by it: the
+// arithmetic here and in slope_branches is part of the result.
+__device__ __forceinline__ void cell_prim_rounded(double g, const double* U, double* W) {
+  const double ir = 1.0 / U[RHO];
+  W[MU] = U[MU] * ir;
+  W[MV] = U[MV] * ir;
+  W[MW] = U[MW] * ir;
+  W[EN] = (g - 1.0) * (U[EN] - 0.5 * (U[MU] * U[MU] + U[MV] * U[MV] + U[MW] * U[MW]) * ir);
+  W[RHO] = U[RHO];
 }
 
 // Cotangent Ub of the conservative gas state U for a cotangent Wb of its

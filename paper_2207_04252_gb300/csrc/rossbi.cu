@@ -35,7 +35,7 @@ struct rossbi_grid {
   bool has_disc = false;
   rossbi_disc_params disc{};
   // device tables
-  double *d_rc = nullptr, *d_rf = nullptr, *d_rcoef = nullptr, *d_vol = nullptr, *d_ivol = nullptr;
+  double *d_rc = nullptr, *d_rf = nullptr, *d_rcoef = nullptr, *d_rslope = nullptr, *d_vol = nullptr, *d_ivol = nullptr;
   double *d_area_r = nullptr, *d_area_t = nullptr, *d_area_z = nullptr, *d_aov = nullptr;
   double *d_ir = nullptr, *d_omk = nullptr, *d_grav = nullptr;
   double *d_e0c = nullptr, *d_e0r = nullptr, *d_e0z = nullptr, *d_r0 = nullptr;
@@ -228,7 +228,7 @@ __global__ void eq_prim_kernel(double gamma, const double* e, double* w, size_t 
   for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x) {
     double U[5], W[5];
     for (int f = 0; f < 5; ++f) U[f] = e[f * n + q];
-    gas_prim(gamma, U, W);
+    cell_prim_rounded(gamma, U, W);
     for (int f = 0; f < 5; ++f) w[f * n + q] = W[f];
   }
 }
@@ -1223,7 +1223,7 @@ int rossbi_precision(const rossbi_grid* g) { return g ? g->desc.precision : -1; 
 
 void rossbi_destroy(rossbi_grid* g) {
   if (!g) return;
-  double* tabs[] = {g->d_rc, g->d_rf, g->d_rcoef, g->d_vol, g->d_ivol, g->d_area_r, g->d_area_t,
+  double* tabs[] = {g->d_rc, g->d_rf, g->d_rcoef, g->d_rslope, g->d_vol, g->d_ivol, g->d_area_r, g->d_area_t,
                     g->d_area_z, g->d_aov, g->d_ir, g->d_omk, g->d_grav, g->d_e0c, g->d_e0r, g->d_e0z, g->d_r0, g->d_partials, g->d_sums};
   for (double* p : tabs)
     if (p) cudaFree(p);
@@ -1288,7 +1288,7 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   const int nr = d.nr;
   const double dy = (d.x1[1] - d.x0[1]) / d.nth;
   const double dz = (d.x1[2] - d.x0[2]) / d.nz;
-  std::vector<double> rc(nr + 2 * GH), rf(nr + 2 * GH + 1), rcoef((size_t)(nr + 2) * RCW, 0.0);
+  std::vector<double> rc(nr + 2 * GH), rf(nr + 2 * GH + 1), rcoef((size_t)(nr + 2) * RCW, 0.0), rslope((size_t)(nr + 2) * 9);
   for (int i = -GH; i < nr + GH; ++i) rc[i + GH] = axis0_centre(d, i);
   for (int i = -GH; i <= nr + GH; ++i) rf[i + GH] = axis0_face(d, i);
   for (int i = -1; i <= nr; ++i) {  // parabola weights (Sect. 2.7)
@@ -1307,6 +1307,16 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
     w[4] = hp * (dr - hp) / (dl * dx);
     w[5] = hp * (dl + hp) / (dr * dx);
     w[6] = up / lo;
+    double* v = &rslope[(size_t)(i + 1) * 9];
+    v[0] = 1.0 / (x0 - xm);
+    v[1] = 1.0 / (xp - x0);
+    v[2] = 1.0 / (xp - xm);
+    v[3] = x0 - xm;
+    v[4] = xp - x0;
+    v[5] = fm - x0;
+    v[6] = fp - x0;
+    v[7] = -std::min(2.0 * (x0 - fm), x0 - xm);
+    v[8] = std::min(2.0 * (fp - x0), xp - x0);
   }
   std::vector<double> vol(nr), ivol(nr), ar(nr + 1), at(nr), az(nr), maxA(nr);
   if (d.geometry == ROSSBI_GEOM_CYL) {  // Sect. 2.2 finite volumes of the cylindrical mesh
@@ -1347,6 +1357,7 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
     if ((st = upload(&g->d_rc, rc, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_rf, rf, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_rcoef, rcoef, g->stream)) != ROSSBI_OK) break;
+    if ((st = upload(&g->d_rslope, rslope, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_vol, vol, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_ivol, ivol, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_area_r, ar, g->stream)) != ROSSBI_OK) break;
@@ -1389,6 +1400,7 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   dg.rc = g->d_rc;
   dg.rf = g->d_rf;
   dg.rcoef = g->d_rcoef;
+  dg.rslope = g->d_rslope;
   dg.vol = g->d_vol;
   dg.ivol = g->d_ivol;
   dg.area_r = g->d_area_r;

@@ -103,6 +103,44 @@ __device__ __forceinline__ unsigned parabola_branches(double em, double e0, doub
          (a ? 4u : 0u) | (b ? 8u : 0u);
 }
 
+// The branches (as parabola_branches) decided on slopes: s the minmod slope,
+// the parabola's face deviation against s times the limiter's reach.  v =
+// {1/(x0-xm), 1/(xp-x0), 1/(xp-xm), x0-xm, xp-x0, fm-x0, fp-x0, -h-, h+}.
+// For the adjoint of the primitive option, see cell_prim_rounded; its branches
+// must not depend on how the weights are arranged for speed.
+__device__ __forceinline__ double slope_minmod(double a, double b) {
+  if (a * b <= 0.0) return 0.0;
+  return fabs(a) < fabs(b) ? a : b;
+}
+__device__ __forceinline__ unsigned slope_branches(double em, double e0, double ep, const double* v) {
+  const double sm = (e0 - em) * v[0];
+  const double sp = (ep - e0) * v[1];
+  const double s = slope_minmod(sm, sp);
+  const double a = (sp - sm) * v[2];
+  const double b = (sp * v[3] + sm * v[4]) * v[2];
+  const double A = v[5] * (a * v[5] + b), B = s * v[7];
+  const double C = v[6] * (a * v[6] + b), D = s * v[8];
+  return (sm * sp > 0.0 ? 1u : 0u) | (fabs(sm) < fabs(sp) ? 2u : 0u) | (fabs(A) < fabs(B) ? 4u : 0u) |
+         (fabs(C) < fabs(D) ? 8u : 0u);
+}
+template <int D>
+__device__ __forceinline__ void slope_weights(const DevGrid& g, int gi, double* v) {
+  if (D == 0) {
+    const int c = gi < -1 ? -1 : (gi > g.nr ? g.nr : gi);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) v[q] = g.rslope[(c + 1) * 9 + q];
+  } else {
+    const double h = g.dx[D];
+    v[0] = v[1] = 1.0 / h;
+    v[2] = 0.5 / h;
+    v[3] = v[4] = h;
+    v[5] = -0.5 * h;
+    v[6] = 0.5 * h;
+    v[7] = -h;
+    v[8] = h;
+  }
+}
+
 // Parabola weights of a cell of axis 0 (the uniform axes 1, 2 need none).
 template <class T, int D>
 __device__ __forceinline__ void parabola_weights(const T* rcoef, int gi, int nr, T* w) {
@@ -433,7 +471,7 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
     double U[5], W[5];
 #pragma unroll
     for (int f = 0; f < 5; ++f) U[f] = a.in[f][lin];
-    if (RC == RECON_PRIM) gas_prim(g.gamma, U, W);
+    if (RC == RECON_PRIM) cell_prim_rounded(g.gamma, U, W);
     const double* e0 = RC == RECON_PRIM ? g.w0c : g.e0c;
 #pragma unroll
     for (int f = 0; f < 5; ++f) {
