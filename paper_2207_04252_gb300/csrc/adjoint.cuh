@@ -22,6 +22,14 @@
 // one down by a shuffle, back-propagates its own reconstruction and passes
 // the neighbour contributions up and down by shuffles; every sum has a fixed
 // order, so the result is deterministic.
+//
+// The FP64 pipe bounds the flux kernel.  With six tangents through the Riemann
+// solution it took 255 registers, eight warps per SM and, for a gradient through
+// two bi-fluid steps of 128 x 256 x 32 cells, most of 159 ms; with the closed
+// reverse of the near solution, the gas before the dust (168 registers, twelve
+// warps per SM) and lines by the axis (launch.cuh) the gradient takes 41 ms, a
+// third of it in the flux kernels (1.44, 0.94 and 1.50 ms a stage along r, theta
+// and z), the rest in forward stages and the point kernels.
 #pragma once
 #include "stage_full.cuh"
 
@@ -352,7 +360,7 @@ static __device__ __noinline__ RFaceVjp riemann_vjp_general(double g, double rl,
 // the cotangent of p* passes to the side states through f_L + f_R + u_R - u_L
 // = 0.  About 40 FP64 operations after the forward's 55, where six tangents
 // carried through the solution took over a thousand.
-template <int D>
+template <int D, int RC>
 __device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL, const double* WR, const double* Fb,
                                              double* WLb, double* WRb, unsigned& status) {
   constexpr int n = Axes<D>::n, t1 = Axes<D>::t1, t2 = Axes<D>::t2;
@@ -363,8 +371,16 @@ __device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL
   const FluxCot F{Fb[RHO], Fb[n], Fb[t1], Fb[t2], Fb[EN]};
   const double dP = pr - pl;
   NearStar<double> s;
-  const int kind = near_riemann<true>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, narrow(WL[n]),
+  int kind = near_riemann<true>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, narrow(WL[n]),
                                         narrow(WR[n]), s);
+  // A contact at rest (the wall face beside an equilibrium ghost, both of whose
+  // states the limiter makes the equilibrium's) has its two sides' derivatives
+  // to choose from by nothing but the rounding of u*.  With primitive departures
+  // such faces are usual; the general solver, whose rounding does not depend on
+  // how this one is arranged, decides them.
+  if (RC == RECON_PRIM && kind >= NEAR_STAR_L &&
+      fabsf(narrow(s.us)) <= 1e-14f * sqrtf(narrow(C.gamma) * narrow(pl) / narrow(rl)))
+    kind = NEAR_GENERAL;
   if (kind == NEAR_GENERAL) {
     const RFaceVjp o = riemann_vjp_general(C.gamma, rl, WL[n], pl, WL[t1], WL[t2], rr, WR[n], pr, WR[t1], WR[t2], F);
     status |= o.status;
@@ -823,14 +839,15 @@ __global__ void __launch_bounds__(L * NL, 2) adj_flux_kernel(const AdjFluxArgs a
   bool fallback = false;
   {
     double qm[5], qp[5];
-#pragma unroll
-    for (int f = 0; f < 5; ++f)
-      br[f] = parabola_branches<UNI>(sv(f, p), sv(f, p + 1), sv(f, p + 2), w, qm[f], qp[f]);
     if (RC == RECON_PRIM) {
       double v[9];
       slope_weights<D>(g, gi, v);
 #pragma unroll
-      for (int f = 0; f < 5; ++f) br[f] = slope_branches(sv(f, p), sv(f, p + 1), sv(f, p + 2), v);
+      for (int f = 0; f < 5; ++f) br[f] = slope_branches(sv(f, p), sv(f, p + 1), sv(f, p + 2), v, qm[f], qp[f]);
+    } else {
+#pragma unroll
+      for (int f = 0; f < 5; ++f)
+        br[f] = parabola_branches<UNI>(sv(f, p), sv(f, p + 1), sv(f, p + 2), w, qm[f], qp[f]);
     }
     auto face_states = [&]() {
       if (g.has_eq) {  // its radial and vertical velocities are zero
@@ -890,7 +907,7 @@ __global__ void __launch_bounds__(L * NL, 2) adj_flux_kernel(const AdjFluxArgs a
         Fb[f] = flux_cot(f);
       }
       if (has_face) {
-        gas_flux_vjp<D>(g.near, WL, WR, Fb, ULb, URb, status);
+        gas_flux_vjp<D, RC>(g.near, WL, WR, Fb, ULb, URb, status);
       } else {
 #pragma unroll
         for (int f = 0; f < 5; ++f) ULb[f] = URb[f] = 0.0;

@@ -49,7 +49,7 @@ auto by_tile(int t, F&& f) {
 // and 21), as the FP64 pipe, which bounds these kernels, takes chunks at one
 // rate.  Grids of some thousand main tiles keep the main tile; at 19 main
 // tiles (the Sod tube, 256 x 4 x 4) 15 % of the SMs had all the work: 240 us per
-// step against 30 with the small tile.  More than one dust species: the main
+// step against 92 with the small tile.  More than one dust species: the main
 // tile only (the others are not instantiated).
 template <class T>
 constexpr long tile_chunks() {

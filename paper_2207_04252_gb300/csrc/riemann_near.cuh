@@ -25,7 +25,9 @@
 //
 // What bounds the callers: in FP64 the two-lane FP64 pipe, which sees about
 // 55 operations here against 250 to 300 of the FP64 Newton iteration with its
-// two branches; in float the issue slots.
+// two branches; in float the issue slots.  A step of the gas disc, 128 x 256 x 32
+// cells in double, went from 10.8 to 3.8 ms with this and the parabola of
+// stage_full.cuh; the bi-fluid one in float, 512 x 1024 x 128, from 28.9 to 19.6.
 #pragma once
 #include <cstring>
 

@@ -14,6 +14,18 @@
 // subtracts the balanced residual R0 (Sect. 2.8), applies the RK stage update
 // (Sect. 2.5) and the semi-implicit drag (Sect. 2.9), and in stage 2 fuses the
 // CFL rate of the new state.
+//
+// The FP64 pipe (two lanes per SM and clock) bounds it, at 84 % busy in the main
+// tile, not memory (9 % of a copy's bandwidth).  So what needs no 64-bit rounding
+// runs on the bits or in float (narrow.cuh), the Riemann solution near p_K is a
+// series (riemann_near.cuh), the parabola is two weights per side on
+// differences, divisions are one reciprocal per density, and the tile is the
+// one with the fewest idle lanes that leaves two blocks to an SM (14 x 6 x 6:
+// 1.27 lanes per cell; 14 x 14 x 6 has 1.21, but at one block of 12 warps per SM
+// took 4.69 ms where this takes 4.53).  One step:
+//   gas and dust, 128 x 256 x 32 (with CFL step, copy and sums): 14.4 -> 4.56 ms;
+//   gas disc, 128 x 256 x 32, two steps: 10.8 -> 3.04 ms;
+//   cylindrical explosion, 1600 x 3200: 29.4 -> 8.35 ms.
 #pragma once
 #include "device_common.cuh"
 
@@ -103,16 +115,19 @@ __device__ __forceinline__ unsigned parabola_branches(double em, double e0, doub
          (a ? 4u : 0u) | (b ? 8u : 0u);
 }
 
-// The branches (as parabola_branches) decided on slopes: s the minmod slope,
-// the parabola's face deviation against s times the limiter's reach.  v =
-// {1/(x0-xm), 1/(xp-x0), 1/(xp-xm), x0-xm, xp-x0, fm-x0, fp-x0, -h-, h+}.
-// For the adjoint of the primitive option, see cell_prim_rounded; its branches
-// must not depend on how the weights are arranged for speed.
+// parabola_branches on slopes: s the minmod slope, the parabola's face deviation
+// against s times the limiter's reach.  v = {1/(x0-xm), 1/(xp-x0), 1/(xp-xm),
+// x0-xm, xp-x0, fm-x0, fp-x0, -h-, h+}.  For the adjoint of the primitive option,
+// see cell_prim_rounded: neither its branches nor the rounding of its face values
+// may depend on how the weights are arranged for speed.  (Beside an equilibrium
+// ghost the limited velocity of a wall's face is e0 - e0, whose rounding decides
+// which side of the contact the face takes.)
 __device__ __forceinline__ double slope_minmod(double a, double b) {
   if (a * b <= 0.0) return 0.0;
   return fabs(a) < fabs(b) ? a : b;
 }
-__device__ __forceinline__ unsigned slope_branches(double em, double e0, double ep, const double* v) {
+__device__ __forceinline__ unsigned slope_branches(double em, double e0, double ep, const double* v, double& qm,
+                                                   double& qp) {
   const double sm = (e0 - em) * v[0];
   const double sp = (ep - e0) * v[1];
   const double s = slope_minmod(sm, sp);
@@ -120,6 +135,8 @@ __device__ __forceinline__ unsigned slope_branches(double em, double e0, double 
   const double b = (sp * v[3] + sm * v[4]) * v[2];
   const double A = v[5] * (a * v[5] + b), B = s * v[7];
   const double C = v[6] * (a * v[6] + b), D = s * v[8];
+  qm = e0 + slope_minmod(A, B);
+  qp = e0 + slope_minmod(C, D);
   return (sm * sp > 0.0 ? 1u : 0u) | (fabs(sm) < fabs(sp) ? 2u : 0u) | (fabs(A) < fabs(B) ? 4u : 0u) |
          (fabs(C) < fabs(D) ? 8u : 0u);
 }
