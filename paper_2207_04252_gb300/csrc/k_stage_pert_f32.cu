@@ -27,13 +27,17 @@ cudaError_t launch_nt(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
 }
 
 // Two blocks of 12 warps share an SM where their shared memory allows it (up to
-// nine fields) and there are tiles for them; otherwise one block
-// takes the SM, of 24 warps: more fields (133 KB and up), or a grid of at most one tile per
-// SM (32 x 48 x 32: 207 -> 153 us for four steps).
+// nine fields) and there are tiles for them; otherwise one block of 24 warps
+// takes the SM: more fields (133 KB and up), or a grid of few tiles, where a
+// tile's latency counts more than the overlap of one block's staging with
+// another's sweeps.  Four steps with dust, two narrow blocks against a wide one:
+// 152 tiles 223 / 165 us, 300 230 / 214, 456 308 / 281, 512 319 / 307, 600
+// 346 / 333 (without dust 281 / 288), 760 404 / 409, 912 436 / 484, 4800
+// 1808 / 2254; the line lies at three tiles per SM of 152.
 template <int NF, class P, bool XT, int RC>
 cudaError_t launch(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
   if constexpr (NF <= 9) {
-    if (nblocks > a.sms) return launch_nt<NF, P32_NT, P32_MINB, P, XT, RC>(a, nblocks, s);
+    if (nblocks > 3 * a.sms) return launch_nt<NF, P32_NT, P32_MINB, P, XT, RC>(a, nblocks, s);
   }
   return launch_nt<NF, P32_WIDE_NT, 1, P, XT, RC>(a, nblocks, s);
 }
