@@ -94,9 +94,12 @@ def _traffic(kernel_tag, cells):
 
 
 KERNEL_SOURCES = {  # files that define the kernel and its launcher, and the launch-configuration line's token
-    "stage_fp32": (("device_common.cuh", "stage_full.cuh", "stage_pert.cuh", "k_stage_pert_f32.cu"), "P32_TR ="),
-    "stage_fp64pert": (("device_common.cuh", "stage_full.cuh", "stage_pert.cuh", "k_stage_pert_f64.cu"), "P32_TR ="),
-    "stage_fp64": (("device_common.cuh", "stage_full.cuh", "k_stage_full.cu"), "F64_TR ="),
+    "stage_fp32": (("device_common.cuh", "narrow.cuh", "riemann_near.cuh", "stage_full.cuh", "stage_pert.cuh",
+                    "stage_f32.cuh", "k_stage_pert_f32.cu"), "P32_TR ="),
+    "stage_fp64pert": (("device_common.cuh", "narrow.cuh", "riemann_near.cuh", "stage_full.cuh", "stage_pert.cuh",
+                        "k_stage_pert_f64.cu"), "using TileMain ="),
+    "stage_fp64": (("device_common.cuh", "narrow.cuh", "riemann_near.cuh", "stage_full.cuh", "k_stage_full.cu"),
+                   "using TileMain ="),
 }
 
 
@@ -596,7 +599,7 @@ def run_ours(args):
                            "l2": "inputs larger than L2 (no flush needed)", "indirect_x_ref": args.indirect,
                            "recon": args.recon},
                 "roofline": roofline, "roofline_issue": roofline_issue, "roofline_alu": roofline_alu, "e2e": e2e,
-                "gpu_launches": (7 if args.indirect else 3) * args.steps, "clocks": clocks,
+                "gpu_launches": (6 if args.indirect else 2) * args.steps, "clocks": clocks,
                 "status": R.status_string(status)}
         if args.precision == "fp32" and not args.no_extras:
             fp64 = measure_fp64(R, workloads, w, torch)
