@@ -16,15 +16,15 @@
 // CFL rate of the new state.
 //
 // The FP64 pipe (two lanes per SM and clock) bounds it, at 84 % busy in the main
-// tile, not memory (9 % of a copy's bandwidth).  So what needs no 64-bit rounding
+// tile, not memory (2 % of a copy's bandwidth).  So what needs no 64-bit rounding
 // runs on the bits or in float (narrow.cuh), the Riemann solution near p_K is a
 // series (riemann_near.cuh), the parabola is two weights per side on
 // differences, divisions are one reciprocal per density, and the tile is the
 // one with the fewest idle lanes that leaves two blocks to an SM (14 x 6 x 6:
 // 1.27 lanes per cell; 14 x 14 x 6 has 1.21, but at one block of 12 warps per SM
 // took 4.69 ms where this takes 4.53).  One step:
-//   gas and dust, 128 x 256 x 32 (with CFL step, copy and sums): 14.4 -> 4.56 ms;
-//   gas disc, 128 x 256 x 32, two steps: 10.8 -> 3.04 ms;
+//   gas and dust, 128 x 256 x 32: 14.4 -> 4.53 ms;
+//   gas disc, 128 x 256 x 32, with the next step's dt and the sums: 10.8 -> 3.03 ms;
 //   cylindrical explosion, 1600 x 3200: 29.4 -> 8.35 ms.
 #pragma once
 #include "device_common.cuh"
