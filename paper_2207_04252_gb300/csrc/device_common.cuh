@@ -399,10 +399,6 @@ static __device__ __noinline__ RFace riemann_general(double g, double rl, double
   return o;
 }
 
-__device__ __forceinline__ double gas_pressure(double g, double mu, double mv, double mw, double en, double rho) {
-  return (g - 1.0) * (en - 0.5 * (mu * mu + mv * mv + mw * mw) / rho);
-}
-
 // Primitive gas state (u, v, w, P, rho), in the field slots MU, MV, MW, EN,
 // RHO, of a conservative gas state; returns 1 / rho (NaN for rho = 0, which
 // leaves a P that fails every positivity test).

@@ -648,7 +648,6 @@ PertArgs<T> pert_args(rossbi_grid* g) {
   a.tile = g->tile;
   a.gam = (T)g->dg.gamma;
   a.om = (T)g->dg.omega;
-  a.cfl = (T)g->dg.cfl;
   a.gm1 = (T)(g->dg.gamma - 1.0);
   a.g_gm1 = (T)g->dg.near.g_gm1;
   return a;

@@ -427,7 +427,7 @@ struct PertArgs {
   // the grid's and the drag's parameters in the state precision, converted
   // once on the host (GB300's FP64 pipe is narrow: per-use conversions of the
   // double originals cost latency in the float kernel)
-  T gam, gm1, g_gm1, om, cfl, kappa;
+  T gam, gm1, g_gm1, om, kappa;
   T ist[ND_MAX], irr[ND_MAX];  // 1 / (St x factor), 1 / (rho_s r_p x factor) of each dust species
 };
 
