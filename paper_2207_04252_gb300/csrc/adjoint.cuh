@@ -506,7 +506,7 @@ __device__ __forceinline__ double drag_vjp(const DevGrid& g, int i, const double
   const double ig = recip(rg), id = recip(rd);
   double P = 0.0;
   if (d.law != 0) P = (g.gamma - 1.0) * fma(-0.5 * ig, fma(U[MU], U[MU], fma(U[MV], U[MV], U[MW] * U[MW])), U[EN]);
-  const double a = tau * inv_stopping_time<true>(g, i, rg, P, d, 0);
+  const double a = tau * inv_stopping_time<true>(g, i, rg, ig, P, d, 0);
   // the momentum that changes hands is K (v_d - v_g), K = rho_d a / (1 + k),
   // k = a (1 + rho_d / rho_g)
   const double eps = rd * ig, q = recip(1.0 + fma(a, eps, a)), aq = a * q, K = rd * aq;

@@ -581,16 +581,16 @@ struct DragArgs {
 };
 
 // 1 / t_s of dust species s (Stokes number St x st_factor[s]) in a cell of
-// radial index i with gas density rg and pressure P (Sect. 2.9): drag law 0
+// radial index i with gas density rg (ig = 1 / rg) and pressure P (Sect. 2.9): drag law 0
 // t_s = St / Omega_K(r) (the Box: St); laws 1 and 2 Epstein t_s = rho_s r_p /
-// (rho_g c_s), rho_s r_p proportional to St, with rho_g c_s = sqrt(gamma P
-// rho_g); law 2 (compiled in with XT) adds the Stokes regime of Sect. 2.9:
+// (rho_g c_s), rho_s r_p proportional to St, with c_s = sqrt(gamma P / rho_g)
+// (gamma P rho_g underflows in a thin atmosphere); law 2 (compiled in with XT) adds the Stokes regime of Sect. 2.9:
 // above r_p = 9 lambda / 4 the Epstein time grows by (4/9) r_p / lambda.
 template <bool XT>
-__device__ __forceinline__ double inv_stopping_time(const DevGrid& g, int i, double rg, double P, const DragArgs& d,
-                                                    int s) {
+__device__ __forceinline__ double inv_stopping_time(const DevGrid& g, int i, double rg, double ig, double P,
+                                                    const DragArgs& d, int s) {
   if (d.law == 0) return g.omk[i] * d.ist[s];
-  double it = root(g.gamma * P * rg) * d.irr[s];
+  double it = rg * root(g.gamma * P * ig) * d.irr[s];
   if (XT && d.law == 2) {
     const double x = d.kappa * rg;
     if (positive(x - 2.25)) it *= 2.25 * recip(x);
@@ -619,7 +619,7 @@ __device__ __forceinline__ void apply_drag(const DevGrid& g, int i, double* U, d
   if constexpr (ND == 1) {
     const double rd = U[DRHO];
     if (!positive(rd)) return;
-    const double a = tau * inv_stopping_time<XT>(g, i, rg, P, d, 0);
+    const double a = tau * inv_stopping_time<XT>(g, i, rg, ig, P, d, 0);
     const double K = rd * a * recip(1.0 + fma(a * rd, ig, a));
     double dE = 0.0;
 #pragma unroll
@@ -640,7 +640,7 @@ __device__ __forceinline__ void apply_drag(const DevGrid& g, int i, double* U, d
       const int b = 5 + 4 * s;
       a[s] = h[s] = 0.0;
       if (!positive(U[b + 3])) continue;
-      a[s] = tau * inv_stopping_time<XT>(g, i, rg, P, d, s);
+      a[s] = tau * inv_stopping_time<XT>(g, i, rg, ig, P, d, s);
       h[s] = recip(1.0 + a[s]);
       const double w = a[s] * h[s];
       den = fma(U[b + 3], w, den);

@@ -27,6 +27,9 @@ __device__ __forceinline__ bool non_negative(double x) {
 }
 __device__ __forceinline__ bool non_negative(float x) { return x >= 0.0f; }
 
+// x is a positive normal number (not subnormal, infinite or NaN).
+__device__ __forceinline__ bool positive_normal(double x) { return (unsigned)((__double2hiint(x) >> 20) - 1) < 0x7feu; }
+
 // |a| < |b| (magnitudes of non-NaN values order like their bits).
 __device__ __forceinline__ bool mag_less(double a, double b) {
   return (__double_as_longlong(a) & 0x7fffffffffffffffll) < (__double_as_longlong(b) & 0x7fffffffffffffffll);
@@ -114,14 +117,21 @@ __device__ __forceinline__ double refine_recip(double x, double y) { return fma(
 __device__ __forceinline__ double refine_recip_sqrt(double x, double y) {
   return fma(scale_down<1>(y), fma(-(x * y), y, 1.0), y);
 }
-// sqrt(x), x > 0
+// sqrt(x) of any x.  Squares of slow velocities underflow, so subnormal
+// arguments are ordinary ones here, and the approximation flushes them to an
+// infinite x^-1/2; the float form is the hardware's root of every value.
 __device__ __forceinline__ double root(double x) {
+  if (!positive_normal(x)) return sqrt(x);
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double t = x * y, e = fma(-t, y, 1.0);
   return fma(t * e, fma(0.375, e, 0.5), t);
 }
-__device__ __forceinline__ float root(float x) { return x * recip_sqrt(x); }
+__device__ __forceinline__ float root(float x) {
+  float y;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 
 // ---------------------------------------------------------------- two floats at a time (the packed arithmetic of sm_100 and later)
 typedef unsigned long long f32x2;

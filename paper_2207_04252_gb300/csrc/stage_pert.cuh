@@ -652,11 +652,11 @@ __device__ __forceinline__ void pert_sources(const PertArgs<T>& a, const PCell<T
 }
 
 // 1 / t_s of dust species s in a perturbation-form cell (as inv_stopping_time
-// of the full-state kernel; gas density rg, pressure p).
+// of the full-state kernel; gas density rg, ig = 1 / rg, pressure p).
 template <class T, bool XT>
-__device__ __forceinline__ T pert_inv_stopping_time(const PertArgs<T>& a, int i, T rg, T p, int s) {
+__device__ __forceinline__ T pert_inv_stopping_time(const PertArgs<T>& a, int i, T rg, T ig, T p, int s) {
   if (a.drag.law == 0) return a.t.omk[i] * a.ist[s];
-  T it = root(a.gam * p * rg) * a.irr[s];
+  T it = rg * root(a.gam * p * ig) * a.irr[s];
   if (XT && a.drag.law == 2) {  // Stokes regime of Sect. 2.9 above r_p = 9 lambda / 4
     const T x = a.kappa * rg;
     if (positive(x - T(2.25))) it *= T(2.25) * recip(x);
@@ -687,7 +687,7 @@ __device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& 
   if constexpr (NF == 9) {
     const T rd = q[DRHO];
     if (!positive(rd)) return;
-    const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, p, 0);
+    const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, ig, p, 0);
     const T K = rd * ak * recip(T(1) + ak * (T(1) + rd * ig));
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -706,7 +706,7 @@ __device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& 
       const T rd = q[b + 3];
       wk[s] = T(0);
       if (!positive(rd)) continue;
-      const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, p, s);
+      const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, ig, p, s);
       wk[s] = ak * recip(T(1) + ak);
       den += rd * wk[s];
 #pragma unroll
