@@ -371,15 +371,15 @@ __device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL
   const FluxCot F{Fb[RHO], Fb[n], Fb[t1], Fb[t2], Fb[EN]};
   const double dP = pr - pl;
   NearStar<double> s;
-  int kind = near_riemann<true>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, narrow(WL[n]),
-                                        narrow(WR[n]), s);
+  int kind = near_riemann<true>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, WL[n],
+                                        WR[n], s);
   // A contact at rest (the wall face beside an equilibrium ghost, both of whose
   // states the limiter makes the equilibrium's) has its two sides' derivatives
   // to choose from by nothing but the rounding of u*.  With primitive departures
   // such faces are usual; the general solver, whose rounding does not depend on
   // how this one is arranged, decides them.
   if (RC == RECON_PRIM && kind >= NEAR_STAR_L &&
-      fabsf(narrow(s.us)) <= 1e-14f * sqrtf(narrow(C.gamma) * narrow(pl) / narrow(rl)))
+      fabsf(narrow(s.us)) <= 1e-14f * narrow(C.gamma * (pl * s.ircl)))
     kind = NEAR_GENERAL;
   if (kind == NEAR_GENERAL) {
     const RFaceVjp o = riemann_vjp_general(C.gamma, rl, WL[n], pl, WL[t1], WL[t2], rr, WR[n], pr, WR[t1], WR[t2], F);

@@ -67,19 +67,22 @@ __device__ __forceinline__ float min_xorsign(float a, float b) {
 
 // double -> float by truncation, flushed to 0 below and held at FLT_MAX above
 // float's range; float -> double, exact for normal values, subnormals to 0.
-__device__ __forceinline__ float narrow(double x) {
+// `bias` other than the formats' own 896 scales by a power of two on the way,
+// narrow(x, 896 + k) = x / 2^k and widen(y, 896 + k) = y 2^k (0 < bias < 1792:
+// zero stays zero, and the widened value is a normal number).
+constexpr int FLOAT_BIAS = 896;
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ float narrow(double x, int bias = FLOAT_BIAS) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned e = (hi >> 20) & 0x7ffu;
-  unsigned b = __funnelshift_l(lo, hi & 0x7fffffffu, 3) - (896u << 23);
-  b = e - 897u < 254u ? b & 0x7fffffffu : (e < 897u ? 0u : 0x7f7fffffu);
+  const int e = exponent(x) - bias;
+  unsigned b = __funnelshift_l(lo, hi & 0x7fffffffu, 3) - ((unsigned)bias << 23);
+  b = (unsigned)(e - 1) < 254u ? b & 0x7fffffffu : (e < 1 ? 0u : 0x7f7fffffu);
   return __uint_as_float(b | (hi & 0x80000000u));
 }
 __device__ __forceinline__ float narrow(float x) { return x; }
-template <class T> __device__ __forceinline__ T widen(float x);
-template <> __device__ __forceinline__ float widen<float>(float x) { return x; }
-template <> __device__ __forceinline__ double widen<double>(float x) {
+__device__ __forceinline__ double widen(float x, int bias = FLOAT_BIAS) {
   const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-  const unsigned hi = m < 0x00800000u ? 0u : (m >> 3) + (896u << 20);
+  const unsigned hi = m < 0x00800000u ? 0u : (m >> 3) + ((unsigned)bias << 20);
   return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(m < 0x00800000u ? 0u : b << 29));
 }
 

@@ -118,7 +118,7 @@ __device__ __forceinline__ double near_sum(const double (&c)[2][NEAR_N], const f
   float t = shock ? ct[1][NEAR_T - 1] : ct[0][NEAR_T - 1];
 #pragma unroll
   for (int k = NEAR_T - 2; k >= 0; --k) t = fmaf(t, xf, shock ? ct[1][k] : ct[0][k]);
-  double v = widen<double>(t);
+  double v = widen(t);
 #pragma unroll
   for (int k = NEAR_N - 1; k >= 2; --k) v = fma(v, x, shock ? c[1][k] : c[0][k]);
   return fma(fma(v, x, c[0][1]), x, c[0][0]);
@@ -142,25 +142,33 @@ struct NearStar {
 // a fan or a shock may sit on the face; the caller then takes the general
 // solver.  (rl, pl), (rr, pr): densities and pressures (a float state that is
 // not positive comes back as NEAR_GENERAL; a double one is the caller's to sort out); dP = p_R -
-// p_L, ul, ur velocities about u0, dU = u_R - u_L; ulf, urf the full
-// velocities in float.
+// p_L, ul, ur velocities about u0, dU = u_R - u_L; vl, vr the full
+// velocities.
 // EXACT_INV: s.irc and s.ip rounded to the last bits (the adjoint's use of
 // them). The solution itself takes them to about 2^-43: they multiply p* - p_K,
 // at most 2^-7 p, so the star state keeps its last bits; one Newton step each
 // from the float values, five and two FP64 operations instead of seven and three.
 template <bool EXACT_INV = false>
 __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double ul, double pl, double rr, double ur,
-                                            double pr, double dP, double dU, double u0, bool has_u0, float ulf,
-                                            float urf, NearStar<double>& s) {
+                                            double pr, double dP, double dU, double u0, bool has_u0, double vl,
+                                            double vr, NearStar<double>& s) {
   using T = double;
-  const float plf = narrow(pl), prf = narrow(pr), rlf = narrow(rl), rrf = narrow(rr);
-  // doubles beyond float's comfortable range: the general solver
-  if (!(fmaxf(fmaxf(plf, prf), fmaxf(rlf, rrf)) < 1e30f)) return NEAR_GENERAL;
+  // The float work is in units in which p_L and the sound speed are of order
+  // one: pressures by 2^k (bias bp), velocities by 2^m (bias bu), densities by
+  // 2^(k - 2m).  In the caller's units the small steps of a small pressure would
+  // be below float's range.  p and rho beyond 2^500, whose product may leave
+  // the range of double, and densities 2^80 apart go to the general solver.
+  const int ep = exponent(pl), er = exponent(rl);
+  if ((unsigned)(ep - 523) > 1000u || (unsigned)(er - 523) > 1000u) return NEAR_GENERAL;
+  const int m = (ep - er) >> 1, bp = ep - 127, bu = FLOAT_BIAS + m, br = bp - 2 * m;
+  const float plf = narrow(pl, bp), prf = narrow(pr, bp), rlf = narrow(rl, br), rrf = narrow(rr, br);
+  if (!(rrf > 0x1p-80f && rrf < 0x1p80f)) return NEAR_GENERAL;
+  const float ulf = narrow(vl, bu), urf = narrow(vr, bu);
   const float gl = C.gammaf * plf, gr = C.gammaf * prf;
   const float il = recip_sqrt(gl) * recip_sqrt(rlf), ir = recip_sqrt(gr) * recip_sqrt(rrf);  // 1 / (rho c)
   const float cl = gl * il, cr = gr * ir;
   const float ipl = recip(plf), ipr = recip(prf);
-  const float dPf = narrow(dP), dUf = narrow(dU);
+  const float dPf = narrow(dP, bp), dUf = narrow(dU, bu);
   // linear (acoustic) star pressure d = p* - p_L
   float d = (dPf * ir - dUf) * recip(il + ir);
   float xl = d * ipl, xr = (d - dPf) * ipr;
@@ -188,12 +196,13 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
       s.ipl = recip(pl);
       s.ipr = recip(pr);
     } else {
-      s.ircl = refine_recip_sqrt(C.gamma * (pl * rl), widen<T>(il));
-      s.ircr = refine_recip_sqrt(C.gamma * (pr * rr), widen<T>(ir));
-      s.ipl = refine_recip(pl, widen<T>(ipl));
-      s.ipr = refine_recip(pr, widen<T>(ipr));
+      const int bq = 2 * FLOAT_BIAS - bp, bi = bq + m;  // of 1/p, 1/(rho c)
+      s.ircl = refine_recip_sqrt(C.gamma * (pl * rl), widen(il, bi));
+      s.ircr = refine_recip_sqrt(C.gamma * (pr * rr), widen(ir, bi));
+      s.ipl = refine_recip(pl, widen(ipl, bq));
+      s.ipr = refine_recip(pr, widen(ipr, bq));
     }
-    T dd = widen<T>(d), f1 = T(0), f2 = T(0);
+    T dd = widen(d, bp), f1 = T(0), f2 = T(0);
     float step = 0.0f;
     bool more = true;
     for (int it = 0; it < 4 && more; ++it) {
@@ -202,14 +211,14 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
       const bool sl = !sign_bit(yl), sr = !sign_bit(yr);
       f1 = dd * s.ircl * near_sum(C.s, C.st, sl, yl);
       f2 = dr * s.ircr * near_sum(C.s, C.st, sr, yr);
-      step = -narrow(f1 + f2 + dU) * iD;
-      dd += widen<T>(step);
+      step = -narrow(f1 + f2 + dU, bu) * iD;
+      dd += widen(step, bp);
       more = !(fabsf(step) <= small);
     }
     if (more) return NEAR_GENERAL;
     s.d = dd;
-    s.fl = f1 + widen<T>(tl * step);
-    s.fr = f2 + widen<T>(tr * step);
+    s.fl = f1 + widen(tl * step, bu);
+    s.fr = f2 + widen(tr * step, bu);
     s.us = ul - s.fl;
   }
   // u* = u_L - f_L = u_R + f_R: the side that the face lies on gives it

@@ -466,7 +466,7 @@ __device__ __forceinline__ bool pert_face(const PertArgs<T>& a, const PEq<T>& Em
   int kind = NEAR_GENERAL;
   if (sizeof(T) == 4 || (positive(rl) && positive(rr) && positive(pl) && positive(pr)))
     kind = near_riemann(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
-                           narrow(un0 + wl[n]), narrow(un0 + wm[n]), st);
+                           un0 + wl[n], un0 + wm[n], st);
   if (!GENERAL && kind == NEAR_GENERAL) return true;
   const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
   T d[3], drho = left ? wl[RHO] : wm[RHO], dp = left ? wl[EN] : wm[EN];
