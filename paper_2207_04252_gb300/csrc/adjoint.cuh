@@ -371,7 +371,7 @@ __device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL
   const FluxCot F{Fb[RHO], Fb[n], Fb[t1], Fb[t2], Fb[EN]};
   const double dP = pr - pl;
   NearStar<double> s;
-  int kind = near_riemann<true>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, WL[n],
+  int kind = near_riemann<NEAR_INVERSES>(C, rl, WL[n], pl, rr, WR[n], pr, dP, WR[n] - WL[n], 0.0, false, WL[n],
                                         WR[n], s);
   // A contact at rest (the wall face beside an equilibrium ghost, both of whose
   // states the limiter makes the equilibrium's) has its two sides' derivatives

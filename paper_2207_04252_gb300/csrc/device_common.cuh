@@ -467,7 +467,7 @@ __device__ __forceinline__ void gas_face_flux(const NearCoef& C, double area, co
     return;
   }
   NearStar<double> s;
-  const int kind = near_riemann(C, WL[RHO], WL[n], WL[EN], WR[RHO], WR[n], WR[EN], WR[EN] - WL[EN],
+  const int kind = near_riemann<NEAR_STATE>(C, WL[RHO], WL[n], WL[EN], WR[RHO], WR[n], WR[EN], WR[EN] - WL[EN],
                                         WR[n] - WL[n], 0.0, false, WL[n], WR[n], s);
   const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
   double rho = left ? WL[RHO] : WR[RHO], u = left ? WL[n] : WR[n], p = left ? WL[EN] : WR[EN];

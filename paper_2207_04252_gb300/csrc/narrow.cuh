@@ -115,7 +115,7 @@ __device__ __forceinline__ float recip_sqrt(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// One Newton step of 1/x and x^-1/2 from y (error squared: 2^-22 -> 2^-43).
+// One Newton step of 1/x and x^-1/2 from y (error e of y: e^2 and 3 e^2 / 2).
 __device__ __forceinline__ double refine_recip(double x, double y) { return fma(y, fma(-x, y, 1.0), y); }
 __device__ __forceinline__ double refine_recip_sqrt(double x, double y) {
   return fma(scale_down<1>(y), fma(-(x * y), y, 1.0), y);

@@ -17,9 +17,23 @@
 // In double the Newton iteration runs in float and its result is corrected by
 // FP64 residuals: step = -F/F' with F in FP64 and the quotient in float.  A
 // step has a relative error of about 2^-22, so the iteration ends once it is
-// below 2^-31 p (one evaluation of F for |x| up to about 2^-9, two beyond)
-// and p* is then exact to the last bits, as the FP64 iteration's is.  The
-// series are summed in double to x^3, the rest (below 2^-30 of the sum at
+// below 2^-31 p (one evaluation of F for |x| up to about 2^-9, two beyond).
+// What the caller does with the solution sets how far it is taken:
+//   NEAR_STATE       the star state.  1/(rho c) and 1/p to about 2^-42, one Newton
+//                    step from the float values (five and two FP64 operations
+//                    instead of seven and three): they multiply p* - p_K, so p* is
+//                    within 2^-53 p + 2^-42 |p* - p_K| (2^-49 p at |x| = 1/128);
+//   NEAR_INVERSES    the same with 1/(rho c) and 1/p to their last bits (the adjoint);
+//   NEAR_DEPARTURES  p* - p_K, u* - u_K and rho* - rho_K to their own last bits (the
+//                    perturbation forms, whose result they are): the linear
+//                    solution is taken in FP64, the float iteration gives only
+//                    what S - 1 adds to it (|x| of it and less, and nothing that
+//                    float's range could lose), and the residuals go on to 2^-31
+//                    of the larger |p* - p_K|: one evaluation for |x| up to about
+//                    2^-10.  Twelve FP64 operations a face more than NEAR_STATE, 1.7 %
+//                    of a step of 93 x 131 x 37 bi-fluid cells (2.64 -> 2.69 ms); a
+//                    second evaluation in place of the linear solution took 4.8 %.
+// The series are summed in double to x^3, the rest (below 2^-30 of the sum at
 // |x| = 1/128) in float: 1/128 is where float's rounding of the tail reaches
 // 2^-54 of the sum; each power of two more takes another FP64 term per sum.
 //
@@ -98,12 +112,16 @@ inline NearCoef near_coef(double gamma) {
   return c;
 }
 
-// Float series to x^4; the branches share the first two coefficients.
-__device__ __forceinline__ float near_sum_f(const float (&c)[2][5], bool shock, float x) {
+// Float series to x^4, less its constant and over x; the branches share the
+// first two coefficients.
+__device__ __forceinline__ float near_slope_f(const float (&c)[2][5], bool shock, float x) {
   float t = shock ? c[1][4] : c[0][4];
 #pragma unroll
   for (int k = 3; k >= 2; --k) t = fmaf(t, x, shock ? c[1][k] : c[0][k]);
-  return fmaf(fmaf(t, x, c[0][1]), x, c[0][0]);
+  return fmaf(t, x, c[0][1]);
+}
+__device__ __forceinline__ float near_sum_f(const float (&c)[2][5], bool shock, float x) {
+  return fmaf(near_slope_f(c, shock, x), x, c[0][0]);
 }
 // The same to x^3 (truncation below 2^-26 at |x| = 1/64).
 template <int N>
@@ -126,6 +144,8 @@ __device__ __forceinline__ double near_sum(const double (&c)[2][NEAR_N], const f
 
 enum { NEAR_GENERAL = 0, NEAR_LEFT = 1, NEAR_RIGHT = 2, NEAR_STAR_L = 3, NEAR_STAR_R = 4 };
 
+enum { NEAR_STATE, NEAR_INVERSES, NEAR_DEPARTURES };
+
 // What the solution needs beyond the face state (the adjoint reads it).
 template <class T>
 struct NearStar {
@@ -144,11 +164,7 @@ struct NearStar {
 // not positive comes back as NEAR_GENERAL; a double one is the caller's to sort out); dP = p_R -
 // p_L, ul, ur velocities about u0, dU = u_R - u_L; vl, vr the full
 // velocities.
-// EXACT_INV: s.irc and s.ip rounded to the last bits (the adjoint's use of
-// them). The solution itself takes them to about 2^-43: they multiply p* - p_K,
-// at most 2^-7 p, so the star state keeps its last bits; one Newton step each
-// from the float values, five and two FP64 operations instead of seven and three.
-template <bool EXACT_INV = false>
+template <int WHAT>
 __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double ul, double pl, double rr, double ur,
                                             double pr, double dP, double dU, double u0, bool has_u0, double vl,
                                             double vr, NearStar<double>& s) {
@@ -178,6 +194,18 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
   if (ulf >= 1.1f * cl) return NEAR_LEFT;
   if (-urf >= 1.1f * cr) return NEAR_RIGHT;
   if (!(X <= NEAR_XD)) return NEAR_GENERAL;
+  if (WHAT == NEAR_STATE) {
+    const int bq = 2 * FLOAT_BIAS - bp, bi = bq + m;  // of 1/p, 1/(rho c)
+    s.ircl = refine_recip_sqrt(C.gamma * (pl * rl), widen(il, bi));
+    s.ircr = refine_recip_sqrt(C.gamma * (pr * rr), widen(ir, bi));
+    s.ipl = refine_recip(pl, widen(ipl, bq));
+    s.ipr = refine_recip(pr, widen(ipr, bq));
+  } else {
+    s.ircl = recip_sqrt(C.gamma * (pl * rl));
+    s.ircr = recip_sqrt(C.gamma * (pr * rr));
+    s.ipl = recip(pl);
+    s.ipr = recip(pr);
+  }
   {
     float tl = 0.0f, tr = 0.0f;
 #pragma unroll
@@ -189,20 +217,18 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
       tr = ir * near_sum_f(C.tf, sr, xr);
       d -= (d * il * near_sum_f(C.sf, sl, xl) + (d - dPf) * ir * near_sum_f(C.sf, sr, xr) + dUf) * recip(tl + tr);
     }
-    const float iD = recip(tl + tr), small = 4.6e-10f * fminf(plf, prf);
-    if constexpr (EXACT_INV) {
-      s.ircl = recip_sqrt(C.gamma * (pl * rl));
-      s.ircr = recip_sqrt(C.gamma * (pr * rr));
-      s.ipl = recip(pl);
-      s.ipr = recip(pr);
+    const float iD = recip(tl + tr);
+    const float small = 4.6e-10f * (WHAT == NEAR_DEPARTURES ? fmaxf(fabsf(d), fabsf(d - dPf)) : fminf(plf, prf));
+    T dd, f1 = T(0), f2 = T(0);
+    if (WHAT == NEAR_DEPARTURES) {
+      xl = d * ipl;
+      xr = (d - dPf) * ipr;
+      const float ql = d * il * (xl * near_slope_f(C.sf, d > 0.0f, xl));
+      const float qr = (d - dPf) * ir * (xr * near_slope_f(C.sf, d > dPf, xr));
+      dd = fma(fma(dP, s.ircr, -dU), recip(s.ircl + s.ircr), widen(-(ql + qr) * recip(il + ir), bp));
     } else {
-      const int bq = 2 * FLOAT_BIAS - bp, bi = bq + m;  // of 1/p, 1/(rho c)
-      s.ircl = refine_recip_sqrt(C.gamma * (pl * rl), widen(il, bi));
-      s.ircr = refine_recip_sqrt(C.gamma * (pr * rr), widen(ir, bi));
-      s.ipl = refine_recip(pl, widen(ipl, bq));
-      s.ipr = refine_recip(pr, widen(ipr, bq));
+      dd = widen(d, bp);
     }
-    T dd = widen(d, bp), f1 = T(0), f2 = T(0);
     float step = 0.0f;
     bool more = true;
     for (int it = 0; it < 4 && more; ++it) {
@@ -219,8 +245,8 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
     s.d = dd;
     s.fl = f1 + widen(tl * step, bu);
     s.fr = f2 + widen(tr * step, bu);
-    s.us = ul - s.fl;
   }
+  s.us = ul - s.fl;
   // u* = u_L - f_L = u_R + f_R: the side that the face lies on gives it
   const bool left = !sign_bit(has_u0 ? u0 + s.us : s.us);
   if (!left) s.us = ur + s.fr;
@@ -236,6 +262,7 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
 
 // The same in float, the two sides in the halves of packed values (they take
 // the same operations).
+template <int WHAT>
 __device__ __forceinline__ int near_riemann(const NearCoef& C, float rl, float ul, float pl, float rr, float ur,
                                             float pr, float dP, float dU, float u0, bool has_u0, float ulf, float urf,
                                             NearStar<float>& s) {

@@ -465,7 +465,7 @@ __device__ __forceinline__ bool pert_face(const PertArgs<T>& a, const PEq<T>& Em
   NearStar<T> st;
   int kind = NEAR_GENERAL;
   if (sizeof(T) == 4 || (positive(rl) && positive(rr) && positive(pl) && positive(pr)))
-    kind = near_riemann(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
+    kind = near_riemann<NEAR_DEPARTURES>(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
                            un0 + wl[n], un0 + wm[n], st);
   if (!GENERAL && kind == NEAR_GENERAL) return true;
   const bool left = kind == NEAR_LEFT || kind == NEAR_STAR_L;
