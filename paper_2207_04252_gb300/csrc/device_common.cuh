@@ -400,8 +400,7 @@ static __device__ __noinline__ RFace riemann_general(double g, double rl, double
 }
 
 // Primitive gas state (u, v, w, P, rho), in the field slots MU, MV, MW, EN,
-// RHO, of a conservative gas state; returns 1 / rho (NaN for rho = 0, which
-// leaves a P that fails every positivity test).
+// RHO, of a conservative gas state; returns 1 / rho.
 __device__ __forceinline__ double gas_prim(double g, const double* U, double* W) {
   const double ir = recip(U[RHO]);
   W[MU] = U[MU] * ir;

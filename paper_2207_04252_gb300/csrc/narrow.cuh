@@ -65,6 +65,13 @@ __device__ __forceinline__ float min_xorsign(float a, float b) {
   return r;
 }
 
+// The smaller value, NaN if either is.
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // double -> float by truncation, flushed to 0 below and held at FLT_MAX above
 // float's range; float -> double, exact for normal values, subnormals to 0.
 // `bias` other than the formats' own 896 scales by a power of two on the way,
@@ -91,21 +98,31 @@ __device__ __forceinline__ double widen(float x, int bias = FLOAT_BIAS) {
 // e = 1 - x y for 1/x; y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 for x^-1/2)
 // from the PTX approximation, whose error of about 2^-20 it takes below
 // 2^-59: three and five FP64 operations, where the correctly rounded division
-// and square root with their scaling take 8 and more.  Zero, infinite and
-// subnormal arguments give NaN: the callers test positivity first.
+// and square root with their scaling take 8 and more.  recip() takes every
+// value: where the approximation is zero or not finite (zero, subnormal,
+// infinite or NaN arguments and those above 2^1022) it divides.
 __device__ __forceinline__ double recip(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  if ((unsigned)(exponent(y) - 1) >= 0x7feu) return 1.0 / x;
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
+// x^-1/2 of a positive normal number.
 __device__ __forceinline__ double recip_sqrt(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-(x * y), y, 1.0);
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
+// The hardware's approximation in float; recip_normal() without the scaling of
+// subnormal arguments (infinite) and results (zero).
 __device__ __forceinline__ float recip(float x) {
+  float y;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float recip_normal(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;

@@ -183,10 +183,10 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
   const float gl = C.gammaf * plf, gr = C.gammaf * prf;
   const float il = recip_sqrt(gl) * recip_sqrt(rlf), ir = recip_sqrt(gr) * recip_sqrt(rrf);  // 1 / (rho c)
   const float cl = gl * il, cr = gr * ir;
-  const float ipl = recip(plf), ipr = recip(prf);
+  const float ipl = recip_normal(plf), ipr = recip_normal(prf);
   const float dPf = narrow(dP, bp), dUf = narrow(dU, bu);
   // linear (acoustic) star pressure d = p* - p_L
-  float d = (dPf * ir - dUf) * recip(il + ir);
+  float d = (dPf * ir - dUf) * recip_normal(il + ir);
   float xl = d * ipl, xr = (d - dPf) * ipr;
   float X = fabsf(xl) + fabsf(xr);
   if (!(X <= 2.0f * NEAR_XF)) return NEAR_GENERAL;  // NaN too
@@ -215,9 +215,9 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
       xr = (d - dPf) * ipr;
       tl = il * near_sum_f(C.tf, sl, xl);
       tr = ir * near_sum_f(C.tf, sr, xr);
-      d -= (d * il * near_sum_f(C.sf, sl, xl) + (d - dPf) * ir * near_sum_f(C.sf, sr, xr) + dUf) * recip(tl + tr);
+      d -= (d * il * near_sum_f(C.sf, sl, xl) + (d - dPf) * ir * near_sum_f(C.sf, sr, xr) + dUf) * recip_normal(tl + tr);
     }
-    const float iD = recip(tl + tr);
+    const float iD = recip_normal(tl + tr);
     const float small = 4.6e-10f * (WHAT == NEAR_DEPARTURES ? fmaxf(fabsf(d), fabsf(d - dPf)) : fminf(plf, prf));
     T dd, f1 = T(0), f2 = T(0);
     if (WHAT == NEAR_DEPARTURES) {
@@ -225,7 +225,7 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double
       xr = (d - dPf) * ipr;
       const float ql = d * il * (xl * near_slope_f(C.sf, d > 0.0f, xl));
       const float qr = (d - dPf) * ir * (xr * near_slope_f(C.sf, d > dPf, xr));
-      dd = fma(fma(dP, s.ircr, -dU), recip(s.ircl + s.ircr), widen(-(ql + qr) * recip(il + ir), bp));
+      dd = fma(fma(dP, s.ircr, -dU), recip(s.ircl + s.ircr), widen(-(ql + qr) * recip_normal(il + ir), bp));
     } else {
       dd = widen(d, bp);
     }
@@ -272,14 +272,17 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, float rl, float u
   const f32x2 i2 = mul2(pack2(recip_sqrt(gl), recip_sqrt(gr)), pack2(recip_sqrt(rl), recip_sqrt(rr)));  // 1 / (rho c)
   unpack2(i2, il, ir);
   unpack2(mul2(g2, i2), cl, cr);
-  s.ipl = recip(pl);
-  s.ipr = recip(pr);
+  s.ipl = recip_normal(pl);
+  s.ipr = recip_normal(pr);
   const f32x2 ip2 = pack2(s.ipl, s.ipr);
   // linear (acoustic) star pressure d = p* - p_L
-  float d = (dP * ir - dU) * recip(il + ir);
+  const float sum = il + ir;
+  float d = (dP * ir - dU) * recip_normal(sum);
   unpack2(mul2(pack2(d, d - dP), ip2), xl, xr);
   const float X = fabsf(xl) + fabsf(xr);
-  if (!(X <= 2.0f * NEAR_XF)) return NEAR_GENERAL;  // NaN too: a state that is not positive
+  // NaN too: a state that is not positive; a sum beyond 2^126: densities or
+  // pressures so small (subnormal, too) that their inverses leave float's range
+  if (!(X <= 2.0f * NEAR_XF) || !(sum < 0x1p126f)) return NEAR_GENERAL;
   if (ulf >= 1.1f * cl) return NEAR_LEFT;
   if (-urf >= 1.1f * cr) return NEAR_RIGHT;
   if (!(X <= NEAR_XF)) return NEAR_GENERAL;
@@ -298,7 +301,7 @@ __device__ __forceinline__ int near_riemann(const NearCoef& C, float rl, float u
     f32x2 f2 = mul2(mul2(d2, i2), S);
     unpack2(f2, fl, fr);
     unpack2(t2, tl, tr);
-    const float step = -(fl + fr + dU) * recip(tl + tr);
+    const float step = -(fl + fr + dU) * recip_normal(tl + tr);
     d += step;
     unpack2(fma2(t2, pack2(step, step), f2), fl, fr);
   };

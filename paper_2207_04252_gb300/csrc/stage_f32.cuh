@@ -153,7 +153,7 @@ struct F32Tile {
         const int s = (zb + u) * M::PLANE + at;
         if (RC == RECON_PRIM && inside[u]) {
           float w[5];
-          face_prim(a.gm1, eq[u][0], eq[u][1], v[u], w);
+          face_prim(a.gm1, eq[u][1], v[u], recip(eq[u][0] + v[u][RHO]), w);
 #pragma unroll
           for (int f = 0; f < 4; ++f) v[u][f] = w[f];
         }
@@ -217,9 +217,9 @@ struct F32Tile {
   // lines of L lanes).  Lane p of a line reconstructs cell p - 1, takes the
   // upper face state of its lower neighbour by a shuffle, solves its lower
   // face and takes the flux of its upper face by a second shuffle.
-  // Returns whether the lane's face needs the general solver; its flux then
-  // counts as zero until the chunk is taken again with REDO, which solves the
-  // faces of the `again` lanes and adds their fluxes.
+  // Returns whether the lane's face needs the general solver or a flat
+  // reconstruction; its flux then counts as zero until the chunk is taken again
+  // with REDO, which solves the faces of the `again` lanes and adds their fluxes.
   template <int D, class P, bool REDO>
   __device__ __forceinline__ bool chunk(const PertArgs<float>& a, float* sm, int base, bool again, unsigned& status,
                                         unsigned& nfallback) const {
@@ -305,7 +305,7 @@ struct F32Tile {
             unpack2(up[q], qp[2 * q], qp[2 * q + 1]);
           }
         }
-        auto face_states = [&]() {
+        auto face_states = [&](auto reciprocal) {
           if (RC == RECON_PRIM) {
 #pragma unroll
             for (int f = 0; f < 5; ++f) {
@@ -313,19 +313,25 @@ struct F32Tile {
               wp[f] = qp[f];
             }
           } else {
-            face_prim(a.gm1, Em.rho, Em.v, qm, wm);
-            face_prim(a.gm1, fp.x, fp.y, qp, wp);
+            face_prim(a.gm1, Em.v, qm, reciprocal(Em.rho + qm[RHO]), wm);
+            face_prim(a.gm1, fp.y, qp, reciprocal(fp.x + qp[RHO]), wp);
           }
-          return positive(fminf(Em.rho + wm[RHO], fp.x + wp[RHO])) && positive(fminf(Em.p + wm[EN], fp.z + wp[EN]));
+          return positive(min_nan(Em.rho + wm[RHO], fp.x + wp[RHO])) &&
+                 positive(min_nan(Em.p + wm[EN], fp.z + wp[EN]));
         };
-        if (!face_states()) {  // positivity fallback: flat reconstruction of the gas fields
+        if constexpr (!REDO) {
+          // states that are not physical (or seem so by a subnormal density): NaN
+          // leaves both faces of the cell to redo()
+          if (!face_states([](float x) { return recip_normal(x); })) wm[EN] = wp[EN] = __int_as_float(0x7fffffff);
+        } else if (!face_states([](float x) { return recip(x); })) {
+          // positivity fallback: flat reconstruction of the gas fields
           const float4 e = reinterpret_cast<const float4*>(sm)[s];
           qm[0] = qp[0] = e.x;
           qm[1] = qp[1] = e.y;
           qm[2] = qp[2] = e.z;
           qm[3] = qp[3] = e.w;
           qm[RHO] = qp[RHO] = sm[M::rho + sr];
-          face_states();
+          face_states([](float x) { return recip(x); });
         }
       }
       float F[5], wl[5];
@@ -408,8 +414,8 @@ struct F32Tile {
   }
 
   // The faces for the general solver (near a strong wave or in the sonic band)
-  // of all three sweeps, for blocks that have any; sweep by sweep, so that every
-  // sum has one order.  Out of line and after the sweeps: with no call in their
+  // and those of cells whose reconstruction is not physical, of all three sweeps,
+  // for blocks that have any; sweep by sweep, so that every sum has one order.  Out of line and after the sweeps: with no call in their
   // loops the kernel takes 80 registers and 24 warps share an SM; with the
   // solver called from the loops it took 128 (16 warps), and spilled at fewer.
   struct Word2 {
@@ -425,14 +431,37 @@ struct F32Tile {
     return w;
   }
 
+  // The update of a cell.  THIN: with reciprocals of any density; the others are
+  // cheaper and right for normal ones, so a cell below 2^-120 (which no stage takes
+  // from there to a subnormal density) goes through an out-of-line copy.
+  struct Updated {
+    float rate;
+    unsigned status;
+  };
   template <bool XT>
+  static __device__ __noinline__ Updated update_thin(const PertArgs<float>& a, const float* sm, int cidx, float tau) {
+    Updated u{0.0f, 0};
+    F32Tile(a, blockIdx.x).template update<XT, true>(a, sm, cidx, tau, u.rate, u.status);
+    return u;
+  }
+  template <bool XT, bool THIN = false>
   __device__ __forceinline__ void update(const PertArgs<float>& a, const float* sm, int cidx, float tau, float& rate,
                                          unsigned& status) const {
     const int x = cidx % TR, y = (cidx / TR) % TT, z = cidx / (TR * TT);
     const int gi = i0 + x, gj = j0 + y, gk = k0 + z;
     if (gi >= a.g.nr || gj >= a.g.nth || gk >= a.g.nz) return;
     const int s = (z + 2) * M::PLANE + (y + 2) * M::ROW + (x + 2), core = z * M::CPLANE + y * M::CROW + x;
+    const PCell<float> ce = cell_eq(a.t, a.g, gi, gk);
     float e[5], dust[NF > 5 ? M::ND : 1][4], G[NF];
+    e[RHO] = sm[M::rho + (z + 2) * M::RPLANE + (y + 2) * M::RROW + (x + 2)];
+    if constexpr (!THIN) {
+      if (!(ce.rho0 + e[RHO] >= 0x1p-120f)) {
+        const Updated u = update_thin<XT>(a, sm, cidx, tau);
+        rate = fmaxf(rate, u.rate);
+        status |= u.status;
+        return;
+      }
+    }
     auto quad = [&](int at, float* q) {
       const float4 v = reinterpret_cast<const float4*>(sm)[at];
       q[0] = v.x;
@@ -441,7 +470,6 @@ struct F32Tile {
       q[3] = v.w;
     };
     quad(s, e);
-    e[RHO] = sm[M::rho + (z + 2) * M::RPLANE + (y + 2) * M::RROW + (x + 2)];
     quad(M::acc(0) / 4 + core, G);
     G[RHO] = sm[M::acc_rho + z * M::CRPLANE + y * M::CRROW + x];
 #pragma unroll
@@ -449,7 +477,8 @@ struct F32Tile {
       quad(M::quad(q) / 4 + s, dust[q - 1]);
       quad(M::acc(q) / 4 + core, G + 1 + 4 * q);
     }
-    pert_update<float, NF, RC, XT>(a, gi, gj, gk, e, dust, G, tau, rate, status);
+    pert_update<float, NF, RC, XT>(a, ce, gi, gj, gk, e, dust, G, tau, rate, status,
+                                   [](float x) { return THIN ? recip(x) : recip_normal(x); });
   }
 };
 

@@ -436,10 +436,9 @@ struct PertArgs {
 // density rho0 and azimuthal velocity v0 (r and z velocities zero):
 // rho = rho0 + rho', du = (m' - rho' u0)/rho,
 // dP = (gamma-1)(E' - [rho' |u0|^2/2 + rho u0.du + rho |du|^2/2]).
-// Returns 1 / rho.
+// ir = 1 / rho.
 template <class T>
-__device__ __forceinline__ T face_prim(T gm1, T rho0, T v0, const T* q, T* w) {
-  const T ir = recip(rho0 + q[RHO]);
+__device__ __forceinline__ void face_prim(T gm1, T v0, const T* q, T ir, T* w) {
   const T m1 = q[MV] - q[RHO] * v0;  // rho dv
   w[MU] = q[MU] * ir;
   w[MV] = m1 * ir;
@@ -447,7 +446,6 @@ __device__ __forceinline__ T face_prim(T gm1, T rho0, T v0, const T* q, T* w) {
   const T ke = q[MU] * w[MU] + m1 * w[MV] + q[MW] * w[MW];
   w[EN] = gm1 * (q[EN] - (v0 * (T(0.5) * q[RHO] * v0 + m1) + T(0.5) * ke));
   w[RHO] = q[RHO];
-  return ir;
 }
 
 // Area times the gas flux perturbation through a face normal to axis D of
@@ -552,8 +550,8 @@ __device__ __forceinline__ void sweep_pert_gas(const PertArgs<double>& a, const 
             wp[f] = qp[f];
           }
         } else {
-          face_prim(a.gm1, Em.rho, Em.v, qm, wm);
-          face_prim(a.gm1, Ep.rho, Ep.v, qp, wp);
+          face_prim(a.gm1, Em.v, qm, recip(Em.rho + qm[RHO]), wm);
+          face_prim(a.gm1, Ep.v, qp, recip(Ep.rho + qp[RHO]), wp);
         }
         return positive(Em.rho + wm[RHO]) && positive(Ep.rho + wp[RHO]) && positive(Em.p + wm[EN]) &&
                positive(Ep.p + wp[EN]);
@@ -760,17 +758,17 @@ __device__ __forceinline__ T pert_cell_rate(const PertArgs<T>& a, const PCell<T>
 // departures, or primitive ones with RC = RECON_PRIM), the primitives of its
 // dust and its flux divergence G, raising the thread's CFL rate.  XT: the
 // optional terms (indirect gravity, wave-killing zones) are compiled in; the
-// plain instantiation carries none of their code.
-template <class T, int NF, int RC, bool XT>
-__device__ __forceinline__ void pert_update(const PertArgs<T>& a, int gi, int gj, int gk, const T* e,
-                                            const T (*dust)[4], T* G, T tau, T& rate, unsigned& status) {
+// plain instantiation carries none of their code.  ce: the cell's equilibrium;
+// inverse(x): 1 / x, for the densities.
+template <class T, int NF, int RC, bool XT, class I>
+__device__ __forceinline__ void pert_update(const PertArgs<T>& a, const PCell<T>& ce, int gi, int gj, int gk, const T* e,
+                                            const T (*dust)[4], T* G, T tau, T& rate, unsigned& status, I&& inverse) {
   constexpr int ND = NF > 5 ? (NF - 5) / 4 : 1;
   const DevGrid& g = a.g;
   const size_t lin = ((size_t)gk * g.nth + gj) * g.nr + gi;
-  const PCell<T> ce = cell_eq(a.t, g, gi, gk);
   T w[5];  // primitive perturbations
   if (RC == RECON_CONS) {
-    face_prim(a.gm1, ce.rho0, ce.v0, e, w);
+    face_prim(a.gm1, ce.v0, e, inverse(ce.rho0 + e[RHO]), w);
   } else {
 #pragma unroll
     for (int f = 0; f < 5; ++f) w[f] = e[f];
@@ -794,9 +792,9 @@ __device__ __forceinline__ void pert_update(const PertArgs<T>& a, int gi, int gj
     const T b = !a.stage2 && RC == RECON_CONS && f < 5 ? e[f] : a.base[f][lin];
     E[f] = b + tv * G[f];
   }
-  if (NF > 5 || a.stage2) ig = recip(ce.rho0 + E[RHO]);
+  if (NF > 5 || a.stage2) ig = inverse(ce.rho0 + E[RHO]);
 #pragma unroll
-  for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = recip(E[b + 3]);
+  for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = inverse(E[b + 3]);
   if constexpr (NF > 5) pert_drag<T, NF, XT>(a, ce, gi, E, tau, ig, id);
 #pragma unroll
   for (int f = 0; f < NF; ++f) a.out[f][lin] = E[f];
@@ -840,7 +838,7 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<dou
     for (int f = 0; f < 5; ++f) q[f] = a.in[f][lin];
     if (RC == RECON_PRIM) {
       const PEq<double> eq = g.has_eq ? load_eq(a.t.cen + 8 * ((size_t)c[2] * g.nr + c[0])) : PEq<double>{};
-      face_prim(a.gm1, eq.rho, eq.v, q, w);
+      face_prim(a.gm1, eq.v, q, recip(eq.rho + q[RHO]), w);
     }
 #pragma unroll
     for (int f = 0; f < 5; ++f) sE[f * BOX + idx] = RC == RECON_PRIM ? w[f] : q[f];
@@ -873,7 +871,8 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<dou
       for (int q = 0; q < 3; ++q) d[q] = a.in[b + q][lin] * id;
     }
     // e is the state as it is stored, whatever the sweeps reconstructed from
-    pert_update<double, NF, RECON_CONS, XT>(a, gi, gj, gk, e, dust, G, s_tau, rate, status);
+    pert_update<double, NF, RECON_CONS, XT>(a, cell_eq(a.t, g, gi, gk), gi, gj, gk, e, dust, G, s_tau, rate, status,
+                                            [](double x) { return recip(x); });
   }
   if (a.stage2) raise_rate(a.rate_out, rate);
   if (status) atomicOr(a.status, status);

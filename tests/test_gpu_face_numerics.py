@@ -1,6 +1,8 @@
 """Rounding of the arithmetic that the kernels write themselves, function by function.
 
-The Riemann solution near p_K, and its departures from the side states, against
+Reciprocals and roots against numpy's correctly rounded ones over the exponent
+range; the conversions and predicates on bits against the casts and
+comparisons that they stand for, at the ends of the ranges too; the Riemann solution near p_K, and its departures from the side states, against
 a Newton iteration in long double.
 """
 import ctypes
@@ -11,6 +13,8 @@ import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
+
+TINY32, TINY64 = np.finfo(np.float32).tiny, np.finfo(np.float64).tiny
 
 
 @pytest.fixture(scope="module")
@@ -32,10 +36,73 @@ def probe(tmp_path_factory):
             assert fn(*head, ctypes.c_int(n), ctypes.c_void_p(a.data_ptr()), ctypes.c_void_p(out.data_ptr())) == 0
             return out.cpu().numpy()
 
+        def scalar(self, op, x):
+            return self._run(lib.probe_scalar, ctypes.c_int(op), x=x, rows=0)
+
         def near(self, gamma, x):
             return self._run(lib.probe_near, ctypes.c_double(gamma), x=x, rows=6)
 
     return Probe()
+
+
+def _sweep(lo, hi, n=200000, seed=0):
+    """Random mantissas over the binary exponents lo ... hi, and the powers of two themselves."""
+    rng = np.random.default_rng(seed)
+    e = rng.integers(lo, hi + 1, n)
+    return np.concatenate([np.ldexp(1.0 + rng.random(n), e), np.ldexp(1.0, np.arange(lo, hi + 1))])
+
+
+def _ulps(got, want):
+    return float((np.abs(got - want) / np.spacing(np.abs(want))).max())
+
+
+def test_double_reciprocals_and_roots(probe):
+    # one third-order step leaves 2^-59 of the value (0.03 ulp); its last operation and the one
+    # before it round: within 1 ulp of the correctly rounded result, within 2 for the longer x^-1/2
+    x = _sweep(-1020, 1020)
+    assert _ulps(probe.scalar(0, x), 1.0 / x) <= 1.0
+    assert _ulps(probe.scalar(1, x), (1.0 / np.sqrt(x.astype(np.longdouble))).astype(np.float64)) <= 2.0
+    assert _ulps(probe.scalar(2, x), np.sqrt(x)) <= 1.0
+
+
+def test_double_roots_and_reciprocals_at_the_ends(probe):
+    x = np.array([0.0, 5e-324, 1e-310, 6e-309, TINY64, np.finfo(np.float64).max, np.inf, np.nan, -1.0])
+    with np.errstate(all="ignore"):
+        np.testing.assert_allclose(probe.scalar(2, x), np.sqrt(x), rtol=2.3e-16)
+        got, want = probe.scalar(0, x), 1.0 / x
+    np.testing.assert_allclose(got, want, rtol=2.3e-16)
+
+
+def test_float_reciprocals_and_roots(probe):
+    # the hardware's approximations: 1 ulp for the reciprocal, 2 for x^-1/2 and the root
+    x = _sweep(-125, 125).astype(np.float32)
+    v = x.astype(np.float64)
+    for op, want, bar in ((7, 1.0 / v, 1.0), (8, np.sqrt(v), 2.0), (9, 1.0 / np.sqrt(v), 2.0)):
+        err = np.abs(probe.scalar(op, v) - want) / np.spacing(want.astype(np.float32)).astype(np.float64)
+        assert err.max() <= bar + 0.5, (op, err.max())
+    ends = np.array([0.0, 1e-45, 1e-40, 5e-39, TINY32, np.finfo(np.float32).max, np.inf, np.nan, -1.0], dtype=np.float32)
+    with np.errstate(all="ignore"):
+        np.testing.assert_allclose(probe.scalar(8, ends.astype(np.float64)), np.sqrt(ends), rtol=3e-7)
+        np.testing.assert_allclose(probe.scalar(7, ends.astype(np.float64)), np.float32(1.0) / ends, rtol=3e-7, atol=2e-45)
+
+
+def test_conversions_and_predicates(probe):
+    x = np.concatenate([_sweep(-200, 200), _sweep(-1022, 1022, seed=1)])
+    x = np.concatenate([x, -x, [0.0, -0.0, 5e-324, -5e-324, TINY64, np.inf, -np.inf]])
+    big, low = np.abs(x) >= 2.0 ** 128, np.abs(x) < TINY32
+    cut = (np.ascontiguousarray(x).view(np.int64) & ~np.int64((1 << 29) - 1)).view(np.float64)  # towards zero
+    want = np.where(big, np.copysign(np.finfo(np.float32).max, x), np.where(low, np.copysign(0.0, x), cut))
+    assert np.array_equal(probe.scalar(3, x), want)
+    f = want[~big]
+    assert np.array_equal(probe.scalar(4, f), f)
+    assert np.array_equal(probe.scalar(4, np.array([1e-45, -1e-40, 0.0])), np.zeros(3))
+    y = np.append(x, np.nan)
+    with np.errstate(invalid="ignore"):
+        bits = (y > 0) * 1 + (y >= 0) * 2 + np.signbit(y) * 4
+    assert np.array_equal(probe.scalar(5, y), bits)
+    y = x[np.isfinite(x)]
+    want = np.where(np.abs(y) >= 8.0 * TINY64, y / 8.0, 0.0)
+    assert np.array_equal(probe.scalar(6, y), want)
 
 
 def _star(g, v):
