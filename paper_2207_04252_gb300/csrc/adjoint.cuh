@@ -502,7 +502,7 @@ __device__ __forceinline__ double drag_vjp(const DevGrid& g, int i, const double
 #pragma unroll
   for (int f = 0; f < 9; ++f) li[f] = lo[f];
   const double rg = U[RHO], rd = U[DRHO];
-  if (!positive(rd) || !positive(rg)) return 0.0;
+  if (!has_mass(rd) || !positive(rg)) return 0.0;
   const double ig = recip(rg), id = recip(rd);
   double P = 0.0;
   if (d.law != 0) P = (g.gamma - 1.0) * fma(-0.5 * ig, fma(U[MU], U[MU], fma(U[MV], U[MV], U[MW] * U[MW])), U[EN]);
@@ -571,7 +571,7 @@ __device__ __forceinline__ void sources_vjp(const DevGrid& g, int i, int k, cons
     out[EN] += sg;
     out[RHO] += fma(s[MU], fma(-v, vr, A1), fma(0.5 * sg, fma(u, u, fma(v, v, w * w)), fma(s[MV] * u, vr, s[MW] * fz)));
   }
-  if (g.nf > 5 && positive(U[DRHO])) {
+  if (g.nf > 5 && has_mass(U[DRHO])) {
     const double iq = recip(U[DRHO]);
     const double u = U[DMU] * iq, v = U[DMV] * iq, vr = v * ir;
     out[DMU] -= s[DMV] * (vr + Om2);
@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(ADJ_PT_NT) adj_point_kernel(const AdjPointArgs
         src[MV] -= s[EN] * gt;
         double P = -(s[MU] * E[RHO] + s[EN] * E[MU]);
         double Q = -(s[MV] * E[RHO] + s[EN] * E[MV]);
-        if (NF == 9 && E[DRHO] > 0.0) {
+        if (NF == 9 && has_mass(E[DRHO])) {
           src[DRHO] -= s[DMU] * gr + s[DMV] * gt;
           P -= s[DMU] * E[DRHO];
           Q -= s[DMV] * E[DRHO];
@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(L * NL, 2) adj_flux_kernel(const AdjFluxArgs a
       dst[(size_t)f * PE * NLP] = g.has_eq ? v - e0[((size_t)f * g.nz + c[2]) * g.nr + c[0]] : v;
     }
     if (NF == 9) {  // the dust as primitives (u, v, w, rho_d)
-      const double rd = a.E[DRHO][lin], id = positive(rd) ? recip(rd) : 0.0;
+      const double rd = a.E[DRHO][lin], id = has_mass(rd) ? recip(rd) : 0.0;
 #pragma unroll
       for (int q = 0; q < 3; ++q) dst[(size_t)(DMU + q) * PE * NLP] = a.E[DMU + q][lin] * id;
       dst[(size_t)DRHO * PE * NLP] = rd;
@@ -977,7 +977,7 @@ __global__ void __launch_bounds__(L * NL, 2) adj_flux_kernel(const AdjFluxArgs a
       tot[q] = gather(tm, t0, tp);
     }
     if (own) {  // the primitives' cotangents back to (rho_d u, rho_d v, rho_d w, rho_d)
-      const double rd = sv(8, p + 1), id = positive(rd) ? recip(rd) : 0.0;
+      const double rd = sv(8, p + 1), id = has_mass(rd) ? recip(rd) : 0.0;
       double rb = tot[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {

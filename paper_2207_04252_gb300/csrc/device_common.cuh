@@ -559,7 +559,7 @@ __device__ __forceinline__ void add_sources(const DevGrid& g, int i, int j, int 
 #pragma unroll
   for (int b = 5; b < NF; b += 4) {  // each dust species
     const double v = Vd[(b - 5) / 4], rd = U[b + 3];
-    if (!positive(rd)) continue;
+    if (!has_mass(rd)) continue;
     G[b] = fma(V, fma(U[b + 1], fma(v, ir, Om2), rd * ar), G[b]);
     double sd = -U[b] * fma(v, ir, Om2);
     if (ind) sd -= rd * gt;
@@ -617,7 +617,7 @@ __device__ __forceinline__ void apply_drag(const DevGrid& g, int i, double* U, d
     P = (g.gamma - 1.0) * fma(-0.5 * ig, fma(U[MU], U[MU], fma(U[MV], U[MV], U[MW] * U[MW])), U[EN]);
   if constexpr (ND == 1) {
     const double rd = U[DRHO];
-    if (!positive(rd)) return;
+    if (!has_mass(rd)) return;
     const double a = tau * inv_stopping_time<XT>(g, i, rg, ig, P, d, 0);
     const double K = rd * a * recip(1.0 + fma(a * rd, ig, a));
     double dE = 0.0;
@@ -638,7 +638,7 @@ __device__ __forceinline__ void apply_drag(const DevGrid& g, int i, double* U, d
     for (int s = 0; s < ND; ++s) {
       const int b = 5 + 4 * s;
       a[s] = h[s] = 0.0;
-      if (!positive(U[b + 3])) continue;
+      if (!has_mass(U[b + 3])) continue;
       a[s] = tau * inv_stopping_time<XT>(g, i, rg, ig, P, d, s);
       h[s] = recip(1.0 + a[s]);
       const double w = a[s] * h[s];
@@ -655,7 +655,7 @@ __device__ __forceinline__ void apply_drag(const DevGrid& g, int i, double* U, d
 #pragma unroll
       for (int s = 0; s < ND; ++s) {
         const int b = 5 + 4 * s;
-        if (!positive(U[b + 3])) continue;
+        if (!has_mass(U[b + 3])) continue;
         U[b + c] = h[s] * fma(U[b + 3] * a[s], vg, U[b + c]);
       }
       dE = fma(0.5 * X, fma(U[MU + c], ig, vg), dE);
@@ -682,7 +682,7 @@ __device__ __forceinline__ double cell_rate(const DevGrid& g, int i, const doubl
   for (int b = 5; b < NF; b += 4) {
     const double j = id[(b - 5) / 4], ud = U[b] * j, vd = U[b + 1] * j, wd = U[b + 2] * j;
     const double d2 = fma(ud, ud, fma(vd, vd, wd * wd));
-    if (positive(U[b + 3]) && positive(d2)) {
+    if (has_mass(U[b + 3]) && positive(d2)) {
       const double vel = root(d2);
       if (mag_less(rate, vel)) rate = vel;
     }

@@ -30,6 +30,20 @@ __device__ __forceinline__ bool non_negative(float x) { return x >= 0.0f; }
 // x is a positive normal number (not subnormal, infinite or NaN).
 __device__ __forceinline__ bool positive_normal(double x) { return (unsigned)((__double2hiint(x) >> 20) - 1) < 0x7feu; }
 
+// A dust cell has mass where its density is a normal number (or infinite): the
+// reciprocal of a subnormal one may overflow.
+__device__ __forceinline__ bool has_mass(double rho) {
+  return (unsigned long long)(__double_as_longlong(rho) - 0x0010000000000000ll) <= 0x7fe0000000000000ull;
+}
+__device__ __forceinline__ bool has_mass(float rho) { return rho >= 0x1p-126f; }
+// A dust density after a stage, negative subnormal ones as zero: a cell that has
+// mass in the first stage's input but not in the second's leaves its neighbours
+// short by less than the smallest normal number.
+__device__ __forceinline__ double dust_density(double rho) {
+  return (unsigned)__double2hiint(rho) >> 20 == 0x800u ? 0.0 : rho;
+}
+__device__ __forceinline__ float dust_density(float rho) { return rho > -0x1p-126f ? fmaxf(rho, 0.0f) : rho; }
+
 // |a| < |b| (magnitudes of non-NaN values order like their bits).
 __device__ __forceinline__ bool mag_less(double a, double b) {
   return (__double_as_longlong(a) & 0x7fffffffffffffffll) < (__double_as_longlong(b) & 0x7fffffffffffffffll);

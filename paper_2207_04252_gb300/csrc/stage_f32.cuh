@@ -161,7 +161,7 @@ struct F32Tile {
         sm[M::rho + (zb + u) * M::RPLANE + (y + 2) * M::RROW + (x + 2)] = v[u][RHO];
 #pragma unroll
         for (int b = 5; b < NF; b += 4) {
-          const float rd = v[u][b + 3], id = positive(rd) ? recip(rd) : 0.0f;
+          const float rd = v[u][b + 3], id = has_mass(rd) ? recip_normal(rd) : 0.0f;
           reinterpret_cast<float4*>(sm + M::quad((b - 1) / 4))[s] =
               make_float4(v[u][b] * id, v[u][b + 1] * id, v[u][b + 2] * id, rd);
         }

@@ -378,7 +378,7 @@ __device__ __forceinline__ void dust_species(const DevGrid& g, const double* con
         return;
       }
       const size_t lin = ((size_t)c[2] * g.nth + c[1]) * g.nr + c[0];
-      const double rd = in[b + 3][lin], id = positive(rd) ? recip(rd) : 0.0;
+      const double rd = in[b + 3][lin], id = has_mass(rd) ? recip(rd) : 0.0;
 #pragma unroll
       for (int q = 0; q < 3; ++q) sE[q * BOX + idx] = in[b + q][lin] * id;
       sE[3 * BOX + idx] = rd;
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
 #pragma unroll
       for (int b = 5; b < NF; b += 4) {
         bad |= !non_negative(U[b + 3]);
-        Vd[(b - 5) / 4] = positive(U[b + 3]) ? U[b + 1] * recip(U[b + 3]) : 0.0;
+        Vd[(b - 5) / 4] = has_mass(U[b + 3]) ? U[b + 1] * recip(U[b + 3]) : 0.0;
       }
       if (bad) status |= STATUS_NONPHYSICAL;
       if (g.geom == GEOM_CYL) add_sources<XT, NF>(g, gi, gj, gk, U, W, Vd, G);
@@ -558,7 +558,10 @@ __global__ void __launch_bounds__(NT, MINB) stage_full_kernel(const StageArgs a)
     for (int f = 0; f < NF; ++f) E[f] = fma(tv, G[f], a.base[f][lin]);
     if (NF > 5 || a.stage2) ig = recip(E[RHO]);
 #pragma unroll
-    for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = recip(E[b + 3]);
+    for (int b = 5; b < NF; b += 4) {
+      E[b + 3] = dust_density(E[b + 3]);
+      id[(b - 5) / 4] = recip(E[b + 3]);
+    }
     if constexpr (NF > 5) apply_drag<XT, ND>(g, gi, E, tau, a.drag, ig, id);
 #pragma unroll
     for (int f = 0; f < NF; ++f) a.out[f][lin] = E[f];

@@ -636,7 +636,7 @@ __device__ __forceinline__ void pert_sources(const PertArgs<T>& a, const PCell<T
 #pragma unroll
   for (int b = 5; b < NF; b += 4) {  // each dust species
     const T* d = dust[(b - 5) / 4];
-    const T Vr = positive(d[3]) ? V * d[3] : T(0);
+    const T Vr = has_mass(d[3]) ? V * d[3] : T(0);
     const T dvd = d[1] - c.v0;  // v_d - v0
     T s0 = c.Cr + dvd * (c.cor + dvd * c.ir), s1 = -d[0] * (d[1] * c.ir + Om2);
     if (ind) {
@@ -684,7 +684,7 @@ __device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& 
   T dE = T(0);
   if constexpr (NF == 9) {
     const T rd = q[DRHO];
-    if (!positive(rd)) return;
+    if (!has_mass(rd)) return;
     const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, ig, p, 0);
     const T K = rd * ak * recip(T(1) + ak * (T(1) + rd * ig));
 #pragma unroll
@@ -703,7 +703,7 @@ __device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& 
       const int b = 5 + 4 * s;
       const T rd = q[b + 3];
       wk[s] = T(0);
-      if (!positive(rd)) continue;
+      if (!has_mass(rd)) continue;
       const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, ig, p, s);
       wk[s] = ak * recip(T(1) + ak);
       den += rd * wk[s];
@@ -718,7 +718,7 @@ __device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& 
       for (int s = 0; s < ND; ++s) {
         const int b = 5 + 4 * s;
         const T rd = q[b + 3];
-        if (!positive(rd)) continue;
+        if (!has_mass(rd)) continue;
         const T rel = (q[b + k] - rd * u0[k]) * id[s] - dug[k];  // v_k - v_g
         q[b + k] += rd * wk[s] * (D - rel);
       }
@@ -745,7 +745,7 @@ __device__ __forceinline__ T pert_cell_rate(const PertArgs<T>& a, const PCell<T>
   for (int b = 5; b < NF; b += 4) {
     const T j = id[(b - 5) / 4], ud = q[b] * j, vd = q[b + 1] * j, wd = q[b + 2] * j;
     const T d2 = ud * ud + vd * vd + wd * wd;
-    if (positive(q[b + 3]) && positive(d2)) {
+    if (has_mass(q[b + 3]) && positive(d2)) {
       const T vel = root(d2);
       if (!(vel <= rate)) rate = vel;
     }
@@ -794,7 +794,10 @@ __device__ __forceinline__ void pert_update(const PertArgs<T>& a, const PCell<T>
   }
   if (NF > 5 || a.stage2) ig = inverse(ce.rho0 + E[RHO]);
 #pragma unroll
-  for (int b = 5; b < NF; b += 4) id[(b - 5) / 4] = inverse(E[b + 3]);
+  for (int b = 5; b < NF; b += 4) {
+    E[b + 3] = dust_density(E[b + 3]);
+    id[(b - 5) / 4] = inverse(E[b + 3]);
+  }
   if constexpr (NF > 5) pert_drag<T, NF, XT>(a, ce, gi, E, tau, ig, id);
 #pragma unroll
   for (int f = 0; f < NF; ++f) a.out[f][lin] = E[f];
@@ -866,7 +869,7 @@ __global__ void __launch_bounds__(NT, MINB) stage_pert_kernel(const PertArgs<dou
     for (int b = 5; b < NF; b += 4) {
       double* d = dust[(b - 5) / 4];
       d[3] = a.in[b + 3][lin];
-      const double id = positive(d[3]) ? recip(d[3]) : 0.0;
+      const double id = has_mass(d[3]) ? recip(d[3]) : 0.0;
 #pragma unroll
       for (int q = 0; q < 3; ++q) d[q] = a.in[b + q][lin] * id;
     }
