@@ -668,6 +668,7 @@ void set_pert_drag(PertArgs<T>& a, const DragArgs& drag) {
 // that the Stokes number holds at r = 1, z = 0).
 rossbi_status drag_args(rossbi_grid* g, const rossbi_dust_params* dust, DragArgs& drag) {
   drag = DragArgs{};
+  double unit = 0.0;  // rho_s r_p of St = 1
   if (g->nf > 5) {
     drag.stokes = dust->stokes;
     drag.law = dust->drag_law;
@@ -682,13 +683,20 @@ rossbi_status drag_args(rossbi_grid* g, const rossbi_dust_params* dust, DragArgs
       if (!g->has_disc) return ROSSBI_ERR_ARG;
       double rho1, vth1, p1;
       equilibrium_prim(g->desc, g->disc, 1.0, 0.0, rho1, vth1, p1);
-      drag.rhos_rp = dust->stokes * rho1 * std::sqrt(g->desc.gamma * p1 / rho1) / std::sqrt(g->desc.gm);
+      const double cs1 = std::sqrt(g->desc.gamma * p1 / rho1), om1 = std::sqrt(g->desc.gm);
+      drag.rhos_rp = dust->stokes * rho1 * cs1 / om1;
+      unit = rho1 * cs1 / om1;
     } else if (dust->drag_law != 0) {
       return ROSSBI_ERR_ARG;
     }
+    // A Stokes number below `least` stops the dust to a part in 10^14 (of the
+    // state's 10^7) or 10^190 in any step worth taking: it is taken as `least`,
+    // whose inverse is a number in the state's precision.
+    const double least = g->desc.precision == ROSSBI_FP32_PERT ? 0x1p-66 : 0x1p-660;
     for (int s = 0; s < ND_MAX; ++s) {
-      drag.ist[s] = 1.0 / (drag.stokes * g->dg.st_factor[s]);
-      drag.irr[s] = 1.0 / (drag.rhos_rp * g->dg.st_factor[s]);
+      const double f = g->dg.st_factor[s], st = drag.stokes * f;
+      drag.ist[s] = 1.0 / std::max(st, least);
+      drag.irr[s] = 1.0 / (st > least ? drag.rhos_rp * f : least * unit);
     }
   }
   return ROSSBI_OK;
