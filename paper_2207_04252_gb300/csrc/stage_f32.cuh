@@ -92,125 +92,16 @@ struct F32Smem {
   __host__ __device__ static constexpr int face(int axis) { return axis == 0 ? face0 : (axis == 1 ? face1 : face2); }
 };
 
-template <int NF, int TR, int TT, int TZ, int NT, int RC>
-struct F32Tile {
+// The sweeps' work on a tile, whatever the block's shape (so that both shapes share
+// one copy of redo(), and with it the bits of its results).
+template <int NF, int TR, int TT, int TZ, int RC>
+struct F32Lines {
   using M = F32Smem<NF, TR, TT, TZ>;
   int i0, j0, k0;
   bool full;  // the tile lies within the grid
-  __device__ __forceinline__ F32Tile(const PertArgs<float>& a, int tile) {
+  __device__ __forceinline__ F32Lines(const PertArgs<float>& a, int tile) {
     a.order.origin(tile, TR, TT, TZ, i0, j0, k0);
     full = i0 + TR <= a.g.nr && j0 + TT <= a.g.nth && k0 + TZ <= a.g.nz;
-  }
-
-  // The tile and its halo as deviations: the gas as conservative departures (or,
-  // with RC = RECON_PRIM, primitive ones), the dust as primitives, converted
-  // once here.  Each thread owns one (r, theta) position of the box and walks
-  // its z planes (half of them where the block has two threads per position),
-  // so that an index costs one addition; the loads of a batch of planes are all
-  // in flight before the first is used.  Equilibrium ghosts are zero departures.
-  __device__ __forceinline__ void stage(const PertArgs<float>& a, float* sm) const {
-    constexpr int COLS = M::BX * M::BY, HALVES = NT >= 2 * COLS ? 2 : 1, NB = NF <= 9 ? 5 : 2;
-    static_assert(COLS <= NT && M::BZ % 2 == 0, "a thread per (r, theta) position of the box");
-    const DevGrid& g = a.g;
-    if (threadIdx.x >= HALVES * COLS) return;
-    const int half = HALVES == 2 && threadIdx.x >= COLS ? 1 : 0, pos = (int)threadIdx.x - half * COLS;
-    const int x = pos % M::BX - 2, y = pos / M::BX - 2;
-    const bool side = x < 0 || x >= TR, end = y < 0 || y >= TT;
-    if (side && end) return;  // no sweep reads the box's edges and corners
-    int ci = i0 + x, cj = j0 + y;
-    const bool in = resolve_axis(g, 0, ci) && resolve_axis(g, 1, cj);
-    const int first = side || end ? 2 : 0, last = side || end ? TZ + 2 : M::BZ;
-    const int z0 = HALVES == 2 && half ? M::BZ / 2 : 0, z1 = HALVES == 2 && !half ? M::BZ / 2 : M::BZ;
-    const size_t plane = (size_t)g.nth * g.nr, row = (size_t)cj * g.nr + ci;
-    const int at = (y + 2) * M::ROW + (x + 2);
-#pragma unroll 1
-    for (int zb = z0; zb < z1; zb += NB) {
-      float v[NB][NF], eq[NB][2];
-      bool use[NB], inside[NB];
-#pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        const int z = zb + u;
-        int ck = k0 + z - 2;
-        use[u] = z < z1 && z >= first && z < last;
-        inside[u] = use[u] && resolve_axis(g, 2, ck) && in;
-        if (inside[u]) {
-          const size_t lin = (size_t)ck * plane + row;
-#pragma unroll
-          for (int f = 0; f < NF; ++f) v[u][f] = a.in[f][lin];
-          if (RC == RECON_PRIM) {
-            const float* c = a.t.cen + 8 * ((size_t)ck * g.nr + ci);
-            eq[u][0] = g.has_eq ? c[0] : 0.0f;
-            eq[u][1] = g.has_eq ? c[1] : 0.0f;
-          }
-        } else {
-#pragma unroll
-          for (int f = 0; f < NF; ++f) v[u][f] = 0.0f;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < NB; ++u) {
-        if (!use[u]) continue;
-        const int s = (zb + u) * M::PLANE + at;
-        if (RC == RECON_PRIM && inside[u]) {
-          float w[5];
-          face_prim(a.gm1, eq[u][1], v[u], recip(eq[u][0] + v[u][RHO]), w);
-#pragma unroll
-          for (int f = 0; f < 4; ++f) v[u][f] = w[f];
-        }
-        reinterpret_cast<float4*>(sm)[s] = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
-        sm[M::rho + (zb + u) * M::RPLANE + (y + 2) * M::RROW + (x + 2)] = v[u][RHO];
-#pragma unroll
-        for (int b = 5; b < NF; b += 4) {
-          const float rd = v[u][b + 3], id = has_mass(rd) ? recip_normal(rd) : 0.0f;
-          reinterpret_cast<float4*>(sm + M::quad((b - 1) / 4))[s] =
-              make_float4(v[u][b] * id, v[u][b + 1] * id, v[u][b + 2] * id, rd);
-        }
-      }
-    }
-  }
-
-  // The tables of the tile's faces and cells, indices clamped to the grid, by
-  // asynchronous copies (in flight while the box is staged).
-  __device__ __forceinline__ void tables(const PertArgs<float>& a, float* sm) const {
-    const DevGrid& g = a.g;
-    constexpr int N0 = (TR + 3) * TZ, N1 = N0 + TR * TZ, N2 = N1 + TR * (TZ + 3);
-    for (int q = threadIdx.x; q < N2; q += NT) {
-      const int at = q < N1 ? q : N1 + (q - N1) / TR * M::ZROW + (q - N1) % TR;
-      float4* dst = reinterpret_cast<float4*>(sm + M::face0) + at;
-      if (!g.has_eq) {
-        *dst = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      } else {
-        size_t o;
-        const float* t;
-        if (q < N0) {
-          const int f = clampi(i0 - 1 + q % (TR + 3), 0, g.nr), k = clampi(k0 + q / (TR + 3), 0, g.nz - 1);
-          t = a.t.face[0];
-          o = (size_t)k * (g.nr + 1) + f;
-        } else if (q < N1) {
-          const int c = q - N0, i = clampi(i0 + c % TR, 0, g.nr - 1), k = clampi(k0 + c / TR, 0, g.nz - 1);
-          t = a.t.face[1];
-          o = (size_t)k * g.nr + i;
-        } else {
-          const int c = q - N1, i = clampi(i0 + c % TR, 0, g.nr - 1), f = clampi(k0 - 1 + c / TR, 0, g.nz);
-          t = a.t.face[2];
-          o = (size_t)f * g.nr + i;
-        }
-        copy_async<16>(dst, t + 4 * o);
-      }
-    }
-    constexpr int W = RCW / 4 * (TR + 2);  // 16-byte pieces of the weights, then the areas one by one
-    for (int q = threadIdx.x; q < W + 3 * TR + 1; q += NT) {
-      if (q < W) {
-        const int c = i0 - 1 + q / (RCW / 4);  // weights of cells -1 .. nr are tabulated
-        copy_async<16>(sm + M::wgt + 4 * (q % (RCW / 4) * (TR + 2) + q / (RCW / 4)), a.t.rcoef + (size_t)((c > g.nr ? g.nr : c) + 1) * RCW + 4 * (q % (RCW / 4)));
-      } else {
-        const int n = q - W;
-        const float* t = n < TR + 1 ? a.t.area_r + clampi(i0 + n, 0, g.nr)
-                                    : (n < 2 * TR + 1 ? a.t.area_t + clampi(i0 + n - TR - 1, 0, g.nr - 1)
-                                                      : a.t.area_z + clampi(i0 + n - 2 * TR - 1, 0, g.nr - 1));
-        copy_async<4>(sm + M::area + n, t);
-      }
-    }
   }
 
   // One 32-lane chunk of the sweep along axis D: items base .. base + 31 (whole
@@ -392,45 +283,169 @@ struct F32Tile {
   static __host__ __device__ constexpr int items() {
     return (D == 0 ? TT * TZ : (D == 1 ? TR * TZ : TR * TT)) * pow2ceil((D == 0 ? TR : (D == 1 ? TT : TZ)) + 2);
   }
-  // The sweep along axis D, chunks spread over the warps; sets bit BITS D + n of
-  // `left` where the lane's face of the warp's n-th chunk is left to redo().
-  static constexpr int BITS = 10;
-  template <int D, class P>
-  __device__ __forceinline__ void sweep(const PertArgs<float>& a, float* sm, unsigned& left) const {
-    static_assert((items<D>() + NT - 1) / NT <= BITS, "a bit per chunk");
-    unsigned bit = 1u << (BITS * D), status = 0, nfallback = 0;
-#pragma unroll 1
-    for (int base = threadIdx.x & ~31; base < items<D>(); base += NT, bit <<= 1)
-      if (chunk<D, P, false>(a, sm, base, false, status, nfallback)) left |= bit;
-  }
+  static constexpr int BITS = 10;  // chunks of a warp and sweep at most
   template <int D, class P>
   __device__ __forceinline__ void resweep(const PertArgs<float>& a, float* sm, unsigned left, unsigned& status,
                                           unsigned& nfallback) const {
     unsigned bit = 1u << (BITS * D);
 #pragma unroll 1
-    for (int base = threadIdx.x & ~31; base < items<D>(); base += NT, bit <<= 1)
+    for (int base = threadIdx.x & ~31; base < items<D>(); base += blockDim.x, bit <<= 1)
       if (__any_sync(0xffffffffu, left & bit)) chunk<D, P, true>(a, sm, base, left & bit, status, nfallback);
     __syncthreads();
   }
 
   // The faces for the general solver (near a strong wave or in the sonic band)
   // and those of cells whose reconstruction is not physical, of all three sweeps,
-  // for blocks that have any; sweep by sweep, so that every sum has one order.  Out of line and after the sweeps: with no call in their
-  // loops the kernel takes 80 registers and 24 warps share an SM; with the
-  // solver called from the loops it took 128 (16 warps), and spilled at fewer.
+  // for blocks that have any; sweep by sweep, so that every sum has one order.
+  // Out of line and after the sweeps: with no call in their loops the kernel takes
+  // 80 registers and 24 warps share an SM; with the solver called from the loops
+  // it took 128 (16 warps), and spilled at fewer.  The solver is in line here, as
+  // every face takes it: around a call the faces' states go to local memory.  A step
+  // of 280 x 180 x 48 bi-fluid cells with jumps of 10 % at all faces, the most that
+  // this can cost: 1.51 ms, 1.66 with a call, 1.58 with 16 warps and an FP32 Newton
+  // iteration on every face.
   struct Word2 {
     unsigned status, nfallback;
   };
   template <class P>
   static __device__ __noinline__ Word2 redo(const PertArgs<float>& a, float* sm, unsigned left) {
-    const F32Tile t(a, blockIdx.x);
+    const F32Lines t(a, blockIdx.x);
     Word2 w{0, 0};
     t.template resweep<0, P>(a, sm, left, w.status, w.nfallback);
     t.template resweep<1, P>(a, sm, left, w.status, w.nfallback);
     t.template resweep<2, P>(a, sm, left, w.status, w.nfallback);
     return w;
   }
+};
 
+template <int NF, int TR, int TT, int TZ, int NT, int RC>
+struct F32Tile : F32Lines<NF, TR, TT, TZ, RC> {
+  using Base = F32Lines<NF, TR, TT, TZ, RC>;
+  using M = typename Base::M;
+  using Base::i0, Base::j0, Base::k0;
+  using Base::Base;
+
+  // The tile and its halo as deviations: the gas as conservative departures (or,
+  // with RC = RECON_PRIM, primitive ones), the dust as primitives, converted
+  // once here.  Each thread owns one (r, theta) position of the box and walks
+  // its z planes (half of them where the block has two threads per position),
+  // so that an index costs one addition; the loads of a batch of planes are all
+  // in flight before the first is used.  Equilibrium ghosts are zero departures.
+  __device__ __forceinline__ void stage(const PertArgs<float>& a, float* sm) const {
+    constexpr int COLS = M::BX * M::BY, HALVES = NT >= 2 * COLS ? 2 : 1, NB = NF <= 9 ? 5 : 2;
+    static_assert(COLS <= NT && M::BZ % 2 == 0, "a thread per (r, theta) position of the box");
+    const DevGrid& g = a.g;
+    if (threadIdx.x >= HALVES * COLS) return;
+    const int half = HALVES == 2 && threadIdx.x >= COLS ? 1 : 0, pos = (int)threadIdx.x - half * COLS;
+    const int x = pos % M::BX - 2, y = pos / M::BX - 2;
+    const bool side = x < 0 || x >= TR, end = y < 0 || y >= TT;
+    if (side && end) return;  // no sweep reads the box's edges and corners
+    int ci = i0 + x, cj = j0 + y;
+    const bool in = resolve_axis(g, 0, ci) && resolve_axis(g, 1, cj);
+    const int first = side || end ? 2 : 0, last = side || end ? TZ + 2 : M::BZ;
+    const int z0 = HALVES == 2 && half ? M::BZ / 2 : 0, z1 = HALVES == 2 && !half ? M::BZ / 2 : M::BZ;
+    const size_t plane = (size_t)g.nth * g.nr, row = (size_t)cj * g.nr + ci;
+    const int at = (y + 2) * M::ROW + (x + 2);
+#pragma unroll 1
+    for (int zb = z0; zb < z1; zb += NB) {
+      float v[NB][NF], eq[NB][2];
+      bool use[NB], inside[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        const int z = zb + u;
+        int ck = k0 + z - 2;
+        use[u] = z < z1 && z >= first && z < last;
+        inside[u] = use[u] && resolve_axis(g, 2, ck) && in;
+        if (inside[u]) {
+          const size_t lin = (size_t)ck * plane + row;
+#pragma unroll
+          for (int f = 0; f < NF; ++f) v[u][f] = a.in[f][lin];
+          if (RC == RECON_PRIM) {
+            const float* c = a.t.cen + 8 * ((size_t)ck * g.nr + ci);
+            eq[u][0] = g.has_eq ? c[0] : 0.0f;
+            eq[u][1] = g.has_eq ? c[1] : 0.0f;
+          }
+        } else {
+#pragma unroll
+          for (int f = 0; f < NF; ++f) v[u][f] = 0.0f;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < NB; ++u) {
+        if (!use[u]) continue;
+        const int s = (zb + u) * M::PLANE + at;
+        if (RC == RECON_PRIM && inside[u]) {
+          float w[5];
+          face_prim(a.gm1, eq[u][1], v[u], recip(eq[u][0] + v[u][RHO]), w);
+#pragma unroll
+          for (int f = 0; f < 4; ++f) v[u][f] = w[f];
+        }
+        reinterpret_cast<float4*>(sm)[s] = make_float4(v[u][0], v[u][1], v[u][2], v[u][3]);
+        sm[M::rho + (zb + u) * M::RPLANE + (y + 2) * M::RROW + (x + 2)] = v[u][RHO];
+#pragma unroll
+        for (int b = 5; b < NF; b += 4) {
+          const float rd = v[u][b + 3], id = has_mass(rd) ? recip_normal(rd) : 0.0f;
+          reinterpret_cast<float4*>(sm + M::quad((b - 1) / 4))[s] =
+              make_float4(v[u][b] * id, v[u][b + 1] * id, v[u][b + 2] * id, rd);
+        }
+      }
+    }
+  }
+
+  // The tables of the tile's faces and cells, indices clamped to the grid, by
+  // asynchronous copies (in flight while the box is staged).
+  __device__ __forceinline__ void tables(const PertArgs<float>& a, float* sm) const {
+    const DevGrid& g = a.g;
+    constexpr int N0 = (TR + 3) * TZ, N1 = N0 + TR * TZ, N2 = N1 + TR * (TZ + 3);
+    for (int q = threadIdx.x; q < N2; q += NT) {
+      const int at = q < N1 ? q : N1 + (q - N1) / TR * M::ZROW + (q - N1) % TR;
+      float4* dst = reinterpret_cast<float4*>(sm + M::face0) + at;
+      if (!g.has_eq) {
+        *dst = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      } else {
+        size_t o;
+        const float* t;
+        if (q < N0) {
+          const int f = clampi(i0 - 1 + q % (TR + 3), 0, g.nr), k = clampi(k0 + q / (TR + 3), 0, g.nz - 1);
+          t = a.t.face[0];
+          o = (size_t)k * (g.nr + 1) + f;
+        } else if (q < N1) {
+          const int c = q - N0, i = clampi(i0 + c % TR, 0, g.nr - 1), k = clampi(k0 + c / TR, 0, g.nz - 1);
+          t = a.t.face[1];
+          o = (size_t)k * g.nr + i;
+        } else {
+          const int c = q - N1, i = clampi(i0 + c % TR, 0, g.nr - 1), f = clampi(k0 - 1 + c / TR, 0, g.nz);
+          t = a.t.face[2];
+          o = (size_t)f * g.nr + i;
+        }
+        copy_async<16>(dst, t + 4 * o);
+      }
+    }
+    constexpr int W = RCW / 4 * (TR + 2);  // 16-byte pieces of the weights, then the areas one by one
+    for (int q = threadIdx.x; q < W + 3 * TR + 1; q += NT) {
+      if (q < W) {
+        const int c = i0 - 1 + q / (RCW / 4);  // weights of cells -1 .. nr are tabulated
+        copy_async<16>(sm + M::wgt + 4 * (q % (RCW / 4) * (TR + 2) + q / (RCW / 4)), a.t.rcoef + (size_t)((c > g.nr ? g.nr : c) + 1) * RCW + 4 * (q % (RCW / 4)));
+      } else {
+        const int n = q - W;
+        const float* t = n < TR + 1 ? a.t.area_r + clampi(i0 + n, 0, g.nr)
+                                    : (n < 2 * TR + 1 ? a.t.area_t + clampi(i0 + n - TR - 1, 0, g.nr - 1)
+                                                      : a.t.area_z + clampi(i0 + n - 2 * TR - 1, 0, g.nr - 1));
+        copy_async<4>(sm + M::area + n, t);
+      }
+    }
+  }
+
+  // The sweep along axis D, chunks spread over the warps; sets bit BITS D + n of
+  // `left` where the lane's face of the warp's n-th chunk is left to redo().
+  template <int D, class P>
+  __device__ __forceinline__ void sweep(const PertArgs<float>& a, float* sm, unsigned& left) const {
+    static_assert((Base::template items<D>() + NT - 1) / NT <= Base::BITS, "a bit per chunk");
+    unsigned bit = 1u << (Base::BITS * D), status = 0, nfallback = 0;
+#pragma unroll 1
+    for (int base = threadIdx.x & ~31; base < Base::template items<D>(); base += NT, bit <<= 1)
+      if (this->template chunk<D, P, false>(a, sm, base, false, status, nfallback)) left |= bit;
+  }
   // The update of a cell.  THIN: with reciprocals of any density; the others are
   // cheaper and right for normal ones, so a cell below 2^-120 (which no stage takes
   // from there to a subnormal density) goes through an out-of-line copy.

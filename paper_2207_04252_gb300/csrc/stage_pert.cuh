@@ -147,12 +147,12 @@ struct PFace {
 // Perturbation of one side of a face, with the full values the wave pattern needs.
 template <class T>
 struct PSide {
-  T drho, dun, dp;      // perturbations
-  T rho, un, p, c, dc;  // full values and c - c0
+  T drho, dun, dp;  // perturbations
+  T rho, un, p, c;  // full values
 };
 
 template <class T>
-__device__ __forceinline__ PSide<T> pert_side(T g, const PFace<T>& W0, T drho, T dun, T dp, bool has_eq) {
+__device__ __forceinline__ PSide<T> pert_side(T g, const PFace<T>& W0, T drho, T dun, T dp) {
   PSide<T> s;
   s.drho = drho;
   s.dun = dun;
@@ -161,7 +161,6 @@ __device__ __forceinline__ PSide<T> pert_side(T g, const PFace<T>& W0, T drho, T
   s.p = W0.p + dp;
   s.un = W0.un + dun;
   s.c = Math<T>::sqrt_(g * s.p / s.rho);
-  s.dc = has_eq ? W0.c * sqrt1pm1((dp * W0.rho - W0.p * drho) / (W0.p * s.rho)) : s.c;
   return s;
 }
 
@@ -201,27 +200,29 @@ __device__ __forceinline__ void pert_pressure_fn(T g, const PSide<T>& K, const P
 }
 
 template <class T, class P>
-__device__ __forceinline__ void fan_pert(T g, const PFace<T>& W0, const PSide<T>& K, bool left, T& drho, T& dun,
-                                         T& dp) {
+__device__ __forceinline__ void fan_pert(T g, const PFace<T>& W0, const PSide<T>& K, bool has_eq, bool left, T& drho,
+                                         T& dun, T& dp) {
   const T g6 = (g - T(1)) / (g + T(1));
+  // c - c0
+  const T dc = has_eq ? W0.c * sqrt1pm1((K.dp * W0.rho - W0.p * K.drho) / (W0.p * K.rho)) : K.c;
   if (left) {  // (u_L - c_L) = (u0 - c0) + du_L - dc_L
-    const T y = g6 * (W0.un_mc + K.dun - K.dc) / K.c;
+    const T y = g6 * (W0.un_mc + K.dun - dc) / K.c;
     drho = K.drho + K.rho * P::fan_rho(y, g);
     dp = K.dp + K.p * P::fan_p(y, g);
-    dun = -W0.un_mc + K.dc + K.c * y;
+    dun = -W0.un_mc + dc + K.c * y;
   } else {     // (-u_R - c_R) = -(u0 + c0) - du_R - dc_R
-    const T y = g6 * (-W0.un_pc - K.dun - K.dc) / K.c;
+    const T y = g6 * (-W0.un_pc - K.dun - dc) / K.c;
     drho = K.drho + K.rho * P::fan_rho(y, g);
     dp = K.dp + K.p * P::fan_p(y, g);
-    dun = -W0.un_pc - K.dc - K.c * y;
+    dun = -W0.un_pc - dc - K.c * y;
   }
 }
 
 // Perturbation of the face state of the exact Riemann solution.  Returns
 // 0 on success, 1 when the caller must use the FP64 full-state solver.
 template <class T, class P>
-__device__ __forceinline__ int pert_riemann(T g, const PFace<T>& W0, const PSide<T>& L, const PSide<T>& R, T& drho,
-                                            T& dun, T& dp, int& side) {
+__device__ __forceinline__ int pert_riemann(T g, const PFace<T>& W0, const PSide<T>& L, const PSide<T>& R, bool has_eq,
+                                            T& drho, T& dun, T& dp, int& side) {
   if (T(2) / (g - T(1)) * (L.c + R.c) <= R.un - L.un) return 1;  // vacuum generation
   const T du = R.dun - L.dun;
   const T floor_p = T(1e-8) * fmin(L.p, R.p);
@@ -287,7 +288,7 @@ __device__ __forceinline__ int pert_riemann(T g, const PFace<T>& W0, const PSide
       const T r = rar(x);
       const T cs = L.c * (T(1) + r);
       if (us - cs < T(0)) { drho = L.drho + L.rho * P::dens(x, g, r); dun = dus; dp = d; return 0; }
-      fan_pert<T, P>(g, W0, L, true, drho, dun, dp);
+      fan_pert<T, P>(g, W0, L, has_eq, true, drho, dun, dp);
       return 0;
     }
     if (L.un - L.c * Math<T>::sqrt_(T(1) + (g + T(1)) / (T(2) * g) * x) >= T(0)) {
@@ -313,7 +314,7 @@ __device__ __forceinline__ int pert_riemann(T g, const PFace<T>& W0, const PSide
   const T r = rar(x);
   const T cs = R.c * (T(1) + r);
   if (us + cs > T(0)) { drho = R.drho + R.rho * P::dens(x, g, r); dun = dus; dp = d; return 0; }
-  fan_pert<T, P>(g, W0, R, false, drho, dun, dp);
+  fan_pert<T, P>(g, W0, R, has_eq, false, drho, dun, dp);
   return 0;
 }
 
@@ -385,11 +386,9 @@ __device__ __noinline__ PStar<T> pert_fallback_fp64(T g, const PFace<T> W0, cons
   return o;
 }
 
-// The general solver of a face: near a strong wave or in the sonic band.  One
-// out-of-line copy serves the three sweep directions; arguments and result by
-// value.
+// The general solver of a face: near a strong wave or in the sonic band.
 template <class T, class P>
-__device__ __noinline__ PStar<T> pert_general(T g, const PFace<T> W0, T lr, T lu, T lp, T rr, T ru, T rp,
+__device__ __forceinline__ PStar<T> pert_general(T g, const PFace<T> W0, T lr, T lu, T lp, T rr, T ru, T rp,
                                               bool has_eq) {
   PStar<T> o;
   o.side = 0;
@@ -399,12 +398,20 @@ __device__ __noinline__ PStar<T> pert_general(T g, const PFace<T> W0, T lr, T lu
     o.status = STATUS_NONPHYSICAL;
     return o;
   }
-  const PSide<T> L = pert_side(g, W0, lr, lu, lp, has_eq), R = pert_side(g, W0, rr, ru, rp, has_eq);
-  if (pert_riemann<T, P>(g, W0, L, R, o.drho, o.dun, o.dp, o.side) != 0) {
+  const PSide<T> L = pert_side(g, W0, lr, lu, lp), R = pert_side(g, W0, rr, ru, rp);
+  if (pert_riemann<T, P>(g, W0, L, R, has_eq, o.drho, o.dun, o.dp, o.side) != 0) {
     o = pert_fallback_fp64(g, W0, L, R);
     o.fallback = 1;
   }
   return o;
+}
+
+// The same out of line for the double kernel, whose sweeps mostly pass it by: one
+// copy serves the three directions; arguments and result by value.
+template <class T, class P>
+__device__ __noinline__ PStar<T> pert_general_call(T g, const PFace<T> W0, T lr, T lu, T lp, T rr, T ru, T rp,
+                                                   bool has_eq) {
+  return pert_general<T, P>(g, W0, lr, lu, lp, rr, ru, rp, has_eq);
 }
 
 template <class T>
@@ -452,7 +459,8 @@ __device__ __forceinline__ void face_prim(T gm1, T v0, const T* q, T ir, T* w) {
 // equilibrium Em, from the primitive perturbations wl, wm of its left and right
 // states; wave_at(): the face's place in the table of wave speeds.  Returns
 // whether the face needs the general solver; with GENERAL = false F is then
-// left as it is.
+// left as it is.  In float GENERAL = true takes the general solver at once: its
+// faces are those that the other one has left.
 template <class T, int D, class P, bool GENERAL, class W>
 __device__ __forceinline__ bool pert_face(const PertArgs<T>& a, const PEq<T>& Em, T area, const T* wl, const T* wm,
                                           W&& wave_at, T* F, unsigned& status, unsigned& nfallback) {
@@ -462,7 +470,7 @@ __device__ __forceinline__ bool pert_face(const PertArgs<T>& a, const PEq<T>& Em
   const T rl = Em.rho + wl[RHO], pl = Em.p + wl[EN], rr = Em.rho + wm[RHO], pr = Em.p + wm[EN];
   NearStar<T> st;
   int kind = NEAR_GENERAL;
-  if (sizeof(T) == 4 || (positive(rl) && positive(rr) && positive(pl) && positive(pr)))
+  if (sizeof(T) == 4 ? !GENERAL : positive(rl) && positive(rr) && positive(pl) && positive(pr))
     kind = near_riemann<NEAR_DEPARTURES>(g.near, rl, wl[n], pl, rr, wm[n], pr, wm[EN] - wl[EN], wm[n] - wl[n], un0, D == 1,
                            un0 + wl[n], un0 + wm[n], st);
   if (!GENERAL && kind == NEAR_GENERAL) return true;
@@ -484,7 +492,8 @@ __device__ __forceinline__ bool pert_face(const PertArgs<T>& a, const PEq<T>& Em
       W0.un_mc = wv[1];
       W0.un_pc = wv[2];
     }
-    const PStar<T> o = pert_general<T, P>(a.gam, W0, wl[RHO], wl[n], wl[EN], wm[RHO], wm[n], wm[EN], g.has_eq != 0);
+    constexpr auto solve = sizeof(T) == 4 ? pert_general<T, P> : pert_general_call<T, P>;
+    const PStar<T> o = solve(a.gam, W0, wl[RHO], wl[n], wl[EN], wm[RHO], wm[n], wm[EN], g.has_eq != 0);
     status |= o.status;
     nfallback += o.fallback;
     ok = !(o.status & STATUS_NONPHYSICAL);
