@@ -4,7 +4,15 @@
 // limiter branches, the wave pattern and sampling of the exact Riemann
 // solution, the dust upwinding and the positivity fallback are held at the
 // branch the forward values take; the star pressure's derivative follows from
-// the implicit function theorem at the converged p*.  For one stage
+// the implicit function theorem at the converged p*.  Where rounding alone decides
+// a branch, both sides' derivatives belong to the same forward value.  Conservative
+// departures take the forward's own expressions there too.  With primitive ones
+// such states are usual (the pressure departure of an isobaric one, the velocities
+// of a wall's face beside an equilibrium ghost); their branches come from
+// expressions of the adjoint's own, slope_branches and for contacts at rest
+// riemann_jac, which do not move when the forward is arranged for speed, so that
+// the side taken there may be the other one than in the forward's rounding.  For
+// one stage
 //     Y = E_base + tau (G(E_in) - R0) / V,    E_out = D(Y)   (drag),
 // a cotangent lambda_out on E_out gives mu = D'(Y)^T lambda_out on Y and on
 // E_base, the weighted cotangent mu' = tau / V mu on G, and

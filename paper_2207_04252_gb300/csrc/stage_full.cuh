@@ -117,9 +117,10 @@ __device__ __forceinline__ unsigned parabola_branches(double em, double e0, doub
 
 // parabola_branches on slopes: s the minmod slope, the parabola's face deviation
 // against s times the limiter's reach.  v = {1/(x0-xm), 1/(xp-x0), 1/(xp-xm),
-// x0-xm, xp-x0, fm-x0, fp-x0, -h-, h+}.  For the adjoint of the primitive option,
-// see cell_prim_rounded: neither its branches nor the rounding of its face values
-// may depend on how the weights are arranged for speed.  (Beside an equilibrium
+// x0-xm, xp-x0, fm-x0, fp-x0, -h-, h+}.  For the adjoint of the primitive option
+// only (the forward takes parabola(), equal to rounding), see cell_prim_rounded:
+// neither its branches nor the rounding of its face values may depend on how the
+// forward's weights are arranged for speed.  (Beside an equilibrium
 // ghost the limited velocity of a wall's face is e0 - e0, whose rounding decides
 // which side of the contact the face takes.)
 __device__ __forceinline__ double slope_minmod(double a, double b) {
