@@ -10,7 +10,7 @@
 // such states are usual (the pressure departure of an isobaric one, the velocities
 // of a wall's face beside an equilibrium ghost); their branches come from
 // expressions of the adjoint's own, slope_branches and for contacts at rest
-// riemann_jac, which do not move when the forward is arranged for speed, so that
+// riemann_vjp_general, which do not move when the forward is arranged for speed, so that
 // the side taken there may be the other one than in the forward's rounding.  For
 // one stage
 //     Y = E_base + tau (G(E_in) - R0) / V,    E_out = D(Y)   (drag),
@@ -43,286 +43,7 @@
 
 namespace rossbi {
 
-// ------------------------------------------------------------------ forward-mode number, 6 tangents
-// Tangents with respect to the primitive face states (rho_L, u_L, p_L, rho_R, u_R, p_R).
-struct J6 {
-  double v;
-  double d[6];
-};
-
-__device__ __forceinline__ J6 jc(double v) {
-  J6 r;
-  r.v = v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = 0.0;
-  return r;
-}
-__device__ __forceinline__ J6 jv(double v, int k) {
-  J6 r = jc(v);
-  r.d[k] = 1.0;
-  return r;
-}
-__device__ __forceinline__ J6 operator+(const J6& a, const J6& b) {
-  J6 r;
-  r.v = a.v + b.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = a.d[q] + b.d[q];
-  return r;
-}
-__device__ __forceinline__ J6 operator-(const J6& a, const J6& b) {
-  J6 r;
-  r.v = a.v - b.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = a.d[q] - b.d[q];
-  return r;
-}
-__device__ __forceinline__ J6 operator*(const J6& a, const J6& b) {
-  J6 r;
-  r.v = a.v * b.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = a.d[q] * b.v + a.v * b.d[q];
-  return r;
-}
-__device__ __forceinline__ J6 operator/(const J6& a, const J6& b) {
-  J6 r;
-  r.v = a.v / b.v;
-  const double ib = 1.0 / b.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = (a.d[q] - r.v * b.d[q]) * ib;
-  return r;
-}
-__device__ __forceinline__ J6 operator+(const J6& a, double b) {
-  J6 r = a;
-  r.v = a.v + b;
-  return r;
-}
-__device__ __forceinline__ J6 operator-(const J6& a, double b) {
-  J6 r = a;
-  r.v = a.v - b;
-  return r;
-}
-__device__ __forceinline__ J6 operator*(const J6& a, double b) {
-  J6 r;
-  r.v = a.v * b;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = a.d[q] * b;
-  return r;
-}
-__device__ __forceinline__ J6 operator*(double a, const J6& b) {
-  J6 r;
-  r.v = a * b.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = a * b.d[q];
-  return r;
-}
-__device__ __forceinline__ J6 operator/(const J6& a, double b) {
-  J6 r;
-  r.v = a.v / b;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = a.d[q] / b;
-  return r;
-}
-__device__ __forceinline__ J6 operator/(double a, const J6& b) {
-  J6 r;
-  r.v = a / b.v;
-  const double s = -r.v / b.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = s * b.d[q];
-  return r;
-}
-__device__ __forceinline__ J6 jsqrt(const J6& a) {
-  J6 r;
-  r.v = sqrt(a.v);
-  const double s = 0.5 / r.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = s * a.d[q];
-  return r;
-}
-__device__ __forceinline__ J6 jpow(const J6& a, double e) {
-  J6 r;
-  r.v = pow(a.v, e);
-  const double s = e * r.v / a.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = s * a.d[q];
-  return r;
-}
-
-// a^e with its value v given (computed elsewhere, e.g. as a polynomial).
-__device__ __forceinline__ J6 jpow_v(const J6& a, double e, double v) {
-  J6 r;
-  r.v = v;
-  const double s = e * v / a.v;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) r.d[q] = s * a.d[q];
-  return r;
-}
-
-// ------------------------------------------------------------------ Riemann solution and its Jacobian
-struct JSide {
-  J6 rho, u, p, c;
-};
-
-// f_K(p) at a fixed p (its tangent: the partials in the side's state) and the
-// value of df_K/dp; the value arithmetic is that of pressure_fn.
-// G75 (gamma = 7/5): zK = (p / p_K)^(1/7) is given.
-template <bool G75>
-__device__ __forceinline__ void pressure_fn_jac(double g, const JSide& K, double p, J6& f, double& fd, double zK) {
-  if (p <= K.p.v) {
-    const J6 prat = jc(p) / K.p;
-    const J6 e = G75 ? jpow_v(prat, 1.0 / 7.0, zK) : jpow(prat, (g - 1.0) / (2.0 * g));
-    f = 2.0 * K.c / (g - 1.0) * (e - 1.0);
-    fd = e.v / (prat.v * K.rho.v * K.c.v);
-  } else {
-    const J6 A = 2.0 / ((g + 1.0) * K.rho);
-    const J6 B = (g - 1.0) / (g + 1.0) * K.p;
-    const J6 q = jsqrt(A / (B + p));
-    f = (jc(p) - K.p) * q;
-    fd = (1.0 - 0.5 * (p - K.p.v) / (B.v + p)) * q.v;
-  }
-}
-
-template <bool G75>
-__device__ __forceinline__ void fan_jac(double g, const JSide& K, double sgn, J6& rho, J6& u, J6& p) {
-  const J6 cf = 2.0 / (g + 1.0) * (K.c + sgn * 0.5 * (g - 1.0) * K.u);
-  u = sgn * cf;
-  const J6 ratio = cf / K.c;
-  if (G75) {  // exponents 5 and 7
-    const double r = ratio.v, r2 = r * r, r5 = r2 * r2 * r;
-    rho = K.rho * jpow_v(ratio, 5.0, r5);
-    p = K.p * jpow_v(ratio, 7.0, r5 * r2);
-  } else {
-    rho = K.rho * jpow(ratio, 2.0 / (g - 1.0));
-    p = K.p * jpow(ratio, 2.0 * g / (g - 1.0));
-  }
-}
-
-// The face state of riemann_face (riemann_face_g75 for G75) together with its
-// Jacobian in the six primitive inputs.  Branch decisions are taken on the
-// same values; for gamma = 7/5 the powers come from z = (p/p_L)^(1/7) as in
-// the forward solver.
-template <bool G75>
-__device__ __noinline__ int riemann_jac(double g, double rl, double ul, double pl, double rr, double ur, double pr,
-                                        J6& rho, J6& u, J6& p, unsigned& status) {
-  const JSide L{jv(rl, 0), jv(ul, 1), jv(pl, 2), jsqrt(g * jv(pl, 2) / jv(rl, 0))};
-  const JSide R{jv(rr, 3), jv(ur, 4), jv(pr, 5), jsqrt(g * jv(pr, 5) / jv(rr, 3))};
-  const double cl = L.c.v, cr = R.c.v;
-  if (2.0 / (g - 1.0) * (cl + cr) <= ur - ul) {  // vacuum
-    const double sl_star = ul + 2.0 * cl / (g - 1.0);
-    const double sr_star = ur - 2.0 * cr / (g - 1.0);
-    if (0.0 <= sl_star) {
-      if (0.0 <= ul - cl) { rho = L.rho; u = L.u; p = L.p; }
-      else fan_jac<G75>(g, L, 1.0, rho, u, p);
-      return -1;
-    }
-    if (0.0 >= sr_star) {
-      if (0.0 >= ur + cr) { rho = R.rho; u = R.u; p = R.p; }
-      else fan_jac<G75>(g, R, -1.0, rho, u, p);
-      return 1;
-    }
-    rho = u = p = jc(0.0);
-    return 0;
-  }
-  // Newton on the star pressure, values only (same arithmetic as the forward)
-  const RSide Lv{rl, ul, pl, cl}, Rv{rr, ur, pr, cr};
-  const double pfloor = 1e-8 * fmin(pl, pr);
-  double ps = fmax(pfloor, 0.5 * (pl + pr) - 0.125 * (ur - ul) * (rl + rr) * (cl + cr));
-  bool conv = false;
-  double zl = 0.0, zr = 0.0;
-  if (G75) {
-    const double k = root7(pl / pr);
-    double z = root7(ps / pl);
-    double fl, fdl, fr, fdr, step;
-    conv = newton_z_g75(Lv, Rv, ur - ul, pfloor, k, ps, z, fl, fdl, fr, fdr, step);  // the forward's iteration
-    zl = z;
-    zr = z * k;
-  } else {
-    for (int it = 0; it < 100; ++it) {
-      double fl, fdl, fr, fdr;
-      pressure_fn(g, Lv, ps, fl, fdl);
-      pressure_fn(g, Rv, ps, fr, fdr);
-      const double pn = fmax(pfloor, ps - (fl + fr + ur - ul) / (fdl + fdr));
-      const double change = 2.0 * fabs(pn - ps) / (pn + ps);
-      ps = pn;
-      if (change <= 1e-12) { conv = true; break; }
-    }
-  }
-  if (!conv) status |= STATUS_RIEMANN;
-  // implicit function theorem: f_L(p*) + f_R(p*) + u_R - u_L = 0
-  J6 FL, FR;
-  double dl, dr;
-  pressure_fn_jac<G75>(g, L, ps, FL, dl, zl);
-  pressure_fn_jac<G75>(g, R, ps, FR, dr, zr);
-  J6 PS = jc(ps);
-  if (ps == pfloor) {
-    PS = 1e-8 * (pl <= pr ? L.p : R.p);
-  } else {
-    const double iD = -1.0 / (dl + dr);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) PS.d[q] = (FL.d[q] + FR.d[q] + R.u.d[q] - L.u.d[q]) * iD;
-  }
-#pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    FL.d[q] += dl * PS.d[q];
-    FR.d[q] += dr * PS.d[q];
-  }
-  const J6 US = 0.5 * (L.u + R.u) + 0.5 * (FR - FL);
-  if (0.0 <= US.v) {
-    if (ps <= pl) {
-      if (0.0 <= ul - cl) { rho = L.rho; u = L.u; p = L.p; return -1; }
-      const J6 ratio = PS / L.p;
-      if (0.0 > US.v - cl * (G75 ? zl : pow(ratio.v, (g - 1.0) / (2.0 * g)))) {
-        if (G75) {
-          const double z2 = zl * zl;
-          rho = L.rho * jpow_v(ratio, 5.0 / 7.0, z2 * z2 * zl);
-        } else {
-          rho = L.rho * jpow(ratio, 1.0 / g);
-        }
-        u = US; p = PS; return -1;
-      }
-      fan_jac<G75>(g, L, 1.0, rho, u, p);
-      return -1;
-    }
-    const J6 ratio = PS / L.p;
-    if (0.0 <= ul - cl * sqrt((g + 1.0) / (2.0 * g) * ratio.v + (g - 1.0) / (2.0 * g))) {
-      rho = L.rho; u = L.u; p = L.p; return -1;
-    }
-    const double g6 = (g - 1.0) / (g + 1.0);
-    rho = L.rho * (ratio + g6) / (ratio * g6 + 1.0); u = US; p = PS;
-    return -1;
-  }
-  if (ps > pr) {
-    const J6 ratio = PS / R.p;
-    if (0.0 >= ur + cr * sqrt((g + 1.0) / (2.0 * g) * ratio.v + (g - 1.0) / (2.0 * g))) {
-      rho = R.rho; u = R.u; p = R.p; return 1;
-    }
-    const double g6 = (g - 1.0) / (g + 1.0);
-    rho = R.rho * (ratio + g6) / (ratio * g6 + 1.0); u = US; p = PS;
-    return 1;
-  }
-  if (0.0 >= ur + cr) { rho = R.rho; u = R.u; p = R.p; return 1; }
-  const J6 ratio = PS / R.p;
-  if (0.0 <= US.v + cr * (G75 ? zr : pow(ratio.v, (g - 1.0) / (2.0 * g)))) {
-    if (G75) {
-      const double z2 = zr * zr;
-      rho = R.rho * jpow_v(ratio, 5.0 / 7.0, z2 * z2 * zr);
-    } else {
-      rho = R.rho * jpow(ratio, 1.0 / g);
-    }
-    u = US; p = PS; return 1;
-  }
-  fan_jac<G75>(g, R, -1.0, rho, u, p);
-  return 1;
-}
-
 // ------------------------------------------------------------------ face flux adjoints
-// Cotangents (rho, u, p)_L, (rho, u, p)_R of the Riemann solution for the
-// cotangents (rb, ub, pb) of the face state, by the six-tangent Jacobian, and
-// the side; out of line, by value: the faces that near_riemann hands back.
-struct RFaceVjp {
-  double rho, u, p, b[6];
-  int side;
-  unsigned status;
-};
 struct FluxCot {  // cotangent of the flux in face order: mass, normal and transverse momenta, energy
   double m, n, t1, t2, e;
 };
@@ -340,23 +61,162 @@ __device__ __forceinline__ void flux_state_vjp(double g_gm1, double rho, double 
   ut1b = fma(F.t1, m, Fm * ut1);
   ut2b = fma(F.t2, m, Fm * ut2);
 }
-static __device__ __noinline__ RFaceVjp riemann_vjp_general(double g, double rl, double ul, double pl, double l1,
-                                                            double l2, double rr, double ur, double pr, double r1,
-                                                            double r2, const FluxCot F) {
-  RFaceVjp o;
-  o.status = 0;
-  J6 Rs, Us, Ps;
-  o.side = g == 1.4 ? riemann_jac<true>(g, rl, ul, pl, rr, ur, pr, Rs, Us, Ps, o.status)
-                    : riemann_jac<false>(g, rl, ul, pl, rr, ur, pr, Rs, Us, Ps, o.status);
-  o.rho = Rs.v;
-  o.u = Us.v;
-  o.p = Ps.v;
+
+// f_K and df_K/dp at the star pressure; for gamma = 7/5 zK = (p / p_K)^(1/7) is given.
+template <bool G75>
+__device__ __forceinline__ void pressure_fn_at(double g, const RSide& K, double p, double zK, double& f, double& fd) {
+  if (p <= K.p) {
+    const double prat = p / K.p;
+    const double e = G75 ? zK : pow(prat, (g - 1.0) / (2.0 * g));
+    f = 2.0 * K.c / (g - 1.0) * (e - 1.0);
+    fd = e / (prat * K.rho * K.c);
+  } else {
+    const double A = 2.0 / ((g + 1.0) * K.rho);
+    const double B = (g - 1.0) / (g + 1.0) * K.p;
+    const double q = sqrt(A / (B + p));
+    f = (p - K.p) * q;
+    fd = (1.0 - 0.5 * (p - K.p) / (B + p)) * q;
+  }
+}
+
+// The general Riemann solution of a face (riemann_face) with its reverse: the
+// face's mass flux, the side whose transverse velocity it carries, and the
+// cotangents b of (rho, u, p)_L and (rho, u, p)_R for the cotangent F of the flux;
+// l1, l2, r1, r2 the transverse velocities.  The wave pattern picks one of four
+// closed forms in the side K that the face lies on (its own state, a fan, the star
+// state behind a rarefaction or a shock); f_K enters by df_K/drho_K = -f_K / (2
+// rho_K) and p* f_K' + p_K df_K/dp_K = f_K / 2, as in gas_flux_vjp.  An adjoint step
+// of 140 x 96 x 36 cells with jumps of 3 % at all faces takes 19.6 ms; six tangents
+// carried through the solution took 26.9 (21.2 in a kernel of 255 registers without
+// the near solution).
+struct RFaceVjp {
+  double m, b[6];
+  int side;
+  unsigned status;
+};
+template <bool G75>
+__device__ __forceinline__ RFaceVjp riemann_vjp(double g, double g_gm1, const RSide& L, const RSide& R, double l1,
+                                                double l2, double r1, double r2, const FluxCot& F) {
+  enum { OWN, FAN, RAREFACTION, SHOCK };
+  RFaceVjp o{};
+  int what = OWN;
+  double ps = 0.0, us = 0.0, fl = 0.0, fdl = 0.0, fr = 0.0, fdr = 0.0, zl = 0.0, zr = 0.0;
+  const double pfloor = 1e-8 * fmin(L.p, R.p), t = 2.0 * (g_gm1 - 1.0);  // 2 / (gamma - 1)
+  if (t * (L.c + R.c) <= R.u - L.u) {  // vacuum
+    if (0.0 <= L.u + t * L.c) {
+      o.side = -1;
+      what = 0.0 <= L.u - L.c ? OWN : FAN;
+    } else if (0.0 >= R.u - t * R.c) {
+      o.side = 1;
+      what = 0.0 >= R.u + R.c ? OWN : FAN;
+    } else {
+      return o;
+    }
+  } else {
+    ps = fmax(pfloor, 0.5 * (L.p + R.p) - 0.125 * (R.u - L.u) * (L.rho + R.rho) * (L.c + R.c));
+    bool conv = false;
+    if (G75) {
+      const double k = root7(L.p / R.p);
+      double z = root7(ps / L.p), step;
+      conv = newton_z_g75(L, R, R.u - L.u, pfloor, k, ps, z, fl, fdl, fr, fdr, step);  // the forward's iteration
+      zl = z;
+      zr = z * k;
+    } else {
+      for (int it = 0; it < 100; ++it) {
+        pressure_fn(g, L, ps, fl, fdl);
+        pressure_fn(g, R, ps, fr, fdr);
+        const double pn = fmax(pfloor, ps - (fl + fr + R.u - L.u) / (fdl + fdr));
+        const double change = 2.0 * fabs(pn - ps) / (pn + ps);
+        ps = pn;
+        if (change <= 1e-12) {
+          conv = true;
+          break;
+        }
+      }
+    }
+    if (!conv) o.status = STATUS_RIEMANN;
+    pressure_fn_at<G75>(g, L, ps, zl, fl, fdl);
+    pressure_fn_at<G75>(g, R, ps, zr, fr, fdr);
+    us = 0.5 * (L.u + R.u) + 0.5 * (fr - fl);
+    o.side = 0.0 <= us ? -1 : 1;
+    // the same on either side with the axis turned round: v towards the face
+    const RSide& K = o.side < 0 ? L : R;
+    const double sgn = o.side < 0 ? 1.0 : -1.0, v = sgn * K.u, ratio = ps / K.p;
+    if (ps > K.p) {
+      what = 0.0 <= v - K.c * sqrt((g + 1.0) / (2.0 * g) * ratio + (g - 1.0) / (2.0 * g)) ? OWN : SHOCK;
+    } else if (0.0 <= v - K.c) {
+      what = OWN;
+    } else {
+      const double tail = sgn * us - K.c * (G75 ? (o.side < 0 ? zl : zr) : pow(ratio, (g - 1.0) / (2.0 * g)));
+      what = (o.side < 0 ? 0.0 > tail : 0.0 >= tail) ? RAREFACTION : FAN;
+    }
+  }
+  const bool left = o.side < 0;
+  const RSide K = left ? L : R;
+  const double sgn = left ? 1.0 : -1.0, ipk = recip(K.p);
+  double rho = K.rho, u = K.u, p = K.p, h = 1.0, dh = 0.0, cf = 0.0;  // h(x) = rho* / rho_K, x = p* / p_K
+  if (what == FAN) {
+    cf = 2.0 / (g + 1.0) * (K.c + sgn * 0.5 * (g - 1.0) * K.u);
+    const double r = cf / K.c;
+    u = sgn * cf;
+    rho *= G75 ? r * r * (r * r) * r : pow(r, 2.0 / (g - 1.0));
+    p *= G75 ? r * r * (r * r) * (r * r * r) : pow(r, 2.0 * g / (g - 1.0));
+  } else if (what != OWN) {
+    const double x = ps * ipk, g6 = (g - 1.0) / (g + 1.0);
+    u = us;
+    p = ps;
+    if (what == RAREFACTION) {
+      const double z = left ? zl : zr;
+      h = G75 ? z * z * (z * z) * z : pow(x, 1.0 / g);
+      dh = h * recip(g * x);
+    } else {
+      const double i = recip(x * g6 + 1.0);
+      h = (x + g6) * i;
+      dh = (1.0 - g6 * g6) * i * i;
+    }
+    rho *= h;
+  }
   double rb, ub, pb, t1b, t2b;
-  const double ut1 = o.side < 0 ? l1 : (o.side > 0 ? r1 : 0.0), ut2 = o.side < 0 ? l2 : (o.side > 0 ? r2 : 0.0);
-  flux_state_vjp(g / (g - 1.0), o.rho, o.u, o.p, ut1, ut2, F, rb, ub, pb, t1b, t2b);
-#pragma unroll
-  for (int q = 0; q < 6; ++q) o.b[q] = rb * Rs.d[q] + ub * Us.d[q] + pb * Ps.d[q];
+  flux_state_vjp(g_gm1, rho, u, p, left ? l1 : r1, left ? l2 : r2, F, rb, ub, pb, t1b, t2b);
+  o.m = rho * u;
+  double kr = rb, ku = ub, kp = pb;  // cotangents of K
+  double* b = o.b;
+  if (what == FAN) {
+    const double q = 2.0 / (g - 1.0) * (rb * rho + g * (pb * p));  // cotangent of log(cf / c)
+    const double cfb = sgn * ub + q / cf, cb = 2.0 / (g + 1.0) * cfb - q / K.c;
+    ku = cfb * (sgn * (g - 1.0) / (g + 1.0));
+    kr = (rb * rho - 0.5 * cb * K.c) / K.rho;
+    kp = (pb * p + 0.5 * cb * K.c) * ipk;
+  } else if (what != OWN) {
+    const double hb = rb * K.rho * dh * ipk, gu = 0.5 * ub;
+    const double psb = pb + hb + gu * (fdr - fdl);
+    kr = rb * h;
+    ku = 0.0;
+    kp = -hb * (ps * ipk);
+    const bool floor = ps == pfloor;
+    const double lam = floor ? 0.0 : -psb * recip(fdl + fdr), pm = floor ? 1e-8 * psb : 0.0;
+    const double flb = lam - gu, frb = lam + gu;
+    b[0] = -0.5 * flb * fl * recip(L.rho);
+    b[1] = gu - lam;
+    b[2] = flb * (0.5 * fl - ps * fdl) * recip(L.p) + (L.p <= R.p ? pm : 0.0);
+    b[3] = -0.5 * frb * fr * recip(R.rho);
+    b[4] = gu + lam;
+    b[5] = frb * (0.5 * fr - ps * fdr) * recip(R.p) + (L.p <= R.p ? 0.0 : pm);
+  }
+  b[0] += left ? kr : 0.0;
+  b[1] += left ? ku : 0.0;
+  b[2] += left ? kp : 0.0;
+  b[3] += left ? 0.0 : kr;
+  b[4] += left ? 0.0 : ku;
+  b[5] += left ? 0.0 : kp;
   return o;
+}
+static __device__ __noinline__ RFaceVjp riemann_vjp_general(double g, double g_gm1, double rl, double ul, double pl,
+                                                            double l1, double l2, double rr, double ur, double pr,
+                                                            double r1, double r2, const FluxCot F) {
+  const RSide L{rl, ul, pl, sqrt(g * pl / rl)}, R{rr, ur, pr, sqrt(g * pr / rr)};
+  return g == 1.4 ? riemann_vjp<true>(g, g_gm1, L, R, l1, l2, r1, r2, F)
+                  : riemann_vjp<false>(g, g_gm1, L, R, l1, l2, r1, r2, F);
 }
 
 // Cotangents of the primitive face states (u, v, w, P, rho in the field
@@ -390,7 +250,8 @@ __device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL
       fabsf(narrow(s.us)) <= 1e-14f * narrow(C.gamma * (pl * s.ircl)))
     kind = NEAR_GENERAL;
   if (kind == NEAR_GENERAL) {
-    const RFaceVjp o = riemann_vjp_general(C.gamma, rl, WL[n], pl, WL[t1], WL[t2], rr, WR[n], pr, WR[t1], WR[t2], F);
+    const RFaceVjp o =
+        riemann_vjp_general(C.gamma, C.g_gm1, rl, WL[n], pl, WL[t1], WL[t2], rr, WR[n], pr, WR[t1], WR[t2], F);
     status |= o.status;
     WLb[RHO] = o.b[0];
     WLb[n] = o.b[1];
@@ -398,7 +259,7 @@ __device__ __forceinline__ void gas_flux_vjp(const NearCoef& C, const double* WL
     WRb[RHO] = o.b[3];
     WRb[n] = o.b[4];
     WRb[EN] = o.b[5];
-    const double m = o.rho * o.u, Fm = F.e * m;
+    const double m = o.m, Fm = F.e * m;
     if (o.side < 0) {
       WLb[t1] = F.t1 * m + Fm * WL[t1];
       WLb[t2] = F.t2 * m + Fm * WL[t2];
