@@ -153,7 +153,7 @@ __device__ __forceinline__ double refine_recip_sqrt(double x, double y) {
 }
 // sqrt(x) of any x.  Squares of slow velocities underflow, so subnormal
 // arguments are ordinary ones here, and the approximation flushes them to an
-// infinite x^-1/2; the float form is the hardware's root of every value.
+// infinite x^-1/2.
 __device__ __forceinline__ double root(double x) {
   if (!positive_normal(x)) return sqrt(x);
   double y;
@@ -164,7 +164,7 @@ __device__ __forceinline__ double root(double x) {
 __device__ __forceinline__ float root(float x) {
   float y;
   asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
+  return x >= 0x1p-126f && x <= 0x1.fffffep127f ? x * recip_sqrt(x) : y;
 }
 
 // ---------------------------------------------------------------- two floats at a time (the packed arithmetic of sm_100 and later)
