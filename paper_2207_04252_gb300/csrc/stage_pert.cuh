@@ -660,13 +660,13 @@ __device__ __forceinline__ void pert_sources(const PertArgs<T>& a, const PCell<T
 
 // 1 / t_s of dust species s in a perturbation-form cell (as inv_stopping_time
 // of the full-state kernel; gas density rg, ig = 1 / rg, pressure p).
-template <class T, bool XT>
-__device__ __forceinline__ T pert_inv_stopping_time(const PertArgs<T>& a, int i, T rg, T ig, T p, int s) {
+template <class T, bool XT, class I>
+__device__ __forceinline__ T pert_inv_stopping_time(const PertArgs<T>& a, int i, T rg, T ig, T p, int s, I&& inverse) {
   if (a.drag.law == 0) return a.t.omk[i] * a.ist[s];
   T it = rg * root(a.gam * p * ig) * a.irr[s];
   if (XT && a.drag.law == 2) {  // Stokes regime of Sect. 2.9 above r_p = 9 lambda / 4
     const T x = a.kappa * rg;
-    if (positive(x - T(2.25))) it *= T(2.25) * recip(x);
+    if (positive(x - T(2.25))) it *= T(2.25) * inverse(x);
   }
   return it;
 }
@@ -676,10 +676,11 @@ __device__ __forceinline__ T pert_inv_stopping_time(const PertArgs<T>& a, int i,
 // velocity moves by D = sum rho_k w_k (v_k - v_g) / (rho_g + sum rho_k w_k)
 // and species k by w_k (D - (v_k - v_g)), w_k = a_k / (1 + a_k), every
 // quantity a difference of velocities, never the large u0 itself.
-// ig = 1 / rho_g, id = 1 / rho_d of each species (any value without mass).
-template <class T, int NF, bool XT>
+// ig = 1 / rho_g, id = 1 / rho_d of each species (any value without mass);
+// inverse(x): 1 / x.
+template <class T, int NF, bool XT, class I>
 __device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& c, int i, T* q, T tau, T ig,
-                                          const T* id) {
+                                          const T* id, I&& inverse) {
   const T rg = c.rho0 + q[RHO];
   if (!positive(rg)) return;
   const T m1 = q[MV] - q[RHO] * c.v0;
@@ -694,8 +695,8 @@ __device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& 
   if constexpr (NF == 9) {
     const T rd = q[DRHO];
     if (!has_mass(rd)) return;
-    const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, ig, p, 0);
-    const T K = rd * ak * recip(T(1) + ak * (T(1) + rd * ig));
+    const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, ig, p, 0, inverse);
+    const T K = rd * ak * inverse(T(1) + ak * (T(1) + rd * ig));
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const T vd = (q[DMU + k] - rd * u0[k]) * id[0];  // v_d - u0
@@ -713,13 +714,13 @@ __device__ __forceinline__ void pert_drag(const PertArgs<T>& a, const PCell<T>& 
       const T rd = q[b + 3];
       wk[s] = T(0);
       if (!has_mass(rd)) continue;
-      const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, ig, p, s);
-      wk[s] = ak * recip(T(1) + ak);
+      const T ak = tau * pert_inv_stopping_time<T, XT>(a, i, rg, ig, p, s, inverse);
+      wk[s] = ak * inverse(T(1) + ak);
       den += rd * wk[s];
 #pragma unroll
       for (int k = 0; k < 3; ++k) num[k] += rd * wk[s] * ((q[b + k] - rd * u0[k]) * id[s] - dug[k]);
     }
-    const T iden = recip(den);
+    const T iden = inverse(den);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const T D = num[k] * iden;  // v_g' - v_g
@@ -768,7 +769,7 @@ __device__ __forceinline__ T pert_cell_rate(const PertArgs<T>& a, const PCell<T>
 // dust and its flux divergence G, raising the thread's CFL rate.  XT: the
 // optional terms (indirect gravity, wave-killing zones) are compiled in; the
 // plain instantiation carries none of their code.  ce: the cell's equilibrium;
-// inverse(x): 1 / x, for the densities.
+// inverse(x): 1 / x.
 template <class T, int NF, int RC, bool XT, class I>
 __device__ __forceinline__ void pert_update(const PertArgs<T>& a, const PCell<T>& ce, int gi, int gj, int gk, const T* e,
                                             const T (*dust)[4], T* G, T tau, T& rate, unsigned& status, I&& inverse) {
@@ -807,7 +808,7 @@ __device__ __forceinline__ void pert_update(const PertArgs<T>& a, const PCell<T>
     E[b + 3] = dust_density(E[b + 3]);
     id[(b - 5) / 4] = inverse(E[b + 3]);
   }
-  if constexpr (NF > 5) pert_drag<T, NF, XT>(a, ce, gi, E, tau, ig, id);
+  if constexpr (NF > 5) pert_drag<T, NF, XT>(a, ce, gi, E, tau, ig, id, inverse);
 #pragma unroll
   for (int f = 0; f < NF; ++f) a.out[f][lin] = E[f];
   bool bad = false;
