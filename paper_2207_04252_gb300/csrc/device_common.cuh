@@ -22,7 +22,6 @@ enum { STATUS_NONPHYSICAL = 1u, STATUS_RIEMANN = 2u };
 // on the departures of the primitive variables (rho, u, v, w, P).
 enum { RECON_CONS = 0, RECON_PRIM = 1 };
 
-constexpr int GH = 2;   // ghost offset of the axis-0 coordinate tables
 constexpr int RCW = 8;  // parabola weights per axis-0 cell
 
 // Grid data the kernels read.  Passed by value as a kernel parameter; the
@@ -32,9 +31,7 @@ struct DevGrid {
   int recon;             // RECON_CONS or RECON_PRIM
   int bc_lo[3], bc_hi[3];
   double gamma, gm, omega, cfl;
-  double x0[3], dx[3];   // uniform axes 1, 2 (and axis 0 of the Box): origin, spacing
-  const double* rc;      // axis-0 cell centres,  index i + GH, i in [-GH, nr + GH)
-  const double* rf;      // axis-0 lower faces,   index i + GH, i in [-GH, nr + GH]
+  double dx[3];          // spacing of the uniform axes 1, 2 (and axis 0 of the Box)
   const double* rcoef;   // axis-0 parabola weights for cells i in [-1, nr]: RCW per cell at (i + 1) * RCW
   const double* rslope;  // axis-0 slopes and distances for slope_branches: 9 per cell at (i + 1) * 9
   const double* vol;     // V(i)

@@ -33,7 +33,9 @@ cudaError_t launch_nt(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
 // another's sweeps.  Four steps with dust, two narrow blocks against a wide one:
 // 152 tiles 223 / 165 us, 300 230 / 214, 456 308 / 281, 512 319 / 307, 600
 // 346 / 333 (without dust 281 / 288), 760 404 / 409, 912 436 / 484, 4800
-// 1808 / 2254; the line lies at three tiles per SM of 152.
+// 1808 / 2254: the lines cross between three and four tiles per SM of 152 without
+// dust and between four and five with it.  One rule at three for both: beyond it
+// the narrow blocks lose 4 % at most.
 template <int NF, class P, bool XT, int RC>
 cudaError_t launch(const PertArgs<float>& a, int nblocks, cudaStream_t s) {
   if constexpr (NF <= 9) {

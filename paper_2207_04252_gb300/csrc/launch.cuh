@@ -48,7 +48,7 @@ auto by_tile(int t, F&& f) {
 // in 32-lane chunks of its sweeps (60 for a main tile, whose sweeps have 18, 21
 // and 21), as the FP64 pipe, which bounds these kernels, takes chunks at one
 // rate.  Grids of some thousand main tiles keep the main tile; at 19 main
-// tiles (the Sod tube, 256 x 4 x 4) 15 % of the SMs had all the work: 240 us per
+// tiles (the Sod tube, 256 x 4 x 4) an eighth of the SMs had all the work: 240 us per
 // step against 92 with the small tile.  More than one dust species: the main
 // tile only (the others are not instantiated).
 template <class T>

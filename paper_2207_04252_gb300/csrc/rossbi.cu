@@ -35,7 +35,7 @@ struct rossbi_grid {
   bool has_disc = false;
   rossbi_disc_params disc{};
   // device tables
-  double *d_rc = nullptr, *d_rf = nullptr, *d_rcoef = nullptr, *d_rslope = nullptr, *d_vol = nullptr, *d_ivol = nullptr;
+  double *d_rcoef = nullptr, *d_rslope = nullptr, *d_vol = nullptr, *d_ivol = nullptr;
   double *d_area_r = nullptr, *d_area_t = nullptr, *d_area_z = nullptr, *d_aov = nullptr;
   double *d_ir = nullptr, *d_omk = nullptr, *d_grav = nullptr;
   double *d_e0c = nullptr, *d_e0r = nullptr, *d_e0z = nullptr, *d_r0 = nullptr;
@@ -1242,7 +1242,7 @@ int rossbi_precision(const rossbi_grid* g) { return g ? g->desc.precision : -1; 
 
 void rossbi_destroy(rossbi_grid* g) {
   if (!g) return;
-  double* tabs[] = {g->d_rc, g->d_rf, g->d_rcoef, g->d_rslope, g->d_vol, g->d_ivol, g->d_area_r, g->d_area_t,
+  double* tabs[] = {g->d_rcoef, g->d_rslope, g->d_vol, g->d_ivol, g->d_area_r, g->d_area_t,
                     g->d_area_z, g->d_aov, g->d_ir, g->d_omk, g->d_grav, g->d_e0c, g->d_e0r, g->d_e0z, g->d_r0, g->d_partials, g->d_sums};
   for (double* p : tabs)
     if (p) cudaFree(p);
@@ -1307,6 +1307,7 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   const int nr = d.nr;
   const double dy = (d.x1[1] - d.x0[1]) / d.nth;
   const double dz = (d.x1[2] - d.x0[2]) / d.nz;
+  constexpr int GH = 2;  // ghosts of the axis-0 coordinates
   std::vector<double> rc(nr + 2 * GH), rf(nr + 2 * GH + 1), rcoef((size_t)(nr + 2) * RCW, 0.0), rslope((size_t)(nr + 2) * 9);
   for (int i = -GH; i < nr + GH; ++i) rc[i + GH] = axis0_centre(d, i);
   for (int i = -GH; i <= nr + GH; ++i) rf[i + GH] = axis0_face(d, i);
@@ -1373,8 +1374,6 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   }
   rossbi_status st = ROSSBI_OK;
   do {
-    if ((st = upload(&g->d_rc, rc, g->stream)) != ROSSBI_OK) break;
-    if ((st = upload(&g->d_rf, rf, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_rcoef, rcoef, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_rslope, rslope, g->stream)) != ROSSBI_OK) break;
     if ((st = upload(&g->d_vol, vol, g->stream)) != ROSSBI_OK) break;
@@ -1409,15 +1408,12 @@ rossbi_status rossbi_init_grid(const rossbi_grid_desc* desc, void* cuda_stream, 
   for (int a = 0; a < 3; ++a) {
     dg.bc_lo[a] = d.bc_lo[a];
     dg.bc_hi[a] = d.bc_hi[a];
-    dg.x0[a] = d.x0[a];
     dg.dx[a] = (d.x1[a] - d.x0[a]) / (a == 0 ? d.nr : (a == 1 ? d.nth : d.nz));
   }
   dg.gamma = d.gamma;
   dg.gm = d.gm;
   dg.omega = d.geometry == ROSSBI_GEOM_CYL ? d.omega_frame : 0.0;
   dg.cfl = d.cfl;
-  dg.rc = g->d_rc;
-  dg.rf = g->d_rf;
   dg.rcoef = g->d_rcoef;
   dg.rslope = g->d_rslope;
   dg.vol = g->d_vol;
