@@ -1,10 +1,9 @@
 #!/usr/bin/env python
 """Throughput of the RoSSBi3D time step on GB300, in cell-updates/s.
 
-A step is one full midpoint-RK2 update (two fused stage launches plus the
-conservation-sum finalisation) of the whole grid of the synthetic workload,
-with the state resident in HBM and the CFL step kept on the device.  The
-state (2.4 GB in the default FP32 perturbation form, 4.8 GB in FP64, for the
+A step is one full midpoint-RK2 update (two fused stage launches) of the whole
+grid of the synthetic workload, with the state resident in HBM and the CFL step
+kept on the device.  The state (2.4 GB in the default FP32 perturbation form, 4.8 GB in FP64, for the
 512x1024x128 bi-fluid grid) is far larger than L2, so no flush is needed
 between steps.  The line also carries the FP64 form's throughput on the same
 grid, the FP32 form's relative L1 error against the FP64 form over the timed

@@ -36,7 +36,7 @@
 // two bi-fluid steps of 128 x 256 x 32 cells, most of 159 ms; with the closed
 // reverse of the near solution, the gas before the dust (168 registers, twelve
 // warps per SM) and lines by the axis (launch.cuh) the gradient takes 41 ms, a
-// third of it in the flux kernels (1.44, 0.94 and 1.50 ms a stage along r, theta
+// third of it in the flux kernels (1.40, 0.95 and 1.38 ms a stage along r, theta
 // and z), the rest in forward stages and the point kernels.
 #pragma once
 #include "stage_full.cuh"

@@ -144,7 +144,7 @@ __device__ __forceinline__ double near_sum(const double (&c)[2][NEAR_N], const f
 
 enum { NEAR_GENERAL = 0, NEAR_LEFT = 1, NEAR_RIGHT = 2, NEAR_STAR_L = 3, NEAR_STAR_R = 4 };
 
-enum { NEAR_STATE, NEAR_INVERSES, NEAR_DEPARTURES };
+enum { NEAR_STATE, NEAR_INVERSES, NEAR_DEPARTURES };  // what the solution is for, see above
 
 // What the solution needs beyond the face state (the adjoint reads it).
 template <class T>
@@ -161,9 +161,9 @@ struct NearStar {
 // side; s is set), or NEAR_GENERAL: not near, or within the sonic band where
 // a fan or a shock may sit on the face; the caller then takes the general
 // solver.  (rl, pl), (rr, pr): densities and pressures (a float state that is
-// not positive comes back as NEAR_GENERAL; a double one is the caller's to sort out); dP = p_R -
-// p_L, ul, ur velocities about u0, dU = u_R - u_L; vl, vr the full
-// velocities.
+// not positive comes back as NEAR_GENERAL; a double one is the caller's to sort
+// out); dP = p_R - p_L, ul, ur velocities about u0, dU = u_R - u_L; vl, vr the
+// full velocities; WHAT: one of the three above (the float solution has one way).
 template <int WHAT>
 __device__ __forceinline__ int near_riemann(const NearCoef& C, double rl, double ul, double pl, double rr, double ur,
                                             double pr, double dP, double dU, double u0, bool has_u0, double vl,

@@ -19,7 +19,7 @@
 //     is out of line, after the sweeps (redo).
 // A bi-fluid step of 512 x 1024 x 128 cells (12.1 GB that it cannot do without,
 // 1.8 ms of a copy's rate) took 28.9 ms with single-word staging and an FP32
-// Newton iteration on every face, and takes 12.8: 166 -> 69 warp instructions
+// Newton iteration on every face, and takes 12.8: 166 -> 73 warp instructions
 // per cell and stage.  A step of 256 x 512 x 64: 3.6 -> 1.55 ms.
 #pragma once
 #include "stage_pert.cuh"
